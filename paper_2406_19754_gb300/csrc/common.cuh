@@ -54,6 +54,32 @@ struct Arena {
 
 // ------------------------------------------------------------------ SELL
 
+// Column coding of one slice's index block (w ELL columns of 32 slots):
+//   IX_PLAIN   32 w int32 columns (128 w bytes)
+//   IX_DELTA   w int32 bases (padded to 16 bytes), then 32 w uint16: the column
+//              is base[k] + delta (about 68 w bytes)
+//   IX_OFFSET  w int32 offsets (padded to 16 bytes): the column of row i is
+//              i + offset[k]
+//   IX_CLAMP   the same, clamped into range (padding of boundary slices)
+// Every coding yields the columns of Sell::col, so a row's sum is the same
+// bits whichever a slice uses.
+// Slices wider than RING_MAX_WIDTH ELL columns do not fit a stage of the ring.
+constexpr int RING_MAX_WIDTH = 56;
+__host__ __device__ constexpr int ring_tile(int q) { return 8 >> q; }  // slices per tile, q = 0..2
+enum { IX_PLAIN = 0, IX_DELTA = 1, IX_OFFSET = 2, IX_CLAMP = 3 };
+
+// Start of slice s: first slot, and byte offset of its index block (a
+// multiple of 16) with the IX_* code in the low two bits.
+struct alignas(16) SliceRec {
+  int64_t slot;
+  int64_t ix;
+};
+
+__host__ __device__ inline int64_t ix_bytes(int mode, int64_t w) {
+  const int64_t head = (4 * w + 15) & ~(int64_t)15;
+  return mode >= IX_OFFSET ? head : mode == IX_DELTA ? head + 64 * w : 128 * w;
+}
+
 // Sliced ELLPACK (Sec. 2.2, "Hacked ELLPACK"): rows in slices of C rows,
 // each slice an ELLPACK block of width = its longest row, stored column
 // major (entry k of row r of slice s at sliceptr[s] + k * C + r).  Padding
@@ -62,7 +88,7 @@ struct Arena {
 // [row0[s], row0[s+1]) (at most C rows) and belongs to system sys[s].
 // Without systems row0/sys are null and slice s covers rows [s*C, s*C + C).
 struct Sell {
-  int64_t n = 0, nslices = 0, nnz_pad = 0;
+  int64_t n = 0, ncols = 0, nslices = 0, nnz_pad = 0;
   int C = 32, tpr = 1;
   int wmax = 0;  // widest slice (ELL columns)
   int64_t* sliceptr = nullptr;
@@ -78,6 +104,14 @@ struct Sell {
   // The kernels stream d16 (2 bytes a slot) instead of col (4 bytes).
   uint16_t* d16 = nullptr;
   int32_t* kbase = nullptr;
+  // Packed column indices of the shared-memory ring streams (ring.cuh; null
+  // when the matrix is not built for them): rec[s] says where slice s's
+  // values and index block start and how the block is coded.
+  // ring_tile(q) consecutive slices hold at most tile_w[q] ELL columns and
+  // tile_ix[q] index bytes.
+  SliceRec* rec = nullptr;
+  unsigned char* ix = nullptr;
+  int tile_w[3] = {}, tile_ix[3] = {};
 };
 
 template <typename V>
@@ -95,6 +129,9 @@ struct SellView {
   const int32_t* sys;
   const uint16_t* d16;   // compressed columns, or null
   const int32_t* kbase;
+  const SliceRec* rec;   // packed indices of the ring streams, or null
+  const unsigned char* ix;
+  int32_t ncols;
   const int* act;        // batched PCG: per-system "still iterating" flags, or null
   // false for a slice of a system whose solve has stopped (its results are
   // not used), so the kernels skip it
@@ -514,10 +551,12 @@ int scan_exclusive_i32(Arena& ar, const int32_t* in, int32_t* out, int64_t n, in
 int scan_exclusive_i64(Arena& ar, const int64_t* in, int64_t* out, int64_t n, int64_t* total,
                        cudaStream_t s);
 
-// SELL conversion (sell.cu)
+// SELL conversion (sell.cu).  ring: also pack the column indices for the
+// shared-memory ring streams (slice height 32, one thread per row).
 int sell_from_csr(Arena& ar, int64_t n, int64_t ncols, const int64_t* rowptr, const int32_t* col,
                   const double* val, int C, int tpr, Sell& out, cudaStream_t s,
-                  const std::vector<int64_t>* sys_off = nullptr, bool compress = true);
+                  const std::vector<int64_t>* sys_off = nullptr, bool compress = true,
+                  bool ring = false);
 int sell_make_copies(Arena& ar, Sell& A, int vstore, cudaStream_t s);
 // Builds A.d16 / A.kbase from A.col (left null when a slice's column offsets
 // exceed 16 bits).  Synchronous.

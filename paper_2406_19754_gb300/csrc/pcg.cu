@@ -97,30 +97,33 @@ __global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
 
 // k_spmv_dot on the shared-memory ring of ring.cuh (one system, one thread
 // per row): the same row sums; (p, q) per thread over the warp's slices.
-__global__ void __launch_bounds__(RING_THREADS, 4)
-    k_spmv_dot_ring(SellView<double> A, const double* __restrict__ p, double* __restrict__ q,
-                    Reduce red, PcgScalars* sc, RingGeom g, RingRows rows, int* fail) {
+__global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
+    k_spmv_dot_ring(const __grid_constant__ SellView<double> A, const double* __restrict__ p,
+                    double* __restrict__ q, Reduce red, PcgScalars* sc,
+                    const __grid_constant__ RingGeom g, const __grid_constant__ RingRows rows,
+                    int* fail) {
   extern __shared__ unsigned char ring_smem[];
   if (*(volatile int*)fail) return;  // the host resets the reduction ticket
   double d[1] = {0.0};
-  RingWarp<double> ring(A, g, rows, ring_smem);
-  ring.start();
-  for (int64_t sl = ring.first; sl < A.nslices; sl += ring.nwt) {
-    const int64_t i = sl * 32 + ring.lane;
-    const bool has = i < A.n;
-    const double pi = has ? __ldg(p + i) : 0.0;  // overlaps the wait
-    if (!ring.wait()) {
-      if (ring.lane == 0) ring_fail(fail, &sc->status);
-      ring.drain();
-      break;
+  TileRing<double> ring(A, g, rows, ring_smem);
+  if (ring.producer()) {
+    ring.produce(fail, &sc->status);
+  } else {
+    for (int64_t t = blockIdx.x; t < ring.ntiles; t += gridDim.x) {
+      if (!ring.wait(t)) {
+        if (ring.lane == 0) ring_fail(fail, &sc->status);
+        break;
+      }
+      if (ring.sl < A.nslices) {
+        const int64_t i = ring.sl * 32 + ring.lane;
+        const double acc = ring_row_sum<double>(ring, i, [&](int j) { return __ldg(p + j); });
+        if (i < A.n) {
+          q[i] = acc;
+          d[0] += ring.template row<double>(0, i) * acc;
+        }
+      }
+      ring.release();
     }
-    const double acc =
-        ring_row_sum<double>(ring, ring.width(), [&](int j) { return __ldg(p + j); });
-    if (has) {
-      q[i] = acc;
-      d[0] += pi * acc;
-    }
-    ring.release();
   }
   grid_reduce<1>(d, red, PqEpi{sc});
 }
@@ -212,11 +215,13 @@ static int launch_spmv_dot(const amg_handle* H, cudaStream_t s) {
   const int grid = sell_grid(sell_groups(L.A), H->num_sms);
   const SellView<double> v = view<double>(L.A, L.A.v64);
   if (H->opt.stream_ring && !H->batched) {
-    RingGeom g = ring_plan(L.A, 8, ring_stages(H), RingRows());
+    RingRows rows;
+    rows.add(H->p, (int)sizeof(double));
+    RingGeom g = ring_plan(L.A, 8, ring_stages(H), rows, true);
     if (g.D) {
       AMG_TRY(ring_prepare((const void*)k_spmv_dot_ring, g, L.A.nslices, H->num_sms));
-      k_spmv_dot_ring<<<g.grid, RING_THREADS, g.smem, s>>>(v, H->p, H->q, H->red, H->sc, g,
-                                                           RingRows(), H->wait_fail);
+      k_spmv_dot_ring<<<g.grid, g.threads(), g.smem, s>>>(v, H->p, H->q, H->red, H->sc, g,
+                                                          rows, H->wait_fail);
       AMG_LAUNCH_CHECK();
       return AMG_OK;
     }

@@ -1,5 +1,6 @@
 // Host side of the shared-memory ring streams (ring.cuh): which matrices
 // qualify, the ring's geometry, and the kernels' shared-memory limit.
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <utility>
@@ -8,39 +9,66 @@
 
 namespace amg {
 
-RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows) {
-  RingGeom g;
-  if (M.C != 32 || M.tpr != 1 || M.row0 || M.d16 || M.wmax <= 0 || M.nslices <= 0) return g;
-  if (vbytes != 2 && vbytes != 4 && vbytes != 8) return g;
-  if (stages == 0) stages = RING_DEFAULT_STAGES;
-  if (stages < 2 || stages > RING_MAX_STAGES || rows.n > RING_MAX_ROWS) return g;
+// Stages and tile: the largest tile (8, 4 or 2 slices, one consumer warp
+// each) that leaves room for the warps of RING_CTAS_PER_SM CTAs of 8 slices
+// per SM, else for half of them.  Three stages while the SM's rings then stay
+// within half of its unified memory, so that the rest caches the gathered
+// vector, else two: measured at 256^3 (FP32), the level-0 pre-smoother (9 KB
+// stages) took 0.136 ms with three against 0.143 with two, the level-1 one of
+// a diffusion matrix (18 KB stages) 0.092 against 0.080.
+constexpr size_t RING_L1_SPLIT = 128 * 1024;
+
+RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows, bool dots) {
+  RingGeom none;
+  if (M.C != 32 || M.tpr != 1 || M.row0 || !M.rec || M.wmax <= 0 || M.nslices <= 0) return none;
+  if (vbytes != 2 && vbytes != 4 && vbytes != 8) return none;
+  if (stages == 1 || stages > RING_MAX_STAGES || rows.n > RING_MAX_ROWS) return none;
+  uint32_t direct = 0;
   for (int k = 0; k < rows.n; ++k) {
-    if (rows.esz[k] != 4 && rows.esz[k] != 8) return g;
-    if (((uintptr_t)rows.p[k] & 15u) != 0) return g;  // bulk copies start 16-byte aligned
+    if (rows.esz[k] != 4 && rows.esz[k] != 8) return none;
+    if (((uintptr_t)rows.p[k] & 15u) != 0) direct |= 1u << k;  // no bulk copy from there
   }
   auto up = [](size_t v) { return (v + 127) & ~(size_t)127; };
-  // values, columns, per-row vectors; every block starts on 128 bytes
-  size_t off = up((size_t)M.wmax * 32 * (size_t)vbytes);
-  g.coff = (uint32_t)off;
-  off = up(off + (size_t)M.wmax * 128);
-  for (int k = 0; k < rows.n; ++k) {
-    g.roff[k] = (uint32_t)off;
-    off = up(off + 32 * (size_t)rows.esz[k]);
-  }
-  const size_t stage = off;
-  const size_t tables = (size_t)RING_WARPS * RING_MAX_STAGES * (8 + 4);  // barriers, widths
-  const size_t smem = (size_t)RING_WARPS * stages * stage + tables + RING_ALIGN_SLACK;
-  if (smem > RING_SMEM_PER_CTA) return g;
-  g.D = stages;
-  g.stage = (uint32_t)stage;
-  g.smem = smem;
-  return g;
+  // values, index blocks, records, per-row vectors; every part starts on 128 bytes
+  auto plan = [&](int q, int D) {
+    RingGeom g;
+    g.tile = ring_tile(q);
+    size_t off = up((size_t)M.tile_w[q] * 32 * (size_t)vbytes);
+    g.coff = (uint32_t)off;
+    off = up(off + (size_t)M.tile_ix[q]);
+    g.soff = (uint32_t)off;
+    off = up(off + 16 * (size_t)(g.tile + 1));
+    for (int k = 0; k < rows.n; ++k) {
+      g.roff[k] = (uint32_t)off;
+      off = up(off + 32 * (size_t)(g.tile * rows.esz[k]));
+    }
+    g.D = D;
+    g.direct = direct;
+    g.stage = (uint32_t)off;
+    g.smem = (size_t)D * off + 2 * RING_MAX_STAGES * 8 + RING_ALIGN_SLACK;
+    return g;
+  };
+  // smaller tiles where 8 slices a CTA would leave SMs without work (two
+  // CTAs on each of 152); with dot products 8 slices, the blocks of the
+  // per-lane kernels, so that both sum small levels alike
+  const int q0 = dots || M.nslices >= 304 * ring_tile(0) ? 0
+                 : M.nslices >= 304 * ring_tile(1)       ? 1
+                                                         : 2;
+  for (int ctas : {RING_CTAS_PER_SM, 2})
+    for (int q = q0; q < 3; ++q) {
+      const int c = ctas * ring_tile(0) / ring_tile(q);  // the same number of warps
+      const size_t smem = c * (plan(q, 3).smem + 1024);
+      const RingGeom g = plan(q, stages ? stages : smem <= RING_L1_SPLIT ? 3 : 2);
+      if (g.smem <= RING_SMEM_PER_CTA && (size_t)c * (g.smem + 1024) <= RING_SMEM_PER_SM)
+        return g;
+    }
+  return none;
 }
 
 int ring_prepare(const void* fn, RingGeom& g, int64_t nslices, int num_sms) {
   static std::mutex mu;
   static std::map<std::pair<const void*, int>, bool> attr;
-  static std::map<std::pair<const void*, size_t>, int> occ;
+  static std::map<std::pair<const void*, std::pair<size_t, int>>, int> occ;
   int dev = 0;
   AMG_CUDA_TRY(cudaGetDevice(&dev));
   int per_sm = 0;
@@ -55,17 +83,17 @@ int ring_prepare(const void* fn, RingGeom& g, int64_t nslices, int num_sms) {
                                         (int)cudaSharedmemCarveoutMaxShared));
       done = true;
     }
-    int& nb = occ[{fn, g.smem}];  // the same on every device of one kind
+    int& nb = occ[{fn, {g.smem, g.tile}}];  // the same on every device of one kind
     if (!nb) {
-      AMG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, RING_THREADS,
-                                                                 g.smem));
+      AMG_CUDA_TRY(
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, g.threads(), g.smem));
       if (nb < 1) nb = -1;
     }
     per_sm = nb;
   }
   if (per_sm < 1) return AMG_ERR_UNSUPPORTED;
-  const int64_t need = (nslices + RING_WARPS - 1) / RING_WARPS;  // one slice per warp
-  const int64_t full = (int64_t)num_sms * per_sm;
+  const int64_t need = (nslices + g.tile - 1) / g.tile;  // one tile per CTA
+  const int64_t full = (int64_t)num_sms * std::min(per_sm, 16);  // grid reductions hold 16 per SM
   g.grid = (int)(need < full ? need : full);
   return AMG_OK;
 }

@@ -2,49 +2,71 @@
 //
 // The level operators are HBM streams (Sec. 2.1: sparse kernels move O(1)
 // bytes per flop), and a warp that loads its slice entry by entry keeps only
-// a few loads in flight, so DRAM latency bounds it.  Here every warp owns a
-// ring of D stages in shared memory; one lane starts the copy of a whole
-// slice (values and column indices, each one contiguous block of the
-// column-major slice) with cp.async.bulk, completion counted in bytes on the
-// stage's mbarrier, D - 1 slices ahead of the one being consumed.  The lanes
-// then read their row's entries from shared memory and gather the vector
-// through L2.  Slices of a warp: gw, gw + W, gw + 2W, ... (W warps in the
-// grid), the same slice order as the grid-stride kernels.
+// a few loads in flight, so DRAM latency bounds it.  Here every CTA owns a
+// ring of D stages in shared memory.  A producer warp copies whole tiles of
+// consecutive slices (values, index blocks, slice records: each one contiguous
+// range) with cp.async.bulk, completion counted in bytes on the stage's "full"
+// mbarrier; each consumer warp takes one slice of the tile, its lanes read
+// their row's entries from shared memory and gather the vector through L2, and
+// the warp then arrives on the stage's "empty" mbarrier.  Tiles of a CTA: b,
+// b + G, b + 2G, ... (G CTAs in the grid).
 //
-// The slice's 32 entries of the kernel's per-row vectors (b, s, r, the
-// aggregate map, ...) come with it, so every DRAM stream of the loop is a
-// bulk copy started D - 1 slices ahead; the ragged last slice reads those
+// The 32 entries per slice of the kernel's per-row vectors (b, s, r, the
+// aggregate map, ...) come with the tile, so every DRAM stream of the loop is
+// a bulk copy started D - 1 tiles ahead; the ragged last tile reads those
 // from global memory instead (its copy would run past the vectors' end).
 //
+// What bounds it: with a ring per warp (every warp refilling its own two
+// stages slice by slice) the FP32 level-0 pre-smoother issued 241 warp
+// instructions a slice of 7 entries a row, more than half of them to manage
+// the ring, and its time did not move when a third of its bytes went.
+//
+// Column indices are a third of an FP64 operator's stream and half of an FP32
+// one's, and the columns of 32 consecutive rows say almost the same thing 32
+// times.  Each slice's index block takes the smallest coding that holds its
+// columns (IX_* in common.cuh): one offset per ELL column where the rows share
+// their offsets (every slice of a stencil matrix: 4 bytes instead of 128),
+// 16-bit deltas from a base per ELL column where the columns lie close (A P
+// and the coarse levels: 68 instead of 128), else plain columns.  In the
+// per-lane kernels fewer index bytes did not pay (each load then carries less,
+// and their number bounds them); here the copies are whole blocks, so bytes
+// are what counts.
+//
 // Requirements (checked on the host by ring_plan): one thread per row and
-// slice height 32 (lane = row of the slice), one system (no row0), plain
-// int32 columns, and a widest slice that fits a stage.  Slice s starts at
-// sliceptr[s], a multiple of 32, so both copies start on 16-byte boundaries
-// and have sizes that are multiples of 16 bytes (32 w values of 2, 4 or 8
-// bytes; 32 w int32 columns); the per-row copies are 32 entries of 4 or 8
-// bytes at offset 32 s entries of 256-byte aligned vectors.
+// slice height 32 (lane = row of the slice), one system (no row0), packed
+// indices (Sell::rec), and tiles that fit a stage.  Slice s starts at slot
+// rec[s].slot, a multiple of 32, and its index block at a multiple of 16 bytes,
+// so all copies start on 16-byte boundaries and have sizes that are multiples
+// of 16 bytes (32 w values of 2, 4 or 8 bytes; ix_bytes; 16-byte records); the
+// per-row copies are 32 tile entries of 4 or 8 bytes at offset 32 tile t
+// entries of 256-byte aligned vectors.
 //
 // Bounded waits: a wait for a stage gives up after RING_WAIT_NS of
-// %globaltimer, sets the handle's sticky failure flag, waits (bounded) for
-// the warp's other copies in flight and leaves the loop; later launches see
-// the flag and return at once, and pcg_solve reports AMG_ERR_DEVICE_CHECK.
+// %globaltimer and sets the handle's sticky failure flag; the warp leaves its
+// loop, and the producer waits (bounded) for the copies in flight before the
+// CTA ends.  Later launches see the flag and return at once, and pcg_solve
+// reports AMG_ERR_DEVICE_CHECK.
 #pragma once
 
 #include "sellk.cuh"
 
 namespace amg {
 
-constexpr int RING_WARPS = 8;                      // warps per CTA
-constexpr int RING_THREADS = RING_WARPS * 32;
 constexpr int RING_MAX_STAGES = 4;
+constexpr int RING_MAX_TILE = 8;  // slices per tile = consumer warps per CTA
+// CTAs per SM that the streaming kernels are compiled for: 36 warps of 56
+// registers.  Five or six CTAs leave 40 and 32 registers, too few to keep a
+// row's gathers in flight together (256^3 FP32 solve 158.7 -> 175 and 193 ms).
+constexpr int RING_CTAS_PER_SM = 4;
+constexpr int RING_MAX_THREADS = (RING_MAX_TILE + 1) * 32;
 constexpr unsigned long long RING_WAIT_NS = 1000000000ull;  // 1 s
 constexpr size_t RING_SMEM_PER_CTA = 112 * 1024;   // at least two CTAs per SM
-constexpr int RING_DEFAULT_STAGES = 2;
+constexpr size_t RING_SMEM_PER_SM = 227 * 1024;
 constexpr size_t RING_ALIGN_SLACK = 128;
 
-constexpr int RING_MAX_ROWS = 5;  // per-row vectors staged with each slice
+constexpr int RING_MAX_ROWS = 5;  // per-row vectors staged with each tile
 
-// Per-row vectors copied into the stage with each slice (the slice's 32
+// Per-row vectors copied into the stage with each tile (the tile's
 // consecutive entries of each): base pointers and element sizes.
 struct RingRows {
   const void* p[RING_MAX_ROWS] = {};
@@ -57,15 +79,20 @@ struct RingRows {
   }
 };
 
-// Ring geometry of one launch (host-computed).  A stage holds the slice's
-// values, its columns, then 32 entries of each per-row vector.
+// Ring geometry of one launch (host-computed).  A stage holds the tile's
+// values, its index blocks, its slice records, then its entries of each
+// per-row vector.
 struct RingGeom {
-  int D = 0;            // stages per warp (0: not eligible)
+  int D = 0;            // stages per CTA (0: not eligible)
+  int tile = 0;         // slices per tile
   uint32_t stage = 0;   // bytes per stage
-  uint32_t coff = 0;    // offset of the columns within a stage
+  uint32_t coff = 0;    // offset of the index blocks within a stage
+  uint32_t soff = 0;    // offset of the slice records
   uint32_t roff[RING_MAX_ROWS] = {};  // offsets of the per-row vectors
+  uint32_t direct = 0;  // bit k: row vector k starts off a 16-byte boundary, read directly
   int grid = 0;         // CTAs (ring_prepare)
   size_t smem = 0;      // dynamic shared memory per CTA
+  int threads() const { return (tile + 1) * 32; }
 };
 
 // ------------------------------------------------------------------ PTX wrappers
@@ -137,143 +164,192 @@ __device__ __forceinline__ void bulk_copy_g2s(uint32_t dst, const void* src, uin
       : "memory");
 }
 
-// ------------------------------------------------------------------ per-warp ring
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
 
-// One warp's ring over the slices gw, gw + nwt, ... of a SELL matrix with
-// slice height 32.  Lane 0 issues, every lane consumes.  Usage:
-//   RingWarp<V> ring(A, g, smem);  ring.start();
-//   for (int64_t sl = ring.first; sl < A.nslices; sl += ring.nwt) {
-//     if (!ring.wait()) { ...report...; ring.drain(); break; }  // gave up
-//     ... ring.width(), ring.val(k), ring.col(k) of slice sl ...
-//     ring.release();                   // stage free: refill with sl + D nwt
+// ------------------------------------------------------------------ the CTA's ring
+
+// Usage (every thread of the CTA):
+//   TileRing<V> ring(A, g, rows, smem);
+//   if (ring.producer()) ring.produce(fail, status);
+//   else for (int64_t t = blockIdx.x; t < ring.ntiles; t += gridDim.x) {
+//     if (!ring.wait(t)) { report; break; }
+//     if (ring.sl < A.nslices) { ... ring_row_sum(ring, i, g, init) of slice sl ... }
+//     ring.release();
 //   }
-// Every copy issued is consumed before the loop ends, so none is in flight
-// when the kernel returns (drain() covers the loop left early).
 template <typename V>
-struct RingWarp {
+struct TileRing {
   const SellView<V>& A;
   const RingGeom& g;
   const RingRows& rows;
-  unsigned char* base;  // this warp's first stage
-  uint32_t bar0;        // this warp's first barrier (shared address)
-  int* widths;          // per stage: ELL width of the slice it holds
-  int64_t first, nwt, cur;
+  unsigned char* base;   // first stage
+  uint32_t bars;         // shared address: full[D], then empty[D]
+  int64_t ntiles;
+  int warp, lane;
+  // consumer state
   int stage = 0;
-  uint32_t phase = 0;   // parity of the current stage's next completion
-  int lane;
-  uint64_t pol;
-  bool ok = true;
-  int64_t nbeg = 0, nend = 0;  // lane 0: bounds of the slice release() copies next
+  uint32_t phase = 0;
+  int64_t sl = 0, t = 0;
+  const unsigned char* st = nullptr;  // current stage
+  const unsigned char* vals = nullptr;
+  const int32_t* ixb = nullptr;
+  int wm = 0;  // (ELL width << 2) | IX_* code
+  bool full_tile = false;
 
-  __device__ __forceinline__ RingWarp(const SellView<V>& A_, const RingGeom& g_,
+  __device__ __forceinline__ TileRing(const SellView<V>& A_, const RingGeom& g_,
                                       const RingRows& rows_, unsigned char* smem_raw)
       : A(A_), g(g_), rows(rows_) {
     // 128-byte aligned start (the launch adds RING_ALIGN_SLACK bytes)
-    unsigned char* smem =
-        smem_raw + ((128u - (smem_addr(smem_raw) & 127u)) & 127u);
-    const int warp = threadIdx.x >> 5;
+    base = smem_raw + ((128u - (smem_addr(smem_raw) & 127u)) & 127u);
+    bars = smem_addr(base) + (uint32_t)g.D * g.stage;
+    warp = threadIdx.x >> 5;
     lane = threadIdx.x & 31;
-    base = smem + (size_t)warp * g.D * g.stage;
-    uint64_t* bars = (uint64_t*)(smem + (size_t)RING_WARPS * g.D * g.stage);
-    bar0 = smem_addr(bars + warp * RING_MAX_STAGES);
-    widths = (int*)(bars + RING_WARPS * RING_MAX_STAGES) + warp * RING_MAX_STAGES;
-    nwt = (int64_t)gridDim.x * RING_WARPS;
-    first = (int64_t)blockIdx.x * RING_WARPS + warp;
-    cur = first;
-    pol = l2_evict_first();
-  }
-
-  __device__ __forceinline__ uint32_t bar(int d) const { return bar0 + 8u * (uint32_t)d; }
-
-  // Slice sl has 32 rows (not the ragged last slice): its per-row vectors
-  // come with it; the last slice's are read from global memory.
-  __device__ __forceinline__ bool full(int64_t sl) const { return (sl + 1) * 32 <= A.n; }
-
-  // lane 0: copy slice sl = [beg, end) (and its per-row vectors) into stage d
-  __device__ __forceinline__ void issue(int64_t sl, int d, int64_t beg, int64_t end) {
-    const int w = (int)((end - beg) >> 5);
-    widths[d] = w;
-    const uint32_t vb = (uint32_t)w * 32u * (uint32_t)sizeof(V), cb = (uint32_t)w * 128u;
-    const bool f = full(sl);
-    uint32_t rb = 0;
-#pragma unroll
-    for (int k = 0; k < RING_MAX_ROWS; ++k)
-      if (f && k < rows.n) rb += 32u * (uint32_t)rows.esz[k];
-    const uint32_t dst = smem_addr(base + (size_t)d * g.stage);
-    mbar_arrive_expect_tx(bar(d), vb + cb + rb);
-    if (w > 0) {
-      bulk_copy_g2s(dst, A.val + beg, vb, bar(d), pol);
-      bulk_copy_g2s(dst + g.coff, A.col + beg, cb, bar(d), pol);
-    }
-#pragma unroll
-    for (int k = 0; k < RING_MAX_ROWS; ++k)
-      if (f && k < rows.n)
-        bulk_copy_g2s(dst + g.roff[k], (const unsigned char*)rows.p[k] + sl * 32 * rows.esz[k],
-                      32u * (uint32_t)rows.esz[k], bar(d), pol);
-  }
-
-  // barriers initialised, the first D slices on their way
-  __device__ __forceinline__ void start() {
-    if (lane == 0) {
-      for (int d = 0; d < g.D; ++d) mbar_init(bar(d), 1);
-      mbar_init_fence();
+    ntiles = (A.nslices + g.tile - 1) / g.tile;
+    if (threadIdx.x == 0) {
       for (int d = 0; d < g.D; ++d) {
-        const int64_t sl = first + (int64_t)d * nwt;
-        if (sl < A.nslices) issue(sl, d, __ldg(A.sliceptr + sl), __ldg(A.sliceptr + sl + 1));
+        mbar_init(full(d), 1);
+        mbar_init(empty(d), (uint32_t)g.tile);
       }
+      mbar_init_fence();
     }
-    __syncwarp();
+    __syncthreads();
   }
 
-  // Waits for the current slice.  Lane 0 first loads the bounds of the slice
-  // that release() will copy next, so that load's latency passes during the
-  // wait and the slice's arithmetic instead of delaying the copy.
-  __device__ __forceinline__ bool wait() {
-    const int64_t nxt = cur + (int64_t)g.D * nwt;
-    if (lane == 0 && nxt < A.nslices) {
-      nbeg = __ldg(A.sliceptr + nxt);
-      nend = __ldg(A.sliceptr + nxt + 1);
-    }
-    ok = mbar_wait_bounded(bar(stage), phase);
-    return __all_sync(0xffffffffu, ok);
+  __device__ __forceinline__ uint32_t full(int d) const { return bars + 8u * (uint32_t)d; }
+  __device__ __forceinline__ uint32_t empty(int d) const {
+    return bars + 8u * (uint32_t)(RING_MAX_STAGES + d);
+  }
+  __device__ __forceinline__ bool producer() const { return warp == g.tile; }
+  __device__ __forceinline__ bool is_full(int64_t tt) const {
+    return (tt + 1) * g.tile * 32 <= A.n;
+  }
+  __device__ __forceinline__ bool staged(bool f, int k) const {
+    return f && k < rows.n && !((g.direct >> k) & 1u);
+  }
+  __device__ __forceinline__ SliceRec load_rec(int64_t s) const {
+    const longlong2 r = __ldg((const longlong2*)(A.rec + (s < A.nslices ? s : A.nslices)));
+    return SliceRec{r.x, r.y};
   }
 
-  __device__ __forceinline__ int width() const { return widths[stage]; }
-  __device__ __forceinline__ V val(int k) const {
-    return ((const V*)(base + (size_t)stage * g.stage))[k * 32 + lane];
+  // The producer warp: lane 0 copies every tile of this CTA, a stage as soon
+  // as its consumers have left it.  The next tile's bounds are loaded a tile
+  // ahead.
+  __device__ __forceinline__ void produce(int* fail, int* status) {
+    if (lane != 0) return;
+    const uint64_t pol = l2_evict_first();
+    int64_t tt = blockIdx.x;
+    if (tt >= ntiles) return;
+    SliceRec b = load_rec(tt * g.tile), e = load_rec(tt * g.tile + g.tile);
+    int d = 0, issued = 0;
+    uint32_t ph = 1;  // the first pass over the stages does not wait
+    for (;;) {
+      const int64_t nx = tt + gridDim.x;
+      SliceRec nb = {0, 0}, ne = {0, 0};
+      if (nx < ntiles) {
+        nb = load_rec(nx * g.tile);
+        ne = load_rec(nx * g.tile + g.tile);
+      }
+      if (issued >= g.D && !mbar_wait_bounded(empty(d), ph)) {
+        atomicExch(fail, 1);
+        if (status) atomicCAS(status, 0, AMG_ERR_DEVICE_CHECK);
+        break;
+      }
+      const int64_t ib = b.ix & ~(int64_t)3;
+      const uint32_t vb = (uint32_t)(e.slot - b.slot) * (uint32_t)sizeof(V);
+      const uint32_t cb = (uint32_t)((e.ix & ~(int64_t)3) - ib);
+      const int64_t s0 = tt * g.tile;
+      const uint32_t ns = (uint32_t)(A.nslices - s0 < g.tile ? A.nslices - s0 : g.tile);
+      const bool f = is_full(tt);
+      uint32_t rb = 0;
+#pragma unroll
+      for (int k = 0; k < RING_MAX_ROWS; ++k)
+        if (staged(f, k)) rb += 32u * (uint32_t)(g.tile * rows.esz[k]);
+      const uint32_t dst = smem_addr(base) + (uint32_t)d * g.stage, fb = full(d);
+      mbar_arrive_expect_tx(fb, vb + cb + 16u * (ns + 1) + rb);
+      bulk_copy_g2s(dst + g.soff, A.rec + s0, 16u * (ns + 1), fb, pol);
+      if (vb > 0) {
+        bulk_copy_g2s(dst, A.val + b.slot, vb, fb, pol);
+        bulk_copy_g2s(dst + g.coff, A.ix + ib, cb, fb, pol);
+      }
+#pragma unroll
+      for (int k = 0; k < RING_MAX_ROWS; ++k)
+        if (staged(f, k))
+          bulk_copy_g2s(dst + g.roff[k],
+                        (const unsigned char*)rows.p[k] + s0 * 32 * rows.esz[k],
+                        32u * (uint32_t)(g.tile * rows.esz[k]), fb, pol);
+      ++issued;
+      if (++d == g.D) {
+        d = 0;
+        ph ^= 1u;
+      }
+      tt = nx;
+      if (tt >= ntiles) break;
+      b = nb;
+      e = ne;
+    }
+    // every copy has landed before the CTA can end (consumers that gave up
+    // leave stages unread)
+    for (int k = issued > g.D ? issued - g.D : 0; k < issued; ++k)
+      if (!mbar_wait_bounded(full(k % g.D), (uint32_t)(k / g.D) & 1u)) break;
   }
-  __device__ __forceinline__ int32_t col(int k) const {
-    return ((const int32_t*)(base + (size_t)stage * g.stage + g.coff))[k * 32 + lane];
+
+  // Waits for tile tt; false if the wait gave up.
+  __device__ __forceinline__ bool wait(int64_t tt) {
+    if (!__all_sync(0xffffffffu, mbar_wait_bounded(full(stage), phase))) return false;
+    t = tt;
+    sl = tt * g.tile + warp;
+    st = base + (size_t)stage * g.stage;
+    full_tile = is_full(tt);
+    if (sl < A.nslices) {
+      const SliceRec* r = (const SliceRec*)(st + g.soff);
+      const SliceRec r0 = r[0], rw = r[warp], rn = r[warp + 1];
+      vals = st + (size_t)(rw.slot - r0.slot) * sizeof(V);
+      ixb = (const int32_t*)(st + g.coff + ((rw.ix & ~(int64_t)3) - (r0.ix & ~(int64_t)3)));
+      wm = ((int)(rn.slot - rw.slot) >> 5 << 2) | (int)(rw.ix & 3);
+    }
+    return true;
   }
-  // entry i = 32 cur + lane of per-row vector k (element type X = its type)
+
+  __device__ __forceinline__ V val(int k) const { return ((const V*)vals)[k * 32 + lane]; }
+  // entry i = 32 sl + lane of per-row vector k (element type X = its type)
   template <typename X>
-  __device__ __forceinline__ X row(int k, bool f, int64_t i) const {
-    if (f) return ((const X*)(base + (size_t)stage * g.stage + g.roff[k]))[lane];
+  __device__ __forceinline__ X row(int k, int64_t i) const {
+    if (staged(full_tile, k)) return ((const X*)(st + g.roff[k]))[warp * 32 + lane];
     return __ldg((const X*)rows.p[k] + i);
   }
 
-  // every lane is done with the current stage: refill it, move on
+  // every lane is done with the stage
   __device__ __forceinline__ void release() {
     __syncwarp();
-    const int64_t nxt = cur + (int64_t)g.D * nwt;
-    if (lane == 0 && nxt < A.nslices) issue(nxt, stage, nbeg, nend);
-    cur += nwt;
+    if (lane == 0) mbar_arrive(empty(stage));
     if (++stage == g.D) {
       stage = 0;
       phase ^= 1u;
     }
   }
+};
 
-  // After a wait that gave up: wait (bounded) for the copies still in
-  // flight, so none lands in shared memory after the CTA has exited.
-  __device__ __forceinline__ void drain() {
-    for (int d = 0; d < g.D; ++d) {
-      const int64_t sl = cur + (int64_t)d * nwt;
-      if (sl >= A.nslices) break;
-      const int st = (stage + d) % g.D;
-      const uint32_t ph = phase ^ (uint32_t)((stage + d) / g.D);
-      if (!mbar_wait_bounded(bar(st), ph)) break;
-    }
+// Columns of this lane's row in the current stage, by the slice's coding.
+struct IxPlain {
+  const int32_t* c;
+  __device__ __forceinline__ int32_t operator()(int k) const { return c[k * 32]; }
+};
+struct IxDelta {
+  const int32_t* base;
+  const uint16_t* d;
+  __device__ __forceinline__ int32_t operator()(int k) const { return base[k] + (int)d[k * 32]; }
+};
+struct IxOffset {
+  const int32_t* off;
+  int32_t i;  // this lane's row
+  __device__ __forceinline__ int32_t operator()(int k) const { return i + off[k]; }
+};
+struct IxClamp {
+  const int32_t* off;
+  int32_t i, last;  // the clamp only ever moves padding
+  __device__ __forceinline__ int32_t operator()(int k) const {
+    return min(max(i + off[k], 0), last);
   }
 };
 
@@ -281,11 +357,12 @@ struct RingWarp {
 // values) for k = k0 .. k0 + N - 1, k ascending: the N gathers issue
 // together, then the FMAs follow in order.  Exactly N FMAs: on GB300's FP64
 // pipe a predicated-off FMA would still cost its cycles.
-template <int N, bool NEG, typename T, typename V, typename G>
-__device__ __forceinline__ T ring_chunk(const RingWarp<V>& ring, int k0, T acc, G g) {
+template <int N, bool NEG, typename T, typename V, typename I, typename G>
+__device__ __forceinline__ T ring_chunk(const TileRing<V>& ring, const I& ix, int k0, T acc,
+                                        G g) {
   T x[N];
 #pragma unroll
-  for (int u = 0; u < N; ++u) x[u] = g(ring.col(k0 + u));
+  for (int u = 0; u < N; ++u) x[u] = g(ix(k0 + u));
 #pragma unroll
   for (int u = 0; u < N; ++u) {
     const T a = to_f(ring.val(k0 + u), T(0));
@@ -294,26 +371,45 @@ __device__ __forceinline__ T ring_chunk(const RingWarp<V>& ring, int k0, T acc, 
   return acc;
 }
 
-// init + sum_k a_k g(col_k) (NEG: init - sum) over the w entries of this
-// lane's row in the current stage, k ascending (the per-lane kernels'
-// order): chunks of 8 and one remainder chunk of the exact length (w is
+// Chunks of 8 and one remainder chunk of the exact length (w is
 // warp-uniform).
-template <typename T, bool NEG = false, typename V, typename G>
-__device__ __forceinline__ T ring_row_sum(const RingWarp<V>& ring, int w, G g, T init = T(0)) {
-  T acc = init;
+template <bool NEG, typename T, typename V, typename I, typename G>
+__device__ __forceinline__ T ring_chunks(const TileRing<V>& ring, const I& ix, int w, T acc,
+                                         G g) {
   int k0 = 0;
-  for (; k0 + 8 <= w; k0 += 8) acc = ring_chunk<8, NEG>(ring, k0, acc, g);
+  for (; k0 + 8 <= w; k0 += 8) acc = ring_chunk<8, NEG>(ring, ix, k0, acc, g);
   switch (w - k0) {
-    case 1: acc = ring_chunk<1, NEG>(ring, k0, acc, g); break;
-    case 2: acc = ring_chunk<2, NEG>(ring, k0, acc, g); break;
-    case 3: acc = ring_chunk<3, NEG>(ring, k0, acc, g); break;
-    case 4: acc = ring_chunk<4, NEG>(ring, k0, acc, g); break;
-    case 5: acc = ring_chunk<5, NEG>(ring, k0, acc, g); break;
-    case 6: acc = ring_chunk<6, NEG>(ring, k0, acc, g); break;
-    case 7: acc = ring_chunk<7, NEG>(ring, k0, acc, g); break;
+    case 1: acc = ring_chunk<1, NEG>(ring, ix, k0, acc, g); break;
+    case 2: acc = ring_chunk<2, NEG>(ring, ix, k0, acc, g); break;
+    case 3: acc = ring_chunk<3, NEG>(ring, ix, k0, acc, g); break;
+    case 4: acc = ring_chunk<4, NEG>(ring, ix, k0, acc, g); break;
+    case 5: acc = ring_chunk<5, NEG>(ring, ix, k0, acc, g); break;
+    case 6: acc = ring_chunk<6, NEG>(ring, ix, k0, acc, g); break;
+    case 7: acc = ring_chunk<7, NEG>(ring, ix, k0, acc, g); break;
     default: break;
   }
   return acc;
+}
+
+// init + sum_k a_k g(col_k) (NEG: init - sum) over the entries of this
+// lane's row i in the current stage, k ascending (the per-lane kernels'
+// order).
+template <typename T, bool NEG = false, typename V, typename G>
+__device__ __forceinline__ T ring_row_sum(const TileRing<V>& ring, int64_t i, G g,
+                                          T init = T(0)) {
+  const int w = ring.wm >> 2;
+  const int32_t* c = ring.ixb;
+  switch (ring.wm & 3) {
+    case IX_OFFSET:
+      return ring_chunks<NEG>(ring, IxOffset{c, (int32_t)i}, w, init, g);
+    case IX_CLAMP:
+      return ring_chunks<NEG>(ring, IxClamp{c, (int32_t)i, ring.A.ncols - 1}, w, init, g);
+    case IX_DELTA:
+      return ring_chunks<NEG>(
+          ring, IxDelta{c, (const uint16_t*)(c + ((w + 3) & ~3)) + ring.lane}, w, init, g);
+    default:
+      return ring_chunks<NEG>(ring, IxPlain{c + ring.lane}, w, init, g);
+  }
 }
 
 // A bounded wait gave up: the handle's sticky flag, and the PCG status
@@ -325,12 +421,14 @@ __device__ __forceinline__ void ring_fail(int* fail, int* status) {
 
 // Geometry for streaming M (values of `vbytes` bytes) with the ring, or
 // D = 0 when M does not qualify.  stages: 2..RING_MAX_STAGES, or 0 for the
-// default.  The grid is left to ring_launch_grid.  Host code.
-RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows);
+// default.  dots: the kernel also sums dot products over its grid.  The grid
+// is left to ring_prepare.  Host code.
+RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows,
+                   bool dots = false);
 
 // Prepares kernel `fn` for a launch with geometry g on the current device
 // (shared-memory limit, once per device and kernel) and sets g.grid to the
-// CTAs that are co-resident (occupancy query), at most one slice per warp.
+// CTAs that are co-resident (occupancy query), at most one tile per CTA.
 // Host code.
 int ring_prepare(const void* fn, RingGeom& g, int64_t nslices, int num_sms);
 

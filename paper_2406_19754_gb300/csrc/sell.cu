@@ -1,4 +1,6 @@
 // CSR -> sliced-ELL conversion and the plain FP64 SpMV (y = alpha A x + beta y).
+#include <algorithm>
+
 #include "sellk.cuh"
 
 namespace amg {
@@ -139,6 +141,168 @@ __global__ void k_sell_fill(int64_t n, int64_t ncols, int64_t nslices, int C,
   }
 }
 
+// Slices of 32 rows, one warp per slice and one lane per row (the kernels
+// above give a whole slice to one thread, whose pointer walk over 32 rows is
+// a chain of dependent loads: 0.28 ms a matrix, averaged over a 128^3
+// hierarchy; a warp steps all rows at once and finds the smallest offset by
+// one reduction).  The merge is slice_offsets' own: at each step the smallest
+// col - row among the rows' next entries is one ELL column, and the rows that
+// hold it step on.
+struct SliceLane {
+  int64_t i, beg;
+  int len, w;
+  bool has;
+  __device__ __forceinline__ SliceLane(int64_t s, int64_t n, const int64_t* row0,
+                                       const int64_t* rowptr) {
+    int64_t sb, se;
+    slice_rows(s, 32, n, row0, &sb, &se);
+    i = sb + (threadIdx.x & 31);
+    has = i < se;
+    beg = has ? rowptr[i] : 0;
+    len = has ? (int)(rowptr[i + 1] - beg) : 0;
+    w = __reduce_max_sync(0xffffffffu, len);
+  }
+};
+
+// Per slice: packed[s] = (w << 32) | (index block bytes / 16) for one scan of
+// both, and the layout: bit 2 = aligned, low bits = the index block's coding
+// (ring: aligned slices store one offset per ELL column, others 16-bit deltas
+// if every ELL column's columns lie within 65535, else plain columns).
+__global__ void k_sell_widths32(int64_t n, int64_t ncols, int64_t nslices, const int64_t* row0,
+                                const int64_t* rowptr, const int32_t* col, int ring,
+                                int64_t* packed, uint8_t* layout, int* wmax) {
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  __shared__ int wm;
+  if (threadIdx.x == 0) wm = 0;
+  __syncthreads();
+  int wl = 0;
+  for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nslices; s += nw) {
+    const SliceLane ln(s, n, row0, rowptr);
+    bool aligned = ln.w > 0;
+    int pos = 0, cnt = 0, umin = 0, umax = 0;
+    while (aligned) {
+      const int o = pos < ln.len ? col[ln.beg + pos] - (int32_t)ln.i : INT32_MAX;
+      const int m = __reduce_min_sync(0xffffffffu, o);
+      if (m == INT32_MAX) break;
+      aligned = cnt < ln.w;
+      umin = cnt ? min(umin, m) : m;
+      umax = cnt ? max(umax, m) : m;
+      ++cnt;
+      if (o == m) ++pos;
+    }
+    // offsets that leave [0, ncols) from some lane (only padding can) are clamped
+    const int64_t i0 = ln.i - (threadIdx.x & 31);
+    int mode = i0 + umin < 0 || i0 + 31 + umax >= ncols ? IX_CLAMP : IX_OFFSET;
+    if (!aligned) {
+      mode = IX_DELTA;
+      const int32_t pad = ln.len > 0 ? col[ln.beg + ln.len - 1]
+                                     : (int32_t)(ln.i < ncols ? ln.i : ncols - 1);
+      for (int k = 0; ring && k < ln.w; ++k) {
+        const int32_t c = k < ln.len ? col[ln.beg + k] : pad;
+        const int32_t lo = __reduce_min_sync(0xffffffffu, c);
+        const int32_t hi = __reduce_max_sync(0xffffffffu, c);
+        if (hi - lo > 65535) {
+          mode = IX_PLAIN;
+          break;
+        }
+      }
+    }
+    const int64_t ib = ring ? ix_bytes(mode, ln.w) : 0;
+    if ((threadIdx.x & 31) == 0) {
+      packed[s] = ((int64_t)ln.w << 32) | (ib >> 4);
+      layout[s] = (uint8_t)(mode | (aligned ? 4 : 0));
+    }
+    wl = max(wl, ln.w);
+  }
+  if ((threadIdx.x & 31) == 0) atomicMax(&wm, wl);
+  __syncthreads();
+  if (threadIdx.x == 0 && wm > 0) atomicMax(wmax, wm);
+}
+
+// Slots, slice pointers, and (ring) records, index blocks and the largest
+// tiles (tmax: ELL columns and index bytes per ring_tile(q)).  pk:
+// exclusive scan of `packed`; total: its grand total.
+__global__ void k_sell_fill32(int64_t n, int64_t ncols, int64_t nslices, const int64_t* row0,
+                              const int64_t* rowptr, const int32_t* col, const double* val,
+                              const int64_t* pk, int64_t total, const uint8_t* layout,
+                              int64_t* sliceptr, int32_t* ocol, double* oval, SliceRec* rec,
+                              unsigned char* ix, int* tmax) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  __shared__ int tm[6];
+  if (threadIdx.x < 6) tm[threadIdx.x] = 0;
+  __syncthreads();
+  for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nslices; s += nw) {
+    const SliceLane ln(s, n, row0, rowptr);
+    const int64_t beg = (pk[s] >> 32) * 32, ib = (pk[s] & 0xffffffffll) << 4;
+    const int mode = layout[s] & 3;
+    const bool aligned = layout[s] & 4;
+    if (lane == 0) {
+      sliceptr[s] = beg;
+      if (rec) rec[s] = SliceRec{beg, ib | mode};
+      if (s == nslices - 1) {
+        sliceptr[nslices] = (total >> 32) * 32;
+        if (rec) rec[nslices] = SliceRec{(total >> 32) * 32, (total & 0xffffffffll) << 4};
+      }
+      for (int q = 0; rec && q < 3; ++q)
+        if (s % ring_tile(q) == 0) {
+          const int64_t e = s + ring_tile(q) < nslices ? pk[s + ring_tile(q)] : total;
+          atomicMax(&tm[q], (int)((e >> 32) - (pk[s] >> 32)));
+          atomicMax(&tm[3 + q], (int)(((e & 0xffffffffll) << 4) - ib));
+        }
+    }
+    int32_t* head = rec ? (int32_t*)(ix + ib) : nullptr;
+    if (aligned) {
+      // ELL column k holds offset u_k; padding reads column i + u_k clamped
+      // into range (value 0; rows past the slice's last use that row)
+      const int64_t last = ln.i - lane + __popc(__ballot_sync(0xffffffffu, ln.has)) - 1;
+      const int64_t ir = ln.has ? ln.i : last;
+      int pos = 0;
+      for (int k = 0; k < ln.w; ++k) {
+        const int32_t c = pos < ln.len ? col[ln.beg + pos] : 0;
+        const int o = pos < ln.len ? c - (int32_t)ln.i : INT32_MAX;
+        const int m = __reduce_min_sync(0xffffffffu, o);
+        const int64_t dst = beg + (int64_t)k * 32 + lane;
+        // a slice with fewer distinct offsets than its longest row cannot be:
+        // m is an offset here for every k < w
+        if (o == m && pos < ln.len) {
+          ocol[dst] = c;
+          oval[dst] = val[ln.beg + pos];
+          ++pos;
+        } else {
+          int64_t cc = ir + m;
+          cc = cc < 0 ? 0 : cc >= ncols ? ncols - 1 : cc;
+          ocol[dst] = (int32_t)cc;
+          oval[dst] = 0.0;
+        }
+        if (rec && lane == 0) head[k] = m;
+      }
+      continue;
+    }
+    // sorted: k-th entry in ELL column k; padding (value 0) reads the row's
+    // last column, else the row itself
+    const int32_t pad = ln.len > 0 ? col[ln.beg + ln.len - 1]
+                                   : (int32_t)(ln.i < ncols ? ln.i : ncols - 1);
+    uint16_t* d = rec && mode == IX_DELTA ? (uint16_t*)(ix + ib + ((4 * ln.w + 15) & ~15))
+                                          : nullptr;
+    for (int k = 0; k < ln.w; ++k) {
+      const int64_t dst = beg + (int64_t)k * 32 + lane;
+      const int32_t c = k < ln.len ? col[ln.beg + k] : pad;
+      ocol[dst] = c;
+      oval[dst] = k < ln.len ? val[ln.beg + k] : 0.0;
+      if (d) {
+        const int32_t lo = __reduce_min_sync(0xffffffffu, c);
+        if (lane == 0) head[k] = lo;
+        d[k * 32 + lane] = (uint16_t)(c - lo);
+      } else if (rec) {
+        head[k * 32 + lane] = c;
+      }
+    }
+  }
+  __syncthreads();
+  if (tmax && threadIdx.x < 6 && tm[threadIdx.x] > 0) atomicMax(tmax + threadIdx.x, tm[threadIdx.x]);
+}
+
 // Column compression, one thread per slice: for each ELL column k the base is
 // the smallest column of its C slots and every slot stores its offset from it.
 // A slice whose offsets do not fit 16 bits raises *wide (the caller then
@@ -174,9 +338,58 @@ __global__ void k_to_bf16(int64_t n, const double* in, __nv_bfloat16* out) {
     out[i] = __float2bfloat16_rn((float)in[i]);
 }
 
+// Slices of 32 rows (out.n, ncols, nslices, row0 are set): sizes by one warp
+// per slice, one scan of slots and index bytes together, one fill.
+static int sell_from_csr32(Arena& ar, const int64_t* rowptr, const int32_t* col,
+                           const double* val, Sell& out, cudaStream_t s, bool compress,
+                           bool ring) {
+  int64_t *packed = nullptr, *pk = nullptr;
+  uint8_t* layout = nullptr;
+  int* mx = nullptr;  // widest slice; then the largest tiles (k_sell_fill32)
+  AMG_TRY(ar.alloc_n(&packed, out.nslices));
+  AMG_TRY(ar.alloc_n(&pk, out.nslices));
+  AMG_TRY(ar.alloc_n(&layout, out.nslices));
+  AMG_TRY(ar.alloc_n(&mx, 7));
+  AMG_TRY(ar.alloc_n(&out.sliceptr, out.nslices + 1));
+  AMG_CUDA_TRY(cudaMemsetAsync(mx, 0, 7 * sizeof(int), s));
+  const unsigned g = (unsigned)std::min<int64_t>((out.nslices + 7) / 8, 2048);
+  k_sell_widths32<<<g, 256, 0, s>>>(out.n, out.ncols, out.nslices, out.row0, rowptr, col, ring,
+                                    packed, layout, mx);
+  AMG_LAUNCH_CHECK();
+  int mx_h[7] = {};
+  AMG_CUDA_TRY(cudaMemcpyAsync(mx_h, mx, sizeof(int), cudaMemcpyDeviceToHost, s));
+  int64_t total = 0;
+  AMG_TRY(scan_exclusive_i64(ar, packed, pk, out.nslices, &total, s));  // synchronises
+  out.wmax = mx_h[0];
+  out.nnz_pad = (total >> 32) * 32;
+  ring = ring && out.wmax <= RING_MAX_WIDTH;
+  AMG_TRY(ar.alloc_n(&out.col, out.nnz_pad));
+  AMG_TRY(ar.alloc_n(&out.v64, out.nnz_pad));
+  if (ring) {
+    AMG_TRY(ar.alloc_n(&out.rec, out.nslices + 1));
+    AMG_TRY(ar.alloc_n(&out.ix, (total & 0xffffffffll) << 4));
+  }
+  k_sell_fill32<<<g, 256, 0, s>>>(out.n, out.ncols, out.nslices, out.row0, rowptr, col, val, pk,
+                                  total, layout, out.sliceptr, out.col, out.v64, out.rec,
+                                  out.ix, ring ? mx + 1 : nullptr);
+  AMG_LAUNCH_CHECK();
+  AMG_CUDA_TRY(cudaMemcpyAsync(mx_h, mx, sizeof(mx_h), cudaMemcpyDeviceToHost, s));
+  if (compress && out.tpr <= 8) AMG_TRY(sell_compress(ar, out, s));
+  AMG_CUDA_TRY(cudaStreamSynchronize(s));  // the CSR may go when this returns
+  for (int q = 0; q < 3; ++q) {
+    out.tile_w[q] = mx_h[1 + q];
+    out.tile_ix[q] = mx_h[4 + q];
+  }
+  ar.release(packed);
+  ar.release(pk);
+  ar.release(layout);
+  ar.release(mx);
+  return AMG_OK;
+}
+
 int sell_from_csr(Arena& ar, int64_t n, int64_t ncols, const int64_t* rowptr, const int32_t* col,
                   const double* val, int C, int tpr, Sell& out, cudaStream_t s,
-                  const std::vector<int64_t>* sys_off, bool compress) {
+                  const std::vector<int64_t>* sys_off, bool compress, bool ring) {
   if (n <= 0 || ncols <= 0) return AMG_ERR_ARG;
   // heights 1..64 and 1..32 threads per row, powers of two; batched systems
   // keep one slice per warp (slice height x threads per row = 32)
@@ -184,6 +397,7 @@ int sell_from_csr(Arena& ar, int64_t n, int64_t ncols, const int64_t* rowptr, co
     return AMG_ERR_ARG;
   if (sys_off && sys_off->size() >= 2 && C * tpr != 32) return AMG_ERR_ARG;
   out.n = n;
+  out.ncols = ncols;
   out.C = C;
   out.tpr = tpr;
   out.nslices = (n + C - 1) / C;
@@ -206,6 +420,8 @@ int sell_from_csr(Arena& ar, int64_t n, int64_t ncols, const int64_t* rowptr, co
                                  cudaMemcpyHostToDevice, s));
     AMG_CUDA_TRY(cudaStreamSynchronize(s));  // host vectors go out of scope
   }
+  if (C == 32)
+    return sell_from_csr32(ar, rowptr, col, val, out, s, compress, ring && tpr == 1);
   int64_t* slen = nullptr;
   uint8_t* aligned = nullptr;
   int* wmax = nullptr;

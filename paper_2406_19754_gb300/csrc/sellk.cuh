@@ -158,6 +158,9 @@ inline SellView<V> view(const Sell& A, const V* val) {
   v.sys = A.sys;
   v.d16 = A.d16;
   v.kbase = A.kbase;
+  v.rec = A.rec;
+  v.ix = A.ix;
+  v.ncols = (int32_t)A.ncols;
   v.act = nullptr;
   return v;
 }

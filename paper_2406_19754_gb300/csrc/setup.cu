@@ -864,7 +864,7 @@ static int build_ah(Arena& ar, Level& L, int num_sms, cudaStream_t s) {
 }
 
 static int build_ap(Arena& ar, Level& L, const int64_t* rp, const int32_t* ci, const double* va,
-                    bool compress, int num_sms, cudaStream_t s) {
+                    bool compress, bool ring, int num_sms, cudaStream_t s) {
   const int64_t n = L.n;
   int64_t* cnt = nullptr;
   int64_t* rp_ap = nullptr;
@@ -884,7 +884,7 @@ static int build_ap(Arena& ar, Level& L, const int64_t* rp, const int32_t* ci, c
   AMG_LAUNCH_CHECK();
   L.ap_nnz = total;
   AMG_TRY(sell_from_csr(ar, n, L.nc, rp_ap, ci_ap, va_ap, L.A.C, L.A.tpr, L.AP, s,
-                        L.sys_off.empty() ? nullptr : &L.sys_off, compress));
+                        L.sys_off.empty() ? nullptr : &L.sys_off, compress, ring));
   if (L.vstore != VAL_F64) AMG_TRY(sell_make_copies(ar, L.AP, L.vstore, s));
   AMG_CUDA_TRY(cudaStreamSynchronize(s));
   ar.release(cnt);
@@ -1054,7 +1054,8 @@ static std::vector<Layout> tune_candidates(bool wide, bool batched) {
 
 static void release_sell(Arena& ar, Sell& A) {
   for (void* p : {(void*)A.sliceptr, (void*)A.col, (void*)A.v64, (void*)A.v32, (void*)A.v16,
-                  (void*)A.row0, (void*)A.sys, (void*)A.d16, (void*)A.kbase})
+                  (void*)A.row0, (void*)A.sys, (void*)A.d16, (void*)A.kbase, (void*)A.rec,
+                  (void*)A.ix})
     ar.release(p);
   A = Sell();
 }
@@ -1345,14 +1346,17 @@ int setup_hierarchy(amg_handle* H, const amg_csr* A, cudaStream_t s, const amg_h
     const bool smooth = l + 1 < H->L.size();  // a level with a coarser one
     auto build = [&](Layout lay) -> int {
       const bool cmp = o.compress_columns != 0;
+      // the ring streams plain-column matrices of one system
+      const bool ring = o.stream_ring != 0 && !cmp && !H->batched &&
+                        (l == 0 || L.vstore != VAL_BF16);
       AMG_TRY(sell_from_csr(ar, L.n, L.n, rp, ci, va, lay.C, lay.tpr, L.A, s,
-                            H->batched ? &L.sys_off : nullptr, cmp));
+                            H->batched ? &L.sys_off : nullptr, cmp, ring));
       if (smooth) {
         AMG_TRY(build_ah(ar, L, sms, s));
         if (o.smooth_prolongator)
           AMG_TRY(build_smoothed_ops(ar, L, cmp, s));
         else
-          AMG_TRY(build_ap(ar, L, rp, ci, va, cmp, sms, s));
+          AMG_TRY(build_ap(ar, L, rp, ci, va, cmp, ring, sms, s));
       }
       return AMG_OK;
     };

@@ -115,6 +115,9 @@ __device__ __forceinline__ SellView<V> dview(const SellDesc& d) {
   v.sys = d.sys;
   v.d16 = d.d16;
   v.kbase = d.kbase;
+  v.rec = nullptr;
+  v.ix = nullptr;
+  v.ncols = 0;
   v.act = d.act;
   return v;
 }

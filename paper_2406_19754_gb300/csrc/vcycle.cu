@@ -136,88 +136,142 @@ __global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
   }
 }
 
-// k_pre and k_post (one sweep, one system, one thread per row, FP64 or FP32
+// k_pre, k_post and the sweeps (one system, one thread per row, FP64 or FP32
 // operator values) on the shared-memory ring of ring.cuh: the same row
 // arithmetic in the same order, so the same bits as the per-lane-load
 // kernels; the dot products of the level-0 post-smoother are summed per
 // thread over the warp's slices, then per block and over blocks, as there
-// (with this launch's grid).  k_pre loads its row's b before waiting for the
-// slice; k_post's row operands s, r, b, agg (and q for the second dot
-// product) come with the slice (per-row vectors of the ring).
+// (with this launch's grid).  The rows' own operands (s, r, b, agg, ...) come
+// with the tile (per-row vectors of the ring).
 template <typename V, typename T, typename BT>
-__global__ void __launch_bounds__(RING_THREADS, 4)
-    k_pre_ring(SellView<V> Ah, const BT* __restrict__ b, T* __restrict__ r, RingGeom g,
-               RingRows rows, int* fail) {
+__global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
+    k_pre_ring(const __grid_constant__ SellView<V> Ah, const BT* __restrict__ b,
+               T* __restrict__ r, const __grid_constant__ RingGeom g,
+               const __grid_constant__ RingRows rows, int* fail) {
   extern __shared__ unsigned char ring_smem[];
   if (*(volatile int*)fail) return;
-  RingWarp<V> ring(Ah, g, rows, ring_smem);
-  ring.start();
-  for (int64_t sl = ring.first; sl < Ah.nslices; sl += ring.nwt) {
-    const int64_t i = sl * 32 + ring.lane;
-    const bool has = i < Ah.n;
-    const T bi = has ? to_f(__ldg(b + i), T(0)) : T(0);  // overlaps the wait
-    if (!ring.wait()) {
+  TileRing<V> ring(Ah, g, rows, ring_smem);
+  if (ring.producer()) {
+    ring.produce(fail, nullptr);
+    return;
+  }
+  for (int64_t t = blockIdx.x; t < ring.ntiles; t += gridDim.x) {
+    if (!ring.wait(t)) {
       if (ring.lane == 0) ring_fail(fail, nullptr);
-      ring.drain();
       return;
     }
-    // pre_slice's arithmetic: from b_i down by negated FMAs
-    const T acc = ring_row_sum<T, true>(
-        ring, ring.width(), [&](int j) { return to_f(__ldg(b + j), T(0)); }, bi);
-    if (has) r[i] = acc;
+    if (ring.sl < Ah.nslices) {
+      const int64_t i = ring.sl * 32 + ring.lane;
+      const bool has = i < Ah.n;
+      const T bi = has ? to_f(ring.template row<BT>(0, i), T(0)) : T(0);
+      // pre_slice's arithmetic: from b_i down by negated FMAs
+      const T acc = ring_row_sum<T, true>(
+          ring, i, [&](int j) { return to_f(__ldg(b + j), T(0)); }, bi);
+      if (has) r[i] = acc;
+    }
     ring.release();
   }
 }
 
-template <typename V, typename T, typename BT, typename XT, int NDOT>
-__global__ void __launch_bounds__(RING_THREADS, 4)
-    k_post_ring(SellView<V> AP, const BT* __restrict__ b, const T* __restrict__ s,
-                const T* __restrict__ r, const int32_t* __restrict__ agg,
-                const T* __restrict__ xc, XT* __restrict__ x, const double* __restrict__ q,
-                Reduce red, PcgScalars* sc, RingGeom g, RingRows rows, int* fail) {
+// MS: several sweeps (xp the pre-smoothed x, e receives r - AP x_c), as in
+// k_post; per-row operands in the order s, r, b (MS: xp), agg, q.
+template <typename V, typename T, typename BT, typename XT, int NDOT, bool MS>
+__global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
+    k_post_ring(const __grid_constant__ SellView<V> AP, const T* __restrict__ xc,
+                XT* __restrict__ x, Reduce red, PcgScalars* sc,
+                const __grid_constant__ RingGeom g, const __grid_constant__ RingRows rows,
+                int* fail, T* __restrict__ e) {
   extern __shared__ unsigned char ring_smem[];
   if (*(volatile int*)fail) return;  // the host resets the reduction ticket
   constexpr int ND = NDOT > 0 ? NDOT : 1;
   double d[ND];
 #pragma unroll
   for (int k = 0; k < ND; ++k) d[k] = 0.0;
-  RingWarp<V> ring(AP, g, rows, ring_smem);
-  ring.start();
-  for (int64_t sl = ring.first; sl < AP.nslices; sl += ring.nwt) {
-    if (!ring.wait()) {
-      if (ring.lane == 0) ring_fail(fail, NDOT > 0 ? &sc->status : nullptr);
-      ring.drain();
-      break;
+  TileRing<V> ring(AP, g, rows, ring_smem);
+  if (ring.producer()) {
+    ring.produce(fail, NDOT > 0 ? &sc->status : nullptr);
+  } else {
+    for (int64_t t = blockIdx.x; t < ring.ntiles; t += gridDim.x) {
+      if (!ring.wait(t)) {
+        if (ring.lane == 0) ring_fail(fail, NDOT > 0 ? &sc->status : nullptr);
+        break;
+      }
+      if (ring.sl < AP.nslices) {
+        const int64_t i = ring.sl * 32 + ring.lane;
+        const bool has = i < AP.n;
+        // x_c of the row's own aggregate: gathered with the row's entries
+        const T xci = has ? __ldg(xc + ring.template row<int32_t>(3, i)) : T(0);
+        const T ri = has ? ring.template row<T>(1, i) : T(0);
+        if constexpr (MS) {
+          const T acc = ring_row_sum<T>(ring, i, [&](int J) { return __ldg(xc + J); });
+          if (has) {
+            const T si = ring.template row<T>(0, i);
+            const T yi = ring.template row<T>(2, i) + xci;
+            const T ei = ri - acc;
+            x[i] = to_f(fma(si, ei, yi), XT(0));
+            e[i] = ei;
+          }
+        } else {
+          // post_slice's arithmetic (one sweep): from b_i + r_i down, then one FMA
+          const BT bi = has ? ring.template row<BT>(2, i) : BT(0);
+          const T init = has ? to_f(bi, T(0)) + ri : T(0);
+          const T acc =
+              ring_row_sum<T, true>(ring, i, [&](int J) { return __ldg(xc + J); }, init);
+          if (has) {
+            const XT zi = to_f(fma(ring.template row<T>(0, i), acc, xci), XT(0));
+            x[i] = zi;
+            if constexpr (NDOT > 0) d[0] += (double)bi * (double)zi;
+            if constexpr (NDOT > 1)
+              d[NDOT > 1 ? 1 : 0] += (double)zi * ring.template row<double>(4, i);
+          }
+        }
+      }
+      ring.release();
     }
-    const bool f = ring.full(sl);
-    const int64_t i = sl * 32 + ring.lane;
-    const bool has = i < AP.n;
-    T si = T(0), ri = T(0);
-    BT bi = BT(0);
-    int32_t ai = 0;
-    double qi = 0.0;
-    if (has) {  // the row's operands, which came with the slice
-      si = ring.template row<T>(0, f, i);
-      ri = ring.template row<T>(1, f, i);
-      bi = ring.template row<BT>(2, f, i);
-      ai = ring.template row<int32_t>(3, f, i);
-      if constexpr (NDOT > 1) qi = ring.template row<double>(4, f, i);
+  }
+  if constexpr (NDOT > 0) grid_reduce<NDOT>(d, red, VcycleDotEpi{sc});
+}
+
+// Further sweeps (k_sweep_pre / k_sweep_post): per-row operands in the order
+// s, r, then (PRE) b before the first of them, else x (POST: y).
+template <bool PRE, typename V, typename T, typename BT, typename YT>
+__global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
+    k_sweep_ring(const __grid_constant__ SellView<V> Ah, const T* __restrict__ r,
+                 T* __restrict__ r_out, YT* __restrict__ x, int first,
+                 const __grid_constant__ RingGeom g, const __grid_constant__ RingRows rows,
+                 int* fail) {
+  extern __shared__ unsigned char ring_smem[];
+  if (*(volatile int*)fail) return;
+  TileRing<V> ring(Ah, g, rows, ring_smem);
+  if (ring.producer()) {
+    ring.produce(fail, nullptr);
+    return;
+  }
+  for (int64_t t = blockIdx.x; t < ring.ntiles; t += gridDim.x) {
+    if (!ring.wait(t)) {
+      if (ring.lane == 0) ring_fail(fail, nullptr);
+      return;
     }
-    // x_c of the row's own aggregate: gathered with the row's entries
-    const T xci = has ? __ldg(xc + ai) : T(0);
-    // post_slice's arithmetic (one sweep): from b_i + r_i down, then one FMA
-    const T init = has ? to_f(bi, T(0)) + ri : T(0);
-    const T acc =
-        ring_row_sum<T, true>(ring, ring.width(), [&](int J) { return __ldg(xc + J); }, init);
-    if (has) {
-      const XT zi = to_f(fma(si, acc, xci), XT(0));
-      x[i] = zi;
-      if constexpr (NDOT > 0) d[0] += (double)bi * (double)zi;
-      if constexpr (NDOT > 1) d[NDOT > 1 ? 1 : 0] += (double)zi * qi;
+    if (ring.sl < Ah.nslices) {
+      const int64_t i = ring.sl * 32 + ring.lane;
+      const bool has = i < Ah.n;
+      const T acc = ring_row_sum<T>(ring, i, [&](int j) { return __ldg(r + j); });
+      if (has) {
+        const T ri = ring.template row<T>(1, i);
+        const T rn = ri - acc;
+        r_out[i] = rn;
+        const T si = ring.template row<T>(0, i);
+        if constexpr (PRE) {
+          const T xi = first ? si * to_f(ring.template row<BT>(2, i), T(0))
+                             : ring.template row<T>(2, i);
+          x[i] = sweep_pre_x(xi, si, ri);
+        } else {
+          x[i] = sweep_post_y(ring.template row<YT>(2, i), si, rn);
+        }
+      }
     }
     ring.release();
   }
-  if constexpr (NDOT > 0) grid_reduce<NDOT>(d, red, VcycleDotEpi{sc});
 }
 
 // Post-smoother of a level with a smoothed prolongator P (Sec. 2.3; A P in
@@ -493,10 +547,12 @@ static int launch_pre(const amg_handle* H, const Level& L, const V* ah, const BT
   // FP64 and FP32 operators (BF16 values keep the per-lane kernels)
   if constexpr (sizeof(V) >= 4) {
     if (!act && H->opt.stream_ring) {
-      RingGeom g = ring_plan(L.A, (int)sizeof(V), ring_stages(H), RingRows());
+      RingRows rows;
+      rows.add(b, (int)sizeof(BT));
+      RingGeom g = ring_plan(L.A, (int)sizeof(V), ring_stages(H), rows);
       if (g.D) {
         AMG_TRY(ring_prepare((const void*)k_pre_ring<V, T, BT>, g, L.A.nslices, H->num_sms));
-        k_pre_ring<V, T, BT><<<g.grid, RING_THREADS, g.smem, s>>>(v, b, r, g, RingRows(),
+        k_pre_ring<V, T, BT><<<g.grid, g.threads(), g.smem, s>>>(v, b, r, g, rows,
                                                                  H->wait_fail);
         AMG_LAUNCH_CHECK();
         return AMG_OK;
@@ -529,6 +585,24 @@ static int launch_post(const amg_handle* H, const Level& L, const V* ap, const B
   const T* sc = (const T*)(sizeof(T) == 8 ? (const void*)L.s64 : (const void*)L.s32);
   const T* r = in.r ? in.r : (const T*)L.r;
   if constexpr (NDOT == 0) {
+    if constexpr (sizeof(V) >= 4) {
+      if (in.xp && !act && H->opt.stream_ring) {
+        RingRows rows;  // as read by k_post_ring<MS>
+        rows.add(sc, (int)sizeof(T));
+        rows.add(r, (int)sizeof(T));
+        rows.add(in.xp, (int)sizeof(T));
+        rows.add(L.agg, (int)sizeof(int32_t));
+        RingGeom g = ring_plan(L.AP, (int)sizeof(V), ring_stages(H), rows);
+        if (g.D) {
+          AMG_TRY(ring_prepare((const void*)k_post_ring<V, T, BT, XT, 0, true>, g, L.AP.nslices,
+                               H->num_sms));
+          k_post_ring<V, T, BT, XT, 0, true><<<g.grid, g.threads(), g.smem, s>>>(
+              v, xc, x, H->red, H->sc, g, rows, H->wait_fail, in.e);
+          AMG_LAUNCH_CHECK();
+          return AMG_OK;
+        }
+      }
+    }
     if (in.xp) {
       AMG_DISPATCH_TPR(sell_code(L.AP),
                        (k_post<TPR, V, T, BT, XT, 0, true><<<grid, SELL_BLOCK, 0, s>>>(
@@ -546,12 +620,12 @@ static int launch_post(const amg_handle* H, const Level& L, const V* ap, const B
       rows.add(b, (int)sizeof(BT));
       rows.add(L.agg, (int)sizeof(int32_t));
       if (NDOT > 1) rows.add(q, (int)sizeof(double));
-      RingGeom g = ring_plan(L.AP, (int)sizeof(V), ring_stages(H), rows);
+      RingGeom g = ring_plan(L.AP, (int)sizeof(V), ring_stages(H), rows, NDOT > 0);
       if (g.D) {
-        AMG_TRY(ring_prepare((const void*)k_post_ring<V, T, BT, XT, NDOT>, g, L.AP.nslices,
-                             H->num_sms));
-        k_post_ring<V, T, BT, XT, NDOT><<<g.grid, RING_THREADS, g.smem, s>>>(
-            v, b, sc, r, L.agg, xc, x, q, H->red, H->sc, g, rows, H->wait_fail);
+        AMG_TRY(ring_prepare((const void*)k_post_ring<V, T, BT, XT, NDOT, false>, g,
+                             L.AP.nslices, H->num_sms));
+        k_post_ring<V, T, BT, XT, NDOT, false><<<g.grid, g.threads(), g.smem, s>>>(
+            v, xc, x, H->red, H->sc, g, rows, H->wait_fail, nullptr);
         AMG_LAUNCH_CHECK();
         return AMG_OK;
       }
@@ -587,6 +661,26 @@ static int launch_sweep(const amg_handle* H, const Level& L, const BT* b, const 
     using V = decltype(vtag);
     SellView<V> v = view<V>(L.A, ah);
     v.act = act;
+    if constexpr (sizeof(V) >= 4) {
+      if (!act && H->opt.stream_ring) {
+        RingRows rows;
+        rows.add(sc, (int)sizeof(T));
+        rows.add(r, (int)sizeof(T));
+        if (PRE && first)
+          rows.add(b, (int)sizeof(BT));
+        else
+          rows.add(x, (int)sizeof(YT));
+        RingGeom g = ring_plan(L.A, (int)sizeof(V), ring_stages(H), rows);
+        if (g.D) {
+          AMG_TRY(ring_prepare((const void*)k_sweep_ring<PRE, V, T, BT, YT>, g, L.A.nslices,
+                               H->num_sms));
+          k_sweep_ring<PRE, V, T, BT, YT><<<g.grid, g.threads(), g.smem, s>>>(
+              v, r, r_out, x, first, g, rows, H->wait_fail);
+          AMG_LAUNCH_CHECK();
+          return AMG_OK;
+        }
+      }
+    }
     if constexpr (PRE) {
       AMG_DISPATCH_TPR(sell_code(L.A), (k_sweep_pre<TPR, V, T, BT><<<grid, SELL_BLOCK, 0, s>>>(
                                             v, sc, b, r, r_out, (T*)x, first)));
