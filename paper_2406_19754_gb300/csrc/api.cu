@@ -192,7 +192,10 @@ static int create(const amg_csr* A, const amg_options* opt, cudaStream_t s, amg_
   AMG_TRY(ar.alloc_n(&H->sc, 1));
   AMG_CUDA_TRY(cudaMemsetAsync(H->sc, 0, sizeof(PcgScalars), s));
   if (!systems) AMG_TRY(pattern_hash(A, &H->pattern, s, H->num_sms));
-  AMG_TRY(setup_hierarchy(H, A, s, like));
+  ar.begin_reuse();
+  AMG_TRY(setup_hierarchy(H, A, s, like));  // on error the caller destroys H
+  AMG_CUDA_TRY(cudaStreamSynchronize(s));
+  ar.end_reuse();
   const int64_t n = A->n;
   AMG_TRY(ar.alloc_n(&H->r, n));
   AMG_TRY(ar.alloc_n(&H->z, n));
@@ -444,7 +447,7 @@ int amg_pairwise_match(const amg_csr* A, int32_t* mate, int* rounds, amg_stream_
   if (rc < 0) return rc;
   if (!mate) return AMG_ERR_ARG;
   Arena ar;
-  rc = match_pairwise(ar, A->n, A->rowptr, A->col, A->val, mate, rounds, (cudaStream_t)stream);
+  rc = match_pairwise(ar, A->n, A->nnz, A->rowptr, A->col, A->val, mate, rounds, (cudaStream_t)stream);
   cudaStreamSynchronize((cudaStream_t)stream);
   ar.release_all();
   return rc;

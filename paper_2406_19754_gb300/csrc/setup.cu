@@ -85,14 +85,45 @@ __device__ __forceinline__ bool heavier(const EdgeKey& a, const EdgeKey& b) {
   return a.hi < b.hi;
 }
 
+// Weight of edge {i, j} from its stored value and the two diagonals.
+__device__ __forceinline__ double match_weight(double a, double di, double dj) {
+  return __dsub_rn(1.0, __ddiv_rn(__dmul_rn(2.0, a), __dadd_rn(di, dj)));
+}
+
+// All edge weights once, into both rows' slots (0, never eligible, where there
+// is none); entry e's weight is w[e - rowptr[0]].  A row is re-examined whenever a neighbour is matched, and each
+// look at an edge from its larger endpoint searched the other row for the
+// stored value and divided again on the reduced-rate FP64 pipe (a 128^3
+// diffusion setup spent 7.3 ms in k_match_cand).
+__global__ void k_match_weights(int64_t n, const int64_t* __restrict__ rowptr,
+                                const int32_t* __restrict__ col, const double* __restrict__ val,
+                                const double* __restrict__ diag, double* __restrict__ w) {
+  const int64_t e0 = rowptr[0];
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t i = (int32_t)t;
+    const double di = diag[i];
+    for (int64_t e = rowptr[i]; e < rowptr[i + 1]; ++e) {
+      const int32_t j = col[e];
+      double a;
+      double c = 0.0;
+      // the entry of the smaller row, found from either side
+      if (j != i && edge_value(rowptr, col, val, i, j, val[e], &a)) c = match_weight(a, di, diag[j]);
+      w[e - e0] = c;
+    }
+  }
+}
+
 // mate[i]: >= 0 matched, -1 active, -2 no eligible partner left (singleton).
 // flag[i]: 1 while i sits on the next frontier list.
 __global__ void k_match_cand(const int32_t* __restrict__ wl, const int* __restrict__ nwl,
                              const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                              const double* __restrict__ val, const double* __restrict__ diag,
-                             const int32_t* __restrict__ mate, int32_t* __restrict__ cand,
-                             int32_t* __restrict__ flag, int* rounds) {
+                             const double* __restrict__ w, const int32_t* __restrict__ mate,
+                             int32_t* __restrict__ cand, int32_t* __restrict__ flag,
+                             int* rounds) {
   const int nw = *nwl;
+  const int64_t e0 = rowptr[0];
   if (blockIdx.x == 0 && threadIdx.x == 0 && nw > 0) ++*rounds;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nw; t += gridDim.x * blockDim.x) {
     const int32_t i = wl[t];
@@ -104,9 +135,14 @@ __global__ void k_match_cand(const int32_t* __restrict__ wl, const int* __restri
     for (int64_t e = rowptr[i]; e < rowptr[i + 1]; ++e) {
       const int32_t j = col[e];
       if (j == i || mate[j] != -1) continue;
-      double a;
-      if (!edge_value(rowptr, col, val, i, j, val[e], &a)) continue;
-      const double c = __dsub_rn(1.0, __ddiv_rn(__dmul_rn(2.0, a), __dadd_rn(di, diag[j])));
+      double c;
+      if (w) {
+        c = w[e - e0];
+      } else {
+        double a;
+        if (!edge_value(rowptr, col, val, i, j, val[e], &a)) continue;
+        c = match_weight(a, di, diag[j]);
+      }
       if (!(c > 0.0)) continue;
       EdgeKey k;
       k.c = c;
@@ -122,9 +158,11 @@ __global__ void k_match_cand(const int32_t* __restrict__ wl, const int* __restri
 }
 
 // Mutual pointers match; a vertex without an eligible neighbour is final.
+// nwl_next: the next frontier's size, cleared for k_match_expand.
 __global__ void k_match_commit(const int32_t* __restrict__ wl, const int* __restrict__ nwl,
-                               const int32_t* __restrict__ cand, int32_t* mate) {
+                               const int32_t* __restrict__ cand, int32_t* mate, int* nwl_next) {
   const int nw = *nwl;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *nwl_next = 0;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nw; t += gridDim.x * blockDim.x) {
     const int32_t i = wl[t];
     if (mate[i] != -1) continue;
@@ -177,12 +215,13 @@ __global__ void k_match_counts(int* cnt, int n) {
 
 // The rounds of locally-dominant matching on caller-provided scratch: cand
 // and flag hold n entries, wl two frontiers of n entries at wl and
-// wl + wl_stride, cnt 4 ints.  Every entry point that matches runs this loop,
+// wl + wl_stride, cnt 4 ints, w every entry's edge weight or null (computed on
+// every look then).  Every entry point that matches runs this loop,
 // so they launch the same kernels in the same order.
 int match_round_loop(int64_t n, const int64_t* rowptr, const int32_t* col, const double* val,
-                     const double* diag, int32_t* mate, int32_t* cand, int32_t* flag,
-                     int32_t* wl, int64_t wl_stride, int* cnt, int* rounds_out, int num_sms,
-                     cudaStream_t s) {
+                     const double* diag, const double* w_edge, int32_t* mate, int32_t* cand,
+                     int32_t* flag, int32_t* wl, int64_t wl_stride, int* cnt, int* rounds_out,
+                     int num_sms, cudaStream_t s) {
   // scratch may hold an earlier call's contents: reset what must start at zero
   AMG_CUDA_TRY(cudaMemsetAsync(mate, 0xFF, sizeof(int32_t) * n, s));
   AMG_CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(int32_t) * n, s));
@@ -194,23 +233,25 @@ int match_round_loop(int64_t n, const int64_t* rowptr, const int32_t* col, const
   int cur = 0;
   int rc = AMG_OK;
   int64_t launched = 0;
+  int work = grid;  // CTAs for the last known frontier (the kernels stride over any size)
   for (;;) {
-    // a batch of rounds between host checks; empty rounds exit immediately
-    for (int r = 0; r < 8; ++r) {
+    // a batch of rounds between host checks; empty rounds exit immediately.
+    // Long runs of rounds (chains on regular grids) get longer batches.
+    const int batch = launched < 32 ? 8 : 16;
+    for (int r = 0; r < batch; ++r) {
       int32_t* w = wl + (int64_t)cur * wl_stride;
       int32_t* wn = wl + (int64_t)(1 - cur) * wl_stride;
-      k_match_cand<<<grid, 256, 0, s>>>(w, cnt + cur, rowptr, col, val, diag, mate, cand, flag,
-                                        cnt + 2);
+      k_match_cand<<<work, 256, 0, s>>>(w, cnt + cur, rowptr, col, val, diag, w_edge, mate, cand,
+                                        flag, cnt + 2);
       AMG_LAUNCH_CHECK();
-      k_match_commit<<<grid, 256, 0, s>>>(w, cnt + cur, cand, mate);
+      k_match_commit<<<work, 256, 0, s>>>(w, cnt + cur, cand, mate, cnt + 1 - cur);
       AMG_LAUNCH_CHECK();
-      AMG_CUDA_TRY(cudaMemsetAsync(cnt + 1 - cur, 0, sizeof(int), s));
-      k_match_expand<<<grid, 256, 0, s>>>(w, cnt + cur, rowptr, col, mate, flag, wn,
+      k_match_expand<<<work, 256, 0, s>>>(w, cnt + cur, rowptr, col, mate, flag, wn,
                                           cnt + 1 - cur);
       AMG_LAUNCH_CHECK();
       cur = 1 - cur;
     }
-    launched += 8;
+    launched += batch;
     int h[4];
     AMG_CUDA_TRY(cudaMemcpyAsync(h, cnt, sizeof(h), cudaMemcpyDeviceToHost, s));
     AMG_CUDA_TRY(cudaStreamSynchronize(s));
@@ -218,6 +259,7 @@ int match_round_loop(int64_t n, const int64_t* rowptr, const int32_t* col, const
       if (rounds_out) *rounds_out = h[2];
       break;
     }
+    work = std::min(grid, grid_for(2 * (int64_t)h[cur], 256, num_sms, 8));
     if (launched > 4 * n + 64) {  // each round matches at least the heaviest edge
       rc = AMG_ERR_DEVICE_CHECK;
       break;
@@ -229,8 +271,8 @@ int match_round_loop(int64_t n, const int64_t* rowptr, const int32_t* col, const
   return rc;
 }
 
-static int match_rounds(Arena& ar, int64_t n, const int64_t* rowptr, const int32_t* col,
-                        const double* val, const double* diag, int32_t* mate, int* rounds_out,
+static int match_rounds(Arena& ar, int64_t n, int64_t nnz, const int64_t* rowptr,
+                        const int32_t* col, const double* val, const double* diag, int32_t* mate, int* rounds_out,
                         int num_sms, cudaStream_t s) {
   int32_t *cand = nullptr, *flag = nullptr, *wl = nullptr;
   int* cnt = nullptr;  // [0], [1]: frontier sizes; [2]: rounds with a non-empty frontier
@@ -238,8 +280,13 @@ static int match_rounds(Arena& ar, int64_t n, const int64_t* rowptr, const int32
   AMG_TRY(ar.alloc_n(&flag, n));
   AMG_TRY(ar.alloc_n(&wl, 2 * n));
   AMG_TRY(ar.alloc_n(&cnt, 4));
-  const int rc = match_round_loop(n, rowptr, col, val, diag, mate, cand, flag, wl, n, cnt,
+  double* w = nullptr;
+  AMG_TRY(ar.alloc_n(&w, nnz));
+  k_match_weights<<<grid_for(n, 256, num_sms, 8), 256, 0, s>>>(n, rowptr, col, val, diag, w);
+  AMG_LAUNCH_CHECK();
+  const int rc = match_round_loop(n, rowptr, col, val, diag, w, mate, cand, flag, wl, n, cnt,
                                   rounds_out, num_sms, s);
+  ar.release(w);
   ar.release(cand);
   ar.release(flag);
   ar.release(wl);
@@ -247,8 +294,8 @@ static int match_rounds(Arena& ar, int64_t n, const int64_t* rowptr, const int32
   return rc;
 }
 
-int match_pairwise(Arena& ar, int64_t n, const int64_t* rowptr, const int32_t* col,
-                   const double* val, int32_t* mate, int* rounds, cudaStream_t s) {
+int match_pairwise(Arena& ar, int64_t n, int64_t nnz, const int64_t* rowptr,
+                   const int32_t* col, const double* val, int32_t* mate, int* rounds, cudaStream_t s) {
   int dev = 0, sms = 0;
   AMG_CUDA_TRY(cudaGetDevice(&dev));
   AMG_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -256,7 +303,7 @@ int match_pairwise(Arena& ar, int64_t n, const int64_t* rowptr, const int32_t* c
   AMG_TRY(ar.alloc_n(&diag, n));
   k_l1_diag<<<grid_for(n, 256, sms, 8), 256, 0, s>>>(n, rowptr, col, val, nullptr, diag);
   AMG_LAUNCH_CHECK();
-  int rc = match_rounds(ar, n, rowptr, col, val, diag, mate, rounds, sms, s);
+  int rc = match_rounds(ar, n, nnz, rowptr, col, val, diag, mate, rounds, sms, s);
   AMG_CUDA_TRY(cudaStreamSynchronize(s));
   ar.release(diag);
   return rc;
@@ -340,9 +387,17 @@ static int build_members(Arena& ar, int64_t n, const int32_t* agg, int64_t nc, i
 // (A_c)_IJ = sum of a_ij over agg(i) = I, agg(j) = J, added left to right in
 // ascending (min(i,j), max(i,j), [i > j]) order.  For each coarse row a team
 // (one warp, or one block for long rows) stages the contributions of its
-// member rows in shared memory, sorts them by (J, min, max, flip) with a
-// bitonic network and adds each J-run sequentially.
+// member rows in shared memory, orders them by (J, min, max, flip) and adds
+// each J-run sequentially.  Rows of up to GAL_SMALL contributions (nearly all
+// rows of stencil hierarchies: 2 or 4 members of 7 to 14 entries) are ordered
+// by rank: each lane counts the smaller keys among all of them (broadcast
+// reads, no exchanges), and the count pass compares aggregates only.  The
+// bitonic network that longer rows use took 15 to 21 compare-exchange steps
+// through shared memory, twice (a 128^3 diffusion setup spent 16.2 ms in it).
 
+constexpr int GAL_SMALL = 64;       // contributions of a rank-ordered row: two per lane
+constexpr int GAL_SMALL_WARPS = 8;
+constexpr int GAL_SMALL_MEMBERS = 32;  // members of such a row: one per lane
 constexpr int GAL_WARP_CAP = 512;   // contributions per warp-staged row
 constexpr int GAL_WARPS = 4;        // warps per block in the warp kernel
 constexpr int GAL_BLOCK_CAP = 8192; // contributions per block-staged row
@@ -397,6 +452,8 @@ struct GalArgs {
   const int64_t* rowptr_c;  // fill pass
   int32_t* col_c;
   double* val_c;
+  int32_t* mid_list;      // rows the warp kernel sorts
+  int* mid_count;
   int32_t* ovf_list;      // rows staged by the block kernel
   int* ovf_count;
   int* status;
@@ -445,6 +502,132 @@ __device__ __forceinline__ int next_pow2(int x) {
   return p;
 }
 
+// Rows of at most GAL_SMALL contributions, one warp each; the others are
+// listed for k_galerkin_warp (count pass) or skipped (fill pass).
+template <bool FILL>
+__global__ void __launch_bounds__(GAL_SMALL_WARPS * 32) k_galerkin_small(GalArgs g) {
+  __shared__ ulonglong2 keys[GAL_SMALL_WARPS][GAL_SMALL];
+  __shared__ double vals[GAL_SMALL_WARPS][GAL_SMALL];
+  __shared__ int32_t cols[GAL_SMALL_WARPS][GAL_SMALL];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  ulonglong2* key = keys[wib];
+  double* sv = vals[wib];
+  int32_t* sj = cols[wib];
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t I = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; I < g.nc; I += nw) {
+    // lane s: member s, its row's bounds, and where its entries go
+    int64_t tot64 = GAL_SMALL + 1;
+    int32_t m = -1;
+    int64_t beg = 0;
+    int len = 0, end = 0;
+    if (g.stride <= GAL_SMALL_MEMBERS) {
+      m = lane < g.stride ? g.members[I * g.stride + lane] : -1;
+      if (m >= 0) {
+        beg = g.rowptr[m];
+        const int64_t l = g.rowptr[m + 1] - beg;
+        len = l <= GAL_SMALL ? (int)l : GAL_SMALL + 1;
+      }
+      end = len;
+      for (int o = 1; o < g.stride; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, end, o);
+        if (lane >= o) end += t;
+      }
+      tot64 = __shfl_sync(0xffffffffu, end, g.stride - 1);
+    }
+    if (tot64 > GAL_SMALL) {
+      if (!FILL && lane == 0) {
+        g.mid_list[atomicAdd(g.mid_count, 1)] = (int32_t)I;
+        g.cnt[I] = 0;
+      }
+      continue;
+    }
+    const int total = (int)tot64;
+    // entries p = lane and lane + 32
+    int32_t J[2];
+    ulonglong2 k[2];
+    double v[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int p = lane + 32 * u;
+      int32_t row = -1;
+      int64_t e = 0;
+      for (int s = 0; s < g.stride; ++s) {
+        const int se = __shfl_sync(0xffffffffu, end, s), sl = __shfl_sync(0xffffffffu, len, s);
+        const int32_t sm = __shfl_sync(0xffffffffu, m, s);
+        const int64_t sb = __shfl_sync(0xffffffffu, beg, s);
+        if (p >= se - sl && p < se) {
+          row = sm;
+          e = sb + (p - (se - sl));
+        }
+      }
+      J[u] = -1;
+      if (row >= 0) {
+        const int32_t j = g.col[e];
+        J[u] = g.agg[j];
+        if constexpr (FILL) {
+          v[u] = g.val[e];
+          k[u].x = ((uint64_t)(uint32_t)J[u] << 32) | (uint32_t)min(row, j);
+          k[u].y = ((uint64_t)(uint32_t)max(row, j) << 1) | (uint64_t)(row > j ? 1 : 0);
+        }
+      }
+    }
+    if constexpr (!FILL) {
+      // distinct aggregates: entries no earlier entry shares its aggregate with
+      sj[lane] = J[0];
+      sj[lane + 32] = J[1];
+      __syncwarp();
+      bool d0 = J[0] >= 0, d1 = J[1] >= 0;
+      for (int t = 0; t < total; ++t) {
+        const int32_t jt = sj[t];
+        if (jt == J[0] && t < lane) d0 = false;
+        if (jt == J[1] && t < lane + 32) d1 = false;
+      }
+      const int c = __popc(__ballot_sync(0xffffffffu, d0)) +
+                    __popc(__ballot_sync(0xffffffffu, d1));
+      if (lane == 0) g.cnt[I] = c;
+      __syncwarp();
+    } else {
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (J[u] >= 0) key[lane + 32 * u] = k[u];
+      __syncwarp();
+      int r0 = 0, r1 = 0;
+      for (int t = 0; t < total; ++t) {
+        const ulonglong2 kt = key[t];
+        r0 += gless(kt.x, kt.y, k[0].x, k[0].y) ? 1 : 0;
+        r1 += gless(kt.x, kt.y, k[1].x, k[1].y) ? 1 : 0;
+      }
+      if (J[0] >= 0) {
+        sv[r0] = v[0];
+        sj[r0] = J[0];
+      }
+      if (J[1] >= 0) {
+        sv[r1] = v[1];
+        sj[r1] = J[1];
+      }
+      __syncwarp();
+      const int64_t off = g.rowptr_c[I];
+      int base = 0;
+      for (int c = 0; c < total; c += 32) {
+        const int p = c + lane;
+        const bool st = p < total && (p == 0 || sj[p] != sj[p - 1]);
+        const unsigned msk = __ballot_sync(0xffffffffu, st);
+        if (st) {
+          const int rank = base + __popc(msk & ((1u << lane) - 1u));
+          const int32_t Jp = sj[p];
+          double s = sv[p];
+          for (int q = p + 1; q < total && sj[q] == Jp; ++q) s = __dadd_rn(s, sv[q]);
+          g.col_c[off + rank] = Jp;
+          g.val_c[off + rank] = s;
+        }
+        base += __popc(msk);
+      }
+      __syncwarp();
+    }
+  }
+}
+
+// The listed rows, one warp each (contributions sorted in shared memory).
 template <bool FILL>
 __global__ void __launch_bounds__(GAL_WARPS * 32) k_galerkin_warp(GalArgs g) {
   extern __shared__ unsigned char smem[];
@@ -454,7 +637,9 @@ __global__ void __launch_bounds__(GAL_WARPS * 32) k_galerkin_warp(GalArgs g) {
   double* v = (double*)((uint64_t*)smem + (size_t)2 * GAL_WARPS * GAL_WARP_CAP) +
               (size_t)wib * GAL_WARP_CAP;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t I = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; I < g.nc; I += nw) {
+  const int64_t nmid = *g.mid_count;
+  for (int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < nmid; q += nw) {
+    const int64_t I = g.mid_list[q];
     const int64_t tot64 = gal_total(g, I);
     if (tot64 > GAL_WARP_CAP) {
       if (!FILL && lane == 0) {
@@ -478,7 +663,7 @@ __global__ void __launch_bounds__(GAL_WARPS * 32) k_galerkin_warp(GalArgs g) {
         const int rank = base + __popc(msk & ((1u << lane) - 1u));
         const uint64_t J = k1[p] >> 32;
         double s = v[p];
-        for (int q = p + 1; q < total && (k1[q] >> 32) == J; ++q) s = __dadd_rn(s, v[q]);
+        for (int f = p + 1; f < total && (k1[f] >> 32) == J; ++f) s = __dadd_rn(s, v[f]);
         g.col_c[off + rank] = (int32_t)J;
         g.val_c[off + rank] = s;
       }
@@ -550,23 +735,33 @@ static int galerkin(Arena& ar, int64_t n, const int64_t* rowptr, const int32_t* 
   AMG_TRY(ar.alloc_n(&g.cnt, nc + 1));
   AMG_CUDA_TRY(cudaMemsetAsync(g.cnt, 0, sizeof(int64_t) * (nc + 1), s));
   AMG_TRY(ar.alloc_n(&g.ovf_list, nc));
-  AMG_TRY(ar.alloc_n(&g.ovf_count, 1));
-  AMG_CUDA_TRY(cudaMemsetAsync(g.ovf_count, 0, sizeof(int), s));
+  AMG_TRY(ar.alloc_n(&g.mid_list, nc));
+  AMG_TRY(ar.alloc_n(&g.ovf_count, 2));
+  AMG_CUDA_TRY(cudaMemsetAsync(g.ovf_count, 0, 2 * sizeof(int), s));
+  g.mid_count = g.ovf_count + 1;
   const size_t wsm = (size_t)GAL_WARPS * GAL_WARP_CAP * 24;
   const size_t bsm = (size_t)GAL_BLOCK_CAP * 24;
   AMG_CUDA_TRY(cudaFuncSetAttribute(k_galerkin_block<false>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsm));
   AMG_CUDA_TRY(cudaFuncSetAttribute(k_galerkin_block<true>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsm));
-  const int wgrid = grid_for(nc * 32, GAL_WARPS * 32, num_sms, 16);
+  const int sgrid = grid_for(nc * 32, GAL_SMALL_WARPS * 32, num_sms, 8);
   g.rowptr_c = nullptr;
   g.col_c = nullptr;
   g.val_c = nullptr;
-  k_galerkin_warp<false><<<wgrid, GAL_WARPS * 32, wsm, s>>>(g);
+  k_galerkin_small<false><<<sgrid, GAL_SMALL_WARPS * 32, 0, s>>>(g);
   AMG_LAUNCH_CHECK();
-  int novf = 0;
-  AMG_CUDA_TRY(cudaMemcpyAsync(&novf, g.ovf_count, sizeof(int), cudaMemcpyDeviceToHost, s));
+  int more[2] = {0, 0};  // rows of the block kernel, of the warp kernel
+  AMG_CUDA_TRY(cudaMemcpyAsync(more, g.ovf_count, sizeof(more), cudaMemcpyDeviceToHost, s));
   AMG_CUDA_TRY(cudaStreamSynchronize(s));
+  const int wgrid = grid_for((int64_t)more[1] * 32, GAL_WARPS * 32, num_sms, 16);
+  if (more[1] > 0) {
+    k_galerkin_warp<false><<<wgrid, GAL_WARPS * 32, wsm, s>>>(g);
+    AMG_LAUNCH_CHECK();
+    AMG_CUDA_TRY(cudaMemcpyAsync(more, g.ovf_count, sizeof(int), cudaMemcpyDeviceToHost, s));
+    AMG_CUDA_TRY(cudaStreamSynchronize(s));
+  }
+  const int novf = more[0];
   if (novf > 0) {
     k_galerkin_block<false><<<std::min(novf, num_sms * 2), GAL_BLOCK_THREADS, bsm, s>>>(g, novf);
     AMG_LAUNCH_CHECK();
@@ -580,14 +775,19 @@ static int galerkin(Arena& ar, int64_t n, const int64_t* rowptr, const int32_t* 
   g.rowptr_c = *rp_c;
   g.col_c = *col_c;
   g.val_c = *val_c;
-  k_galerkin_warp<true><<<wgrid, GAL_WARPS * 32, wsm, s>>>(g);
+  k_galerkin_small<true><<<sgrid, GAL_SMALL_WARPS * 32, 0, s>>>(g);
   AMG_LAUNCH_CHECK();
+  if (more[1] > 0) {
+    k_galerkin_warp<true><<<wgrid, GAL_WARPS * 32, wsm, s>>>(g);
+    AMG_LAUNCH_CHECK();
+  }
   if (novf > 0) {
     k_galerkin_block<true><<<std::min(novf, num_sms * 2), GAL_BLOCK_THREADS, bsm, s>>>(g, novf);
     AMG_LAUNCH_CHECK();
   }
   AMG_CUDA_TRY(cudaStreamSynchronize(s));
   ar.release(g.cnt);
+  ar.release(g.mid_list);
   ar.release(g.ovf_list);
   ar.release(g.ovf_count);
   return AMG_OK;
@@ -613,164 +813,6 @@ __global__ void k_dense_blocks(const int64_t* rowptr, const int32_t* col, const 
       else
         atomicExch(status, AMG_ERR_DEVICE_CHECK);  // an entry coupling two blocks
     }
-}
-
-// Right-looking Cholesky of each block; the dense copy becomes L in its lower
-// triangle.  Then L^-1 (one column per thread) and its transpose.
-__global__ void k_cholesky(const int64_t* brow, const int64_t* bmat, double* dense,
-                           double* Linv_all, double* LinvT_all, int* status) {
-  const int n = (int)(brow[blockIdx.x + 1] - brow[blockIdx.x]);
-  double* a = dense + bmat[blockIdx.x];
-  double* Linv = Linv_all + bmat[blockIdx.x];
-  double* LinvT = LinvT_all + bmat[blockIdx.x];
-  __shared__ int ok;
-  for (int k = 0; k < n; ++k) {
-    if (threadIdx.x == 0) {
-      const double piv = a[(int64_t)k * n + k];
-      ok = piv > 0.0;
-      if (ok) a[(int64_t)k * n + k] = sqrt(piv);
-    }
-    __syncthreads();
-    if (!ok) {
-      if (threadIdx.x == 0) atomicExch(status, AMG_ERR_NOT_SPD);
-      return;
-    }
-    const double lkk = a[(int64_t)k * n + k];
-    for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x)
-      a[(int64_t)i * n + k] = __ddiv_rn(a[(int64_t)i * n + k], lkk);
-    __syncthreads();
-    const int m = n - k - 1;
-    for (int64_t idx = threadIdx.x; idx < (int64_t)m * m; idx += blockDim.x) {
-      const int ii = (int)(idx / m), jj = (int)(idx % m);
-      if (jj <= ii) {
-        const int i = k + 1 + ii, j = k + 1 + jj;
-        a[(int64_t)i * n + j] = __dsub_rn(a[(int64_t)i * n + j],
-                                          __dmul_rn(a[(int64_t)i * n + k], a[(int64_t)j * n + k]));
-      }
-    }
-    __syncthreads();
-  }
-  // column c of L^-1 by forward substitution on e_c
-  for (int c = threadIdx.x; c < n; c += blockDim.x) {
-    for (int i = 0; i < c; ++i) Linv[(int64_t)i * n + c] = 0.0;
-    for (int i = c; i < n; ++i) {
-      double s = (i == c) ? 1.0 : 0.0;
-      for (int k = c; k < i; ++k)
-        s = __dsub_rn(s, __dmul_rn(a[(int64_t)i * n + k], Linv[(int64_t)k * n + c]));
-      Linv[(int64_t)i * n + c] = __ddiv_rn(s, a[(int64_t)i * n + i]);
-    }
-  }
-  __syncthreads();
-  for (int64_t idx = threadIdx.x; idx < (int64_t)n * n; idx += blockDim.x) {
-    const int i = (int)(idx / n), j = (int)(idx % n);
-    LinvT[(int64_t)j * n + i] = Linv[idx];
-  }
-}
-
-// Blocked right-looking Cholesky for large coarsest blocks (several CUDA
-// blocks per step).  Every entry receives the same rank-1 updates, in the
-// same column order and with the same explicitly rounded operations, as in
-// the one-block kernel above, so both produce the same factor bit for bit.
-constexpr int CHOL_NB = 32;
-
-// Factor the diagonal tile [kb, kb+nb) in place (one CUDA block).
-__global__ void k_chol_diag(double* a, int64_t n, int64_t kb, int nb, int* status) {
-  __shared__ int ok;
-  for (int k = 0; k < nb; ++k) {
-    const int64_t kk = kb + k;
-    if (threadIdx.x == 0) {
-      const double piv = a[kk * n + kk];
-      ok = piv > 0.0;
-      if (ok) a[kk * n + kk] = sqrt(piv);
-    }
-    __syncthreads();
-    if (!ok) {
-      if (threadIdx.x == 0) atomicExch(status, AMG_ERR_NOT_SPD);
-      return;
-    }
-    const double lkk = a[kk * n + kk];
-    for (int i = k + 1 + threadIdx.x; i < nb; i += blockDim.x)
-      a[(kb + i) * n + kk] = __ddiv_rn(a[(kb + i) * n + kk], lkk);
-    __syncthreads();
-    const int m = nb - k - 1;
-    for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
-      const int ii = idx / m, jj = idx % m;
-      if (jj <= ii) {
-        const int64_t i = kb + k + 1 + ii, j = kb + k + 1 + jj;
-        a[i * n + j] = __dsub_rn(a[i * n + j], __dmul_rn(a[i * n + kk], a[j * n + kk]));
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// Panel below the tile: row i >= kb+nb, columns k = kb..kb+nb-1 in order.
-__global__ void k_chol_panel(double* a, int64_t n, int64_t kb, int nb) {
-  for (int64_t i = kb + nb + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    for (int k = 0; k < nb; ++k) {
-      const int64_t kk = kb + k;
-      double v = a[i * n + kk];
-      for (int q = 0; q < k; ++q)
-        v = __dsub_rn(v, __dmul_rn(a[i * n + kb + q], a[kk * n + kb + q]));
-      a[i * n + kk] = __ddiv_rn(v, a[kk * n + kk]);
-    }
-  }
-}
-
-// Trailing update: a_ij -= l_ik l_jk for k = kb..kb+nb-1 in order, j <= i.
-__global__ void k_chol_update(double* a, int64_t n, int64_t kb, int nb) {
-  const int64_t t0 = kb + nb, m = n - t0;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < m * m;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t ii = idx / m, jj = idx % m;
-    if (jj > ii) continue;
-    const int64_t i = t0 + ii, j = t0 + jj;
-    double v = a[i * n + j];
-    for (int k = 0; k < nb; ++k)
-      v = __dsub_rn(v, __dmul_rn(a[i * n + kb + k], a[j * n + kb + k]));
-    a[i * n + j] = v;
-  }
-}
-
-// Column c of L^-1 per thread (forward substitution on e_c), then L^-T.
-__global__ void k_tri_inverse(const double* a, int64_t n, double* Linv) {
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-       c += (int64_t)gridDim.x * blockDim.x) {
-    for (int64_t i = 0; i < c; ++i) Linv[i * n + c] = 0.0;
-    for (int64_t i = c; i < n; ++i) {
-      double s = (i == c) ? 1.0 : 0.0;
-      for (int64_t k = c; k < i; ++k) s = __dsub_rn(s, __dmul_rn(a[i * n + k], Linv[k * n + c]));
-      Linv[i * n + c] = __ddiv_rn(s, a[i * n + i]);
-    }
-  }
-}
-
-__global__ void k_transpose(const double* in, int64_t n, double* out) {
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n * n;
-       idx += (int64_t)gridDim.x * blockDim.x)
-    out[(idx % n) * n + idx / n] = in[idx];
-}
-
-static int chol_blocked(double* a, int64_t n, double* Linv, double* LinvT, int* status,
-                        int num_sms, cudaStream_t s) {
-  for (int64_t kb = 0; kb < n; kb += CHOL_NB) {
-    const int nb = (int)std::min<int64_t>(CHOL_NB, n - kb);
-    k_chol_diag<<<1, 256, 0, s>>>(a, n, kb, nb, status);
-    AMG_LAUNCH_CHECK();
-    if (kb + nb < n) {
-      k_chol_panel<<<grid_for(n - kb - nb, 128, num_sms, 4), 128, 0, s>>>(a, n, kb, nb);
-      AMG_LAUNCH_CHECK();
-      const int64_t m = n - kb - nb;
-      k_chol_update<<<grid_for(m * m, 256, num_sms, 8), 256, 0, s>>>(a, n, kb, nb);
-      AMG_LAUNCH_CHECK();
-    }
-  }
-  k_tri_inverse<<<grid_for(n, 64, num_sms, 8), 64, 0, s>>>(a, n, Linv);
-  AMG_LAUNCH_CHECK();
-  k_transpose<<<grid_for(n * n, 256, num_sms, 8), 256, 0, s>>>(Linv, n, LinvT);
-  AMG_LAUNCH_CHECK();
-  return AMG_OK;
 }
 
 // ------------------------------------------------------------------ V-cycle operators
@@ -1167,7 +1209,7 @@ int setup_hierarchy(amg_handle* H, const amg_csr* A, cudaStream_t s, const amg_h
     AMG_TRY(ar.alloc_n(&comp, n));
     k_iota<<<g1, 256, 0, s>>>(n, comp);
     AMG_LAUNCH_CHECK();
-    int64_t cn = n, nc = n;
+    int64_t cn = n, nc = n, cnnz = H->L[l].nnz;
     const int64_t* crp = rp;
     const int32_t* cci = ci;
     const double* cva = va;
@@ -1181,7 +1223,7 @@ int setup_hierarchy(amg_handle* H, const amg_csr* A, cudaStream_t s, const amg_h
     for (int sw = 0; sw < o.sweeps && o.aggregation == 0; ++sw) {
       int32_t *mate = nullptr, *flag = nullptr, *id = nullptr;
       AMG_TRY(ar.alloc_n(&mate, cn));
-      AMG_TRY(match_rounds(ar, cn, crp, cci, cva, cdiag, mate, nullptr, sms, s));
+      AMG_TRY(match_rounds(ar, cn, cnnz, crp, cci, cva, cdiag, mate, nullptr, sms, s));
       AMG_TRY(ar.alloc_n(&flag, cn));
       AMG_TRY(ar.alloc_n(&id, cn));
       const int gc = grid_for(cn, 256, sms, 8);
@@ -1220,6 +1262,7 @@ int setup_hierarchy(amg_handle* H, const amg_csr* A, cudaStream_t s, const amg_h
         cci = t_ci;
         cva = t_va;
         cn = nc;
+        cnnz = n_nnz;
       }
     }
     ar.release(t_rp);
@@ -1296,15 +1339,8 @@ int setup_hierarchy(amg_handle* H, const amg_csr* A, cudaStream_t s, const amg_h
                                  cudaMemcpyHostToDevice, s));
     k_dense_blocks<<<nb, 256, 0, s>>>(rp, ci, va, H->d_brow, H->d_bmat, dense, H->dev_status);
     AMG_LAUNCH_CHECK();
-    if (largest_block(Lc, Lc.n) <= COARSE_SMALL) {  // one CUDA block per diagonal block
-      k_cholesky<<<nb, 1024, 0, s>>>(H->d_brow, H->d_bmat, dense, H->Linv, H->LinvT,
-                                     H->dev_status);
-      AMG_LAUNCH_CHECK();
-    } else {  // large blocks: blocked factorization over the whole GPU, block by block
-      for (int b = 0; b < nb; ++b)
-        AMG_TRY(chol_blocked(dense + bmat[b], brow[b + 1] - brow[b], H->Linv + bmat[b],
-                             H->LinvT + bmat[b], H->dev_status, sms, s));
-    }
+    AMG_TRY(chol_blocks(nb, largest_block(Lc, Lc.n), H->d_brow, H->d_bmat, dense, H->Linv,
+                        H->LinvT, H->dev_status, sms, s));
     int st = read_status(H, s);  // synchronises: brow/bmat copies are done
     ar.release(dense);
     if (st < 0) return st;

@@ -17,6 +17,14 @@ void note_cuda_error(cudaError_t e, const char* what, const char* file, int line
             line, what);
 }
 
+static int device_malloc(void** p, size_t bytes) {
+  const cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaSuccess) return AMG_OK;
+  cudaGetLastError();
+  *p = nullptr;
+  return e == cudaErrorMemoryAllocation ? AMG_ERR_OOM : AMG_ERR_CUDA;
+}
+
 int Arena::alloc(void** p, size_t bytes) {
   *p = nullptr;
   long k = g_fail_after.load();
@@ -27,28 +35,77 @@ int Arena::alloc(void** p, size_t bytes) {
     }
     g_fail_after.store(k - 1);
   }
-  cudaError_t e = cudaMalloc(p, bytes);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    *p = nullptr;
-    return e == cudaErrorMemoryAllocation ? AMG_ERR_OOM : AMG_ERR_CUDA;
+  if (bytes == 0) bytes = 1;
+  bytes = (bytes + 255) & ~(size_t)255;  // every block starts on 256 bytes
+  if (reuse) {
+    const bool small = bytes <= ARENA_SMALL;
+    auto& pool = small ? kept_small : kept;
+    auto it = pool.lower_bound(bytes);
+    // a kept block is taken if little of it is wasted: an eighth of a large one
+    const size_t most = small ? 4 * bytes : bytes + bytes / (bytes > (16u << 20) ? 8 : 2);
+    if (it != pool.end() && it->first <= most) {
+      *p = it->second;
+      blocks[*p] = Block{it->first, small};
+      pool.erase(it);
+      return AMG_OK;
+    }
+    if (small) {
+      if (slab_used + bytes > ARENA_SLAB) {
+        void* s = nullptr;
+        const int rc = device_malloc(&s, ARENA_SLAB);
+        if (rc < 0) return rc;
+        slabs.push_back(s);
+        slab_used = 0;
+      }
+      *p = (unsigned char*)slabs.back() + slab_used;
+      slab_used += bytes;
+      blocks[*p] = Block{bytes, true};
+      return AMG_OK;
+    }
   }
-  blocks.push_back(*p);
+  int rc = device_malloc(p, bytes);
+  if (rc == AMG_ERR_OOM && !kept.empty()) {  // what is kept may be what is missing
+    drop_kept();
+    rc = device_malloc(p, bytes);
+  }
+  if (rc < 0) return rc;
+  blocks[*p] = Block{bytes, false};
   return AMG_OK;
 }
 
 void Arena::release(void* p) {
   if (!p) return;
-  auto it = std::find(blocks.begin(), blocks.end(), p);
-  if (it != blocks.end()) {
+  auto it = blocks.find(p);
+  if (it == blocks.end()) return;
+  const Block b = it->second;
+  blocks.erase(it);
+  if (reuse)
+    (b.slab ? kept_small : kept).emplace(b.bytes, p);
+  else if (!b.slab)
     cudaFree(p);
-    blocks.erase(it);
-  }
+}
+
+void Arena::drop_kept() {
+  for (auto& k : kept) cudaFree(k.second);
+  kept.clear();
+}
+
+void Arena::end_reuse() {
+  reuse = false;
+  drop_kept();
+  kept_small.clear();  // their slabs stay with the arena
+  slab_used = ARENA_SLAB;
 }
 
 void Arena::release_all() {
-  for (void* p : blocks) cudaFree(p);
+  drop_kept();
+  kept_small.clear();
+  for (auto& b : blocks)
+    if (!b.second.slab) cudaFree(b.first);
   blocks.clear();
+  for (void* s : slabs) cudaFree(s);
+  slabs.clear();
+  slab_used = ARENA_SLAB;
 }
 
 int grid_for(int64_t work_items, int threads, int num_sms, int blocks_per_sm) {
