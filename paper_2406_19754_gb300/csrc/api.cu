@@ -103,6 +103,7 @@ static void destroy(amg_handle* H) {
   if (!H) return;
   multi_free(H);
   tg_free(H);
+  ct_free(H);
   if (H->batch.sc_host) cudaFreeHost(H->batch.sc_host);
   if (H->bgraph) cudaGraphExecDestroy(H->bgraph);
   if (H->graph) cudaGraphExecDestroy(H->graph);
@@ -210,6 +211,7 @@ static int create(const amg_csr* A, const amg_options* opt, cudaStream_t s, amg_
     ar.release(cat_va);
   }
   AMG_TRY(tail_init(H, s));
+  AMG_TRY(ct_init(H, s));
   AMG_CUDA_TRY(cudaStreamSynchronize(s));
   return AMG_OK;
 }

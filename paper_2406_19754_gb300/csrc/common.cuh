@@ -355,6 +355,7 @@ struct amg_handle {
   int bloop_maxit = -1;
   int bloop_state = 0;
   void* multi = nullptr;  // multi-RHS workspace (multi.cu)
+  void* ct = nullptr;     // images of the levels in one cluster (ctail.cu)
   void* tg = nullptr;     // two-grid loss workspace and inner solver (twogrid.cu)
   // persistent small-level launch (tail.cu): grid-barrier word, sticky
   // failure flag, and the largest co-resident grid (0: not available)
@@ -695,6 +696,17 @@ int tail_reset(amg_handle* H, cudaStream_t s);
 // up waiting at a barrier, or a streaming kernel gave up waiting for a bulk
 // copy, since the last check, else AMG_OK.
 int tail_check(amg_handle* H, cudaStream_t s);
+
+// The small levels in one thread-block cluster, resident in its shared memory
+// (ctail.cu).  ct_init builds the images after setup; ct_start: the first level
+// that fits, or -1; ct_launch runs levels lt .. coarsest, lt >= ct_start (rfine:
+// the residual of level lt - 1, restricted by the launch itself, or null when
+// level lt's b is already there).
+int ct_init(amg_handle* H, cudaStream_t s);
+void ct_free(amg_handle* H);
+int ct_start(const amg_handle* H);
+template <typename T>
+int ct_launch(const amg_handle* H, int lt, const T* rfine, cudaStream_t s);
 
 // Dense Cholesky factors of the coarsest level's diagonal blocks and their
 // inverses (chol.cu).

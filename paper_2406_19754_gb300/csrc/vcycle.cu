@@ -901,7 +901,12 @@ static int vcycle_levels(const amg_handle* H, const double* r0, double* z0, int 
   };
   // Levels lt .. coarsest run in one persistent launch (tail.cu) when the
   // handle allows it; the others get one launch per step.
-  const int lt = tail_start(H);
+  // Where they fit a cluster's shared memory they run there, and larger levels
+  // above them join the launch (not when timed per level).
+  const int ts = tail_start(H);
+  const int cs = ts >= 0 && !act ? ct_start(H) : -1;
+  const bool cluster = cs > 0 && cs <= ts;
+  const int lt = cluster && !prof ? cs : ts;
   const int ldown = lt >= 0 ? lt : nl - 1;
   // downward: pre-smooth + residual, restriction
   for (int l = 0; l < ldown; ++l) {
@@ -934,6 +939,7 @@ static int vcycle_levels(const amg_handle* H, const double* r0, double* z0, int 
       PROF_END();
       cur[l] = 1 - c;
     }
+    if (cluster && !prof && l == ldown - 1) break;  // the cluster launch restricts
     PROF_BEGIN(l, 1, bytes_restrict(L, vb));
     AMG_TRY(launch_restrict<T>(H, L, rbuf(L, cur[l]), (T*)H->L[l + 1].b, s));
     PROF_END();
@@ -947,7 +953,10 @@ static int vcycle_levels(const amg_handle* H, const double* r0, double* z0, int 
                bytes_post(L, pbytes(L), vb, vb, vb) + 2.0 * (double)(L.nu - 1) * sweep_bytes(L);
     }
     PROF_BEGIN(lt, 4, bytes);
-    AMG_TRY(tail_launch<T>(H, lt, s, act));
+    if (cluster)
+      AMG_TRY(ct_launch<T>(H, lt, prof ? nullptr : rbuf(H->L[lt - 1], cur[lt - 1]), s));
+    else
+      AMG_TRY(tail_launch<T>(H, lt, s, act));
     PROF_END();
   } else {
     PROF_BEGIN(nl - 1, 3, coarse_factor_bytes(H) + mc * 2.0 * vb);
