@@ -621,7 +621,8 @@ __device__ __forceinline__ void rows_sub_v(const SellView<V>& A, bool staged, co
 // R = B - Ah B (as k_m_pre), vector columns.
 template <typename V, typename T>
 __global__ void __launch_bounds__(MROWS_BLOCK, MV_BLOCKS)
-    k_m_pre_v(SellView<V> Ah, int C, int K, const T* __restrict__ B, T* __restrict__ R) {
+    k_m_pre_v(SellView<V> Ah, int C, int K, int sub, const T* __restrict__ B,
+              T* __restrict__ R) {
   constexpr int VW = 16 / sizeof(T);
   __shared__ int32_t scol_all[MROWS_BLOCK / 32][SL_CAP];
   __shared__ T sval_all[MROWS_BLOCK / 32][SL_CAP];
@@ -630,13 +631,14 @@ __global__ void __launch_bounds__(MROWS_BLOCK, MV_BLOCKS)
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int32_t* scol = scol_all[threadIdx.x >> 5];
   T* sval = sval_all[threadIdx.x >> 5];
-  for (int64_t sl = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; sl < Ah.nslices;
-       sl += nw) {
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < Ah.nslices * sub;
+       t += nw) {
+    const int64_t sl = t / sub;
     const int64_t i0 = sl * C;
     const int rows = (int)(Ah.n - i0 < C ? Ah.n - i0 : C);
-    int w;
-    const bool staged = stage_slice(Ah, sl, C, lane, scol, sval, w);
-    for (int p = 0; p < rows; p += RW) {
+    int w = 0;
+    const bool staged = sub == 1 && stage_slice(Ah, sl, C, lane, scol, sval, w);
+    for (int p = (int)(t % sub) * RW; p < rows; p += sub * RW) {
       const bool live = rs < RW && p + rs < rows;
       const int r = live ? p + rs : 0;  // idle lanes shadow row 0 and store nothing
       const int64_t i = i0 + r;
@@ -653,7 +655,8 @@ __global__ void __launch_bounds__(MROWS_BLOCK, MV_BLOCKS)
 // the column sums (B, Z) and (Z, Q) go to epi.
 template <typename V, typename T, typename BT, typename XT, bool DOTS>
 __global__ void __launch_bounds__(MROWS_BLOCK, DOTS ? MV_BLOCKS_DOTS : MV_BLOCKS)
-    k_m_post_v(SellView<V> AP, int C, int K, const BT* __restrict__ B, const T* __restrict__ s,
+    k_m_post_v(SellView<V> AP, int C, int K, int sub, const BT* __restrict__ B,
+               const T* __restrict__ s,
                const T* __restrict__ R, const int32_t* __restrict__ agg,
                const T* __restrict__ Xc, XT* __restrict__ Z, const double* __restrict__ Q,
                double* part, int maxb, unsigned* ticket, MultiRzEpi epi) {
@@ -668,13 +671,14 @@ __global__ void __launch_bounds__(MROWS_BLOCK, DOTS ? MV_BLOCKS_DOTS : MV_BLOCKS
   double d[2][VW];
 #pragma unroll
   for (int k = 0; k < VW; ++k) d[0][k] = d[1][k] = 0.0;
-  for (int64_t sl = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; sl < AP.nslices;
-       sl += nw) {
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < AP.nslices * sub;
+       t += nw) {
+    const int64_t sl = t / sub;
     const int64_t i0 = sl * C;
     const int rows = (int)(AP.n - i0 < C ? AP.n - i0 : C);
-    int w;
-    const bool staged = stage_slice(AP, sl, C, lane, scol, sval, w);
-    for (int p = 0; p < rows; p += RW) {
+    int w = 0;
+    const bool staged = sub == 1 && stage_slice(AP, sl, C, lane, scol, sval, w);
+    for (int p = (int)(t % sub) * RW; p < rows; p += sub * RW) {
       const bool live = rs < RW && p + rs < rows;
       const int r = live ? p + rs : 0;
       const int64_t i = i0 + r;
@@ -766,32 +770,49 @@ __global__ void k_m_restrict_v(int64_t nc, int stride, int K,
 // output element (n <= 3072).  Each dot product is summed exactly as the
 // single-RHS coarse kernel sums it: 32 lane partials over a stride of 32,
 // combined by the same xor-butterfly tree.
-__device__ __forceinline__ double lane_tree(double (&p)[32]) {
+//
+// One warp per row and MC_COLS columns, lane l the terms k = l, l + 32, ... (a
+// thread per element with its 32 partials in an array indexed at run time kept
+// them in local memory: 35 and 32 us a V-cycle for 4 columns of a few hundred
+// rows).
+constexpr int MC_COLS = 4;
+
+// sum over k = k0, k0 + 32, ... < end of row[k] M[k K + c] for MC_COLS columns
+// from c0 (lanes' k0 differ); the sums end up in every lane.
+template <typename BT>
+__device__ __forceinline__ void coarse_cols(const double* __restrict__ row,
+                                            const BT* __restrict__ M, int64_t K, int nc, int k0,
+                                            int end, double (&acc)[MC_COLS]) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
+  for (int q = 0; q < MC_COLS; ++q) acc[q] = 0.0;
+#pragma unroll 4
+  for (int k = k0; k < end; k += 32) {
+    const double a = row[k];
 #pragma unroll
-    for (int l = 0; l < o; ++l) p[l] = p[l] + p[l + o];
-  return p[0];
+    for (int q = 0; q < MC_COLS; ++q)
+      if (q < nc) acc[q] = fma(a, (double)M[(int64_t)k * K + q], acc[q]);
+  }
+#pragma unroll
+  for (int q = 0; q < MC_COLS; ++q) acc[q] = warp_sum(acc[q]);
 }
 
 template <typename BT>
 __global__ void k_m_coarse1(int64_t n, int K, int nblk, const int64_t* __restrict__ brow,
                             const int64_t* __restrict__ bmat, const double* __restrict__ Linv,
                             const BT* __restrict__ B, double* __restrict__ Y) {
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * K;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t gi = t / K;
-    const int c = (int)(t % K);
+  const int lane = threadIdx.x & 31, chunks = (K + MC_COLS - 1) / MC_COLS;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < n * chunks;
+       t += nw) {
+    const int64_t gi = t / chunks;
+    const int c0 = (int)(t % chunks) * MC_COLS, nc = min(MC_COLS, K - c0);
     const int b = coarse_block(brow, nblk, gi);
     const int64_t r0 = brow[b];
     const int m = (int)(brow[b + 1] - r0), i = (int)(gi - r0);
-    const double* L = Linv + bmat[b];
-    double p[32];
-#pragma unroll
-    for (int l = 0; l < 32; ++l) p[l] = 0.0;
-    for (int k = 0; k <= i; ++k)
-      p[k & 31] = fma(L[(int64_t)i * m + k], (double)B[(r0 + k) * K + c], p[k & 31]);
-    Y[t] = lane_tree(p);
+    double acc[MC_COLS];
+    coarse_cols(Linv + bmat[b] + (int64_t)i * m, B + r0 * K + c0, K, nc, lane, i + 1, acc);
+    if (lane == 0)
+      for (int q = 0; q < nc; ++q) Y[gi * K + c0 + q] = acc[q];
   }
 }
 
@@ -799,20 +820,19 @@ template <typename XT>
 __global__ void k_m_coarse2(int64_t n, int K, int nblk, const int64_t* __restrict__ brow,
                             const int64_t* __restrict__ bmat, const double* __restrict__ LinvT,
                             const double* __restrict__ Y, XT* __restrict__ X) {
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * K;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t gk = t / K;
-    const int c = (int)(t % K);
+  const int lane = threadIdx.x & 31, chunks = (K + MC_COLS - 1) / MC_COLS;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < n * chunks;
+       t += nw) {
+    const int64_t gk = t / chunks;
+    const int c0 = (int)(t % chunks) * MC_COLS, nc = min(MC_COLS, K - c0);
     const int b = coarse_block(brow, nblk, gk);
     const int64_t r0 = brow[b];
     const int m = (int)(brow[b + 1] - r0), k = (int)(gk - r0);
-    const double* LT = LinvT + bmat[b];
-    double p[32];
-#pragma unroll
-    for (int l = 0; l < 32; ++l) p[l] = 0.0;
-    for (int i = k; i < m; ++i)
-      p[(i - k) & 31] = fma(LT[(int64_t)k * m + i], Y[(r0 + i) * K + c], p[(i - k) & 31]);
-    X[t] = (XT)lane_tree(p);
+    double acc[MC_COLS];
+    coarse_cols(LinvT + bmat[b] + (int64_t)k * m, Y + r0 * K + c0, K, nc, k + lane, m, acc);
+    if (lane == 0)
+      for (int q = 0; q < nc; ++q) X[gk * K + c0 + q] = (XT)acc[q];
   }
 }
 
@@ -948,7 +968,7 @@ __global__ void __launch_bounds__(MROWS_BLOCK, MV_BLOCKS)
 // Q = A P and (p, q) per column, vector columns (two doubles a lane); see
 // k_m_pre_v for the lane layout.
 __global__ void __launch_bounds__(MROWS_BLOCK, MV_BLOCKS)
-    k_m_spmm_dot_v(SellView<double> A, int C, int K, const double* __restrict__ P,
+    k_m_spmm_dot_v(SellView<double> A, int C, int K, int sub, const double* __restrict__ P,
                    double* __restrict__ Q, double* part, int maxb, unsigned* ticket,
                    MultiPqEpi epi) {
   constexpr int VW = 2;
@@ -960,13 +980,14 @@ __global__ void __launch_bounds__(MROWS_BLOCK, MV_BLOCKS)
   int32_t* scol = scol_all[threadIdx.x >> 5];
   double* sval = sval_all[threadIdx.x >> 5];
   double d[1][VW] = {{0.0, 0.0}};
-  for (int64_t sl = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; sl < A.nslices;
-       sl += nw) {
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < A.nslices * sub;
+       t += nw) {
+    const int64_t sl = t / sub;
     const int64_t i0 = sl * C;
     const int rows = (int)(A.n - i0 < C ? A.n - i0 : C);
-    int w;
-    const bool staged = stage_slice(A, sl, C, lane, scol, sval, w);
-    for (int p = 0; p < rows; p += RW) {
+    int w = 0;
+    const bool staged = sub == 1 && stage_slice(A, sl, C, lane, scol, sval, w);
+    for (int p = (int)(t % sub) * RW; p < rows; p += sub * RW) {
       const bool live = rs < RW && p + rs < rows;
       const int r = live ? p + rs : 0;
       const int64_t i = i0 + r;
@@ -1011,12 +1032,15 @@ struct MultiRrEpi {
   }
 };
 
-// x += alpha_c p; r -= alpha_c q; (r, r) per column (alpha_c = 0 when frozen).
+// r -= alpha_c q; (r, r) per column (alpha_c = 0 when frozen).  The x updates
+// x += alpha_c p wait for the next p update (k_m_p_update), which reads p
+// anyway, or for the end of the solve (k_m_x_pending): both kernels are at
+// their DRAM bound, and this reads P once less an iteration (1.1 of 10.2 GB
+// for 64 columns of 128^3).
 template <int KPL>
 __global__ void __launch_bounds__(MROWS_BLOCK)
-    k_m_update(int64_t n, int K, double* __restrict__ X, double* __restrict__ R,
-               const double* __restrict__ P, const double* __restrict__ Q, const Scal* sc,
-               double* part, int maxb, unsigned* ticket, MultiRrEpi epi,
+    k_m_update(int64_t n, int K, double* __restrict__ R, const double* __restrict__ Q,
+               const Scal* sc, double* part, int maxb, unsigned* ticket, MultiRrEpi epi,
                float* __restrict__ R32) {
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1037,7 +1061,6 @@ __global__ void __launch_bounds__(MROWS_BLOCK)
       rv[q] = 0.0;
       if (act[q]) {
         const int64_t e = i * K + c;
-        X[e] = X[e] + al[q] * P[e];
         const double ri = R[e] - al[q] * Q[e];
         rv[q] = ri;
         R[e] = ri;
@@ -1055,26 +1078,51 @@ __global__ void __launch_bounds__(MROWS_BLOCK)
   cols_reduce<KPL, 1>(d, K, part, maxb, ticket, epi);
 }
 
-// p = z + beta_c p for columns still iterating.
+// The owed x += alpha_c p of the last update, then p = z + beta_c p for columns
+// still iterating.  alpha_c is what the last product set: 0 for columns that
+// took no step, and it is applied here exactly once, whether or not the column
+// has stopped since.
 template <int KPL>
 __global__ void k_m_p_update(int64_t n, int K, double* __restrict__ P, const double* __restrict__ Z,
-                             const Scal* sc) {
+                             double* __restrict__ X, const Scal* sc) {
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  double be[KPL];
-  bool act[KPL];
+  double al[KPL], be[KPL];
+  bool owed[KPL], act[KPL];
 #pragma unroll
   for (int q = 0; q < KPL; ++q) {
     const int c = lane + 32 * q;
+    al[q] = c < K ? sc[c].alpha : 0.0;
+    owed[q] = al[q] != 0.0;
     act[q] = c < K && sc[c].active;
     be[q] = act[q] ? sc[c].beta : 0.0;
   }
   for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += nw)
 #pragma unroll
     for (int q = 0; q < KPL; ++q)
-      if (act[q]) {
+      if (owed[q] || act[q]) {
         const int64_t e = i * K + lane + 32 * q;
-        P[e] = Z[e] + be[q] * P[e];
+        const double p = P[e];
+        if (owed[q]) X[e] = X[e] + al[q] * p;
+        if (act[q]) P[e] = Z[e] + be[q] * p;
+      }
+}
+
+// End of a solve: the x updates still owed.
+template <int KPL>
+__global__ void k_m_x_pending(int64_t n, int K, double* __restrict__ X,
+                              const double* __restrict__ P, const Scal* sc) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  double al[KPL];
+#pragma unroll
+  for (int q = 0; q < KPL; ++q) al[q] = lane + 32 * q < K ? sc[lane + 32 * q].alpha : 0.0;
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += nw)
+#pragma unroll
+    for (int q = 0; q < KPL; ++q)
+      if (al[q] != 0.0) {
+        const int64_t e = i * K + lane + 32 * q;
+        X[e] = X[e] + al[q] * P[e];
       }
 }
 
@@ -1096,6 +1144,19 @@ static int mgrid_mv(const amg_handle* H, int64_t rows) {
   return grid_for(rows * 32, MROWS_BLOCK, H->num_sms, MV_BLOCKS);
 }
 
+// Warps that share a slice in the vector-column kernels, each taking every
+// sub-th group of rows: as many as a launch of `grid` CTAs has to spare.  A
+// warp advances 32 / (K / columns per 16 bytes) rows at a time, one row for 64
+// FP64 columns, so a small level's slices (1,024 of them at 32,768 rows) were
+// walked by few warps, 20 to 25 us a step.  A shared slice is not staged.
+template <typename T>
+static int mv_split(int grid, const Sell& M, int K) {
+  const int rw = 32 / (K / (16 / (int)sizeof(T)));
+  const int64_t passes = (M.C + rw - 1) / rw;
+  const int64_t spare = (int64_t)grid * (MROWS_BLOCK / 32) / std::max<int64_t>(M.nslices, 1);
+  return (int)std::max<int64_t>(1, std::min(passes, spare));
+}
+
 // Smoother launches: the vector-column kernels when vec (VW divides K, all
 // vectors 16-byte aligned), else the per-column ones.
 template <typename V, typename T>
@@ -1103,7 +1164,7 @@ static void m_pre(const amg_handle* H, bool vec, int K, const Level& L, const Se
                   const T* b, T* r, cudaStream_t s) {
   const int g = mgrid_mv(H, L.n);
   if (vec)
-    k_m_pre_v<V, T><<<g, MROWS_BLOCK, 0, s>>>(v, L.A.C, K, b, r);
+    k_m_pre_v<V, T><<<g, MROWS_BLOCK, 0, s>>>(v, L.A.C, K, mv_split<T>(g, L.A, K), b, r);
   else
     AMG_DISPATCH_KPL(K, (k_m_pre<KPL, V, T, T><<<g, MROWS_BLOCK, 0, s>>>(v, L.A.C, K, b, r)));
 }
@@ -1118,7 +1179,8 @@ static void m_post(const amg_handle* H, const MultiWs& W, bool vec, int K, const
   if (vec) {
     const int g = grid_for(L.n * 32, MROWS_BLOCK, H->num_sms, DOTS ? MV_BLOCKS_DOTS : MV_BLOCKS);
     k_m_post_v<V, T, BT, XT, DOTS><<<g, MROWS_BLOCK, 0, s>>>(
-        v, L.AP.C, K, b, sv, rv, L.agg, xc, z, Q, W.part, maxb, W.ticket, epi);
+        v, L.AP.C, K, mv_split<T>(g, L.AP, K), b, sv, rv, L.agg, xc, z, Q, W.part, maxb,
+        W.ticket, epi);
   } else {
     const int g = mgrid_mv(H, L.n);
     AMG_DISPATCH_KPL(K, (k_m_post<KPL, V, T, BT, XT, DOTS><<<g, MROWS_BLOCK, 0, s>>>(
@@ -1138,7 +1200,7 @@ static int m_vcycle(const amg_handle* H, const MultiWs& W, const double* R0, dou
   MultiRzEpi epi{W.sc, beta_form, first ? 1 : 0};
   auto coarse = [&](const auto* b, auto* x) -> int {
     const int64_t n = H->nco;
-    const int g = grid_for(n * K, 256, H->num_sms, 4);
+    const int g = grid_for(n * ((K + MC_COLS - 1) / MC_COLS) * 32, 256, H->num_sms, 8);
     k_m_coarse1<<<g, 256, 0, s>>>(n, K, H->nblk, H->d_brow, H->d_bmat, H->Linv, b, W.cy);
     AMG_LAUNCH_CHECK();
     k_m_coarse2<<<g, 256, 0, s>>>(n, K, H->nblk, H->d_brow, H->d_bmat, H->LinvT, W.cy, x);
@@ -1328,24 +1390,28 @@ int pcg_multi_run(amg_handle* H, int K, const double* B, double* X, const pcg_op
     AMG_CUDA_TRY(cudaMemcpyAsync(W->P, W->Z, sizeof(double) * n * K, cudaMemcpyDeviceToDevice, s));
     for (;;) {
       if (K % 2 == 0)  // two doubles a lane (the workspace is 16-byte aligned)
-        k_m_spmm_dot_v<<<gmv, MROWS_BLOCK, 0, s>>>(A, C, K, W->P, W->Q, W->part, maxb,
+        k_m_spmm_dot_v<<<gmv, MROWS_BLOCK, 0, s>>>(A, C, K, mv_split<double>(gmv, L0.A, K), W->P, W->Q, W->part, maxb,
                                                   W->ticket, pe);
       else
         AMG_DISPATCH_KPL(K, (k_m_spmm_dot<KPL><<<gmv, MROWS_BLOCK, 0, s>>>(
                                 A, C, K, W->P, W->Q, W->part, maxb, W->ticket, pe)));
       AMG_LAUNCH_CHECK();
       AMG_CUDA_TRY(cudaMemsetAsync(W->nactive, 0, sizeof(int), s));
-      AMG_DISPATCH_KPL(K, (k_m_update<KPL><<<g, MROWS_BLOCK, 0, s>>>(n, K, X, W->R, W->P, W->Q,
-                                                                    W->sc, W->part, maxb,
-                                                                    W->ticket, re, W->R32)));
+      AMG_DISPATCH_KPL(K, (k_m_update<KPL><<<g, MROWS_BLOCK, 0, s>>>(
+                                  n, K, W->R, W->Q, W->sc, W->part, maxb, W->ticket, re,
+                                  W->R32)));
       AMG_LAUNCH_CHECK();
       ++k;
       AMG_TRY(read_act());
       if (act == 0 || k >= o->maxit) break;
       AMG_TRY(m_vcycle_any(H, *W, W->R, W->Z, true, W->Q, beta_form, false, s, W->R32));
-      AMG_DISPATCH_KPL(K, (k_m_p_update<KPL><<<g, MROWS_BLOCK, 0, s>>>(n, K, W->P, W->Z, W->sc)));
+      AMG_DISPATCH_KPL(
+          K, (k_m_p_update<KPL><<<g, MROWS_BLOCK, 0, s>>>(n, K, W->P, W->Z, X, W->sc)));
       AMG_LAUNCH_CHECK();
     }
+    AMG_DISPATCH_KPL(K,
+                     (k_m_x_pending<KPL><<<g, MROWS_BLOCK, 0, s>>>(n, K, X, W->P, W->sc)));
+    AMG_LAUNCH_CHECK();
   }
   AMG_CUDA_TRY(cudaEventRecord(H->ev1, s));
   MultiInitEpi te{W->sc, o->tol, o->maxit, W->nactive, 1};
