@@ -544,11 +544,16 @@ def run_ours(a):
     # one per V-cycle profile record, plus the second phase of a coarse solve
     # over a block larger than 1024 rows, the level-0 dot kernel of a
     # one-level hierarchy, and the separate dot kernel of V-cycles with
-    # several sweeps or smoothed prolongators
+    # smoothed prolongators and one sweep.  With a small-level launch, levels
+    # that may join it in one cluster (at most 65534 rows, ctail.cu) are
+    # counted as part of it: a lower bound
     V = len(recs)
+    if not batch and any(r_["kind"] == "tail" for r_ in recs):
+        V = 1 + sum(r_["kind"] != "tail" and H.level_info(r_["level"])[0] > 65534
+                    for r_ in recs)
     if any(r_["kind"] == "coarse" for r_ in recs) and H.level_info(nl - 1)[0] > 1024:
         V += 1
-    if nl == 1 or (not batch and (H.opts.smooth_sweeps > 1 or H.opts.smooth_prolongator)):
+    if nl == 1 or (not batch and H.opts.smooth_prolongator and H.opts.smooth_sweeps == 1):
         V += 1
     if batch:
         launches = (2 + (V + 5) + (it - 1) * (V + 6) + 2) * a.steps
@@ -556,8 +561,9 @@ def run_ours(a):
         launches = None  # the blocked kernels (multi.cu) are not counted here
     else:
         # initial residual, first iteration (V-cycle, SpMV, update), the others
-        # (+ p update), the owed x update, and the loop graph's stopping tests
-        ctl = it if a.graph == "loop" else 0
+        # (+ p update), the owed x update, and the loop graph's first stopping
+        # test (the later ones are part of the update kernel)
+        ctl = 1 if a.graph == "loop" else 0
         launches = (1 + (V + 2) + (it - 1) * (V + 3) + 1 + ctl) * a.steps
     nlaunch = {}  # launches per V-cycle of each (level, kind)
     for _ in range(reps):
@@ -608,6 +614,9 @@ def run_ours(a):
     spmv_ms = e0.elapsed_time(e1) / 10
     lay = H.level_layout(0)
     idx_bytes = 2.0 + 4.0 / lay["slice_height"] if lay["compressed"] else 4.0
+    pre0 = [r_["bytes"] for r_ in recs if r_["level"] == 0 and r_["kind"] == "pre"]
+    if pre0 and a.precision == "f64" and not batch:  # index bytes an entry, as streamed
+        idx_bytes = (pre0[0] - 16.0 * n) / nnz - 8.0
     spmv_gbs = ((8.0 + idx_bytes) * nnz + 16.0 * n) / (spmv_ms * 1e-3) / 1e9
 
     # end to end through the public API from pinned host memory

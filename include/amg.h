@@ -104,8 +104,11 @@ typedef struct amg_options {
                             launch instead of one launch per step: one CTA when
                             the largest of them has at most 16384 rows (and the
                             coarsest level is one block), else a cooperative
-                            grid with bounded grid barriers.  Same results bit
-                            for bit.  0 = off; default 1024 */
+                            grid with bounded grid barriers.  Where these levels
+                            and larger ones above them (at most 65534 rows) fit
+                            the shared memory of a 16-CTA cluster, all of those
+                            run in one launch there.  Same results bit for bit.
+                            0 = off; default 1024 */
   int smooth_sweeps;     /* l1-Jacobi sweeps nu_0 before and after the coarse
                             correction on level 0, 1..8; default 1 (V(1,1)) */
   int variable_cycle;    /* 1: nu_l = nu_0 * 2^l sweeps on level l, the variable
@@ -146,11 +149,12 @@ typedef struct amg_options {
                             In [0, 1) */
   int stream_ring;       /* 1 (default): the level kernels with FP64 or FP32
                             operator values of a one-system hierarchy with one
-                            thread per row (pre- and post-smoother; the FP64
-                            PCG product) stream each slice into a
+                            thread per row (pre- and post-smoother, further
+                            sweeps; the FP64 PCG product) stream tiles of
+                            slices with packed column indices into a
                             shared-memory ring by bulk copies (cp.async.bulk,
                             mbarrier completion), with the library's number of
-                            stages per warp; 2..4: with that many stages;
+                            stages per CTA; 2..4: with that many stages;
                             0: every lane loads its own entries.  Same rows bit
                             for bit; dot products may round differently
                             (another summation order) */
@@ -404,16 +408,19 @@ typedef struct amg_kernel_time {
                     persistent launch of levels >= `level` (all their steps and
                     the coarsest solve), 5 a further smoothing sweep
                     (smooth_sweeps > 1) */
-  double bytes;  /* algorithmic bytes: each matrix entry (value + column index:
-                    4 bytes, or 2 plus a share of the slice column's base when
-                    compressed) and each vector entry read or written once */
+  double bytes;  /* algorithmic bytes: each matrix entry (value + column index as
+                    the kernel streams it: its share of the slices' packed
+                    index blocks, or 4 bytes, or 2 plus a share of the slice
+                    column's base when compressed) and each vector entry read
+                    or written once */
   double ms;     /* device time between CUDA events around the launch */
 } amg_kernel_time;
 
 /*
  * z = B r like amg_vcycle_apply, with a CUDA event pair around every kernel
  * (the paper reports time per iteration; this splits it per kernel).  The
- * kernels are the ones a PCG iteration runs: the level-0 post-smoother also
+ * kernels are the ones a PCG iteration runs, except that levels above
+ * tail_rows are always timed one step at a time: the level-0 post-smoother also
  * forms the dot products PCG fuses into it ((r, z), and (z, q) with an FP32
  * hierarchy, q being internal scratch), and an FP32 hierarchy first copies r
  * to FP32 (untimed) as the CG update does.

@@ -31,7 +31,7 @@ enum { SEG_INIT = 0, SEG_RZ_FIRST = 1, SEG_PQ = 2, SEG_RR = 3, SEG_RZ = 4, SEG_T
 
 // r = b - A x with per-chunk (r, r) and (b, b).
 template <int TPR>
-__global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
+__global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
     k_b_residual(SellView<double> A, int64_t nchunks, const int64_t* __restrict__ chunk_off,
                  const double* __restrict__ b, const double* __restrict__ x,
                  double* __restrict__ r, double* __restrict__ part, float* __restrict__ r32) {
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
 
 // q = A p with per-chunk (p, q); chunks of converged systems are skipped.
 template <int TPR>
-__global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
+__global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
     k_b_spmv_dot(SellView<double> A, int64_t nchunks, const int64_t* __restrict__ chunk_off,
                  const double* __restrict__ p, double* __restrict__ q,
                  double* __restrict__ part, const Scal* __restrict__ sc) {
@@ -219,7 +219,7 @@ static int b_residual(const BatchRun& R, const double* b, const double* x, doubl
                       float* r32, cudaStream_t s) {
   const Level& L = R.H->L[0];
   const Batch& B = R.H->batch;
-  AMG_DISPATCH_TPR(sell_code(L.A), (k_b_residual<TPR><<<chunk_grid(R.H), SELL_BLOCK, 0, s>>>(
+  AMG_DISPATCH_TPR(sell_code(L.A, 8), (k_b_residual<TPR><<<chunk_grid(R.H), SELL_BLOCK, 0, s>>>(
                                 a0(R.H), B.nchunks, B.chunk_off, b, x, r, B.part, r32)));
   AMG_LAUNCH_CHECK();
   return AMG_OK;
@@ -227,7 +227,7 @@ static int b_residual(const BatchRun& R, const double* b, const double* x, doubl
 
 static int b_spmv_dot(const amg_handle* H, cudaStream_t s) {
   const Batch& B = H->batch;
-  AMG_DISPATCH_TPR(sell_code(H->L[0].A),
+  AMG_DISPATCH_TPR(sell_code(H->L[0].A, 8),
                    (k_b_spmv_dot<TPR><<<chunk_grid(H), SELL_BLOCK, 0, s>>>(
                        a0(H), B.nchunks, B.chunk_off, H->p, H->q, B.part, B.sc)));
   AMG_LAUNCH_CHECK();
@@ -310,7 +310,12 @@ static int ensure_bloop(amg_handle* H, const BatchRun& R, double* x) {
   }
   const Batch& B = H->batch;
   const int rc = build_while_graph(
-      H->cap_stream, [&](cudaStream_t cs) { return b_body(R, x, cs); },
+      H->cap_stream,
+      [&](cudaStream_t cs, cudaGraphConditionalHandle h) {
+        const int rb = b_body(R, x, cs);
+        if (rb == AMG_OK) k_b_control<<<1, 1, 0, cs>>>(B.nactive, B.loop_ctl, h);
+        return rb;
+      },
       [&](cudaStream_t cs, cudaGraphConditionalHandle h) {
         k_b_control<<<1, 1, 0, cs>>>(B.nactive, B.loop_ctl, h);
       },

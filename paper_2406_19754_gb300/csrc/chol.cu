@@ -30,7 +30,7 @@ namespace amg {
 namespace {
 
 constexpr int NB = 32;          // panel width
-constexpr int PANEL_THREADS = 128;
+constexpr int PANEL_THREADS = 32;  // a warp per CTA: the rows spread over more SMs' FP64 pipes
 constexpr int TILE_THREADS = 256;
 
 // Block b: rows n, dense row-major a (lower triangle becomes L), L^-1, L^-T.

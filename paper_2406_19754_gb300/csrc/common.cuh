@@ -52,8 +52,10 @@ void note_cuda_error(cudaError_t e, const char* what, const char* file, int line
 // 79 ms of a 128^3 diffusion setup).  Reuse follows stream order, so a block's
 // next user runs after its last one.  end_reuse frees what is still unused;
 // slabs live until release_all.
-constexpr size_t ARENA_SMALL = 64 * 1024;
-constexpr size_t ARENA_SLAB = 2 * 1024 * 1024;
+// Slabs double from ARENA_SLAB_MIN to ARENA_SLAB_MAX bytes.
+constexpr size_t ARENA_SMALL = 1024 * 1024;
+constexpr size_t ARENA_SLAB_MIN = 2 * 1024 * 1024;
+constexpr size_t ARENA_SLAB_MAX = 16 * 1024 * 1024;
 
 struct Arena {
   struct Block {
@@ -63,7 +65,7 @@ struct Arena {
   std::unordered_map<void*, Block> blocks;      // in use
   std::multimap<size_t, void*> kept, kept_small;  // released during reuse
   std::vector<void*> slabs;
-  size_t slab_used = ARENA_SLAB;
+  size_t slab_bytes = 0, slab_used = 0;  // of the last slab
   bool reuse = false;
   int alloc(void** p, size_t bytes);
   template <typename T>
@@ -272,6 +274,9 @@ struct PcgScalars {
   int iter;
   // 1 while x += alpha p of the last update is still to be applied (pcg.cu)
   int x_pending;
+  // the solution vector: captured iterations read it here, so a graph serves
+  // every x (capturing again for another x took 0.3 ms of a 1.8 ms solve)
+  double* x;
 };
 
 // Coarsest blocks up to this many rows are factored and solved by one CUDA
@@ -334,7 +339,6 @@ struct amg_handle {
   // the whole PCG loop as one graph (device-side stopping test in a
   // conditional while node); loop_state 0 untried, 1 built, -1 unavailable
   cudaGraphExec_t loop = nullptr;
-  double* loop_x = nullptr;
   int loop_beta = -2;
   int loop_state = 0;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -735,10 +739,12 @@ int smoothed_prolongator(Arena& ar, int64_t n, const int64_t* A_rp, const int32_
                          const double* A_v, const int32_t* agg, const int64_t* rp, int32_t* ci,
                          double* v, double* w_out, int num_sms, cudaStream_t s);
 
-// exec = [ctl] -> while (condition) { body; ctl }, where ctl launches the
-// kernel that sets the condition through the handle (pcg.cu).
+// exec = [ctl] -> while (condition) { body }, where ctl launches a kernel that
+// sets the condition through the handle, and body's last kernel does so too
+// (pcg.cu).
 // AMG_ERR_UNSUPPORTED if the runtime cannot build it.
-int build_while_graph(cudaStream_t cs, const std::function<int(cudaStream_t)>& body,
+int build_while_graph(cudaStream_t cs,
+                      const std::function<int(cudaStream_t, cudaGraphConditionalHandle)>& body,
                       const std::function<void(cudaStream_t, cudaGraphConditionalHandle)>& ctl,
                       cudaGraphExec_t* out);
 

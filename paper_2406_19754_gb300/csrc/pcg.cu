@@ -35,7 +35,7 @@ struct TrueResEpi {
 
 // r = b - A x with (r, r) and (b, b); mode 1 writes (r, r) to sc->zq only.
 template <int TPR, int MODE>
-__global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
+__global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
     k_residual(SellView<double> A, const double* __restrict__ b, const double* __restrict__ x,
                double* __restrict__ r, Reduce red, PcgScalars* sc, float* __restrict__ r32) {
   const Lanes<TPR> ln;
@@ -77,7 +77,7 @@ struct PqEpi {
 
 // q = A p and (p, q); the last block sets alpha = (r, z) / (p, q).
 template <int TPR>
-__global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
+__global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
     k_spmv_dot(SellView<double> A, const double* __restrict__ p, double* __restrict__ q,
                Reduce red, PcgScalars* sc) {
   const Lanes<TPR> ln;
@@ -128,11 +128,30 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
   grid_reduce<1>(d, red, PqEpi{sc});
 }
 
+// The stopping test of one iteration, on the device: the same decisions as
+// the host loop in pcg_run (a failed (p, q) ends the solve without counting
+// the step; otherwise count it, then stop on an error, on ||r||/||b|| <= tol
+// or at maxit).  Sets the while-node condition: 1 = run another iteration.
+__device__ __forceinline__ void pcg_control(PcgScalars* sc, cudaGraphConditionalHandle h) {
+  unsigned go = 0;
+  if (!sc->pq_fail) {
+    const int k = ++sc->iter;
+    double bnorm = sqrt(sc->bb);
+    if (bnorm == 0.0) bnorm = 1.0;
+    const double rel = sqrt(sc->rr) / bnorm;
+    go = (sc->status < 0 || rel <= sc->tol || k >= sc->maxit) ? 0u : 1u;
+  }
+  cudaGraphSetConditional(h, go);
+}
+
 struct RrEpi {
   PcgScalars* sc;
+  cudaGraphConditionalHandle h;
+  int steer;  // 1: h is the loop graph's while node
   __device__ void operator()(double (&t)[1]) const {
     sc->rr = t[0];
     if (!isfinite(t[0]) && sc->status == 0) sc->status = AMG_ERR_NAN;
+    if (steer) pcg_control(sc, h);
   }
 };
 
@@ -140,23 +159,55 @@ struct RrEpi {
 // V-cycle, so it gathers 4-byte values without converting each one.
 // Skipped after a breakdown.  x null: the x update is deferred to the next
 // p update (k_p_update_x) or to the end of the solve (k_x_pending), which
-// read p anyway; x_pending records that it is owed.
+// read p anyway; x_pending records that it is owed.  steer: the block that
+// completes (r, r) also steers the loop graph's while node h.
+//
+// Bound by DRAM (24 bytes a row, 28 with r32) and by the FP64 pipe: two
+// operations a row, 32 row-operations per SM every 16 clocks.  Each thread
+// takes four rows a step by 16-byte accesses, so enough bytes are in flight,
+// and r32 is rounded on the integer pipe (cvt_n); scalar rows with the
+// hardware conversion took 107 us for 16.8M rows with r32, 74 us without.
 __global__ void k_cg_update(int64_t n, double* __restrict__ x, double* __restrict__ r,
                             const double* __restrict__ p, const double* __restrict__ q, Reduce red,
-                            PcgScalars* sc, float* __restrict__ r32) {
-  if (sc->status < 0) return;  // uniform across the grid: no block reduces
+                            PcgScalars* sc, float* __restrict__ r32,
+                            cudaGraphConditionalHandle h, int steer) {
+  if (sc->status < 0) {  // uniform across the grid: no block reduces
+    if (steer && blockIdx.x == 0 && threadIdx.x == 0) pcg_control(sc, h);
+    return;
+  }
   const double alpha = sc->alpha;
   double d[1] = {0.0};
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    if (x) x[i] = x[i] + alpha * p[i];
-    const double ri = r[i] - alpha * q[i];
-    r[i] = ri;
-    if (r32) r32[i] = (float)ri;
-    d[0] += ri * ri;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x * 4;
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < n; i += step) {
+    if (i + 4 <= n) {  // the workspace vectors start on 256 bytes
+      const double2 q0 = __ldcs((const double2*)(q + i)), q1 = __ldcs((const double2*)(q + i + 2));
+      const double2 r0 = *(const double2*)(r + i), r1 = *(const double2*)(r + i + 2);
+      double v[4] = {r0.x - alpha * q0.x, r0.y - alpha * q0.y, r1.x - alpha * q1.x,
+                     r1.y - alpha * q1.y};
+      *(double2*)(r + i) = make_double2(v[0], v[1]);
+      *(double2*)(r + i + 2) = make_double2(v[2], v[3]);
+      if (r32) {
+        float f[4];
+        cvt_n(v, f);
+        *(float4*)(r32 + i) = make_float4(f[0], f[1], f[2], f[3]);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) d[0] += v[u] * v[u];
+      if (x)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[i + u] = x[i + u] + alpha * p[i + u];
+    } else {
+      for (int64_t k = i; k < n; ++k) {
+        const double ri = r[k] - alpha * q[k];
+        r[k] = ri;
+        if (r32) r32[k] = (float)ri;
+        d[0] += ri * ri;
+        if (x) x[k] = x[k] + alpha * p[k];
+      }
+    }
   }
   if (!x && blockIdx.x == 0 && threadIdx.x == 0) sc->x_pending = 1;
-  grid_reduce<1>(d, red, RrEpi{sc});
+  grid_reduce<1>(d, red, RrEpi{sc, h, steer});
 }
 
 __global__ void k_p_update(int64_t n, double* __restrict__ p, const double* __restrict__ z,
@@ -171,13 +222,24 @@ __global__ void k_p_update(int64_t n, double* __restrict__ p, const double* __re
 // complete one), then p = z + beta p: one pass over p for both.  The same
 // expressions as k_cg_update and k_p_update, so the same bits.
 __global__ void k_p_update_x(int64_t n, double* __restrict__ p, const double* __restrict__ z,
-                             double* __restrict__ x, PcgScalars* sc) {
+                             PcgScalars* sc) {
   const double alpha = sc->alpha, beta = sc->beta;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const double pi = p[i];
-    x[i] = x[i] + alpha * pi;
-    p[i] = z[i] + beta * pi;
+  double* x = sc->x;
+  const bool pairs = ((uintptr_t)x & 15u) == 0;  // p and z start on 256 bytes
+  const int64_t step = (int64_t)gridDim.x * blockDim.x * 2;
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 2; i < n; i += step) {
+    if (pairs && i + 2 <= n) {
+      const double2 pv = *(const double2*)(p + i), zv = __ldcs((const double2*)(z + i));
+      const double2 xv = __ldcs((const double2*)(x + i));
+      __stcs((double2*)(x + i), make_double2(xv.x + alpha * pv.x, xv.y + alpha * pv.y));
+      *(double2*)(p + i) = make_double2(zv.x + beta * pv.x, zv.y + beta * pv.y);
+    } else {
+      for (int64_t k = i; k < n && k < i + 2; ++k) {
+        const double pk = p[k];
+        x[k] = x[k] + alpha * pk;
+        p[k] = z[k] + beta * pk;
+      }
+    }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) sc->x_pending = 0;  // nobody else reads it here
 }
@@ -200,10 +262,10 @@ static int launch_residual(const amg_handle* H, int mode, const double* b, const
   const int grid = sell_grid(sell_groups(L.A), H->num_sms);
   const SellView<double> v = view<double>(L.A, L.A.v64);
   if (mode == 0) {
-    AMG_DISPATCH_TPR(sell_code(L.A), (k_residual<TPR, 0><<<grid, SELL_BLOCK, 0, s>>>(
+    AMG_DISPATCH_TPR(sell_code(L.A, 8), (k_residual<TPR, 0><<<grid, SELL_BLOCK, 0, s>>>(
                                   v, b, x, r, H->red, H->sc, H->r32)));
   } else {
-    AMG_DISPATCH_TPR(sell_code(L.A), (k_residual<TPR, 1><<<grid, SELL_BLOCK, 0, s>>>(
+    AMG_DISPATCH_TPR(sell_code(L.A, 8), (k_residual<TPR, 1><<<grid, SELL_BLOCK, 0, s>>>(
                                   v, b, x, r, H->red, H->sc, nullptr)));
   }
   AMG_LAUNCH_CHECK();
@@ -226,7 +288,7 @@ static int launch_spmv_dot(const amg_handle* H, cudaStream_t s) {
       return AMG_OK;
     }
   }
-  AMG_DISPATCH_TPR(sell_code(L.A),
+  AMG_DISPATCH_TPR(sell_code(L.A, 8),
                    (k_spmv_dot<TPR><<<grid, SELL_BLOCK, 0, s>>>(v, H->p, H->q, H->red, H->sc)));
   AMG_LAUNCH_CHECK();
   return AMG_OK;
@@ -235,10 +297,13 @@ static int launch_spmv_dot(const amg_handle* H, cudaStream_t s) {
 // defer: x += alpha p waits for the next p update (which reads p anyway),
 // saving one pass over p per iteration; the solve then ends with
 // k_x_pending.  Not with per-iteration histories of x.
-static int launch_update(const amg_handle* H, double* x, bool defer, cudaStream_t s) {
+// h: the loop graph's while node, or null outside it.
+static int launch_update(const amg_handle* H, double* x, bool defer, cudaStream_t s,
+                         const cudaGraphConditionalHandle* h = nullptr) {
   const int64_t n = H->L[0].n;
-  k_cg_update<<<grid_for(n, 256, H->num_sms, 8), 256, 0, s>>>(
-      n, defer ? nullptr : x, H->r, H->p, H->q, H->red, H->sc, H->r32);
+  k_cg_update<<<grid_for((n + 3) / 4, 256, H->num_sms, 8), 256, 0, s>>>(
+      n, defer ? nullptr : x, H->r, H->p, H->q, H->red, H->sc, H->r32,
+      h ? *h : cudaGraphConditionalHandle(), h ? 1 : 0);
   AMG_LAUNCH_CHECK();
   return AMG_OK;
 }
@@ -246,21 +311,24 @@ static int launch_update(const amg_handle* H, double* x, bool defer, cudaStream_
 // One iteration after the first: z = B r (+ dots, beta), p = z + beta p
 // (with the owed x update when deferring), q = A p (+ alpha), x/r update
 // (+ (r, r)).
-static int iteration_body(const amg_handle* H, double* x, int dots, bool defer, cudaStream_t s) {
+static int iteration_body(const amg_handle* H, double* x, int dots, bool defer, cudaStream_t s,
+                          const cudaGraphConditionalHandle* h = nullptr) {
   const int64_t n = H->L[0].n;
   AMG_TRY(vcycle_run(H, H->r, H->z, dots, H->q, s, nullptr, H->r32));
   if (defer)
-    k_p_update_x<<<grid_for(n, 256, H->num_sms, 8), 256, 0, s>>>(n, H->p, H->z, x, H->sc);
+    k_p_update_x<<<grid_for((n + 1) / 2, 256, H->num_sms, 8), 256, 0, s>>>(n, H->p, H->z,
+                                                                           H->sc);
   else
     k_p_update<<<grid_for(n, 256, H->num_sms, 8), 256, 0, s>>>(n, H->p, H->z, H->sc);
   AMG_LAUNCH_CHECK();
   AMG_TRY(launch_spmv_dot(H, s));
-  AMG_TRY(launch_update(H, x, defer, s));
+  AMG_TRY(launch_update(H, x, defer, s, h));
   return AMG_OK;
 }
 
 static int ensure_graph(amg_handle* H, double* x, int dots, int beta_form, bool defer) {
-  if (H->graph && H->graph_x == x && H->graph_beta == beta_form &&
+  // a deferred x update goes through sc->x: any x
+  if (H->graph && (defer || H->graph_x == x) && H->graph_beta == beta_form &&
       H->graph_defer == (int)defer)
     return AMG_OK;
   if (H->graph) {
@@ -285,23 +353,12 @@ static int ensure_graph(amg_handle* H, double* x, int dots, int beta_form, bool 
   return AMG_OK;
 }
 
-// The stopping test of one iteration, on the device: the same decisions as
-// the host loop in pcg_run (a failed (p, q) ends the solve without counting
-// the step; otherwise count it, then stop on an error, on ||r||/||b|| <= tol
-// or at maxit).  Sets the while-node condition: 1 = run another iteration.
 __global__ void k_pcg_control(PcgScalars* sc, cudaGraphConditionalHandle h) {
-  unsigned go = 0;
-  if (!sc->pq_fail) {
-    const int k = ++sc->iter;
-    double bnorm = sqrt(sc->bb);
-    if (bnorm == 0.0) bnorm = 1.0;
-    const double rel = sqrt(sc->rr) / bnorm;
-    go = (sc->status < 0 || rel <= sc->tol || k >= sc->maxit) ? 0u : 1u;
-  }
-  cudaGraphSetConditional(h, go);
+  pcg_control(sc, h);
 }
 
-int build_while_graph(cudaStream_t cs, const std::function<int(cudaStream_t)>& body,
+int build_while_graph(cudaStream_t cs,
+                      const std::function<int(cudaStream_t, cudaGraphConditionalHandle)>& body,
                       const std::function<void(cudaStream_t, cudaGraphConditionalHandle)>& ctl,
                       cudaGraphExec_t* out) {
   const cudaStreamCaptureMode mode = cudaStreamCaptureModeThreadLocal;
@@ -331,8 +388,7 @@ int build_while_graph(cudaStream_t cs, const std::function<int(cudaStream_t)>& b
     e = cudaStreamBeginCaptureToGraph(cs, cp.conditional.phGraph_out[0], nullptr, nullptr, 0,
                                       mode);
   if (e == cudaSuccess) {
-    rc = body(cs);
-    if (rc == AMG_OK) ctl(cs, h);
+    rc = body(cs, h);
     cudaGraph_t bcap = nullptr;
     e = cudaStreamEndCapture(cs, &bcap);
   }
@@ -348,32 +404,34 @@ int build_while_graph(cudaStream_t cs, const std::function<int(cudaStream_t)>& b
 }
 
 // The remaining iterations of a solve as one graph: the stopping test, then
-// a conditional while node whose body is one iteration plus the test.  The
-// host waits once per solve instead of once per iteration.
-static int build_loop(amg_handle* H, double* x, int dots, cudaGraphExec_t* out) {
+// a conditional while node whose body is one iteration, whose last kernel also
+// makes the test.  The host waits once per solve instead of once per iteration.
+static int build_loop(amg_handle* H, int dots, cudaGraphExec_t* out) {
   PcgScalars* sc = H->sc;
   return build_while_graph(
-      H->cap_stream, [&](cudaStream_t cs) { return iteration_body(H, x, dots, true, cs); },
+      H->cap_stream,
+      [&](cudaStream_t cs, cudaGraphConditionalHandle h) {
+        return iteration_body(H, nullptr, dots, true, cs, &h);
+      },
       [&](cudaStream_t cs, cudaGraphConditionalHandle h) {
         k_pcg_control<<<1, 1, 0, cs>>>(sc, h);
       },
       out);
 }
 
-// Loop graph for (x, beta form); AMG_ERR_UNSUPPORTED (once, remembered) if
+// Loop graph for a beta form; AMG_ERR_UNSUPPORTED (once, remembered) if
 // the runtime cannot build it, and the caller uses one graph per iteration.
-static int ensure_loop(amg_handle* H, double* x, int dots, int beta_form) {
+static int ensure_loop(amg_handle* H, int dots, int beta_form) {
   if (H->loop_state < 0) return AMG_ERR_UNSUPPORTED;
-  if (H->loop && H->loop_x == x && H->loop_beta == beta_form) return AMG_OK;
+  if (H->loop && H->loop_beta == beta_form) return AMG_OK;
   if (H->loop) {
     cudaGraphExecDestroy(H->loop);
     H->loop = nullptr;
   }
-  const int rc = build_loop(H, x, dots, &H->loop);
+  const int rc = build_loop(H, dots, &H->loop);
   if (rc == AMG_ERR_UNSUPPORTED) H->loop_state = -1;
   if (rc < 0) return rc;
   H->loop_state = 1;
-  H->loop_x = x;
   H->loop_beta = beta_form;
   return AMG_OK;
 }
@@ -394,7 +452,7 @@ int pcg_run(amg_handle* H, const double* b, double* x, const pcg_options* o, pcg
   // one graph for the whole loop unless per-iteration histories are kept
   bool use_loop = false;
   if (o->use_graph == 1 && !o->res_history && !o->x_history) {
-    const int rc = ensure_loop(H, x, dots, beta_form);
+    const int rc = ensure_loop(H, dots, beta_form);
     if (rc < 0 && rc != AMG_ERR_UNSUPPORTED) return rc;
     use_loop = rc == AMG_OK;
   }
@@ -407,6 +465,7 @@ int pcg_run(amg_handle* H, const double* b, double* x, const pcg_options* o, pcg
   init.beta_form = beta_form;
   init.tol = o->tol;
   init.maxit = o->maxit;
+  init.x = x;
   *H->sc_host = init;
   AMG_CUDA_TRY(cudaMemcpyAsync(H->sc, H->sc_host, sizeof(PcgScalars), cudaMemcpyHostToDevice, s));
   AMG_CUDA_TRY(cudaEventRecord(H->ev0, s));

@@ -11,7 +11,7 @@ namespace amg {
 
 // Stages and tile: the largest tile (8, 4 or 2 slices, one consumer warp
 // each) that leaves room for the warps of RING_CTAS_PER_SM CTAs of 8 slices
-// per SM, else for half of them.  Three stages while the SM's rings then stay
+// per SM, else of three, else of two.  Three stages while the SM's rings then stay
 // within half of its unified memory, so that the rest caches the gathered
 // vector, else two: measured at 256^3 (FP32), the level-0 pre-smoother (9 KB
 // stages) took 0.136 ms with three against 0.143 with two, the level-1 one of
@@ -54,7 +54,7 @@ RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows, 
   const int q0 = dots || M.nslices >= 304 * ring_tile(0) ? 0
                  : M.nslices >= 304 * ring_tile(1)       ? 1
                                                          : 2;
-  for (int ctas : {RING_CTAS_PER_SM, 2})
+  for (int ctas : {RING_CTAS_PER_SM, RING_CTAS_PER_SM - 1, 2})
     for (int q = q0; q < 3; ++q) {
       const int c = ctas * ring_tile(0) / ring_tile(q);  // the same number of warps
       const size_t smem = c * (plan(q, 3).smem + 1024);

@@ -501,7 +501,7 @@ int sell_make_copies(Arena& ar, Sell& A, int vstore, cudaStream_t s) {
 }
 
 template <int TPR>
-__global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
+__global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
     k_spmv64(SellView<double> A, double alpha, const double* __restrict__ x, double beta,
              double* __restrict__ y) {
   const Lanes<TPR> ln;
@@ -518,7 +518,7 @@ int sell_spmv64(const Sell& A, double alpha, const double* x, double beta, doubl
                 int num_sms, cudaStream_t s) {
   const int grid = sell_grid(sell_groups(A), num_sms);
   SellView<double> v = view(A, (const double*)A.v64);
-  AMG_DISPATCH_TPR(sell_code(A),
+  AMG_DISPATCH_TPR(sell_code(A, 8),
                    (k_spmv64<TPR><<<grid, SELL_BLOCK, 0, s>>>(v, alpha, x, beta, y)));
   AMG_LAUNCH_CHECK();
   return AMG_OK;

@@ -23,11 +23,22 @@ constexpr int SELL_BLOCK = 256;  // threads per block (8 slices in flight)
 // or 16 and 32 for wide rows) plus SELL_D16 when the matrix stores
 // compressed columns (1..8 threads per row only).
 constexpr int SELL_D16 = 64;
+// ... or plus SELL_IX (one thread per row, slices of 32 rows) when the matrix
+// has packed column indices (Sell::rec): the row's loads are then issued in
+// chunks of its exact length, all values and gathers of up to 8 entries
+// together.  The plain loop takes four entries at a time and the rest one by
+// one, each a column load and the gather that waits for it.
+constexpr int SELL_IX = 128;
+
+// Resident blocks the streaming kernels are compiled for: packed indices keep
+// twice the loads in flight per thread and need the registers for them.
+constexpr int sell_blocks(int code) { return (code & SELL_IX) ? 4 : 8; }
 
 template <int TPR>
 struct Lanes {
-  static constexpr int W = TPR & 63;  // threads per row
+  static constexpr int W = TPR & 63;  // threads per row (1 with SELL_IX)
   static constexpr bool D16 = (TPR & SELL_D16) != 0;
+  static constexpr bool IX = (TPR & SELL_IX) != 0;
   static constexpr int C = 32 / W;
   int r, t;
   __device__ __forceinline__ Lanes() {
@@ -36,6 +47,61 @@ struct Lanes {
     t = lane / C;
   }
 };
+
+// acc (+ or -, NEG) a_k g(col_k) for the N entries k0 .. k0 + N - 1 of this
+// lane's row in a slice with packed indices; val and delta point at the lane's
+// slot of ELL column 0, head at the slice's index block.
+template <int MODE, int N, bool NEG, typename AccT, typename V, typename G>
+__device__ __forceinline__ AccT ix_chunk(const V* __restrict__ val,
+                                         const int32_t* __restrict__ head,
+                                         const uint16_t* __restrict__ delta, int32_t i,
+                                         int32_t last, int lane, int k0, AccT acc, G g) {
+  V a[N];
+  int32_t j[N];
+#pragma unroll
+  for (int u = 0; u < N; ++u) {
+    const int k = k0 + u;
+    a[u] = ld_stream(val + k * 32);
+    if constexpr (MODE == IX_PLAIN)
+      j[u] = ld_stream(head + k * 32 + lane);
+    else if constexpr (MODE == IX_DELTA)
+      j[u] = __ldg(head + k) + (int)ld_stream(delta + k * 32);
+    else if constexpr (MODE == IX_OFFSET)
+      j[u] = i + __ldg(head + k);
+    else
+      j[u] = min(max(i + __ldg(head + k), 0), last);
+  }
+  AccT x[N];
+#pragma unroll
+  for (int u = 0; u < N; ++u) x[u] = g(j[u]);
+#pragma unroll
+  for (int u = 0; u < N; ++u) {
+    const AccT e = to_f(a[u], AccT(0));
+    acc = fma(NEG ? -e : e, x[u], acc);
+  }
+  return acc;
+}
+
+template <int MODE, bool NEG, typename AccT, typename V, typename G>
+__device__ __forceinline__ AccT ix_row(const V* __restrict__ val,
+                                       const int32_t* __restrict__ head, int w, int32_t i,
+                                       int32_t last, int lane, AccT acc, G g) {
+  const uint16_t* delta = (const uint16_t*)(head + ((w + 3) & ~3)) + lane;
+#define AMG_IX_CHUNK(N) ix_chunk<MODE, N, NEG>(val, head, delta, i, last, lane, k0, acc, g)
+  int k0 = 0;
+  for (; k0 + 8 <= w; k0 += 8) acc = AMG_IX_CHUNK(8);
+  switch (w - k0) {
+    case 1: return AMG_IX_CHUNK(1);
+    case 2: return AMG_IX_CHUNK(2);
+    case 3: return AMG_IX_CHUNK(3);
+    case 4: return AMG_IX_CHUNK(4);
+    case 5: return AMG_IX_CHUNK(5);
+    case 6: return AMG_IX_CHUNK(6);
+    case 7: return AMG_IX_CHUNK(7);
+    default: return acc;
+  }
+#undef AMG_IX_CHUNK
+}
 
 // sum_k a_{row,k} * g(col_{row,k}) over the entries of this lane's row in
 // warp row-group s (32/TPR rows), accumulated in AccT.  When the slice height
@@ -53,6 +119,20 @@ template <int TPR, typename AccT, bool NEG = false, typename V, typename G>
 __device__ __forceinline__ AccT sell_row(const SellView<V>& A, int64_t s, const Lanes<TPR>& ln,
                                          G g, AccT init = AccT(0)) {
   constexpr int C = Lanes<TPR>::C, W = Lanes<TPR>::W;
+  if constexpr (Lanes<TPR>::IX) {
+    const longlong2 r0 = __ldg((const longlong2*)(A.rec + s));
+    const int64_t e = __ldg(&A.rec[s + 1].slot);
+    const V* val = A.val + r0.x + ln.r;
+    const int32_t* head = (const int32_t*)(A.ix + (r0.y & ~(int64_t)3));
+    const int w = (int)((e - r0.x) >> 5);
+    const int32_t i = (int32_t)A.rbeg(s, 32) + ln.r, last = A.ncols - 1;
+    switch ((int)(r0.y & 3)) {  // warp-uniform
+      case IX_OFFSET: return ix_row<IX_OFFSET, NEG>(val, head, w, i, last, ln.r, init, g);
+      case IX_CLAMP: return ix_row<IX_CLAMP, NEG>(val, head, w, i, last, ln.r, init, g);
+      case IX_DELTA: return ix_row<IX_DELTA, NEG>(val, head, w, i, last, ln.r, init, g);
+      default: return ix_row<IX_PLAIN, NEG>(val, head, w, i, last, ln.r, init, g);
+    }
+  }
   AccT acc = ln.t == 0 ? init : AccT(0);
   if (!A.row0 && A.C != C) {
     const int64_t i = s * C + ln.r;
@@ -130,11 +210,18 @@ __device__ __forceinline__ AccT sell_row(const SellView<V>& A, int64_t s, const 
     AMG_SELL_CASE(66, __VA_ARGS__)         \
     AMG_SELL_CASE(68, __VA_ARGS__)         \
     AMG_SELL_CASE(72, __VA_ARGS__)         \
+    AMG_SELL_CASE(129, __VA_ARGS__)        \
     default:                               \
       return AMG_ERR_ARG;                  \
   }
 
-inline int sell_code(const Sell& A) { return A.tpr | (A.d16 ? SELL_D16 : 0); }
+// vbytes: size of the values the kernel streams.  Packed indices for FP64 values
+// only: with FP32 ones twice the warps per SM are worth more than exact chunks
+// (batched 12.2M-row pre-smoother 142 us, 169 with them; FP64 product 209, 172
+// with them).
+inline int sell_code(const Sell& A, size_t vbytes) {
+  return A.tpr | (A.rec && vbytes == 8 ? SELL_IX : A.d16 ? SELL_D16 : 0);
+}
 
 // Warp row-groups of 32/tpr rows that the one-warp-per-group kernels iterate
 // over A (see SellView::ngroups).

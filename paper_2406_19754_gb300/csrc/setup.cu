@@ -191,8 +191,17 @@ __global__ void k_match_expand(const int32_t* __restrict__ wl, const int* __rest
       const int32_t v = side == 0 ? i : m;
       for (int64_t e = rowptr[v]; e < rowptr[v + 1]; ++e) {
         const int32_t k = col[e];
-        if (k != v && mate[k] == -1 && atomicExch(&flag[k], 1) == 0)
-          wl_next[atomicAdd(nwl_next, 1)] = k;
+        // most neighbours are on the list already (or matched): look before the
+        // atomic; one counter update per converged group of lanes
+        if (k != v && mate[k] == -1 && *(volatile int32_t*)&flag[k] == 0 &&
+            atomicExch(&flag[k], 1) == 0) {
+          const unsigned m = __activemask();
+          const int lead = __ffs(m) - 1, lane = threadIdx.x & 31;
+          int base = 0;
+          if (lane == lead) base = atomicAdd(nwl_next, __popc(m));
+          base = __shfl_sync(m, base, lead);
+          wl_next[base + __popc(m & ((1u << lane) - 1u))] = k;
+        }
       }
     }
   }
@@ -884,7 +893,7 @@ __global__ void k_scale_cols(int64_t m, const int32_t* __restrict__ col,
       const int64_t e = e0 + u * stride;
       if (e < m) {
         const double v = __dmul_rn(a[u], sj[u]);
-        out64[e] = v;
+        if (out64) out64[e] = v;
         if (out32) out32[e] = (float)v;
         if (out16) out16[e] = __float2bfloat16_rn((float)v);
       }
@@ -894,7 +903,8 @@ __global__ void k_scale_cols(int64_t m, const int32_t* __restrict__ col,
 
 static int build_ah(Arena& ar, Level& L, int num_sms, cudaStream_t s) {
   const int64_t m = L.A.nnz_pad;
-  if (!L.ah64) AMG_TRY(ar.alloc_n(&L.ah64, m));
+  // only the copy the V-cycle reads
+  if (L.vstore == VAL_F64 && !L.ah64) AMG_TRY(ar.alloc_n(&L.ah64, m));
   if (L.vstore == VAL_F32 && !L.ah32) AMG_TRY(ar.alloc_n(&L.ah32, m));
   if (L.vstore == VAL_BF16 && !L.ah16) AMG_TRY(ar.alloc_n(&L.ah16, m));
   int occ = 0;  // a grid of the CTAs that fit at once (no partial second wave)
@@ -1012,17 +1022,25 @@ static int auto_tpr(int64_t rows, int64_t nnz, bool f64) {
   return t;
 }
 
-// Sliced-ELL copies of A P, P (both with A's slices and plain column
-// indices, so one kernel walks both with the same layout code) and R = P^T
+// Sliced-ELL copies of A P, P (both with A's slices, and packed column indices
+// for both or neither, so one kernel walks both with the same layout code) and
+// R = P^T
 // of a smoothed level; R's rows (the fine rows around an aggregate) are
 // long, so it gets its own threads per row (at least 4 once they average 16
 // entries).
-static int build_smoothed_ops(Arena& ar, Level& L, bool compress, cudaStream_t s) {
+static int build_smoothed_ops(Arena& ar, Level& L, bool compress, bool ring, cudaStream_t s) {
   L.ap_nnz = L.q_nnz;
   AMG_TRY(sell_from_csr(ar, L.n, L.nc, L.q_rp, L.q_ci, L.q_v, L.A.C, L.A.tpr, L.AP, s, nullptr,
-                        false));
+                        false, ring));
   AMG_TRY(sell_from_csr(ar, L.n, L.nc, L.p_rp, L.p_ci, L.p_v, L.A.C, L.A.tpr, L.P, s, nullptr,
-                        false));
+                        false, ring));
+  if (!L.AP.rec != !L.P.rec)  // one of them too wide to pack: neither
+    for (Sell* M : {&L.AP, &L.P}) {
+      ar.release(M->rec);
+      ar.release(M->ix);
+      M->rec = nullptr;
+      M->ix = nullptr;
+    }
   const int rt = std::max(auto_tpr(L.nc, L.p_nnz, L.vstore == VAL_F64),
                           L.p_nnz >= 16 * L.nc ? 4 : 1);
   AMG_TRY(sell_from_csr(ar, L.nc, L.n, L.t_rp, L.t_ci, L.t_v, 32 / rt, rt, L.R, s, nullptr,
@@ -1123,7 +1141,7 @@ int set_level0_weights(amg_handle* H, const float* omega, cudaStream_t s) {
   k_smoother_scale<<<grid_for(L.n, 256, H->num_sms, 8), 256, 0, s>>>(L.n, L.dinv, omega, L.s64,
                                                                      L.s32);
   AMG_LAUNCH_CHECK();
-  if (L.ah64) AMG_TRY(build_ah(H->arena, L, H->num_sms, s));
+  if (L.ah64 || L.ah32 || L.ah16) AMG_TRY(build_ah(H->arena, L, H->num_sms, s));
   return AMG_OK;
 }
 
@@ -1382,15 +1400,15 @@ int setup_hierarchy(amg_handle* H, const amg_csr* A, cudaStream_t s, const amg_h
     const bool smooth = l + 1 < H->L.size();  // a level with a coarser one
     auto build = [&](Layout lay) -> int {
       const bool cmp = o.compress_columns != 0;
-      // the ring streams plain-column matrices of one system
-      const bool ring = o.stream_ring != 0 && !cmp && !H->batched &&
+      // packed indices: the ring's kernels, and the batched per-lane ones
+      const bool ring = o.stream_ring != 0 && !cmp &&
                         (l == 0 || L.vstore != VAL_BF16);
       AMG_TRY(sell_from_csr(ar, L.n, L.n, rp, ci, va, lay.C, lay.tpr, L.A, s,
                             H->batched ? &L.sys_off : nullptr, cmp, ring));
       if (smooth) {
         AMG_TRY(build_ah(ar, L, sms, s));
         if (o.smooth_prolongator)
-          AMG_TRY(build_smoothed_ops(ar, L, cmp, s));
+          AMG_TRY(build_smoothed_ops(ar, L, cmp, ring, s));
         else
           AMG_TRY(build_ap(ar, L, rp, ci, va, cmp, ring, sms, s));
       }

@@ -29,7 +29,7 @@
 namespace amg {
 
 template <int TPR>
-__global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
+__global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
     k_tg_smooth(SellView<double> A, const double* __restrict__ s, const double* __restrict__ x,
                 double* __restrict__ out, double* __restrict__ Ax) {
   const Lanes<TPR> ln;
@@ -202,7 +202,7 @@ int twogrid_loss(amg_handle* H, int nsamples, int K, const double* e0, double* l
     return sell_spmv64(L0.A, 1.0, x, 0.0, y, H->num_sms, s);
   };
   auto smooth = [&](const double* x, double* o, double* Ax) -> int {
-    AMG_DISPATCH_TPR(sell_code(L0.A),
+    AMG_DISPATCH_TPR(sell_code(L0.A, 8),
                      (k_tg_smooth<TPR><<<gs, SELL_BLOCK, 0, s>>>(A, sv, x, o, Ax)));
     AMG_LAUNCH_CHECK();
     return AMG_OK;

@@ -50,11 +50,14 @@ int Arena::alloc(void** p, size_t bytes) {
       return AMG_OK;
     }
     if (small) {
-      if (slab_used + bytes > ARENA_SLAB) {
+      if (slab_used + bytes > slab_bytes) {
         void* s = nullptr;
-        const int rc = device_malloc(&s, ARENA_SLAB);
+        const size_t size =
+            std::min(std::max(2 * slab_bytes, ARENA_SLAB_MIN), ARENA_SLAB_MAX);
+        const int rc = device_malloc(&s, size);
         if (rc < 0) return rc;
         slabs.push_back(s);
+        slab_bytes = size;
         slab_used = 0;
       }
       *p = (unsigned char*)slabs.back() + slab_used;
@@ -94,7 +97,6 @@ void Arena::end_reuse() {
   reuse = false;
   drop_kept();
   kept_small.clear();  // their slabs stay with the arena
-  slab_used = ARENA_SLAB;
 }
 
 void Arena::release_all() {
@@ -105,7 +107,7 @@ void Arena::release_all() {
   blocks.clear();
   for (void* s : slabs) cudaFree(s);
   slabs.clear();
-  slab_used = ARENA_SLAB;
+  slab_bytes = slab_used = 0;
 }
 
 int grid_for(int64_t work_items, int threads, int num_sms, int blocks_per_sm) {

@@ -15,7 +15,11 @@
 // b - A y = (b - A S b) - A P x_c.  The level-0 k_post can also reduce (r, z)
 // and (z, q) for the PCG step.
 #include <algorithm>
+#include <map>
+#include <mutex>
+#include <type_traits>
 
+#include "cluster.cuh"
 #include "ring.cuh"
 #include "smooth.cuh"
 
@@ -24,7 +28,7 @@ namespace amg {
 // ------------------------------------------------------------------ kernels
 
 template <int TPR, typename V, typename T, typename BT>
-__global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
+__global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
     k_pre(SellView<V> Ah, const BT* __restrict__ b, T* __restrict__ r) {
   const Lanes<TPR> ln;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -39,6 +43,17 @@ __global__ void k_restrict(int64_t nc, int stride, const int32_t* __restrict__ m
   for (int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; I < nc;
        I += (int64_t)gridDim.x * blockDim.x)
     bc[I] = restrict_sum<LdRO>(members + I * stride, stride, r);
+}
+
+// Aggregates of up to four rows: one 16-byte load of the members, then the
+// gathers together (12.2M rows in batches, FP32: 30.8 -> 26.5 us; no change on
+// large regular grids, where DRAM is the bound).
+template <typename T>
+__global__ void k_restrict4(int64_t nc, const int32_t* __restrict__ members,
+                            const T* __restrict__ r, T* __restrict__ bc) {
+  for (int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; I < nc;
+       I += (int64_t)gridDim.x * blockDim.x)
+    bc[I] = restrict_sum4<LdRO>(members + 4 * I, r);
 }
 
 // Epilogue of the level-0 post-smoother when it feeds PCG: t[0] = (r, z),
@@ -65,7 +80,7 @@ struct VcycleDotEpi {
 // reduction there cost 10% on 256^3 Poisson).  Batched systems use
 // k_post_chunks below.
 template <int TPR, typename V, typename T, typename BT, typename XT, int NDOT, bool MS>
-__global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
+__global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
     k_post(SellView<V> AP, const BT* __restrict__ b, const T* __restrict__ s,
            const T* __restrict__ r, const int32_t* __restrict__ agg, const T* __restrict__ xc,
            XT* __restrict__ x, const double* __restrict__ q, Reduce red, PcgScalars* sc,
@@ -107,7 +122,7 @@ __global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
 // keeps the sums per thread over the chunk's slices and reduces once at its
 // end into part[2 c], part[2 c + 1] (no warp reduction in the slice loop).
 template <int TPR, typename V, typename T, typename BT, typename XT, int NDOT>
-__global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
+__global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
     k_post_chunks(SellView<V> AP, int64_t nchunks, const int64_t* __restrict__ chunk_off,
                   const BT* __restrict__ b, const T* __restrict__ s, const T* __restrict__ r,
                   const int32_t* __restrict__ agg, const T* __restrict__ xc,
@@ -233,24 +248,30 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
 }
 
 // Further sweeps (k_sweep_pre / k_sweep_post): per-row operands in the order
-// s, r, then (PRE) b before the first of them, else x (POST: y).
-template <bool PRE, typename V, typename T, typename BT, typename YT>
+// s, r, then (PRE) b before the first of them, else x (POST: y), and for the
+// last one on level 0 of PCG (NDOT > 0) the right-hand side and q of its dot
+// products (b, y) and (y, q), which otherwise take a pass of their own (50 us
+// on 8M rows).
+template <bool PRE, typename V, typename T, typename BT, typename YT, int NDOT>
 __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
     k_sweep_ring(const __grid_constant__ SellView<V> Ah, const T* __restrict__ r,
                  T* __restrict__ r_out, YT* __restrict__ x, int first,
                  const __grid_constant__ RingGeom g, const __grid_constant__ RingRows rows,
-                 int* fail) {
+                 int* fail, Reduce red, PcgScalars* sc) {
   extern __shared__ unsigned char ring_smem[];
-  if (*(volatile int*)fail) return;
+  if (*(volatile int*)fail) return;  // the host resets the reduction ticket
+  constexpr int ND = NDOT > 0 ? NDOT : 1;
+  double d[ND];
+#pragma unroll
+  for (int k = 0; k < ND; ++k) d[k] = 0.0;
+  int* status = NDOT > 0 ? &sc->status : nullptr;
   TileRing<V> ring(Ah, g, rows, ring_smem);
-  if (ring.producer()) {
-    ring.produce(fail, nullptr);
-    return;
-  }
-  for (int64_t t = blockIdx.x; t < ring.ntiles; t += gridDim.x) {
+  const bool producer = ring.producer();
+  if (producer) ring.produce(fail, status);
+  for (int64_t t = blockIdx.x; !producer && t < ring.ntiles; t += gridDim.x) {
     if (!ring.wait(t)) {
-      if (ring.lane == 0) ring_fail(fail, nullptr);
-      return;
+      if (ring.lane == 0) ring_fail(fail, status);
+      break;
     }
     if (ring.sl < Ah.nslices) {
       const int64_t i = ring.sl * 32 + ring.lane;
@@ -266,12 +287,17 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
                              : ring.template row<T>(2, i);
           x[i] = sweep_pre_x(xi, si, ri);
         } else {
-          x[i] = sweep_post_y(ring.template row<YT>(2, i), si, rn);
+          const YT yi = sweep_post_y(ring.template row<YT>(2, i), si, rn);
+          x[i] = yi;
+          if constexpr (NDOT > 0) d[0] += ring.template row<double>(3, i) * (double)yi;
+          if constexpr (NDOT > 1)
+            d[NDOT > 1 ? 1 : 0] += (double)yi * ring.template row<double>(4, i);
         }
       }
     }
     ring.release();
   }
+  if constexpr (NDOT > 0) grid_reduce<NDOT>(d, red, VcycleDotEpi{sc});
 }
 
 // Post-smoother of a level with a smoothed prolongator P (Sec. 2.3; A P in
@@ -280,7 +306,7 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
 // r - (A P) x_c for further sweeps.  V: stored values, T: V-cycle vectors,
 // BT / XT: this level's b and output (FP64 on level 0).
 template <int TPR, typename V, typename T, typename BT, typename XT>
-__global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
+__global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
     k_post_sm(SellView<V> AQ, SellView<V> P, const BT* __restrict__ b,
               const T* __restrict__ s, const T* __restrict__ r, const T* __restrict__ xc,
               const T* __restrict__ xp, XT* __restrict__ x, T* __restrict__ e) {
@@ -303,7 +329,7 @@ __global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
 
 // b_c = R r for a smoothed level (R = P^T, own slices); V-cycle vector types.
 template <int TPR, typename V, typename T>
-__global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
+__global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
     k_restrict_sm(SellView<V> R, const T* __restrict__ r, T* __restrict__ bc) {
   const Lanes<TPR> ln;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -318,7 +344,7 @@ __global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
 // Pre-smoothing sweeps 2..nu on the residual recurrence: x += S r (x = S b
 // before the first of them), r_out = r - (A S) r.
 template <int TPR, typename V, typename T, typename BT>
-__global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
+__global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
     k_sweep_pre(SellView<V> Ah, const T* __restrict__ s, const BT* __restrict__ b,
                 const T* __restrict__ r, T* __restrict__ r_out, T* __restrict__ x, int first) {
   const Lanes<TPR> ln;
@@ -340,7 +366,7 @@ __global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
 // Post-smoothing sweeps 2..nu: r_out = r - (A S) r (the residual of y after
 // its last update), then y += S r_out.
 template <int TPR, typename V, typename T, typename YT>
-__global__ void __launch_bounds__(SELL_BLOCK, SELL_MIN_BLOCKS)
+__global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
     k_sweep_post(SellView<V> Ah, const T* __restrict__ s, const T* __restrict__ r,
                  T* __restrict__ r_out, YT* __restrict__ y) {
   const Lanes<TPR> ln;
@@ -474,6 +500,34 @@ __global__ void k_coarse_y(int64_t nco, int nblk, const int64_t* __restrict__ br
     coarse_y_row<LdRO>(g, nblk, brow, bmat, Linv_all, b, y);
 }
 
+// The same for one block of at most COARSE_PAIR_ROWS rows: warp g takes rows g
+// and n - 1 - g, n + 1 terms together, so every SM has the same number of FP64
+// operations (the pipe bounds this: 4.3M FMAs a triangle of 2,949 rows), and
+// the vector is converted to FP64 once per CTA instead of once per term.  One
+// row per warp took 33 (y) and 28 us (x).
+constexpr int64_t COARSE_PAIR_ROWS = 5632;  // 44 KB of shared memory
+
+template <bool TRANSPOSED, typename BT, typename XT>
+__global__ void __launch_bounds__(256)
+    k_coarse_pair(int n, const double* __restrict__ M, const BT* __restrict__ v,
+                  XT* __restrict__ out) {
+  extern __shared__ double csh[];
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x; i < n; i += 256) csh[i] = (double)v[i];
+  __syncthreads();
+  const int nw = (int)((gridDim.x * 256) >> 5);
+  for (int g = (int)((blockIdx.x * 256 + threadIdx.x) >> 5); g < (n + 1) / 2; g += nw)
+    for (int h = 0; h < 2; ++h) {
+      const int i = h ? n - 1 - g : g;
+      if (h && i == g) break;
+      const double* row = M + (int64_t)i * n;
+      const double acc = warp_sum(dense_row(row, TRANSPOSED ? i + lane : lane,
+                                            TRANSPOSED ? n : i + 1,
+                                            [&](int64_t k) { return csh[k]; }));
+      if (lane == 0) out[i] = (XT)acc;
+    }
+}
+
 template <typename XT>
 __global__ void k_coarse_x(int64_t nco, int nblk, const int64_t* __restrict__ brow,
                            const int64_t* __restrict__ bmat,
@@ -495,6 +549,134 @@ __global__ void __launch_bounds__(1024, 1)
   coarse_pcg_cta<TPR>(A, sinv, b, xo, w ? w : wsh, maxit, tol);
 }
 
+// The same solve with 32 rows per CTA of one cluster (up to CPCG_CTAS CTAs),
+// their matrix rows in shared memory.  One CTA is bound by its SM: two FP64
+// operations a clock and a block-wide barrier after every step (a 174-row,
+// 15,080-entry level took 225 us, a 31-row one 78 us, through L2).  Warp 0 of
+// each CTA holds its rows' x, r and z; every CTA keeps all of p.  Partial dot
+// products (one per 32 rows, coarse_pcg_cta's warps) and z go to every CTA, so
+// an iteration has two cluster barriers, and every sum is the same tree: the
+// same bits as coarse_pcg_cta.
+constexpr int CPCG_CTAS = 16;
+constexpr int CPCG_ROWS = 32 * CPCG_CTAS;
+
+template <int TPR>
+struct CpcgSmem {
+  static constexpr int W = Lanes<TPR>::W;
+  double p[CPCG_ROWS], z[CPCG_ROWS];
+  double part[3][32];  // (p, q), (r, r), (r, z) of every CTA
+  double q[32];
+  int sp[W + 1];
+  double beta;
+  int stop;
+};
+
+template <int TPR, typename BT, typename XT>
+__global__ void __launch_bounds__(32 * Lanes<TPR>::W)
+    k_coarse_pcg_cluster(SellView<double> A, const double* __restrict__ sinv,
+                         const BT* __restrict__ b, XT* __restrict__ xo, int ctas, int maxit,
+                         double tol) {
+  constexpr int W = Lanes<TPR>::W, C = Lanes<TPR>::C;
+  extern __shared__ __align__(16) unsigned char cp_smem[];
+  CpcgSmem<TPR>& S = *(CpcgSmem<TPR>*)cp_smem;
+  double* val = (double*)(cp_smem + ((sizeof(CpcgSmem<TPR>) + 15) & ~(size_t)15));
+  const int g = (int)cluster_rank(), n = (int)A.n;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // this CTA's W slices of C rows
+  if (threadIdx.x <= W) {
+    const int64_t s0 = (int64_t)g * W, s = s0 + threadIdx.x;
+    S.sp[threadIdx.x] = (int)(A.sliceptr[s < A.nslices ? s : A.nslices] -
+                              A.sliceptr[s0 < A.nslices ? s0 : A.nslices]);
+  }
+  const int64_t base = A.sliceptr[(int64_t)g * W < A.nslices ? (int64_t)g * W : A.nslices];
+  __syncthreads();
+  const int slots = S.sp[W];
+  uint16_t* col = (uint16_t*)(val + slots);
+  for (int e = threadIdx.x; e < slots; e += 32 * W) {
+    val[e] = A.val[base + e];
+    col[e] = (uint16_t)A.col[base + e];
+  }
+  const int i = 32 * g + lane;  // warp 0: this lane's row
+  const bool has = warp == 0 && i < n;
+  const double si = has ? sinv[i] : 0.0;
+  double x = 0.0, r = has ? (double)b[i] : 0.0, z = si * r, rz = 0.0, bnorm = 0.0;
+  const uint32_t o_part = smem_addr(S.part), o_z = smem_addr(S.z);
+  // slot g of partial `which` in every CTA
+  auto send = [&](int which, double v) {
+    v = warp_sum(v);
+    if (lane < ctas) st_cluster(map_rank(o_part + 8u * (uint32_t)(32 * which + g), lane), v);
+  };
+  auto total = [&](int which) { return warp_sum(lane < ctas ? S.part[which][lane] : 0.0); };
+  auto send_z = [&]() {
+    for (int k = 0; has && k < ctas; ++k) st_cluster(map_rank(o_z + 8u * (uint32_t)i, k), z);
+  };
+  cluster_barrier();  // every CTA has started: its memory can be written
+  if (warp == 0) {
+    send(1, has ? r * r : 0.0);
+    send(2, has ? r * z : 0.0);
+    send_z();
+  }
+  cluster_barrier();
+  if (warp == 0) {
+    bnorm = sqrt(total(1));
+    rz = total(2);
+    if (lane == 0) S.stop = !(bnorm > 0.0);
+  }
+  for (int k = threadIdx.x; k < n; k += 32 * W) S.p[k] = S.z[k];
+  __syncthreads();
+  for (int it = 0; it < maxit && !S.stop; ++it) {
+    {  // q = A p on this CTA's rows (sell_row's order)
+      const int s0 = S.sp[warp], w = (S.sp[warp + 1] - s0) / C;
+      const int rr = lane % C, t = lane / C;
+      const double* a = val + s0 + rr;
+      const uint16_t* c = col + s0 + rr;
+      double acc = 0.0;
+#pragma unroll 4
+      for (int k = t; k < w; k += W) acc = fma(a[k * C], S.p[c[k * C]], acc);
+#pragma unroll
+      for (int o = C; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (t == 0) S.q[warp * C + rr] = acc;
+    }
+    __syncthreads();
+    if (warp == 0) send(0, has ? S.p[i] * S.q[lane] : 0.0);
+    cluster_barrier();
+    if (warp == 0) {
+      const double pq = total(0);
+      const bool go = pq > 0.0;
+      if (go) {
+        const double alpha = rz / pq;
+        double d0 = 0.0, d1 = 0.0;
+        if (has) {
+          x = x + alpha * S.p[i];
+          r = r - alpha * S.q[lane];
+          z = si * r;
+          d0 = r * r;
+          d1 = r * z;
+        }
+        send(1, d0);
+        send(2, d1);
+        send_z();
+      } else if (lane == 0) {
+        S.stop = 1;
+      }
+    }
+    cluster_barrier();
+    if (warp == 0 && !S.stop) {
+      const double rr = total(1), rzn = total(2);
+      if (lane == 0) {
+        S.stop = sqrt(rr) <= tol * bnorm;
+        S.beta = rzn / rz;
+      }
+      rz = rzn;
+    }
+    __syncthreads();
+    if (S.stop) break;
+    for (int k = threadIdx.x; k < n; k += 32 * W) S.p[k] = S.z[k] + S.beta * S.p[k];
+    __syncthreads();
+  }
+  if (has) xo[i] = bnorm > 0.0 ? (XT)x : XT(0);
+}
+
 // Largest PCG coarsest level whose work vectors go to shared memory (within
 // the default 48 KB of dynamic shared memory, so no attribute call is needed
 // while a graph is being captured).
@@ -502,16 +684,74 @@ constexpr int64_t COARSE_PCG_SMEM_ROWS = 1152;  // 5 x 1152 doubles = 45 KB, plu
 
 // ------------------------------------------------------------------ driver
 
+constexpr size_t CPCG_SMEM = 200 * 1024;
+
+// Attributes of a cluster PCG kernel, once per device and kernel; *ok: whether
+// a cluster of this launch can be scheduled.
+static int cpcg_prepare(const void* fn, const cudaLaunchConfig_t& cfg, bool* ok) {
+  static std::mutex mu;
+  static std::map<std::pair<const void*, std::pair<int, int>>, bool> known;
+  int dev = 0;
+  AMG_CUDA_TRY(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lock(mu);
+  const auto key = std::make_pair(fn, std::make_pair(dev, (int)cfg.gridDim.x));
+  auto it = known.find(key);
+  if (it == known.end()) {
+    AMG_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    AMG_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)CPCG_SMEM));
+    cudaLaunchConfig_t most = cfg;  // the answer holds for every smaller level
+    most.dynamicSmemBytes = CPCG_SMEM;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, fn, &most) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    it = known.emplace(key, n > 0).first;
+  }
+  *ok = it->second;
+  return AMG_OK;
+}
+
 template <typename BT, typename XT>
 static int coarse_solve(const amg_handle* H, const BT* b, XT* x, cudaStream_t s,
                         const int* act = nullptr) {
   if (H->opt.coarse_solver == 1) {  // PCG with l1-Jacobi (non-batched handles only)
     const Level& Lc = H->L.back();
     const SellView<double> v = view<double>(Lc.A, Lc.A.v64);
+    // 32 rows a CTA: shared memory for the widest possible group of slices
+    const size_t cw = ((sizeof(CpcgSmem<32>) + 15) & ~(size_t)15) + (size_t)Lc.A.wmax * 32 * 10;
+    if (Lc.n <= CPCG_ROWS && Lc.A.C * Lc.A.tpr == 32 && !Lc.A.d16 && cw <= CPCG_SMEM) {
+      int ctas = 1;
+      while (32 * ctas < Lc.n) ctas <<= 1;
+      cudaLaunchAttribute at[1] = {};
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = ctas;
+      at[0].val.clusterDim.y = 1;
+      at[0].val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(ctas);
+      cfg.blockDim = dim3(32 * Lc.A.tpr);
+      cfg.dynamicSmemBytes = cw;
+      cfg.stream = s;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      bool done = false;
+      AMG_DISPATCH_TPR(sell_code(Lc.A, 8), {
+        if constexpr (!Lanes<TPR>::D16) {
+          auto fn = k_coarse_pcg_cluster<TPR, BT, XT>;
+          AMG_TRY(cpcg_prepare((const void*)fn, cfg, &done));
+          if (done)
+            AMG_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, v, (const double*)Lc.s64, b, x, ctas,
+                                            H->opt.coarse_maxit, H->opt.coarse_tol));
+        }
+      });
+      if (done) return AMG_OK;
+    }
     const bool sh = Lc.n <= COARSE_PCG_SMEM_ROWS;
     const size_t smem = sh ? sizeof(double) * 5 * (size_t)Lc.n : 0;
     double* w = sh ? nullptr : H->cpcg;
-    AMG_DISPATCH_TPR(sell_code(Lc.A), (k_coarse_pcg<TPR, BT, XT><<<1, 1024, smem, s>>>(
+    AMG_DISPATCH_TPR(sell_code(Lc.A, 8), (k_coarse_pcg<TPR, BT, XT><<<1, 1024, smem, s>>>(
                                           v, Lc.s64, b, x, w, H->opt.coarse_maxit,
                                           H->opt.coarse_tol)));
     AMG_LAUNCH_CHECK();
@@ -523,6 +763,15 @@ static int coarse_solve(const amg_handle* H, const BT* b, XT* x, cudaStream_t s,
     const size_t sm = sizeof(double) * 2 * (size_t)m;
     k_coarse<BT, XT><<<H->nblk, 1024, sm, s>>>(H->d_brow, H->d_bmat, H->Linv, H->LinvT, b, x,
                                                act);
+    AMG_LAUNCH_CHECK();
+    return AMG_OK;
+  }
+  if (H->nblk == 1 && m <= COARSE_PAIR_ROWS) {
+    const int n = (int)m, g = grid_for((m + 1) / 2 * 32, 256, H->num_sms, 4);
+    const size_t sm = sizeof(double) * (size_t)n;
+    k_coarse_pair<false, BT, double><<<g, 256, sm, s>>>(n, H->Linv, b, H->coarse_y);
+    AMG_LAUNCH_CHECK();
+    k_coarse_pair<true, double, XT><<<g, 256, sm, s>>>(n, H->LinvT, H->coarse_y, x);
     AMG_LAUNCH_CHECK();
     return AMG_OK;
   }
@@ -559,7 +808,7 @@ static int launch_pre(const amg_handle* H, const Level& L, const V* ah, const BT
       }
     }
   }
-  AMG_DISPATCH_TPR(sell_code(L.A),
+  AMG_DISPATCH_TPR(sell_code(L.A, sizeof(V)),
                    (k_pre<TPR, V, T, BT><<<grid, SELL_BLOCK, 0, s>>>(v, b, r)));
   AMG_LAUNCH_CHECK();
   return AMG_OK;
@@ -604,7 +853,7 @@ static int launch_post(const amg_handle* H, const Level& L, const V* ap, const B
       }
     }
     if (in.xp) {
-      AMG_DISPATCH_TPR(sell_code(L.AP),
+      AMG_DISPATCH_TPR(sell_code(L.AP, sizeof(V)),
                        (k_post<TPR, V, T, BT, XT, 0, true><<<grid, SELL_BLOCK, 0, s>>>(
                            v, b, sc, r, L.agg, xc, x, q, H->red, H->sc, in.xp, in.e)));
       AMG_LAUNCH_CHECK();
@@ -636,14 +885,14 @@ static int launch_post(const amg_handle* H, const Level& L, const V* ap, const B
       const Batch& B = H->batch;
       if (!B.chunk_off) return AMG_ERR_ARG;
       const int cg = sell_grid(B.nchunks, H->num_sms);
-      AMG_DISPATCH_TPR(sell_code(L.AP),
+      AMG_DISPATCH_TPR(sell_code(L.AP, sizeof(V)),
                        (k_post_chunks<TPR, V, T, BT, XT, NDOT><<<cg, SELL_BLOCK, 0, s>>>(
                            v, B.nchunks, B.chunk_off, b, sc, r, L.agg, xc, x, q, slice_part)));
       AMG_LAUNCH_CHECK();
       return AMG_OK;
     }
   }
-  AMG_DISPATCH_TPR(sell_code(L.AP),
+  AMG_DISPATCH_TPR(sell_code(L.AP, sizeof(V)),
                    (k_post<TPR, V, T, BT, XT, NDOT, false><<<grid, SELL_BLOCK, 0, s>>>(
                        v, b, sc, r, L.agg, xc, x, q, H->red, H->sc, nullptr, nullptr)));
   AMG_LAUNCH_CHECK();
@@ -652,9 +901,19 @@ static int launch_post(const amg_handle* H, const Level& L, const V* ap, const B
 
 // One further pre- (PRE) or post-smoothing sweep of level L on the residual
 // recurrence (k_sweep_pre / k_sweep_post).
+// dots > 0: the last sweep of level 0 in PCG, with right-hand side r0 and q; it
+// forms the dot products too if it runs on the ring (*fused).
+struct SweepDots {
+  int dots = 0;
+  const double* r0 = nullptr;
+  const double* q = nullptr;
+  bool fused = false;
+};
+
 template <bool PRE, typename T, typename BT, typename YT>
 static int launch_sweep(const amg_handle* H, const Level& L, const BT* b, const T* r, T* r_out,
-                        YT* x, int first, cudaStream_t s, const int* act) {
+                        YT* x, int first, cudaStream_t s, const int* act,
+                        SweepDots* sd = nullptr) {
   const int grid = sell_grid(sell_groups(L.A), H->num_sms);
   const T* sc = (const T*)(sizeof(T) == 8 ? (const void*)L.s64 : (const void*)L.s32);
   auto go = [&](auto vtag, const auto* ah) -> int {
@@ -670,22 +929,36 @@ static int launch_sweep(const amg_handle* H, const Level& L, const BT* b, const 
           rows.add(b, (int)sizeof(BT));
         else
           rows.add(x, (int)sizeof(YT));
-        RingGeom g = ring_plan(L.A, (int)sizeof(V), ring_stages(H), rows);
-        if (g.D) {
-          AMG_TRY(ring_prepare((const void*)k_sweep_ring<PRE, V, T, BT, YT>, g, L.A.nslices,
+        auto run = [&](auto nd) -> int {
+          constexpr int ND = decltype(nd)::value;
+          if (ND > 0) rows.add(sd->r0, (int)sizeof(double));
+          if (ND > 1) rows.add(sd->q, (int)sizeof(double));
+          RingGeom g = ring_plan(L.A, (int)sizeof(V), ring_stages(H), rows, ND > 0);
+          if (!g.D) return 1;
+          AMG_TRY(ring_prepare((const void*)k_sweep_ring<PRE, V, T, BT, YT, ND>, g, L.A.nslices,
                                H->num_sms));
-          k_sweep_ring<PRE, V, T, BT, YT><<<g.grid, g.threads(), g.smem, s>>>(
-              v, r, r_out, x, first, g, rows, H->wait_fail);
+          k_sweep_ring<PRE, V, T, BT, YT, ND><<<g.grid, g.threads(), g.smem, s>>>(
+              v, r, r_out, x, first, g, rows, H->wait_fail, H->red, H->sc);
           AMG_LAUNCH_CHECK();
+          if (ND > 0) sd->fused = true;
           return AMG_OK;
+        };
+        int rc = 1;
+        if constexpr (!PRE && sizeof(YT) == 8) {
+          if (sd && sd->dots == 1) rc = run(std::integral_constant<int, 1>());
+          else if (sd && sd->dots == 2) rc = run(std::integral_constant<int, 2>());
+          else rc = run(std::integral_constant<int, 0>());
+        } else {
+          rc = run(std::integral_constant<int, 0>());
         }
+        if (rc <= 0) return rc;
       }
     }
     if constexpr (PRE) {
-      AMG_DISPATCH_TPR(sell_code(L.A), (k_sweep_pre<TPR, V, T, BT><<<grid, SELL_BLOCK, 0, s>>>(
+      AMG_DISPATCH_TPR(sell_code(L.A, sizeof(V)), (k_sweep_pre<TPR, V, T, BT><<<grid, SELL_BLOCK, 0, s>>>(
                                             v, sc, b, r, r_out, (T*)x, first)));
     } else {
-      AMG_DISPATCH_TPR(sell_code(L.A), (k_sweep_post<TPR, V, T, YT><<<grid, SELL_BLOCK, 0, s>>>(
+      AMG_DISPATCH_TPR(sell_code(L.A, sizeof(V)), (k_sweep_post<TPR, V, T, YT><<<grid, SELL_BLOCK, 0, s>>>(
                                             v, sc, r, r_out, x)));
     }
     AMG_LAUNCH_CHECK();
@@ -715,7 +988,7 @@ static int launch_restrict(const amg_handle* H, const Level& L, const T* r, T* b
     auto go = [&](auto vtag) -> int {
       using V = decltype(vtag);
       const SellView<V> v = view<V>(L.R, sm_vals<V>(L.R));
-      AMG_DISPATCH_TPR(sell_code(L.R),
+      AMG_DISPATCH_TPR(sell_code(L.R, sizeof(V)),
                        (k_restrict_sm<TPR, V, T><<<grid, SELL_BLOCK, 0, s>>>(v, r, bc)));
       AMG_LAUNCH_CHECK();
       return AMG_OK;
@@ -723,8 +996,11 @@ static int launch_restrict(const amg_handle* H, const Level& L, const T* r, T* b
     if constexpr (sizeof(T) == 8) return go(double(0));
     else return L.vstore == VAL_BF16 ? go(__nv_bfloat16()) : go(float(0));
   }
-  k_restrict<T><<<grid_for(L.nc, 256, H->num_sms, 8), 256, 0, s>>>(L.nc, L.stride, L.members, r,
-                                                                   bc);
+  const int grid = grid_for(L.nc, 256, H->num_sms, 8);
+  if (L.stride == 4)  // member tables start on 256 bytes
+    k_restrict4<T><<<grid, 256, 0, s>>>(L.nc, L.members, r, bc);
+  else
+    k_restrict<T><<<grid, 256, 0, s>>>(L.nc, L.stride, L.members, r, bc);
   AMG_LAUNCH_CHECK();
   return AMG_OK;
 }
@@ -744,12 +1020,12 @@ static int launch_post_sm(const amg_handle* H, const Level& L, const BT* b, cons
   const int grid = sell_grid(sell_groups(L.AP), H->num_sms);
   const T* sc = (const T*)(sizeof(T) == 8 ? (const void*)L.s64 : (const void*)L.s32);
   const T* r = in.r ? in.r : (const T*)L.r;
-  if (sell_code(L.AP) != sell_code(L.P)) return AMG_ERR_UNSUPPORTED;
+  if (sell_code(L.AP, 8) != sell_code(L.P, 8)) return AMG_ERR_UNSUPPORTED;
   auto go = [&](auto vtag) -> int {
     using V = decltype(vtag);
     const SellView<V> q = view<V>(L.AP, sm_vals<V>(L.AP));
     const SellView<V> p = view<V>(L.P, sm_vals<V>(L.P));
-    AMG_DISPATCH_TPR(sell_code(L.AP), (k_post_sm<TPR, V, T, BT, XT><<<grid, SELL_BLOCK, 0, s>>>(
+    AMG_DISPATCH_TPR(sell_code(L.AP, sizeof(V)), (k_post_sm<TPR, V, T, BT, XT><<<grid, SELL_BLOCK, 0, s>>>(
                                           q, p, b, sc, r, xc, in.xp, x, in.e)));
     AMG_LAUNCH_CHECK();
     return AMG_OK;
@@ -975,12 +1251,20 @@ static int vcycle_levels(const amg_handle* H, const double* r0, double* z0, int 
     }
     return in;
   };
+  bool dots_done = false;
   auto post_sweeps = [&](const Level& L, int l, auto* y) -> int {
     for (int64_t m = 2; m <= L.nu; ++m) {
       const int c = cur[l];
       PROF_BEGIN(l, 5, sweep_bytes(L));
+      SweepDots sd;  // (r, z) and (z, q) of PCG with level 0's last sweep
+      if (l == 0 && m == L.nu && !slice_part) {
+        sd.dots = dots;
+        sd.r0 = r0;
+        sd.q = q;
+      }
       AMG_TRY((launch_sweep<false, T, T>(H, L, (const T*)nullptr, rbuf(L, c), rbuf(L, 1 - c), y,
-                                         0, s, act)));
+                                         0, s, act, &sd)));
+      dots_done = dots_done || sd.fused;
       PROF_END();
       cur[l] = 1 - c;
     }
@@ -1014,7 +1298,7 @@ static int vcycle_levels(const amg_handle* H, const double* r0, double* z0, int 
   AMG_TRY(rc);
   PROF_END();
   if (L0.nu > 1) AMG_TRY(post_sweeps(L0, 0, z0));
-  if (separate) AMG_TRY(separate_dots());
+  if (separate && !dots_done) AMG_TRY(separate_dots());
   return AMG_OK;
 }
 
