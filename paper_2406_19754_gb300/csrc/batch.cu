@@ -16,6 +16,7 @@
 
 #include <algorithm>
 
+#include "ring.cuh"
 #include "sellk.cuh"
 
 namespace amg {
@@ -78,6 +79,43 @@ __global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
     }
     d = warp_sum(d);
     if ((threadIdx.x & 31) == 0) part[2 * c] = d;
+  }
+}
+
+// k_b_spmv_dot on the ring (chunks of one system, ring.cuh): (p, q) per chunk
+// and warp.
+__global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
+    k_b_spmv_ring(const __grid_constant__ SellView<double> A, const double* __restrict__ p,
+                  double* __restrict__ q, double* __restrict__ part,
+                  const __grid_constant__ RingGeom g, const __grid_constant__ RingRows rows,
+                  const __grid_constant__ RingChunks ch, int* fail) {
+  extern __shared__ unsigned char ring_smem[];
+  if (*(volatile int*)fail) return;
+  TileRing<double, true> ring(A, g, rows, ch, ring_smem);
+  if (ring.producer()) {
+    ring.produce(fail, nullptr);
+    return;
+  }
+  double d = 0.0;
+  while (ring.more()) {
+    if (!ring.wait()) {
+      if (ring.lane == 0) ring_fail(fail, nullptr);
+      return;
+    }
+    if (ring.ended) return;
+    if (ring.slice) {
+      const double acc = ring_row_sum<double>(ring, [&](int j) { return __ldg(p + j); });
+      if (ring.has) {
+        q[ring.i] = acc;
+        d += ring.row<double>(0) * acc;
+      }
+    }
+    if (ring.last) {
+      const double v = warp_sum(d);
+      if (ring.lane == 0) part[2 * (ring.chunk * RING_MAX_TILE + ring.warp)] = v;
+      d = 0.0;
+    }
+    ring.release();
   }
 }
 
@@ -204,8 +242,11 @@ template <int MODE>
 static int seg(const BatchRun& R, cudaStream_t s) {
   const Batch& B = R.H->batch;
   const int grid = std::max(1, std::min(B.nsys, R.H->num_sms * 8));
-  k_b_seg<MODE><<<grid, 256, 0, s>>>(B.nsys, B.sys_chunk, B.part, B.sc, R.tol, R.maxit,
-                                     R.beta_form, B.nactive, B.active);
+  // the post-smoother's and the product's partials may come from the ring
+  const bool ring = B.ring && (MODE == SEG_PQ || MODE == SEG_RZ || MODE == SEG_RZ_FIRST);
+  k_b_seg<MODE><<<grid, 256, 0, s>>>(B.nsys, ring ? B.rsys : B.sys_chunk,
+                                     ring ? B.rpart : B.part, B.sc, R.tol, R.maxit, R.beta_form,
+                                     B.nactive, B.active);
   AMG_LAUNCH_CHECK();
   return AMG_OK;
 }
@@ -227,6 +268,20 @@ static int b_residual(const BatchRun& R, const double* b, const double* x, doubl
 
 static int b_spmv_dot(const amg_handle* H, cudaStream_t s) {
   const Batch& B = H->batch;
+  if (B.ring) {
+    const Level& L = H->L[0];
+    RingRows rows;
+    rows.add(H->p, (int)sizeof(double));
+    RingGeom g = ring_plan(L.A, 8, ring_stages(H), rows, true, true);
+    if (!g.D) return AMG_ERR_UNSUPPORTED;  // Batch::ring said it fits
+    AMG_TRY(ring_prepare((const void*)k_b_spmv_ring, g, L.rch_n, H->num_sms));
+    SellView<double> v = a0(H);
+    v.act = B.active;
+    k_b_spmv_ring<<<g.grid, g.threads(), g.smem, s>>>(
+        v, H->p, H->q, B.rpart, g, rows, RingChunks{L.rch_off, L.rch_n}, H->wait_fail);
+    AMG_LAUNCH_CHECK();
+    return AMG_OK;
+  }
   AMG_DISPATCH_TPR(sell_code(H->L[0].A, 8),
                    (k_b_spmv_dot<TPR><<<chunk_grid(H), SELL_BLOCK, 0, s>>>(
                        a0(H), B.nchunks, B.chunk_off, H->p, H->q, B.part, B.sc)));
@@ -409,6 +464,55 @@ int pcg_batch_run(amg_handle* H, const double* b, double* x, const pcg_options* 
   return tc < 0 ? tc : worst;
 }
 
+// Chunk lists of the ring streams for the levels with enough slices to fill the
+// GPU (eight per CTA, two CTAs on each of 152 SMs; smaller levels stay with the
+// per-lane kernels), about four chunks for each resident CTA and 8 to 128 slices
+// each.  Level 0's kernels with dot products use the ring if all of them fit.
+static int batch_rings(amg_handle* H, cudaStream_t s) {
+  Batch& B = H->batch;
+  if (!H->opt.stream_ring) return AMG_OK;
+  const int nl = (int)H->L.size();
+  for (int l = 0; l < nl - 1; ++l) {
+    Level& L = H->L[l];
+    if (!L.A.rec || !L.A.row0 || !L.AP.rec || L.A.C != 32 || L.A.nslices < 304 * RING_MAX_TILE)
+      continue;
+    int64_t per = L.A.nslices / (4 * RING_CTAS_PER_SM * (int64_t)H->num_sms);
+    per = std::min<int64_t>(std::max<int64_t>(per / RING_MAX_TILE, 1), 16) * RING_MAX_TILE;
+    std::vector<int64_t> off, sys(B.nsys + 1, 0);
+    int64_t sl = 0;
+    for (int k = 0; k < B.nsys; ++k) {
+      sys[k] = (int64_t)off.size() * RING_MAX_TILE;
+      const int64_t end = sl + (L.sys_off[k + 1] - L.sys_off[k] + 31) / 32;
+      for (; sl < end; sl = std::min(sl + per, end)) off.push_back(sl);
+    }
+    if (sl != L.A.nslices) return AMG_ERR_DEVICE_CHECK;
+    L.rch_n = (int64_t)off.size();
+    sys[B.nsys] = L.rch_n * RING_MAX_TILE;
+    off.push_back(sl);
+    AMG_TRY(H->arena.alloc_n(&L.rch_off, L.rch_n + 1));
+    AMG_CUDA_TRY(cudaMemcpyAsync(L.rch_off, off.data(), sizeof(int64_t) * off.size(),
+                                 cudaMemcpyHostToDevice, s));
+    if (l == 0 && L.nu == 1 && L.vstore != VAL_BF16) {
+      const int vb = L.vstore == VAL_F64 ? 8 : 4;
+      RingRows post, prod;  // element sizes as launch_post and b_spmv_dot stage them
+      for (int e : {vb, vb, 8, 4, 8}) post.add(nullptr, e);
+      prod.add(nullptr, 8);
+      B.ring = ring_plan(L.AP, vb, ring_stages(H), post, true, true).D > 0 &&
+               ring_plan(L.A, 8, ring_stages(H), prod, true, true).D > 0;
+      if (B.ring) {
+        AMG_TRY(H->arena.alloc_n(&B.rpart, 2 * L.rch_n * RING_MAX_TILE));
+        AMG_TRY(H->arena.alloc_n(&B.rsys, B.nsys + 1));
+        AMG_CUDA_TRY(cudaMemsetAsync(B.rpart, 0,
+                                     sizeof(double) * 2 * L.rch_n * RING_MAX_TILE, s));
+        AMG_CUDA_TRY(cudaMemcpyAsync(B.rsys, sys.data(), sizeof(int64_t) * sys.size(),
+                                     cudaMemcpyHostToDevice, s));
+      }
+    }
+    AMG_CUDA_TRY(cudaStreamSynchronize(s));  // host vectors go out of scope
+  }
+  return AMG_OK;
+}
+
 // Batch bookkeeping after the hierarchy exists: tile ranges per system.
 int batch_init(amg_handle* H, cudaStream_t s) {
   Batch& B = H->batch;
@@ -449,7 +553,7 @@ int batch_init(amg_handle* H, cudaStream_t s) {
   AMG_CUDA_TRY(cudaMemsetAsync(B.part, 0, sizeof(double) * 2 * B.nchunks, s));
   AMG_CUDA_TRY(cudaMemsetAsync(B.sc, 0, sizeof(Scal) * B.nsys, s));
   AMG_CUDA_TRY(cudaStreamSynchronize(s));
-  return AMG_OK;
+  return batch_rings(H, s);
 }
 
 // ------------------------------------------------------------------ concatenation

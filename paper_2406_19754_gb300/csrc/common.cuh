@@ -141,6 +141,7 @@ struct Sell {
   SliceRec* rec = nullptr;
   unsigned char* ix = nullptr;
   int tile_w[3] = {}, tile_ix[3] = {};
+  int64_t ix_bytes = 0;  // of all index blocks
 };
 
 template <typename V>
@@ -212,8 +213,11 @@ struct Level {
   int64_t nu = 1;
   void* r2 = nullptr;
   void* xp = nullptr;
-  // batched systems: first row of each system on this level (nsys + 1, host)
+  // batched systems: first row of each system on this level (nsys + 1, host),
+  // and the chunks of the ring streams (ring.cuh; none: per-lane kernels)
   std::vector<int64_t> sys_off;
+  int64_t* rch_off = nullptr;
+  int64_t rch_n = 0;
   // smoothed prolongator (option smooth_prolongator, Sec. 2.3): P = (I - w
   // D^-1 A) P_hat (n x nc CSR, kept for export, and sliced ELL with A's
   // slices), its transpose R = P^T as sliced ELL (restriction), and AP above
@@ -250,6 +254,11 @@ struct Batch {
   int64_t* chunk_off = nullptr;  // device, nchunks + 1: first slice of chunk c
   int64_t* sys_chunk = nullptr;  // device, nsys + 1: first chunk of system k
   double* part = nullptr;        // device, 2 * nchunks: per-chunk partial sums
+  // level-0 kernels with dot products on the ring: their partials are two per
+  // ring chunk and warp, system k's from rsys[k] to rsys[k + 1]
+  bool ring = false;
+  double* rpart = nullptr;
+  int64_t* rsys = nullptr;
   struct Scal* sc = nullptr;     // device, nsys
   struct Scal* sc_host = nullptr;  // pinned, nsys
   int* active = nullptr;         // device, nsys: copy of each system's active flag

@@ -101,29 +101,26 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
     k_spmv_dot_ring(const __grid_constant__ SellView<double> A, const double* __restrict__ p,
                     double* __restrict__ q, Reduce red, PcgScalars* sc,
                     const __grid_constant__ RingGeom g, const __grid_constant__ RingRows rows,
-                    int* fail) {
+                    const __grid_constant__ RingChunks ch, int* fail) {
   extern __shared__ unsigned char ring_smem[];
   if (*(volatile int*)fail) return;  // the host resets the reduction ticket
   double d[1] = {0.0};
-  TileRing<double> ring(A, g, rows, ring_smem);
-  if (ring.producer()) {
-    ring.produce(fail, &sc->status);
-  } else {
-    for (int64_t t = blockIdx.x; t < ring.ntiles; t += gridDim.x) {
-      if (!ring.wait(t)) {
-        if (ring.lane == 0) ring_fail(fail, &sc->status);
-        break;
-      }
-      if (ring.sl < A.nslices) {
-        const int64_t i = ring.sl * 32 + ring.lane;
-        const double acc = ring_row_sum<double>(ring, i, [&](int j) { return __ldg(p + j); });
-        if (i < A.n) {
-          q[i] = acc;
-          d[0] += ring.template row<double>(0, i) * acc;
-        }
-      }
-      ring.release();
+  TileRing<double> ring(A, g, rows, ch, ring_smem);
+  const bool producer = ring.producer();
+  if (producer) ring.produce(fail, &sc->status);
+  while (!producer && ring.more()) {
+    if (!ring.wait()) {
+      if (ring.lane == 0) ring_fail(fail, &sc->status);
+      break;
     }
+    if (ring.slice) {
+      const double acc = ring_row_sum<double>(ring, [&](int j) { return __ldg(p + j); });
+      if (ring.has) {
+        q[ring.i] = acc;
+        d[0] += ring.template row<double>(0) * acc;
+      }
+    }
+    ring.release();
   }
   grid_reduce<1>(d, red, PqEpi{sc});
 }
@@ -281,9 +278,9 @@ static int launch_spmv_dot(const amg_handle* H, cudaStream_t s) {
     rows.add(H->p, (int)sizeof(double));
     RingGeom g = ring_plan(L.A, 8, ring_stages(H), rows, true);
     if (g.D) {
-      AMG_TRY(ring_prepare((const void*)k_spmv_dot_ring, g, L.A.nslices, H->num_sms));
+      AMG_TRY(ring_prepare((const void*)k_spmv_dot_ring, g, ring_tiles(g, L.A), H->num_sms));
       k_spmv_dot_ring<<<g.grid, g.threads(), g.smem, s>>>(v, H->p, H->q, H->red, H->sc, g,
-                                                          rows, H->wait_fail);
+                                                          rows, RingChunks(), H->wait_fail);
       AMG_LAUNCH_CHECK();
       return AMG_OK;
     }

@@ -18,9 +18,12 @@ namespace amg {
 // a diffusion matrix (18 KB stages) 0.092 against 0.080.
 constexpr size_t RING_L1_SPLIT = 128 * 1024;
 
-RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows, bool dots) {
+RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows, bool dots,
+                   bool chunked) {
   RingGeom none;
-  if (M.C != 32 || M.tpr != 1 || M.row0 || !M.rec || M.wmax <= 0 || M.nslices <= 0) return none;
+  if (M.C != 32 || M.tpr != 1 || (M.row0 != nullptr) != chunked || !M.rec || M.wmax <= 0 ||
+      M.nslices <= 0)
+    return none;
   if (vbytes != 2 && vbytes != 4 && vbytes != 8) return none;
   if (stages == 1 || stages > RING_MAX_STAGES || rows.n > RING_MAX_ROWS) return none;
   uint32_t direct = 0;
@@ -38,9 +41,14 @@ RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows, 
     off = up(off + (size_t)M.tile_ix[q]);
     g.soff = (uint32_t)off;
     off = up(off + 16 * (size_t)(g.tile + 1));
+    if (chunked) {
+      g.hoff = (uint32_t)off;
+      off = up(off + sizeof(RingTile));
+    }
     for (int k = 0; k < rows.n; ++k) {
       g.roff[k] = (uint32_t)off;
-      off = up(off + 32 * (size_t)(g.tile * rows.esz[k]));
+      // (chunked: up to three rows more on either side of the tile's)
+      off = up(off + (size_t)(32 * g.tile + (chunked ? 8 : 0)) * rows.esz[k]);
     }
     g.D = D;
     g.direct = direct;
@@ -51,11 +59,11 @@ RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows, 
   // smaller tiles where 8 slices a CTA would leave SMs without work (two
   // CTAs on each of 152); with dot products 8 slices, the blocks of the
   // per-lane kernels, so that both sum small levels alike
-  const int q0 = dots || M.nslices >= 304 * ring_tile(0) ? 0
+  const int q0 = dots || chunked || M.nslices >= 304 * ring_tile(0) ? 0
                  : M.nslices >= 304 * ring_tile(1)       ? 1
                                                          : 2;
   for (int ctas : {RING_CTAS_PER_SM, RING_CTAS_PER_SM - 1, 2})
-    for (int q = q0; q < 3; ++q) {
+    for (int q = q0; q < (chunked ? 1 : 3); ++q) {
       const int c = ctas * ring_tile(0) / ring_tile(q);  // the same number of warps
       const size_t smem = c * (plan(q, 3).smem + 1024);
       const RingGeom g = plan(q, stages ? stages : smem <= RING_L1_SPLIT ? 3 : 2);
@@ -65,7 +73,7 @@ RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows, 
   return none;
 }
 
-int ring_prepare(const void* fn, RingGeom& g, int64_t nslices, int num_sms) {
+int ring_prepare(const void* fn, RingGeom& g, int64_t work, int num_sms) {
   static std::mutex mu;
   static std::map<std::pair<const void*, int>, bool> attr;
   static std::map<std::pair<const void*, std::pair<size_t, int>>, int> occ;
@@ -92,9 +100,8 @@ int ring_prepare(const void* fn, RingGeom& g, int64_t nslices, int num_sms) {
     per_sm = nb;
   }
   if (per_sm < 1) return AMG_ERR_UNSUPPORTED;
-  const int64_t need = (nslices + g.tile - 1) / g.tile;  // one tile per CTA
   const int64_t full = (int64_t)num_sms * std::min(per_sm, 16);  // grid reductions hold 16 per SM
-  g.grid = (int)(need < full ? need : full);
+  g.grid = (int)(work < full ? work : full);
   return AMG_OK;
 }
 

@@ -32,9 +32,15 @@
 // and their number bounds them); here the copies are whole blocks, so bytes
 // are what counts.
 //
+// Batched systems (CHUNKED): a CTA takes chunks of consecutive slices of one
+// system, leaves out those of systems that have stopped, and cuts each into
+// tiles; the producer writes what a tile is (RingTile) into its stage, and a
+// last, empty one where the work ends.  A system's rows start anywhere, so the
+// per-row copies start at the 16-byte boundary before them.
+//
 // Requirements (checked on the host by ring_plan): one thread per row and
-// slice height 32 (lane = row of the slice), one system (no row0), packed
-// indices (Sell::rec), and tiles that fit a stage.  Slice s starts at slot
+// slice height 32 (lane = row of the slice), packed indices (Sell::rec), and
+// tiles that fit a stage.  Slice s starts at slot
 // rec[s].slot, a multiple of 32, and its index block at a multiple of 16 bytes,
 // so all copies start on 16-byte boundaries and have sizes that are multiples
 // of 16 bytes (32 w values of 2, 4 or 8 bytes; ix_bytes; 16-byte records); the
@@ -88,11 +94,25 @@ struct RingGeom {
   uint32_t stage = 0;   // bytes per stage
   uint32_t coff = 0;    // offset of the index blocks within a stage
   uint32_t soff = 0;    // offset of the slice records
+  uint32_t hoff = 0;    // offset of the tile's description (CHUNKED)
   uint32_t roff[RING_MAX_ROWS] = {};  // offsets of the per-row vectors
   uint32_t direct = 0;  // bit k: row vector k starts off a 16-byte boundary, read directly
   int grid = 0;         // CTAs (ring_prepare)
   size_t smem = 0;      // dynamic shared memory per CTA
   int threads() const { return (tile + 1) * 32; }
+};
+
+// Chunks of a batched level: chunk c is slices off[c] .. off[c + 1] - 1, all of
+// one system.
+struct RingChunks {
+  const int64_t* off = nullptr;
+  int64_t n = 0;
+};
+// A chunked tile: ns slices (-1: the end of the work) from slice s0 and row r0,
+// `rows` rows; the staged per-row vectors start at row e0.
+struct RingTile {
+  int64_t s0, r0, e0, chunk;
+  int32_t ns, rows, staged, last;  // last: of its chunk
 };
 
 // ------------------------------------------------------------------ PTX wrappers
@@ -171,41 +191,49 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 // ------------------------------------------------------------------ the CTA's ring
 
 // Usage (every thread of the CTA):
-//   TileRing<V> ring(A, g, rows, smem);
+//   TileRing<V, CHUNKED> ring(A, g, rows, chunks, smem);
 //   if (ring.producer()) ring.produce(fail, status);
-//   else for (int64_t t = blockIdx.x; t < ring.ntiles; t += gridDim.x) {
-//     if (!ring.wait(t)) { report; break; }
-//     if (ring.sl < A.nslices) { ... ring_row_sum(ring, i, g, init) of slice sl ... }
+//   else while (ring.more()) {
+//     if (!ring.wait()) { report; break; }
+//     if (ring.ended) break;
+//     if (ring.slice) { ... ring_row_sum(ring, g, init) of row ring.i ... }
 //     ring.release();
 //   }
-template <typename V>
+template <typename V, bool CHUNKED = false>
 struct TileRing {
   const SellView<V>& A;
   const RingGeom& g;
   const RingRows& rows;
+  const RingChunks& ch;
   unsigned char* base;   // first stage
   uint32_t bars;         // shared address: full[D], then empty[D]
-  int64_t ntiles;
+  int64_t ntiles;        // (not CHUNKED)
   int warp, lane;
   // consumer state
   int stage = 0;
   uint32_t phase = 0;
-  int64_t sl = 0, t = 0;
+  int64_t t;             // current tile (not CHUNKED)
+  bool ended = false;    // CHUNKED: no more tiles
+  bool slice = false;    // this warp has a slice of the tile
+  bool has = false;      // this lane has a row: row i
+  bool staged_rows = false, last = false;
+  int64_t i = 0, e0 = 0, chunk = 0;
   const unsigned char* st = nullptr;  // current stage
   const unsigned char* vals = nullptr;
   const int32_t* ixb = nullptr;
   int wm = 0;  // (ELL width << 2) | IX_* code
-  bool full_tile = false;
 
   __device__ __forceinline__ TileRing(const SellView<V>& A_, const RingGeom& g_,
-                                      const RingRows& rows_, unsigned char* smem_raw)
-      : A(A_), g(g_), rows(rows_) {
+                                      const RingRows& rows_, const RingChunks& ch_,
+                                      unsigned char* smem_raw)
+      : A(A_), g(g_), rows(rows_), ch(ch_) {
     // 128-byte aligned start (the launch adds RING_ALIGN_SLACK bytes)
     base = smem_raw + ((128u - (smem_addr(smem_raw) & 127u)) & 127u);
     bars = smem_addr(base) + (uint32_t)g.D * g.stage;
     warp = threadIdx.x >> 5;
     lane = threadIdx.x & 31;
     ntiles = (A.nslices + g.tile - 1) / g.tile;
+    t = blockIdx.x;
     if (threadIdx.x == 0) {
       for (int d = 0; d < g.D; ++d) {
         mbar_init(full(d), 1);
@@ -232,76 +260,151 @@ struct TileRing {
     return SliceRec{r.x, r.y};
   }
 
-  // The producer warp: lane 0 copies every tile of this CTA, a stage as soon
-  // as its consumers have left it.  The next tile's bounds are loaded a tile
-  // ahead.
-  __device__ __forceinline__ void produce(int* fail, int* status) {
-    if (lane != 0) return;
-    const uint64_t pol = l2_evict_first();
-    int64_t tt = blockIdx.x;
-    if (tt >= ntiles) return;
-    SliceRec b = load_rec(tt * g.tile), e = load_rec(tt * g.tile + g.tile);
+  // Producer state: the stage the next copies go to.
+  struct Fill {
     int d = 0, issued = 0;
     uint32_t ph = 1;  // the first pass over the stages does not wait
-    for (;;) {
-      const int64_t nx = tt + gridDim.x;
-      SliceRec nb = {0, 0}, ne = {0, 0};
-      if (nx < ntiles) {
-        nb = load_rec(nx * g.tile);
-        ne = load_rec(nx * g.tile + g.tile);
-      }
-      if (issued >= g.D && !mbar_wait_bounded(empty(d), ph)) {
-        atomicExch(fail, 1);
-        if (status) atomicCAS(status, 0, AMG_ERR_DEVICE_CHECK);
-        break;
-      }
-      const int64_t ib = b.ix & ~(int64_t)3;
-      const uint32_t vb = (uint32_t)(e.slot - b.slot) * (uint32_t)sizeof(V);
-      const uint32_t cb = (uint32_t)((e.ix & ~(int64_t)3) - ib);
-      const int64_t s0 = tt * g.tile;
-      const uint32_t ns = (uint32_t)(A.nslices - s0 < g.tile ? A.nslices - s0 : g.tile);
-      const bool f = is_full(tt);
-      uint32_t rb = 0;
-#pragma unroll
-      for (int k = 0; k < RING_MAX_ROWS; ++k)
-        if (staged(f, k)) rb += 32u * (uint32_t)(g.tile * rows.esz[k]);
-      const uint32_t dst = smem_addr(base) + (uint32_t)d * g.stage, fb = full(d);
-      mbar_arrive_expect_tx(fb, vb + cb + 16u * (ns + 1) + rb);
-      bulk_copy_g2s(dst + g.soff, A.rec + s0, 16u * (ns + 1), fb, pol);
-      if (vb > 0) {
-        bulk_copy_g2s(dst, A.val + b.slot, vb, fb, pol);
-        bulk_copy_g2s(dst + g.coff, A.ix + ib, cb, fb, pol);
-      }
-#pragma unroll
-      for (int k = 0; k < RING_MAX_ROWS; ++k)
-        if (staged(f, k))
-          bulk_copy_g2s(dst + g.roff[k],
-                        (const unsigned char*)rows.p[k] + s0 * 32 * rows.esz[k],
-                        32u * (uint32_t)(g.tile * rows.esz[k]), fb, pol);
-      ++issued;
-      if (++d == g.D) {
-        d = 0;
-        ph ^= 1u;
-      }
-      tt = nx;
-      if (tt >= ntiles) break;
-      b = nb;
-      e = ne;
+  };
+  // Waits until the next stage's consumers have left it; false if that gave up.
+  __device__ __forceinline__ bool claim(const Fill& f, int* fail, int* status) const {
+    if (f.issued < g.D || mbar_wait_bounded(empty(f.d), f.ph)) return true;
+    atomicExch(fail, 1);
+    if (status) atomicCAS(status, 0, AMG_ERR_DEVICE_CHECK);
+    return false;
+  }
+  __device__ __forceinline__ void advance(Fill& f) const {
+    ++f.issued;
+    if (++f.d == g.D) {
+      f.d = 0;
+      f.ph ^= 1u;
     }
-    // every copy has landed before the CTA can end (consumers that gave up
-    // leave stages unread)
-    for (int k = issued > g.D ? issued - g.D : 0; k < issued; ++k)
+  }
+  // Starts the copies of slices s0 .. s0 + ns - 1 (records b .. e) and of rows
+  // r0 .. r0 + nr - 1 of the per-row vectors (if fr).
+  __device__ __forceinline__ void fill(const Fill& f, int64_t s0, uint32_t ns, const SliceRec& b,
+                                       const SliceRec& e, bool fr, int64_t r0, uint32_t nr,
+                                       uint64_t pol) const {
+    const int64_t ib = b.ix & ~(int64_t)3;
+    const uint32_t vb = (uint32_t)(e.slot - b.slot) * (uint32_t)sizeof(V);
+    const uint32_t cb = (uint32_t)((e.ix & ~(int64_t)3) - ib);
+    uint32_t rb = 0;
+#pragma unroll
+    for (int k = 0; k < RING_MAX_ROWS; ++k)
+      if (staged(fr, k)) rb += nr * (uint32_t)rows.esz[k];
+    const uint32_t dst = smem_addr(base) + (uint32_t)f.d * g.stage, fb = full(f.d);
+    mbar_arrive_expect_tx(fb, vb + cb + 16u * (ns + 1) + rb);
+    bulk_copy_g2s(dst + g.soff, A.rec + s0, 16u * (ns + 1), fb, pol);
+    if (vb > 0) {
+      bulk_copy_g2s(dst, A.val + b.slot, vb, fb, pol);
+      bulk_copy_g2s(dst + g.coff, A.ix + ib, cb, fb, pol);
+    }
+#pragma unroll
+    for (int k = 0; k < RING_MAX_ROWS; ++k)
+      if (staged(fr, k))
+        bulk_copy_g2s(dst + g.roff[k], (const unsigned char*)rows.p[k] + r0 * rows.esz[k],
+                      nr * (uint32_t)rows.esz[k], fb, pol);
+  }
+  // Every copy has landed before the CTA can end (consumers that gave up leave
+  // stages unread).
+  __device__ __forceinline__ void drain(const Fill& f) const {
+    for (int k = f.issued > g.D ? f.issued - g.D : 0; k < f.issued; ++k)
       if (!mbar_wait_bounded(full(k % g.D), (uint32_t)(k / g.D) & 1u)) break;
   }
 
-  // Waits for tile tt; false if the wait gave up.
-  __device__ __forceinline__ bool wait(int64_t tt) {
+  // The producer warp: lane 0 copies every tile of this CTA, a stage as soon
+  // as its consumers have left it.
+  __device__ __forceinline__ void produce(int* fail, int* status) {
+    if (lane != 0) return;
+    const uint64_t pol = l2_evict_first();
+    Fill f;
+    if constexpr (CHUNKED) {
+      bool ok = true;
+      for (int64_t c = blockIdx.x; ok && c < ch.n; c += gridDim.x) {
+        const int64_t c0 = __ldg(ch.off + c), c1 = __ldg(ch.off + c + 1);
+        if (!A.live(c0)) continue;  // consumers never see this chunk
+        SliceRec b = load_rec(c0);
+        int64_t r0 = __ldg(A.row0 + c0);
+        for (int64_t s0 = c0; s0 < c1; s0 += g.tile) {
+          const int64_t s1 = s0 + g.tile < c1 ? s0 + g.tile : c1;
+          const SliceRec e = load_rec(s1);
+          const int64_t r1 = __ldg(A.row0 + s1);
+          ok = claim(f, fail, status);
+          if (!ok) break;
+          // whole groups of four rows around the tile's: 16-byte boundaries
+          RingTile h;
+          h.e0 = r0 & ~(int64_t)3;
+          const int64_t e1 = (r1 + 3) & ~(int64_t)3;
+          h.s0 = s0;
+          h.r0 = r0;
+          h.chunk = c;
+          h.ns = (int32_t)(s1 - s0);
+          h.rows = (int32_t)(r1 - r0);
+          h.staged = e1 <= A.n;
+          h.last = s1 == c1;
+          *(RingTile*)(base + (size_t)f.d * g.stage + g.hoff) = h;
+          fill(f, s0, (uint32_t)(s1 - s0), b, e, h.staged != 0, h.e0, (uint32_t)(e1 - h.e0), pol);
+          advance(f);
+          b = e;
+          r0 = r1;
+        }
+      }
+      if (ok && claim(f, fail, status)) {  // the end: an empty stage
+        ((RingTile*)(base + (size_t)f.d * g.stage + g.hoff))->ns = -1;
+        mbar_arrive(full(f.d));
+        advance(f);
+      }
+    } else {
+      int64_t tt = blockIdx.x;
+      if (tt >= ntiles) return;
+      // the next tile's bounds are loaded a tile ahead
+      SliceRec b = load_rec(tt * g.tile), e = load_rec(tt * g.tile + g.tile);
+      for (;;) {
+        const int64_t nx = tt + gridDim.x;
+        SliceRec nb = {0, 0}, ne = {0, 0};
+        if (nx < ntiles) {
+          nb = load_rec(nx * g.tile);
+          ne = load_rec(nx * g.tile + g.tile);
+        }
+        if (!claim(f, fail, status)) break;
+        const int64_t s0 = tt * g.tile;
+        const uint32_t ns = (uint32_t)(A.nslices - s0 < g.tile ? A.nslices - s0 : g.tile);
+        fill(f, s0, ns, b, e, is_full(tt), s0 * 32, 32u * (uint32_t)g.tile, pol);
+        advance(f);
+        tt = nx;
+        if (tt >= ntiles) break;
+        b = nb;
+        e = ne;
+      }
+    }
+    drain(f);
+  }
+
+  __device__ __forceinline__ bool more() const { return CHUNKED || t < ntiles; }
+
+  // Waits for the next tile; false if the wait gave up.
+  __device__ __forceinline__ bool wait() {
     if (!__all_sync(0xffffffffu, mbar_wait_bounded(full(stage), phase))) return false;
-    t = tt;
-    sl = tt * g.tile + warp;
     st = base + (size_t)stage * g.stage;
-    full_tile = is_full(tt);
-    if (sl < A.nslices) {
+    if constexpr (CHUNKED) {
+      const RingTile& h = *(const RingTile*)(st + g.hoff);
+      ended = h.ns < 0;
+      if (ended) return true;
+      slice = warp < h.ns;
+      i = h.r0 + warp * 32 + lane;
+      has = slice && warp * 32 + lane < h.rows;
+      e0 = h.e0;
+      staged_rows = h.staged != 0;
+      last = h.last != 0;
+      chunk = h.chunk;
+    } else {
+      const int64_t sl = t * g.tile + warp;
+      slice = sl < A.nslices;
+      i = sl * 32 + lane;
+      has = i < A.n;
+      e0 = t * g.tile * 32;
+      staged_rows = is_full(t);
+    }
+    if (slice) {
       const SliceRec* r = (const SliceRec*)(st + g.soff);
       const SliceRec r0 = r[0], rw = r[warp], rn = r[warp + 1];
       vals = st + (size_t)(rw.slot - r0.slot) * sizeof(V);
@@ -312,10 +415,10 @@ struct TileRing {
   }
 
   __device__ __forceinline__ V val(int k) const { return ((const V*)vals)[k * 32 + lane]; }
-  // entry i = 32 sl + lane of per-row vector k (element type X = its type)
+  // entry i (this lane's row) of per-row vector k (element type X = its type)
   template <typename X>
-  __device__ __forceinline__ X row(int k, int64_t i) const {
-    if (staged(full_tile, k)) return ((const X*)(st + g.roff[k]))[warp * 32 + lane];
+  __device__ __forceinline__ X row(int k) const {
+    if (staged(staged_rows, k)) return ((const X*)(st + g.roff[k]))[(int)(i - e0)];
     return __ldg((const X*)rows.p[k] + i);
   }
 
@@ -323,6 +426,7 @@ struct TileRing {
   __device__ __forceinline__ void release() {
     __syncwarp();
     if (lane == 0) mbar_arrive(empty(stage));
+    t += gridDim.x;
     if (++stage == g.D) {
       stage = 0;
       phase ^= 1u;
@@ -357,9 +461,8 @@ struct IxClamp {
 // values) for k = k0 .. k0 + N - 1, k ascending: the N gathers issue
 // together, then the FMAs follow in order.  Exactly N FMAs: on GB300's FP64
 // pipe a predicated-off FMA would still cost its cycles.
-template <int N, bool NEG, typename T, typename V, typename I, typename G>
-__device__ __forceinline__ T ring_chunk(const TileRing<V>& ring, const I& ix, int k0, T acc,
-                                        G g) {
+template <int N, bool NEG, typename T, typename R, typename I, typename G>
+__device__ __forceinline__ T ring_chunk(const R& ring, const I& ix, int k0, T acc, G g) {
   T x[N];
 #pragma unroll
   for (int u = 0; u < N; ++u) x[u] = g(ix(k0 + u));
@@ -373,9 +476,8 @@ __device__ __forceinline__ T ring_chunk(const TileRing<V>& ring, const I& ix, in
 
 // Chunks of 8 and one remainder chunk of the exact length (w is
 // warp-uniform).
-template <bool NEG, typename T, typename V, typename I, typename G>
-__device__ __forceinline__ T ring_chunks(const TileRing<V>& ring, const I& ix, int w, T acc,
-                                         G g) {
+template <bool NEG, typename T, typename R, typename I, typename G>
+__device__ __forceinline__ T ring_chunks(const R& ring, const I& ix, int w, T acc, G g) {
   int k0 = 0;
   for (; k0 + 8 <= w; k0 += 8) acc = ring_chunk<8, NEG>(ring, ix, k0, acc, g);
   switch (w - k0) {
@@ -394,9 +496,9 @@ __device__ __forceinline__ T ring_chunks(const TileRing<V>& ring, const I& ix, i
 // init + sum_k a_k g(col_k) (NEG: init - sum) over the entries of this
 // lane's row i in the current stage, k ascending (the per-lane kernels'
 // order).
-template <typename T, bool NEG = false, typename V, typename G>
-__device__ __forceinline__ T ring_row_sum(const TileRing<V>& ring, int64_t i, G g,
-                                          T init = T(0)) {
+template <typename T, bool NEG = false, typename R, typename G>
+__device__ __forceinline__ T ring_row_sum(const R& ring, G g, T init = T(0)) {
+  const int64_t i = ring.i;
   const int w = ring.wm >> 2;
   const int32_t* c = ring.ixb;
   switch (ring.wm & 3) {
@@ -421,15 +523,19 @@ __device__ __forceinline__ void ring_fail(int* fail, int* status) {
 
 // Geometry for streaming M (values of `vbytes` bytes) with the ring, or
 // D = 0 when M does not qualify.  stages: 2..RING_MAX_STAGES, or 0 for the
-// default.  dots: the kernel also sums dot products over its grid.  The grid
-// is left to ring_prepare.  Host code.
+// default.  dots: the kernel also sums dot products over its grid.  chunked:
+// for batched systems (M.row0), which only chunked kernels take.  The grid is
+// left to ring_prepare.  Host code.
 RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows,
-                   bool dots = false);
+                   bool dots = false, bool chunked = false);
 
 // Prepares kernel `fn` for a launch with geometry g on the current device
 // (shared-memory limit, once per device and kernel) and sets g.grid to the
-// CTAs that are co-resident (occupancy query), at most one tile per CTA.
+// CTAs that are co-resident (occupancy query), at most `work` (tiles or chunks).
 // Host code.
-int ring_prepare(const void* fn, RingGeom& g, int64_t nslices, int num_sms);
+int ring_prepare(const void* fn, RingGeom& g, int64_t work, int num_sms);
+inline int64_t ring_tiles(const RingGeom& g, const Sell& M) {
+  return (M.nslices + g.tile - 1) / g.tile;
+}
 
 }  // namespace amg

@@ -245,7 +245,8 @@ __global__ void k_sell_fill32(int64_t n, int64_t ncols, int64_t nslices, const i
         if (rec) rec[nslices] = SliceRec{(total >> 32) * 32, (total & 0xffffffffll) << 4};
       }
       for (int q = 0; rec && q < 3; ++q)
-        if (s % ring_tile(q) == 0) {
+        // (batched systems' tiles start at any slice)
+        if (row0 || s % ring_tile(q) == 0) {
           const int64_t e = s + ring_tile(q) < nslices ? pk[s + ring_tile(q)] : total;
           atomicMax(&tm[q], (int)((e >> 32) - (pk[s] >> 32)));
           atomicMax(&tm[3 + q], (int)(((e & 0xffffffffll) << 4) - ib));
@@ -367,7 +368,8 @@ static int sell_from_csr32(Arena& ar, const int64_t* rowptr, const int32_t* col,
   AMG_TRY(ar.alloc_n(&out.v64, out.nnz_pad));
   if (ring) {
     AMG_TRY(ar.alloc_n(&out.rec, out.nslices + 1));
-    AMG_TRY(ar.alloc_n(&out.ix, (total & 0xffffffffll) << 4));
+    out.ix_bytes = (total & 0xffffffffll) << 4;
+    AMG_TRY(ar.alloc_n(&out.ix, out.ix_bytes));
   }
   k_sell_fill32<<<g, 256, 0, s>>>(out.n, out.ncols, out.nslices, out.row0, rowptr, col, val, pk,
                                   total, layout, out.sliceptr, out.col, out.v64, out.rec,

@@ -15,9 +15,6 @@
 namespace amg {
 
 constexpr int SELL_BLOCK = 256;  // threads per block (8 slices in flight)
-// 8 resident blocks per SM (64 warps, full occupancy): at most 32 registers,
-// which the streaming kernels need to keep enough loads in flight.
-#define SELL_MIN_BLOCKS 8
 
 // Layout code of a SELL kernel instantiation: threads per row (1, 2, 4, 8,
 // or 16 and 32 for wide rows) plus SELL_D16 when the matrix stores
@@ -30,8 +27,10 @@ constexpr int SELL_D16 = 64;
 // one, each a column load and the gather that waits for it.
 constexpr int SELL_IX = 128;
 
-// Resident blocks the streaming kernels are compiled for: packed indices keep
-// twice the loads in flight per thread and need the registers for them.
+// Resident blocks per SM the streaming kernels are compiled for: 8 (64 warps,
+// full occupancy: at most 32 registers, which they need to keep enough loads in
+// flight); packed indices keep twice the loads in flight per thread and need
+// the registers for them.
 constexpr int sell_blocks(int code) { return (code & SELL_IX) ? 4 : 8; }
 
 template <int TPR>

@@ -158,93 +158,104 @@ __global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
 // thread over the warp's slices, then per block and over blocks, as there
 // (with this launch's grid).  The rows' own operands (s, r, b, agg, ...) come
 // with the tile (per-row vectors of the ring).
-template <typename V, typename T, typename BT>
+template <typename V, typename T, typename BT, bool CH>
 __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
     k_pre_ring(const __grid_constant__ SellView<V> Ah, const BT* __restrict__ b,
                T* __restrict__ r, const __grid_constant__ RingGeom g,
-               const __grid_constant__ RingRows rows, int* fail) {
+               const __grid_constant__ RingRows rows, const __grid_constant__ RingChunks ch,
+               int* fail) {
   extern __shared__ unsigned char ring_smem[];
   if (*(volatile int*)fail) return;
-  TileRing<V> ring(Ah, g, rows, ring_smem);
+  TileRing<V, CH> ring(Ah, g, rows, ch, ring_smem);
   if (ring.producer()) {
     ring.produce(fail, nullptr);
     return;
   }
-  for (int64_t t = blockIdx.x; t < ring.ntiles; t += gridDim.x) {
-    if (!ring.wait(t)) {
+  while (ring.more()) {
+    if (!ring.wait()) {
       if (ring.lane == 0) ring_fail(fail, nullptr);
       return;
     }
-    if (ring.sl < Ah.nslices) {
-      const int64_t i = ring.sl * 32 + ring.lane;
-      const bool has = i < Ah.n;
-      const T bi = has ? to_f(ring.template row<BT>(0, i), T(0)) : T(0);
+    if (ring.ended) return;
+    if (ring.slice) {
+      const T bi = ring.has ? to_f(ring.template row<BT>(0), T(0)) : T(0);
       // pre_slice's arithmetic: from b_i down by negated FMAs
       const T acc = ring_row_sum<T, true>(
-          ring, i, [&](int j) { return to_f(__ldg(b + j), T(0)); }, bi);
-      if (has) r[i] = acc;
+          ring, [&](int j) { return to_f(__ldg(b + j), T(0)); }, bi);
+      if (ring.has) r[ring.i] = acc;
     }
     ring.release();
   }
 }
 
 // MS: several sweeps (xp the pre-smoothed x, e receives r - AP x_c), as in
-// k_post; per-row operands in the order s, r, b (MS: xp), agg, q.
-template <typename V, typename T, typename BT, typename XT, int NDOT, bool MS>
+// k_post; per-row operands in the order s, r, b (MS: xp), agg, q.  CH (batched
+// systems): the dot products go to part, two per chunk and warp.
+template <typename V, typename T, typename BT, typename XT, int NDOT, bool MS, bool CH>
 __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
     k_post_ring(const __grid_constant__ SellView<V> AP, const T* __restrict__ xc,
                 XT* __restrict__ x, Reduce red, PcgScalars* sc,
                 const __grid_constant__ RingGeom g, const __grid_constant__ RingRows rows,
-                int* fail, T* __restrict__ e) {
+                const __grid_constant__ RingChunks ch, int* fail, T* __restrict__ e,
+                double* __restrict__ part) {
   extern __shared__ unsigned char ring_smem[];
   if (*(volatile int*)fail) return;  // the host resets the reduction ticket
   constexpr int ND = NDOT > 0 ? NDOT : 1;
   double d[ND];
 #pragma unroll
   for (int k = 0; k < ND; ++k) d[k] = 0.0;
-  TileRing<V> ring(AP, g, rows, ring_smem);
-  if (ring.producer()) {
-    ring.produce(fail, NDOT > 0 ? &sc->status : nullptr);
-  } else {
-    for (int64_t t = blockIdx.x; t < ring.ntiles; t += gridDim.x) {
-      if (!ring.wait(t)) {
-        if (ring.lane == 0) ring_fail(fail, NDOT > 0 ? &sc->status : nullptr);
-        break;
-      }
-      if (ring.sl < AP.nslices) {
-        const int64_t i = ring.sl * 32 + ring.lane;
-        const bool has = i < AP.n;
-        // x_c of the row's own aggregate: gathered with the row's entries
-        const T xci = has ? __ldg(xc + ring.template row<int32_t>(3, i)) : T(0);
-        const T ri = has ? ring.template row<T>(1, i) : T(0);
-        if constexpr (MS) {
-          const T acc = ring_row_sum<T>(ring, i, [&](int J) { return __ldg(xc + J); });
-          if (has) {
-            const T si = ring.template row<T>(0, i);
-            const T yi = ring.template row<T>(2, i) + xci;
-            const T ei = ri - acc;
-            x[i] = to_f(fma(si, ei, yi), XT(0));
-            e[i] = ei;
-          }
-        } else {
-          // post_slice's arithmetic (one sweep): from b_i + r_i down, then one FMA
-          const BT bi = has ? ring.template row<BT>(2, i) : BT(0);
-          const T init = has ? to_f(bi, T(0)) + ri : T(0);
-          const T acc =
-              ring_row_sum<T, true>(ring, i, [&](int J) { return __ldg(xc + J); }, init);
-          if (has) {
-            const XT zi = to_f(fma(ring.template row<T>(0, i), acc, xci), XT(0));
-            x[i] = zi;
-            if constexpr (NDOT > 0) d[0] += (double)bi * (double)zi;
-            if constexpr (NDOT > 1)
-              d[NDOT > 1 ? 1 : 0] += (double)zi * ring.template row<double>(4, i);
-          }
+  int* status = NDOT > 0 && !CH ? &sc->status : nullptr;
+  TileRing<V, CH> ring(AP, g, rows, ch, ring_smem);
+  const bool producer = ring.producer();
+  if (producer) ring.produce(fail, status);
+  while (!producer && ring.more()) {
+    if (!ring.wait()) {
+      if (ring.lane == 0) ring_fail(fail, status);
+      break;
+    }
+    if (ring.ended) break;
+    if (ring.slice) {
+      const bool has = ring.has;
+      const int64_t i = ring.i;
+      // x_c of the row's own aggregate: gathered with the row's entries
+      const T xci = has ? __ldg(xc + ring.template row<int32_t>(3)) : T(0);
+      const T ri = has ? ring.template row<T>(1) : T(0);
+      if constexpr (MS) {
+        const T acc = ring_row_sum<T>(ring, [&](int J) { return __ldg(xc + J); });
+        if (has) {
+          const T si = ring.template row<T>(0);
+          const T yi = ring.template row<T>(2) + xci;
+          const T ei = ri - acc;
+          x[i] = to_f(fma(si, ei, yi), XT(0));
+          e[i] = ei;
+        }
+      } else {
+        // post_slice's arithmetic (one sweep): from b_i + r_i down, then one FMA
+        const BT bi = has ? ring.template row<BT>(2) : BT(0);
+        const T init = has ? to_f(bi, T(0)) + ri : T(0);
+        const T acc = ring_row_sum<T, true>(ring, [&](int J) { return __ldg(xc + J); }, init);
+        if (has) {
+          const XT zi = to_f(fma(ring.template row<T>(0), acc, xci), XT(0));
+          x[i] = zi;
+          if constexpr (NDOT > 0) d[0] += (double)bi * (double)zi;
+          if constexpr (NDOT > 1)
+            d[NDOT > 1 ? 1 : 0] += (double)zi * ring.template row<double>(4);
         }
       }
-      ring.release();
     }
+    if constexpr (CH && NDOT > 0) {
+      if (ring.last) {
+#pragma unroll
+        for (int k = 0; k < NDOT; ++k) {
+          const double v = warp_sum(d[k]);
+          if (ring.lane == 0) part[2 * (ring.chunk * RING_MAX_TILE + ring.warp) + k] = v;
+          d[k] = 0.0;
+        }
+      }
+    }
+    ring.release();
   }
-  if constexpr (NDOT > 0) grid_reduce<NDOT>(d, red, VcycleDotEpi{sc});
+  if constexpr (!CH && NDOT > 0) grid_reduce<NDOT>(d, red, VcycleDotEpi{sc});
 }
 
 // Further sweeps (k_sweep_pre / k_sweep_post): per-row operands in the order
@@ -257,7 +268,7 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
     k_sweep_ring(const __grid_constant__ SellView<V> Ah, const T* __restrict__ r,
                  T* __restrict__ r_out, YT* __restrict__ x, int first,
                  const __grid_constant__ RingGeom g, const __grid_constant__ RingRows rows,
-                 int* fail, Reduce red, PcgScalars* sc) {
+                 const __grid_constant__ RingChunks ch, int* fail, Reduce red, PcgScalars* sc) {
   extern __shared__ unsigned char ring_smem[];
   if (*(volatile int*)fail) return;  // the host resets the reduction ticket
   constexpr int ND = NDOT > 0 ? NDOT : 1;
@@ -265,33 +276,32 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
 #pragma unroll
   for (int k = 0; k < ND; ++k) d[k] = 0.0;
   int* status = NDOT > 0 ? &sc->status : nullptr;
-  TileRing<V> ring(Ah, g, rows, ring_smem);
+  TileRing<V> ring(Ah, g, rows, ch, ring_smem);
   const bool producer = ring.producer();
   if (producer) ring.produce(fail, status);
-  for (int64_t t = blockIdx.x; !producer && t < ring.ntiles; t += gridDim.x) {
-    if (!ring.wait(t)) {
+  while (!producer && ring.more()) {
+    if (!ring.wait()) {
       if (ring.lane == 0) ring_fail(fail, status);
       break;
     }
-    if (ring.sl < Ah.nslices) {
-      const int64_t i = ring.sl * 32 + ring.lane;
-      const bool has = i < Ah.n;
-      const T acc = ring_row_sum<T>(ring, i, [&](int j) { return __ldg(r + j); });
-      if (has) {
-        const T ri = ring.template row<T>(1, i);
+    if (ring.slice) {
+      const T acc = ring_row_sum<T>(ring, [&](int j) { return __ldg(r + j); });
+      if (ring.has) {
+        const int64_t i = ring.i;
+        const T ri = ring.template row<T>(1);
         const T rn = ri - acc;
         r_out[i] = rn;
-        const T si = ring.template row<T>(0, i);
+        const T si = ring.template row<T>(0);
         if constexpr (PRE) {
-          const T xi = first ? si * to_f(ring.template row<BT>(2, i), T(0))
-                             : ring.template row<T>(2, i);
+          const T xi = first ? si * to_f(ring.template row<BT>(2), T(0))
+                             : ring.template row<T>(2);
           x[i] = sweep_pre_x(xi, si, ri);
         } else {
-          const YT yi = sweep_post_y(ring.template row<YT>(2, i), si, rn);
+          const YT yi = sweep_post_y(ring.template row<YT>(2), si, rn);
           x[i] = yi;
-          if constexpr (NDOT > 0) d[0] += ring.template row<double>(3, i) * (double)yi;
+          if constexpr (NDOT > 0) d[0] += ring.template row<double>(3) * (double)yi;
           if constexpr (NDOT > 1)
-            d[NDOT > 1 ? 1 : 0] += (double)yi * ring.template row<double>(4, i);
+            d[NDOT > 1 ? 1 : 0] += (double)yi * ring.template row<double>(4);
         }
       }
     }
@@ -793,16 +803,25 @@ static int launch_pre(const amg_handle* H, const Level& L, const V* ah, const BT
   const int grid = sell_grid(sell_groups(L.A), H->num_sms);
   SellView<V> v = view<V>(L.A, ah);
   v.act = act;
-  // FP64 and FP32 operators (BF16 values keep the per-lane kernels)
+  // FP64 and FP32 operators (BF16 values keep the per-lane kernels); batched
+  // levels where the chunk list says so
   if constexpr (sizeof(V) >= 4) {
-    if (!act && H->opt.stream_ring) {
+    if (H->opt.stream_ring && (H->batched ? L.rch_n > 0 : !act)) {
       RingRows rows;
       rows.add(b, (int)sizeof(BT));
-      RingGeom g = ring_plan(L.A, (int)sizeof(V), ring_stages(H), rows);
+      RingGeom g = ring_plan(L.A, (int)sizeof(V), ring_stages(H), rows, false, H->batched);
+      if (g.D && H->batched) {
+        const auto fn = k_pre_ring<V, T, BT, true>;
+        AMG_TRY(ring_prepare((const void*)fn, g, L.rch_n, H->num_sms));
+        fn<<<g.grid, g.threads(), g.smem, s>>>(v, b, r, g, rows, RingChunks{L.rch_off, L.rch_n},
+                                               H->wait_fail);
+        AMG_LAUNCH_CHECK();
+        return AMG_OK;
+      }
       if (g.D) {
-        AMG_TRY(ring_prepare((const void*)k_pre_ring<V, T, BT>, g, L.A.nslices, H->num_sms));
-        k_pre_ring<V, T, BT><<<g.grid, g.threads(), g.smem, s>>>(v, b, r, g, rows,
-                                                                 H->wait_fail);
+        const auto fn = k_pre_ring<V, T, BT, false>;
+        AMG_TRY(ring_prepare((const void*)fn, g, ring_tiles(g, L.A), H->num_sms));
+        fn<<<g.grid, g.threads(), g.smem, s>>>(v, b, r, g, rows, RingChunks(), H->wait_fail);
         AMG_LAUNCH_CHECK();
         return AMG_OK;
       }
@@ -835,7 +854,7 @@ static int launch_post(const amg_handle* H, const Level& L, const V* ap, const B
   const T* r = in.r ? in.r : (const T*)L.r;
   if constexpr (NDOT == 0) {
     if constexpr (sizeof(V) >= 4) {
-      if (in.xp && !act && H->opt.stream_ring) {
+      if (in.xp && !act && !H->batched && H->opt.stream_ring) {
         RingRows rows;  // as read by k_post_ring<MS>
         rows.add(sc, (int)sizeof(T));
         rows.add(r, (int)sizeof(T));
@@ -843,10 +862,10 @@ static int launch_post(const amg_handle* H, const Level& L, const V* ap, const B
         rows.add(L.agg, (int)sizeof(int32_t));
         RingGeom g = ring_plan(L.AP, (int)sizeof(V), ring_stages(H), rows);
         if (g.D) {
-          AMG_TRY(ring_prepare((const void*)k_post_ring<V, T, BT, XT, 0, true>, g, L.AP.nslices,
-                               H->num_sms));
-          k_post_ring<V, T, BT, XT, 0, true><<<g.grid, g.threads(), g.smem, s>>>(
-              v, xc, x, H->red, H->sc, g, rows, H->wait_fail, in.e);
+          const auto fn = k_post_ring<V, T, BT, XT, 0, true, false>;
+          AMG_TRY(ring_prepare((const void*)fn, g, ring_tiles(g, L.AP), H->num_sms));
+          fn<<<g.grid, g.threads(), g.smem, s>>>(v, xc, x, H->red, H->sc, g, rows, RingChunks(),
+                                                 H->wait_fail, in.e, nullptr);
           AMG_LAUNCH_CHECK();
           return AMG_OK;
         }
@@ -862,22 +881,35 @@ static int launch_post(const amg_handle* H, const Level& L, const V* ap, const B
   }
   if (in.xp) return AMG_ERR_ARG;  // several sweeps: the dot products follow separately
   if constexpr (sizeof(V) >= 4) {  // FP64 and FP32 operators, as for k_pre
-    if (!act && !slice_part && H->opt.stream_ring) {
+    // batched: dot products on the ring only where the whole solve counts on
+    // them there (Batch::ring)
+    const bool bring = H->batched && L.rch_n > 0 && (NDOT == 0 || H->batch.ring);
+    if (H->opt.stream_ring && (H->batched ? bring : !act && !slice_part)) {
       RingRows rows;  // indices 0..4 as read by k_post_ring
       rows.add(sc, (int)sizeof(T));
       rows.add(r, (int)sizeof(T));
       rows.add(b, (int)sizeof(BT));
       rows.add(L.agg, (int)sizeof(int32_t));
       if (NDOT > 1) rows.add(q, (int)sizeof(double));
-      RingGeom g = ring_plan(L.AP, (int)sizeof(V), ring_stages(H), rows, NDOT > 0);
-      if (g.D) {
-        AMG_TRY(ring_prepare((const void*)k_post_ring<V, T, BT, XT, NDOT, false>, g,
-                             L.AP.nslices, H->num_sms));
-        k_post_ring<V, T, BT, XT, NDOT, false><<<g.grid, g.threads(), g.smem, s>>>(
-            v, xc, x, H->red, H->sc, g, rows, H->wait_fail, nullptr);
+      RingGeom g = ring_plan(L.AP, (int)sizeof(V), ring_stages(H), rows, NDOT > 0, H->batched);
+      if (g.D && H->batched) {
+        const auto fn = k_post_ring<V, T, BT, XT, NDOT, false, true>;
+        AMG_TRY(ring_prepare((const void*)fn, g, L.rch_n, H->num_sms));
+        fn<<<g.grid, g.threads(), g.smem, s>>>(v, xc, x, H->red, H->sc, g, rows,
+                                               RingChunks{L.rch_off, L.rch_n}, H->wait_fail,
+                                               nullptr, H->batch.rpart);
         AMG_LAUNCH_CHECK();
         return AMG_OK;
       }
+      if (g.D) {
+        const auto fn = k_post_ring<V, T, BT, XT, NDOT, false, false>;
+        AMG_TRY(ring_prepare((const void*)fn, g, ring_tiles(g, L.AP), H->num_sms));
+        fn<<<g.grid, g.threads(), g.smem, s>>>(v, xc, x, H->red, H->sc, g, rows, RingChunks(),
+                                               H->wait_fail, nullptr, nullptr);
+        AMG_LAUNCH_CHECK();
+        return AMG_OK;
+      }
+      if (H->batched && NDOT > 0) return AMG_ERR_UNSUPPORTED;  // Batch::ring said it fits
     }
   }
   if constexpr (NDOT > 0) {
@@ -921,7 +953,7 @@ static int launch_sweep(const amg_handle* H, const Level& L, const BT* b, const 
     SellView<V> v = view<V>(L.A, ah);
     v.act = act;
     if constexpr (sizeof(V) >= 4) {
-      if (!act && H->opt.stream_ring) {
+      if (!act && !H->batched && H->opt.stream_ring) {
         RingRows rows;
         rows.add(sc, (int)sizeof(T));
         rows.add(r, (int)sizeof(T));
@@ -935,10 +967,10 @@ static int launch_sweep(const amg_handle* H, const Level& L, const BT* b, const 
           if (ND > 1) rows.add(sd->q, (int)sizeof(double));
           RingGeom g = ring_plan(L.A, (int)sizeof(V), ring_stages(H), rows, ND > 0);
           if (!g.D) return 1;
-          AMG_TRY(ring_prepare((const void*)k_sweep_ring<PRE, V, T, BT, YT, ND>, g, L.A.nslices,
-                               H->num_sms));
-          k_sweep_ring<PRE, V, T, BT, YT, ND><<<g.grid, g.threads(), g.smem, s>>>(
-              v, r, r_out, x, first, g, rows, H->wait_fail, H->red, H->sc);
+          const auto fn = k_sweep_ring<PRE, V, T, BT, YT, ND>;
+          AMG_TRY(ring_prepare((const void*)fn, g, ring_tiles(g, L.A), H->num_sms));
+          fn<<<g.grid, g.threads(), g.smem, s>>>(v, r, r_out, x, first, g, rows, RingChunks(),
+                                                 H->wait_fail, H->red, H->sc);
           AMG_LAUNCH_CHECK();
           if (ND > 0) sd->fused = true;
           return AMG_OK;
@@ -1094,8 +1126,9 @@ struct Prof {
 
 // Algorithmic bytes of each V-cycle kernel on one level: operator entries
 // (value + column index) once, every vector once.  mb = bytes of an operator
-// entry (value + 4-byte column, or + 2-byte offset and a share of the 4-byte
-// base per C slots when the columns are compressed), vb = bytes of a V-cycle
+// entry (value + its share of the packed index blocks, or + 4-byte column, or +
+// 2-byte offset and a share of the 4-byte base per C slots when the columns are
+// compressed), vb = bytes of a V-cycle
 // vector element, ib/ob = bytes of the level's input b / output z elements
 // (FP64 on level 0).
 static double bytes_pre(const Level& L, double mb, double vb, double ib) {
@@ -1142,7 +1175,12 @@ static int vcycle_levels(const amg_handle* H, const double* r0, double* z0, int 
   // batched PCG (slice partials requested): skip the systems that stopped
   const int* act = slice_part ? H->batch.active : nullptr;
   auto entry = [&](const Level& L, const Sell& M) {
-    const double idx = M.d16 ? 2.0 + 4.0 / M.C : 4.0;
+    // packed indices where the kernels stream them (FP64 values, and FP32 ones
+    // on the ring), else a plain or compressed column a slot
+    const bool packed = M.rec && (L.vstore == VAL_F64 || (L.vstore == VAL_F32 && !M.row0));
+    const double idx = packed  ? (double)M.ix_bytes / (double)std::max<int64_t>(M.nnz_pad, 1)
+                       : M.d16 ? 2.0 + 4.0 / M.C
+                               : 4.0;
     return idx + (L.vstore == VAL_F64 ? 8.0 : L.vstore == VAL_F32 ? 4.0 : 2.0);
   };
   auto mbytes = [&](const Level& L) { return entry(L, L.A); };
