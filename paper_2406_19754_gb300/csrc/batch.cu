@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
     }
     if (ring.ended) return;
     if (ring.slice) {
-      const double acc = ring_row_sum<double>(ring, [&](int j) { return __ldg(p + j); });
+      const double acc = ring_row_sum<double>(ring, p);
       if (ring.has) {
         q[ring.i] = acc;
         d += ring.row<double>(0) * acc;

@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
       break;
     }
     if (ring.slice) {
-      const double acc = ring_row_sum<double>(ring, [&](int j) { return __ldg(p + j); });
+      const double acc = ring_row_sum<double>(ring, p);
       if (ring.has) {
         q[ring.i] = acc;
         d[0] += ring.template row<double>(0) * acc;

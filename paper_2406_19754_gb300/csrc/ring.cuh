@@ -13,8 +13,10 @@
 //
 // The 32 entries per slice of the kernel's per-row vectors (b, s, r, the
 // aggregate map, ...) come with the tile, so every DRAM stream of the loop is
-// a bulk copy started D - 1 tiles ahead; the ragged last tile reads those
-// from global memory instead (its copy would run past the vectors' end).
+// a bulk copy started D - 1 tiles ahead.  Where no bulk copy can be (the ragged
+// last tile, whose copy would run past the vectors' end; vectors that start off
+// a 16-byte boundary) the producer warp loads and stores the entries itself, so
+// the consumers find them in the stage always.
 //
 // What bounds it: with a ring per warp (every warp refilling its own two
 // stages slice by slice) the FP32 level-0 pre-smoother issued 241 warp
@@ -96,7 +98,7 @@ struct RingGeom {
   uint32_t soff = 0;    // offset of the slice records
   uint32_t hoff = 0;    // offset of the tile's description (CHUNKED)
   uint32_t roff[RING_MAX_ROWS] = {};  // offsets of the per-row vectors
-  uint32_t direct = 0;  // bit k: row vector k starts off a 16-byte boundary, read directly
+  uint32_t direct = 0;  // bit k: row vector k starts off a 16-byte boundary, no bulk copies
   int grid = 0;         // CTAs (ring_prepare)
   size_t smem = 0;      // dynamic shared memory per CTA
   int threads() const { return (tile + 1) * 32; }
@@ -112,7 +114,7 @@ struct RingChunks {
 // `rows` rows; the staged per-row vectors start at row e0.
 struct RingTile {
   int64_t s0, r0, e0, chunk;
-  int32_t ns, rows, staged, last;  // last: of its chunk
+  int32_t ns, rows, last, pad;  // last: of its chunk
 };
 
 // ------------------------------------------------------------------ PTX wrappers
@@ -205,21 +207,21 @@ struct TileRing {
   const RingGeom& g;
   const RingRows& rows;
   const RingChunks& ch;
-  unsigned char* base;   // first stage
-  uint32_t bars;         // shared address: full[D], then empty[D]
-  int64_t ntiles;        // (not CHUNKED)
+  unsigned char* base;  // first stage
+  uint32_t bars;        // shared address: full[D], then empty[D]
   int warp, lane;
-  // consumer state
+  // consumer state; rows and slices are counted in 32 bits (columns are int32)
   int stage = 0;
   uint32_t phase = 0;
-  int64_t t;             // current tile (not CHUNKED)
+  uint32_t t, ntiles;    // current tile, tiles (not CHUNKED)
   bool ended = false;    // CHUNKED: no more tiles
   bool slice = false;    // this warp has a slice of the tile
   bool has = false;      // this lane has a row: row i
-  bool staged_rows = false, last = false;
-  int64_t i = 0, e0 = 0, chunk = 0;
+  bool last = false;     // CHUNKED: last tile of its chunk
+  uint32_t i = 0, j = 0;  // j: the row's place among the staged entries
+  int64_t chunk = 0;
   const unsigned char* st = nullptr;  // current stage
-  const unsigned char* vals = nullptr;
+  const V* vals = nullptr;            // this lane's values
   const int32_t* ixb = nullptr;
   int wm = 0;  // (ELL width << 2) | IX_* code
 
@@ -232,8 +234,9 @@ struct TileRing {
     bars = smem_addr(base) + (uint32_t)g.D * g.stage;
     warp = threadIdx.x >> 5;
     lane = threadIdx.x & 31;
-    ntiles = (A.nslices + g.tile - 1) / g.tile;
+    ntiles = (uint32_t)((A.nslices + g.tile - 1) / g.tile);
     t = blockIdx.x;
+    j = threadIdx.x;
     if (threadIdx.x == 0) {
       for (int d = 0; d < g.D; ++d) {
         mbar_init(full(d), 1);
@@ -249,12 +252,6 @@ struct TileRing {
     return bars + 8u * (uint32_t)(RING_MAX_STAGES + d);
   }
   __device__ __forceinline__ bool producer() const { return warp == g.tile; }
-  __device__ __forceinline__ bool is_full(int64_t tt) const {
-    return (tt + 1) * g.tile * 32 <= A.n;
-  }
-  __device__ __forceinline__ bool staged(bool f, int k) const {
-    return f && k < rows.n && !((g.direct >> k) & 1u);
-  }
   __device__ __forceinline__ SliceRec load_rec(int64_t s) const {
     const longlong2 r = __ldg((const longlong2*)(A.rec + (s < A.nslices ? s : A.nslices)));
     return SliceRec{r.x, r.y};
@@ -265,11 +262,16 @@ struct TileRing {
     int d = 0, issued = 0;
     uint32_t ph = 1;  // the first pass over the stages does not wait
   };
-  // Waits until the next stage's consumers have left it; false if that gave up.
+  // Waits until the next stage's consumers have left it; false if that gave up
+  // (the whole producer warp, same result in every lane).
   __device__ __forceinline__ bool claim(const Fill& f, int* fail, int* status) const {
-    if (f.issued < g.D || mbar_wait_bounded(empty(f.d), f.ph)) return true;
-    atomicExch(fail, 1);
-    if (status) atomicCAS(status, 0, AMG_ERR_DEVICE_CHECK);
+    if (f.issued < g.D ||
+        __all_sync(0xffffffffu, mbar_wait_bounded(empty(f.d), f.ph)))
+      return true;
+    if (lane == 0) {
+      atomicExch(fail, 1);
+      if (status) atomicCAS(status, 0, AMG_ERR_DEVICE_CHECK);
+    }
     return false;
   }
   __device__ __forceinline__ void advance(Fill& f) const {
@@ -279,18 +281,36 @@ struct TileRing {
       f.ph ^= 1u;
     }
   }
-  // Starts the copies of slices s0 .. s0 + ns - 1 (records b .. e) and of rows
-  // r0 .. r0 + nr - 1 of the per-row vectors (if fr).
+  // Fills the stage (whole producer warp): slices s0 .. s0 + ns - 1 (records b
+  // .. e) and nr rows from r0 of the per-row vectors, `bulk` if they may be
+  // copied in bulk (they exist, and r0 and nr suit 16-byte boundaries).
   __device__ __forceinline__ void fill(const Fill& f, int64_t s0, uint32_t ns, const SliceRec& b,
-                                       const SliceRec& e, bool fr, int64_t r0, uint32_t nr,
+                                       const SliceRec& e, bool bulk, int64_t r0, uint32_t nr,
                                        uint64_t pol) const {
+    const uint32_t hand = bulk ? g.direct : ~0u;
+    if (hand) {
+      unsigned char* sp = base + (size_t)f.d * g.stage;
+      for (int k = 0; k < rows.n; ++k) {
+        if (!((hand >> k) & 1u)) continue;
+        if (rows.esz[k] == 8) {
+          const long long* p = (const long long*)rows.p[k] + r0;
+          for (uint32_t u = lane; u < nr; u += 32) ((long long*)(sp + g.roff[k]))[u] = p[u];
+        } else {
+          const int* p = (const int*)rows.p[k] + r0;
+          for (uint32_t u = lane; u < nr; u += 32) ((int*)(sp + g.roff[k]))[u] = p[u];
+        }
+      }
+      __syncwarp();  // before lane 0's arrival publishes the stage
+    }
+    if (lane != 0) return;
     const int64_t ib = b.ix & ~(int64_t)3;
     const uint32_t vb = (uint32_t)(e.slot - b.slot) * (uint32_t)sizeof(V);
     const uint32_t cb = (uint32_t)((e.ix & ~(int64_t)3) - ib);
+    auto staged = [&](int k) { return k < rows.n && !((hand >> k) & 1u); };
     uint32_t rb = 0;
 #pragma unroll
     for (int k = 0; k < RING_MAX_ROWS; ++k)
-      if (staged(fr, k)) rb += nr * (uint32_t)rows.esz[k];
+      if (staged(k)) rb += nr * (uint32_t)rows.esz[k];
     const uint32_t dst = smem_addr(base) + (uint32_t)f.d * g.stage, fb = full(f.d);
     mbar_arrive_expect_tx(fb, vb + cb + 16u * (ns + 1) + rb);
     bulk_copy_g2s(dst + g.soff, A.rec + s0, 16u * (ns + 1), fb, pol);
@@ -300,7 +320,7 @@ struct TileRing {
     }
 #pragma unroll
     for (int k = 0; k < RING_MAX_ROWS; ++k)
-      if (staged(fr, k))
+      if (staged(k))
         bulk_copy_g2s(dst + g.roff[k], (const unsigned char*)rows.p[k] + r0 * rows.esz[k],
                       nr * (uint32_t)rows.esz[k], fb, pol);
   }
@@ -311,10 +331,9 @@ struct TileRing {
       if (!mbar_wait_bounded(full(k % g.D), (uint32_t)(k / g.D) & 1u)) break;
   }
 
-  // The producer warp: lane 0 copies every tile of this CTA, a stage as soon
-  // as its consumers have left it.
+  // The producer warp: copies every tile of this CTA, a stage as soon as its
+  // consumers have left it.
   __device__ __forceinline__ void produce(int* fail, int* status) {
-    if (lane != 0) return;
     const uint64_t pol = l2_evict_first();
     Fill f;
     if constexpr (CHUNKED) {
@@ -339,18 +358,22 @@ struct TileRing {
           h.chunk = c;
           h.ns = (int32_t)(s1 - s0);
           h.rows = (int32_t)(r1 - r0);
-          h.staged = e1 <= A.n;
           h.last = s1 == c1;
-          *(RingTile*)(base + (size_t)f.d * g.stage + g.hoff) = h;
-          fill(f, s0, (uint32_t)(s1 - s0), b, e, h.staged != 0, h.e0, (uint32_t)(e1 - h.e0), pol);
+          h.pad = 0;
+          if (lane == 0) *(RingTile*)(base + (size_t)f.d * g.stage + g.hoff) = h;
+          const bool bulk = e1 <= A.n;
+          fill(f, s0, (uint32_t)(s1 - s0), b, e, bulk, h.e0,
+               (uint32_t)((bulk ? e1 : A.n) - h.e0), pol);
           advance(f);
           b = e;
           r0 = r1;
         }
       }
       if (ok && claim(f, fail, status)) {  // the end: an empty stage
-        ((RingTile*)(base + (size_t)f.d * g.stage + g.hoff))->ns = -1;
-        mbar_arrive(full(f.d));
+        if (lane == 0) {
+          ((RingTile*)(base + (size_t)f.d * g.stage + g.hoff))->ns = -1;
+          mbar_arrive(full(f.d));
+        }
         advance(f);
       }
     } else {
@@ -366,9 +389,10 @@ struct TileRing {
           ne = load_rec(nx * g.tile + g.tile);
         }
         if (!claim(f, fail, status)) break;
-        const int64_t s0 = tt * g.tile;
+        const int64_t s0 = tt * g.tile, nr = A.n - s0 * 32;
         const uint32_t ns = (uint32_t)(A.nslices - s0 < g.tile ? A.nslices - s0 : g.tile);
-        fill(f, s0, ns, b, e, is_full(tt), s0 * 32, 32u * (uint32_t)g.tile, pol);
+        const bool bulk = nr >= 32 * g.tile;
+        fill(f, s0, ns, b, e, bulk, s0 * 32, bulk ? 32u * (uint32_t)g.tile : (uint32_t)nr, pol);
         advance(f);
         tt = nx;
         if (tt >= ntiles) break;
@@ -384,42 +408,39 @@ struct TileRing {
   // Waits for the next tile; false if the wait gave up.
   __device__ __forceinline__ bool wait() {
     if (!__all_sync(0xffffffffu, mbar_wait_bounded(full(stage), phase))) return false;
-    st = base + (size_t)stage * g.stage;
+    st = base + (uint32_t)stage * g.stage;
     if constexpr (CHUNKED) {
       const RingTile& h = *(const RingTile*)(st + g.hoff);
       ended = h.ns < 0;
       if (ended) return true;
       slice = warp < h.ns;
-      i = h.r0 + warp * 32 + lane;
-      has = slice && warp * 32 + lane < h.rows;
-      e0 = h.e0;
-      staged_rows = h.staged != 0;
+      i = (uint32_t)h.r0 + threadIdx.x;
+      has = slice && (int)threadIdx.x < h.rows;
+      j = i - (uint32_t)h.e0;
       last = h.last != 0;
       chunk = h.chunk;
     } else {
-      const int64_t sl = t * g.tile + warp;
-      slice = sl < A.nslices;
-      i = sl * 32 + lane;
-      has = i < A.n;
-      e0 = t * g.tile * 32;
-      staged_rows = is_full(t);
+      const uint32_t s0 = t * (uint32_t)g.tile;
+      slice = s0 + warp < (uint32_t)A.nslices;
+      i = s0 * 32 + threadIdx.x;
+      has = i < (uint32_t)A.n;
     }
     if (slice) {
-      const SliceRec* r = (const SliceRec*)(st + g.soff);
-      const SliceRec r0 = r[0], rw = r[warp], rn = r[warp + 1];
-      vals = st + (size_t)(rw.slot - r0.slot) * sizeof(V);
-      ixb = (const int32_t*)(st + g.coff + ((rw.ix & ~(int64_t)3) - (r0.ix & ~(int64_t)3)));
-      wm = ((int)(rn.slot - rw.slot) >> 5 << 2) | (int)(rw.ix & 3);
+      // low halves: differences within a tile
+      const int4* r = (const int4*)(st + g.soff);
+      const int4 r0 = r[0], rw = r[warp], rn = r[warp + 1];
+      vals = (const V*)(st + (uint32_t)(rw.x - r0.x) * (uint32_t)sizeof(V)) + lane;
+      ixb = (const int32_t*)(st + (g.coff + (uint32_t)((rw.z & ~3) - (r0.z & ~3))));
+      wm = (rn.x - rw.x) >> 5 << 2 | (rw.z & 3);
     }
     return true;
   }
 
-  __device__ __forceinline__ V val(int k) const { return ((const V*)vals)[k * 32 + lane]; }
-  // entry i (this lane's row) of per-row vector k (element type X = its type)
+  __device__ __forceinline__ V val(int k) const { return vals[k * 32]; }
+  // this lane's entry (row i) of per-row vector k, of type X
   template <typename X>
   __device__ __forceinline__ X row(int k) const {
-    if (staged(staged_rows, k)) return ((const X*)(st + g.roff[k]))[(int)(i - e0)];
-    return __ldg((const X*)rows.p[k] + i);
+    return ((const X*)(st + g.roff[k]))[j];
   }
 
   // every lane is done with the stage
@@ -434,38 +455,76 @@ struct TileRing {
   }
 };
 
-// Columns of this lane's row in the current stage, by the slice's coding.
+// Columns k0 .. k0 + N - 1 of this lane's row in the current stage, by the
+// slice's coding, as places from `v` (k0 is a multiple of 4; index blocks start
+// at 16 bytes and hold whole groups of four offsets or bases).
+template <int N>
+__device__ __forceinline__ void ix_heads(const int32_t* c, int k0, int32_t (&o)[N]) {
+  const int4* q = (const int4*)(c + k0);
+#pragma unroll
+  for (int u = 0; u < N; u += 4) {
+    const int4 h = q[u / 4];
+    o[u] = h.x;
+    if (u + 1 < N) o[u + 1 < N ? u + 1 : 0] = h.y;
+    if (u + 2 < N) o[u + 2 < N ? u + 2 : 0] = h.z;
+    if (u + 3 < N) o[u + 3 < N ? u + 3 : 0] = h.w;
+  }
+}
+template <typename X>
 struct IxPlain {
+  const X* v;
   const int32_t* c;
-  __device__ __forceinline__ int32_t operator()(int k) const { return c[k * 32]; }
+  template <int N>
+  __device__ __forceinline__ void load(int k0, int32_t (&o)[N]) const {
+#pragma unroll
+    for (int u = 0; u < N; ++u) o[u] = c[(k0 + u) * 32];
+  }
 };
+template <typename X>
 struct IxDelta {
+  const X* v;
   const int32_t* base;
   const uint16_t* d;
-  __device__ __forceinline__ int32_t operator()(int k) const { return base[k] + (int)d[k * 32]; }
+  template <int N>
+  __device__ __forceinline__ void load(int k0, int32_t (&o)[N]) const {
+    ix_heads<N>(base, k0, o);
+#pragma unroll
+    for (int u = 0; u < N; ++u) o[u] += (int)d[(k0 + u) * 32];
+  }
 };
+template <typename X>
 struct IxOffset {
+  const X* v;  // (at this lane's row)
   const int32_t* off;
-  int32_t i;  // this lane's row
-  __device__ __forceinline__ int32_t operator()(int k) const { return i + off[k]; }
+  template <int N>
+  __device__ __forceinline__ void load(int k0, int32_t (&o)[N]) const {
+    ix_heads<N>(off, k0, o);
+  }
 };
+template <typename X>
 struct IxClamp {
+  const X* v;
   const int32_t* off;
   int32_t i, last;  // the clamp only ever moves padding
-  __device__ __forceinline__ int32_t operator()(int k) const {
-    return min(max(i + off[k], 0), last);
+  template <int N>
+  __device__ __forceinline__ void load(int k0, int32_t (&o)[N]) const {
+    ix_heads<N>(off, k0, o);
+#pragma unroll
+    for (int u = 0; u < N; ++u) o[u] = min(max(i + o[u], 0), last);
   }
 };
 
-// acc + sum of a_k g(col_k) (NEG: acc - sum, by FMAs with the negated
+// acc + sum of a_k v[col_k] (NEG: acc - sum, by FMAs with the negated
 // values) for k = k0 .. k0 + N - 1, k ascending: the N gathers issue
 // together, then the FMAs follow in order.  Exactly N FMAs: on GB300's FP64
 // pipe a predicated-off FMA would still cost its cycles.
-template <int N, bool NEG, typename T, typename R, typename I, typename G>
-__device__ __forceinline__ T ring_chunk(const R& ring, const I& ix, int k0, T acc, G g) {
+template <int N, bool NEG, typename T, typename R, typename I>
+__device__ __forceinline__ T ring_chunk(const R& ring, const I& ix, int k0, T acc) {
+  int32_t o[N];
+  ix.load(k0, o);
   T x[N];
 #pragma unroll
-  for (int u = 0; u < N; ++u) x[u] = g(ix(k0 + u));
+  for (int u = 0; u < N; ++u) x[u] = to_f(__ldg(ix.v + o[u]), T(0));
 #pragma unroll
   for (int u = 0; u < N; ++u) {
     const T a = to_f(ring.val(k0 + u), T(0));
@@ -476,41 +535,41 @@ __device__ __forceinline__ T ring_chunk(const R& ring, const I& ix, int k0, T ac
 
 // Chunks of 8 and one remainder chunk of the exact length (w is
 // warp-uniform).
-template <bool NEG, typename T, typename R, typename I, typename G>
-__device__ __forceinline__ T ring_chunks(const R& ring, const I& ix, int w, T acc, G g) {
+template <bool NEG, typename T, typename R, typename I>
+__device__ __forceinline__ T ring_chunks(const R& ring, const I& ix, int w, T acc) {
   int k0 = 0;
-  for (; k0 + 8 <= w; k0 += 8) acc = ring_chunk<8, NEG>(ring, ix, k0, acc, g);
+  for (; k0 + 8 <= w; k0 += 8) acc = ring_chunk<8, NEG>(ring, ix, k0, acc);
   switch (w - k0) {
-    case 1: acc = ring_chunk<1, NEG>(ring, ix, k0, acc, g); break;
-    case 2: acc = ring_chunk<2, NEG>(ring, ix, k0, acc, g); break;
-    case 3: acc = ring_chunk<3, NEG>(ring, ix, k0, acc, g); break;
-    case 4: acc = ring_chunk<4, NEG>(ring, ix, k0, acc, g); break;
-    case 5: acc = ring_chunk<5, NEG>(ring, ix, k0, acc, g); break;
-    case 6: acc = ring_chunk<6, NEG>(ring, ix, k0, acc, g); break;
-    case 7: acc = ring_chunk<7, NEG>(ring, ix, k0, acc, g); break;
+    case 1: acc = ring_chunk<1, NEG>(ring, ix, k0, acc); break;
+    case 2: acc = ring_chunk<2, NEG>(ring, ix, k0, acc); break;
+    case 3: acc = ring_chunk<3, NEG>(ring, ix, k0, acc); break;
+    case 4: acc = ring_chunk<4, NEG>(ring, ix, k0, acc); break;
+    case 5: acc = ring_chunk<5, NEG>(ring, ix, k0, acc); break;
+    case 6: acc = ring_chunk<6, NEG>(ring, ix, k0, acc); break;
+    case 7: acc = ring_chunk<7, NEG>(ring, ix, k0, acc); break;
     default: break;
   }
   return acc;
 }
 
-// init + sum_k a_k g(col_k) (NEG: init - sum) over the entries of this
+// init + sum_k a_k v[col_k] (NEG: init - sum) over the entries of this
 // lane's row i in the current stage, k ascending (the per-lane kernels'
 // order).
-template <typename T, bool NEG = false, typename R, typename G>
-__device__ __forceinline__ T ring_row_sum(const R& ring, G g, T init = T(0)) {
-  const int64_t i = ring.i;
+template <typename T, bool NEG = false, typename R, typename X>
+__device__ __forceinline__ T ring_row_sum(const R& ring, const X* v, T init = T(0)) {
   const int w = ring.wm >> 2;
   const int32_t* c = ring.ixb;
   switch (ring.wm & 3) {
     case IX_OFFSET:
-      return ring_chunks<NEG>(ring, IxOffset{c, (int32_t)i}, w, init, g);
+      return ring_chunks<NEG>(ring, IxOffset<X>{v + ring.i, c}, w, init);
     case IX_CLAMP:
-      return ring_chunks<NEG>(ring, IxClamp{c, (int32_t)i, ring.A.ncols - 1}, w, init, g);
+      return ring_chunks<NEG>(ring, IxClamp<X>{v, c, (int32_t)ring.i, ring.A.ncols - 1}, w,
+                              init);
     case IX_DELTA:
       return ring_chunks<NEG>(
-          ring, IxDelta{c, (const uint16_t*)(c + ((w + 3) & ~3)) + ring.lane}, w, init, g);
+          ring, IxDelta<X>{v, c, (const uint16_t*)(c + ((w + 3) & ~3)) + ring.lane}, w, init);
     default:
-      return ring_chunks<NEG>(ring, IxPlain{c + ring.lane}, w, init, g);
+      return ring_chunks<NEG>(ring, IxPlain<X>{v, c + ring.lane}, w, init);
   }
 }
 

@@ -180,8 +180,7 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
     if (ring.slice) {
       const T bi = ring.has ? to_f(ring.template row<BT>(0), T(0)) : T(0);
       // pre_slice's arithmetic: from b_i down by negated FMAs
-      const T acc = ring_row_sum<T, true>(
-          ring, [&](int j) { return to_f(__ldg(b + j), T(0)); }, bi);
+      const T acc = ring_row_sum<T, true>(ring, b, bi);
       if (ring.has) r[ring.i] = acc;
     }
     ring.release();
@@ -221,7 +220,7 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
       const T xci = has ? __ldg(xc + ring.template row<int32_t>(3)) : T(0);
       const T ri = has ? ring.template row<T>(1) : T(0);
       if constexpr (MS) {
-        const T acc = ring_row_sum<T>(ring, [&](int J) { return __ldg(xc + J); });
+        const T acc = ring_row_sum<T>(ring, xc);
         if (has) {
           const T si = ring.template row<T>(0);
           const T yi = ring.template row<T>(2) + xci;
@@ -233,7 +232,7 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
         // post_slice's arithmetic (one sweep): from b_i + r_i down, then one FMA
         const BT bi = has ? ring.template row<BT>(2) : BT(0);
         const T init = has ? to_f(bi, T(0)) + ri : T(0);
-        const T acc = ring_row_sum<T, true>(ring, [&](int J) { return __ldg(xc + J); }, init);
+        const T acc = ring_row_sum<T, true>(ring, xc, init);
         if (has) {
           const XT zi = to_f(fma(ring.template row<T>(0), acc, xci), XT(0));
           x[i] = zi;
@@ -285,7 +284,7 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
       break;
     }
     if (ring.slice) {
-      const T acc = ring_row_sum<T>(ring, [&](int j) { return __ldg(r + j); });
+      const T acc = ring_row_sum<T>(ring, r);
       if (ring.has) {
         const int64_t i = ring.i;
         const T ri = ring.template row<T>(1);
