@@ -43,7 +43,7 @@ constexpr int CT_WARPS = CT_THREADS / 32;
 constexpr int CT_MAX_LEVELS = 12;
 constexpr int CT_MAX_ROWS = 65534;        // 0xFFFF marks an empty member slot
 constexpr int CT_PCG_ROWS = CT_THREADS;   // PCG coarsest solve: one row a thread
-constexpr size_t CT_SMEM = 226 * 1024;
+constexpr size_t CT_SMEM = 226 * 1024;    // of 227 KB: static arrays take the rest
 constexpr uint16_t CT_NONE = 0xFFFF;
 
 // One CTA's image of a level: offsets in bytes, the same for every CTA.
@@ -277,16 +277,29 @@ __device__ void ct_cholesky(const CtParams& P, unsigned char* sm, int rank, bool
   }
 }
 
-// Sums over the block's rows (one per thread) by coarse_pcg_cta's tree.
-template <int NV>
-__device__ __forceinline__ void ct_sum(double (&t)[NV], double* tot) {
-  block_sum<NV>(t);
-  if (threadIdx.x == 0)
+// Sums over the block's n rows (one per thread) by coarse_pcg_cta's tree: the
+// lanes of each warp, then the warps; f turns the sums into what every thread
+// reads back from `out`.  Warps without rows would only add zeros and leave
+// their part out, and one thread divides: sixteen warps' shuffled additions
+// and divisions took the SM's FP64 pipe (16 clocks a warp instruction) longer
+// than the rest of an iteration on 33 rows.
+template <int NV, typename F>
+__device__ __forceinline__ void ct_sum(double (&t)[NV], int n, double (*part)[CT_WARPS],
+                                       double* out, F f) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (32 * warp < n) {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) tot[v] = t[v];
+    for (int v = 0; v < NV; ++v) {
+      t[v] = warp_sum(t[v]);
+      if (lane == 0) part[v][warp] = t[v];
+    }
+  }
   __syncthreads();
+  if (warp == 0) {
 #pragma unroll
-  for (int v = 0; v < NV; ++v) t[v] = tot[v];
+    for (int v = 0; v < NV; ++v) t[v] = warp_sum(32 * lane < n ? part[v][lane] : 0.0);
+    if (lane == 0) f(t, out);
+  }
   __syncthreads();
 }
 
@@ -294,7 +307,8 @@ __device__ __forceinline__ void ct_sum(double (&t)[NV], double* tot) {
 // one row per thread (coarse_pcg_cta's arithmetic; rows <= CT_PCG_ROWS).
 template <typename T>
 __device__ void ct_pcg(const CtParams& P, unsigned char* sm) {
-  __shared__ double tot[2];
+  // two sets: a set is rewritten only after the other's sums were read
+  __shared__ double part[2][2][CT_WARPS], out[2][3];
   const uint32_t smb = smem_addr(sm);
   const int n = P.nco, i = threadIdx.x;
   const bool has = i < n;
@@ -306,14 +320,14 @@ __device__ void ct_pcg(const CtParams& P, unsigned char* sm) {
   const CtVec<T> bv{smb + P.o_cb, P.shift_co};
   double x = 0.0, r = has ? (double)bv[i] : 0.0, z = 0.0;
   double t[1] = {has ? r * r : 0.0};
-  ct_sum<1>(t, tot);
-  const double bnorm = sqrt(t[0]);
+  ct_sum<1>(t, n, part[0], out[0], [](const double* v, double* o) { o[0] = sqrt(v[0]); });
+  const double bnorm = out[0][0];
   if (bnorm > 0.0) {
     z = si * r;
     if (has) p[i] = z;
     t[0] = has ? r * z : 0.0;
-    ct_sum<1>(t, tot);
-    double rz = t[0];
+    ct_sum<1>(t, n, part[1], out[1], [](const double* v, double* o) { o[0] = v[0]; });
+    double rz = out[1][0];
     for (int k = 0; k < P.pcg_maxit; ++k) {
       double q = 0.0;
       if (has) {
@@ -324,10 +338,12 @@ __device__ void ct_pcg(const CtParams& P, unsigned char* sm) {
         for (int e = 0; e < w; ++e) q = fma(a[e * 32], p[c[e * 32]], q);
       }
       t[0] = has ? p[i] * q : 0.0;
-      ct_sum<1>(t, tot);
-      const double pq = t[0];
-      if (!(pq > 0.0)) break;
-      const double alpha = rz / pq;
+      ct_sum<1>(t, n, part[0], out[0], [rz](const double* v, double* o) {
+        o[0] = v[0];
+        o[1] = rz / v[0];
+      });
+      if (!(out[0][0] > 0.0)) break;
+      const double alpha = out[0][1];
       double d[2] = {0.0, 0.0};
       if (has) {
         x = x + alpha * p[i];
@@ -336,12 +352,17 @@ __device__ void ct_pcg(const CtParams& P, unsigned char* sm) {
         d[0] += r * r;
         d[1] += r * z;
       }
-      ct_sum<2>(d, tot);
-      if (sqrt(d[0]) <= P.pcg_tol * bnorm) break;
-      const double beta = d[1] / rz;
+      ct_sum<2>(d, n, part[1], out[1],
+                [rz, tol = P.pcg_tol, bnorm](const double* v, double* o) {
+                  o[0] = v[1];
+                  o[1] = v[1] / rz;
+                  o[2] = sqrt(v[0]) <= tol * bnorm ? 1.0 : 0.0;
+                });
+      if (out[1][2] != 0.0) break;
+      rz = out[1][0];
+      const double beta = out[1][1];
       if (has) p[i] = z + beta * p[i];
       __syncthreads();
-      rz = d[1];
     }
   }
   if (has) st_cluster(CtVec<T>{smb + P.o_cx, P.shift_co}.addr(i), bnorm > 0.0 ? (T)x : T(0));
