@@ -408,6 +408,22 @@ __device__ __forceinline__ __nv_bfloat16 ld_stream<__nv_bfloat16>(const __nv_bfl
   return *p;
 }
 
+// Four doubles by one 32-byte access that L2 evicts first (32-byte aligned): a
+// warp's access then covers whole lines, where two 16-byte accesses of a thread
+// each touch half of every sector.
+__device__ __forceinline__ double4_32a ld4_stream(const double* p) {
+  double4_32a v;
+  asm volatile("ld.global.L1::no_allocate.L2::evict_first.v4.f64 {%0, %1, %2, %3}, [%4];"
+               : "=d"(v.x), "=d"(v.y), "=d"(v.z), "=d"(v.w)
+               : "l"(p));
+  return v;
+}
+__device__ __forceinline__ void st4_stream(double* p, const double4_32a& v) {
+  asm volatile("st.global.L1::no_allocate.L2::evict_first.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p),
+               "d"(v.x), "d"(v.y), "d"(v.z), "d"(v.w)
+               : "memory");
+}
+
 __device__ __forceinline__ double to_f(double v, double) { return v; }
 __device__ __forceinline__ float to_f(float v, float) { return v; }
 __device__ __forceinline__ float to_f(double v, float) { return (float)v; }

@@ -161,7 +161,7 @@ struct RrEpi {
 //
 // Bound by DRAM (24 bytes a row, 28 with r32) and by the FP64 pipe: two
 // operations a row, 32 row-operations per SM every 16 clocks.  Each thread
-// takes four rows a step by 16-byte accesses, so enough bytes are in flight,
+// takes four rows a step by 32-byte accesses, so enough bytes are in flight,
 // and r32 is rounded on the integer pipe (cvt_n); scalar rows with the
 // hardware conversion took 107 us for 16.8M rows with r32, 74 us without.
 __global__ void k_cg_update(int64_t n, double* __restrict__ x, double* __restrict__ r,
@@ -177,12 +177,10 @@ __global__ void k_cg_update(int64_t n, double* __restrict__ x, double* __restric
   const int64_t step = (int64_t)gridDim.x * blockDim.x * 4;
   for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < n; i += step) {
     if (i + 4 <= n) {  // the workspace vectors start on 256 bytes
-      const double2 q0 = __ldcs((const double2*)(q + i)), q1 = __ldcs((const double2*)(q + i + 2));
-      const double2 r0 = *(const double2*)(r + i), r1 = *(const double2*)(r + i + 2);
-      double v[4] = {r0.x - alpha * q0.x, r0.y - alpha * q0.y, r1.x - alpha * q1.x,
-                     r1.y - alpha * q1.y};
-      *(double2*)(r + i) = make_double2(v[0], v[1]);
-      *(double2*)(r + i + 2) = make_double2(v[2], v[3]);
+      const double4_32a q4 = ld4_stream(q + i), r4 = *(const double4_32a*)(r + i);
+      double v[4] = {r4.x - alpha * q4.x, r4.y - alpha * q4.y, r4.z - alpha * q4.z,
+                     r4.w - alpha * q4.w};
+      *(double4_32a*)(r + i) = double4_32a{v[0], v[1], v[2], v[3]};
       if (r32) {
         float f[4];
         cvt_n(v, f);
@@ -222,16 +220,25 @@ __global__ void k_p_update_x(int64_t n, double* __restrict__ p, const double* __
                              PcgScalars* sc) {
   const double alpha = sc->alpha, beta = sc->beta;
   double* x = sc->x;
-  const bool pairs = ((uintptr_t)x & 15u) == 0;  // p and z start on 256 bytes
-  const int64_t step = (int64_t)gridDim.x * blockDim.x * 2;
-  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 2; i < n; i += step) {
-    if (pairs && i + 2 <= n) {
-      const double2 pv = *(const double2*)(p + i), zv = __ldcs((const double2*)(z + i));
-      const double2 xv = __ldcs((const double2*)(x + i));
-      __stcs((double2*)(x + i), make_double2(xv.x + alpha * pv.x, xv.y + alpha * pv.y));
-      *(double2*)(p + i) = make_double2(zv.x + beta * pv.x, zv.y + beta * pv.y);
+  // p and z start on 256 bytes, x where the caller put it
+  const bool quads = ((uintptr_t)x & 31u) == 0, pairs = ((uintptr_t)x & 15u) == 0;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x * 4;
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < n; i += step) {
+    if (pairs && i + 4 <= n) {
+      const double4_32a pv = *(const double4_32a*)(p + i), zv = ld4_stream(z + i);
+      if (quads) {
+        const double4_32a xv = ld4_stream(x + i);
+        st4_stream(x + i, double4_32a{xv.x + alpha * pv.x, xv.y + alpha * pv.y,
+                                      xv.z + alpha * pv.z, xv.w + alpha * pv.w});
+      } else {
+        const double2 x0 = __ldcs((const double2*)(x + i)), x1 = __ldcs((const double2*)(x + i + 2));
+        __stcs((double2*)(x + i), make_double2(x0.x + alpha * pv.x, x0.y + alpha * pv.y));
+        __stcs((double2*)(x + i + 2), make_double2(x1.x + alpha * pv.z, x1.y + alpha * pv.w));
+      }
+      *(double4_32a*)(p + i) = double4_32a{zv.x + beta * pv.x, zv.y + beta * pv.y,
+                                           zv.z + beta * pv.z, zv.w + beta * pv.w};
     } else {
-      for (int64_t k = i; k < n && k < i + 2; ++k) {
+      for (int64_t k = i; k < n && k < i + 4; ++k) {
         const double pk = p[k];
         x[k] = x[k] + alpha * pk;
         p[k] = z[k] + beta * pk;
@@ -313,7 +320,7 @@ static int iteration_body(const amg_handle* H, double* x, int dots, bool defer, 
   const int64_t n = H->L[0].n;
   AMG_TRY(vcycle_run(H, H->r, H->z, dots, H->q, s, nullptr, H->r32));
   if (defer)
-    k_p_update_x<<<grid_for((n + 1) / 2, 256, H->num_sms, 8), 256, 0, s>>>(n, H->p, H->z,
+    k_p_update_x<<<grid_for((n + 3) / 4, 256, H->num_sms, 8), 256, 0, s>>>(n, H->p, H->z,
                                                                            H->sc);
   else
     k_p_update<<<grid_for(n, 256, H->num_sms, 8), 256, 0, s>>>(n, H->p, H->z, H->sc);
