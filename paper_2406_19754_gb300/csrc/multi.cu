@@ -480,14 +480,16 @@ __global__ void __launch_bounds__(MROWS_BLOCK, MV_BLOCKS)
       }
       XT zv[KPL];
       cvt_n(zt, zv);
+      double zd[KPL];
+      if constexpr (DOTS) cvt_n(zt, zd);
 #pragma unroll
       for (int q = 0; q < KPL; ++q) {
         const int c = lane + 32 * q;
         if (c < K) {
           Z[i * K + c] = zv[q];
           if (DOTS) {
-            d[0][q] += (double)B[i * K + c] * (double)zv[q];
-            d[1][q] += (double)zv[q] * Q[i * K + c];
+            d[0][q] += (double)B[i * K + c] * zd[q];
+            d[1][q] += zd[q] * Q[i * K + c];
           }
         }
       }
@@ -560,30 +562,34 @@ __device__ __forceinline__ void st_cols(double* __restrict__ p, const double (&o
 }
 
 // acc -= sum_k a_ik X[col_k, c0 ..] for the lane's row (staged slice, or the
-// row's entries from global memory when the slice did not fit the staging);
-// acc += ... with NEG false.
-template <int VW, bool NEG = true, typename V, typename T>
+// row's entries from global memory when the slice did not fit the staging), GRP
+// gathers in flight; acc += ... with NEG false.
+template <int VW, bool NEG = true, int GRP = SL_MAXW, typename V, typename T>
 __device__ __forceinline__ void rows_sub_v(const SellView<V>& A, bool staged, const int32_t* scol,
                                            const T* sval, int C, int w, int r, int64_t i, int K,
                                            int c0, const T* __restrict__ X, T (&acc)[VW]) {
   if (staged) {
-    T g[SL_MAXW][VW];
 #pragma unroll
-    for (int u = 0; u < SL_MAXW; ++u) {
-      if (u < w) {
-        ld_cols(X + (int64_t)scol[u * C + r] * K + c0, g[u]);
-      } else {
+    for (int k0 = 0; k0 < SL_MAXW; k0 += GRP) {
+      if (k0 >= w) break;
+      T g[GRP][VW];
 #pragma unroll
-        for (int k = 0; k < VW; ++k) g[u][k] = T(0);
+      for (int u = 0; u < GRP; ++u) {
+        if (k0 + u < w) {
+          ld_cols(X + (int64_t)scol[(k0 + u) * C + r] * K + c0, g[u]);
+        } else {
+#pragma unroll
+          for (int k = 0; k < VW; ++k) g[u][k] = T(0);
+        }
       }
+#pragma unroll
+      for (int u = 0; u < GRP; ++u)
+        if (k0 + u < w) {
+          const T a = NEG ? -sval[(k0 + u) * C + r] : sval[(k0 + u) * C + r];
+#pragma unroll
+          for (int k = 0; k < VW; ++k) acc[k] = fma(a, g[u][k], acc[k]);
+        }
     }
-#pragma unroll
-    for (int u = 0; u < SL_MAXW; ++u)
-      if (u < w) {
-        const T a = NEG ? -sval[u * C + r] : sval[u * C + r];
-#pragma unroll
-        for (int k = 0; k < VW; ++k) acc[k] = fma(a, g[u][k], acc[k]);
-      }
     return;
   }
   const RowSpan rw = row_span(A, i, C);
@@ -652,7 +658,10 @@ __global__ void __launch_bounds__(MROWS_BLOCK, MV_BLOCKS)
 }
 
 // Z = s (B + R - AP Xc) + Xc[agg] (as k_m_post), vector columns; with DOTS
-// the column sums (B, Z) and (Z, Q) go to epi.
+// the column sums (B, Z) and (Z, Q) go to epi.  Three blocks an SM with DOTS: Q
+// loaded after the gathers and B twice, the level-0 launch took 981 us for 64
+// columns of 128^3; Q before them, B kept, four gathers at a time (for the
+// registers) and Z stored in FP32, 815 us, against 0.49 ms for its bytes.
 template <typename V, typename T, typename BT, typename XT, bool DOTS>
 __global__ void __launch_bounds__(MROWS_BLOCK, DOTS ? MV_BLOCKS_DOTS : MV_BLOCKS)
     k_m_post_v(SellView<V> AP, int C, int K, int sub, const BT* __restrict__ B,
@@ -682,19 +691,19 @@ __global__ void __launch_bounds__(MROWS_BLOCK, DOTS ? MV_BLOCKS_DOTS : MV_BLOCKS
       const bool live = rs < RW && p + rs < rows;
       const int r = live ? p + rs : 0;
       const int64_t i = i0 + r;
-      T acc[VW];
-      {
-        BT bv[VW];
-        T rv[VW];
-        ld_cols(B + i * K + c0, bv);
-        ld_cols(R + i * K + c0, rv);
-        cvt_n(bv, acc);
+      T acc[VW], rv[VW], xv[VW];
+      BT bv[VW];
+      double qv[VW];
+      // (the dot products' operands as well, before the gathers)
+      ld_cols(B + i * K + c0, bv);
+      ld_cols(R + i * K + c0, rv);
+      if constexpr (DOTS) ld_cols(Q + i * K + c0, qv);
+      cvt_n(bv, acc);
 #pragma unroll
-        for (int k = 0; k < VW; ++k) acc[k] = acc[k] + rv[k];
-      }
-      rows_sub_v<VW>(AP, staged, scol, sval, C, w, r, i, K, c0, Xc, acc);
+      for (int k = 0; k < VW; ++k) acc[k] = acc[k] + rv[k];
+      rows_sub_v<VW, true, DOTS ? 4 : SL_MAXW>(AP, staged, scol, sval, C, w, r, i, K, c0, Xc,
+                                               acc);
       const T si = s[i];
-      T xv[VW];
       ld_cols(Xc + (int64_t)agg[i] * K + c0, xv);
 #pragma unroll
       for (int k = 0; k < VW; ++k) xv[k] = fma(si, acc[k], xv[k]);
@@ -703,14 +712,12 @@ __global__ void __launch_bounds__(MROWS_BLOCK, DOTS ? MV_BLOCKS_DOTS : MV_BLOCKS
       if (live) {
         st_cols(Z + i * K + c0, zv);
         if constexpr (DOTS) {
-          BT bv[VW];
-          double qv[VW];
-          ld_cols(B + i * K + c0, bv);
-          ld_cols(Q + i * K + c0, qv);
+          double zd[VW];
+          cvt_n(xv, zd);
 #pragma unroll
           for (int k = 0; k < VW; ++k) {
-            d[0][k] += (double)bv[k] * (double)zv[k];
-            d[1][k] += (double)zv[k] * qv[k];
+            d[0][k] += (double)bv[k] * zd[k];
+            d[1][k] += zd[k] * qv[k];
           }
         }
       }
@@ -1081,9 +1088,11 @@ __global__ void __launch_bounds__(MROWS_BLOCK)
 // The owed x += alpha_c p of the last update, then p = z + beta_c p for columns
 // still iterating.  alpha_c is what the last product set: 0 for columns that
 // took no step, and it is applied here exactly once, whether or not the column
-// has stopped since.
-template <int KPL>
-__global__ void k_m_p_update(int64_t n, int K, double* __restrict__ P, const double* __restrict__ Z,
+// has stopped since.  FIRST: p = z, nothing owed.  An FP32 V-cycle's z is FP32
+// (ZT): kept so, it takes 1.1 GB less an iteration here and in the
+// post-smoother for 64 columns of 128^3, both at their DRAM bound.
+template <int KPL, typename ZT, bool FIRST>
+__global__ void k_m_p_update(int64_t n, int K, double* __restrict__ P, const ZT* __restrict__ Z,
                              double* __restrict__ X, const Scal* sc) {
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1092,20 +1101,153 @@ __global__ void k_m_p_update(int64_t n, int K, double* __restrict__ P, const dou
 #pragma unroll
   for (int q = 0; q < KPL; ++q) {
     const int c = lane + 32 * q;
-    al[q] = c < K ? sc[c].alpha : 0.0;
+    al[q] = !FIRST && c < K ? sc[c].alpha : 0.0;
     owed[q] = al[q] != 0.0;
-    act[q] = c < K && sc[c].active;
-    be[q] = act[q] ? sc[c].beta : 0.0;
+    act[q] = c < K && (FIRST || sc[c].active);
+    be[q] = !FIRST && act[q] ? sc[c].beta : 0.0;
   }
-  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += nw)
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += nw) {
+    ZT zt[KPL];
+    double z[KPL], p[KPL], x[KPL];
+    // every load of the row before the conversions
 #pragma unroll
-    for (int q = 0; q < KPL; ++q)
-      if (owed[q] || act[q]) {
-        const int64_t e = i * K + lane + 32 * q;
-        const double p = P[e];
-        if (owed[q]) X[e] = X[e] + al[q] * p;
-        if (act[q]) P[e] = Z[e] + be[q] * p;
+    for (int q = 0; q < KPL; ++q) {
+      const int64_t e = i * K + lane + 32 * q;
+      zt[q] = act[q] ? Z[e] : ZT(0);
+      p[q] = !FIRST && (owed[q] || act[q]) ? P[e] : 0.0;
+      x[q] = owed[q] ? X[e] : 0.0;
+    }
+    cvt_n(zt, z);
+#pragma unroll
+    for (int q = 0; q < KPL; ++q) {
+      const int64_t e = i * K + lane + 32 * q;
+      if (owed[q]) X[e] = x[q] + al[q] * p[q];
+      if (act[q]) P[e] = FIRST ? z[q] : z[q] + be[q] * p[q];
+    }
+  }
+}
+
+// The same two updates with vector columns: lane (rs, cg) takes columns 2 cg and
+// 2 cg + 1 of one of the RW rows a warp advances by, two such groups of rows at a
+// time, every load before the first conversion.  DRAM bounds both (4.8 and 3.8 GB
+// for 64 columns of 128^3), and one column a lane keeps too little in flight: 943
+// and 627 us for these columns, now 778 and 603 (floors at the copy rate 723 and
+// 562).  For K even and vectors on 16 bytes.
+constexpr int MU_ROWS = 2;
+struct MuLanes {
+  int c0, rs, RW;
+  int64_t i0, step;  // first row, rows of the grid a pass
+  bool on;           // this lane has columns
+  __device__ __forceinline__ MuLanes(int K) {
+    const int lane = threadIdx.x & 31, G = K / 2;
+    RW = 32 / G;
+    rs = lane / G;
+    c0 = lane % G * 2;
+    on = rs < RW;
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    i0 = w * RW + rs;
+    step = (((int64_t)gridDim.x * blockDim.x) >> 5) * RW;
+  }
+};
+__device__ __forceinline__ void mu_load(const double* p, double* o) {
+  const double2 v = *(const double2*)p;
+  o[0] = v.x, o[1] = v.y;
+}
+__device__ __forceinline__ void mu_load(const float* p, float* o) {
+  const float2 v = *(const float2*)p;
+  o[0] = v.x, o[1] = v.y;
+}
+
+__global__ void __launch_bounds__(MROWS_BLOCK)
+    k_m_update_v(int64_t n, int K, double* __restrict__ R, const double* __restrict__ Q,
+                 const Scal* sc, double* part, int maxb, unsigned* ticket, MultiRrEpi epi,
+                 float* __restrict__ R32) {
+  constexpr int U = MU_ROWS;
+  const MuLanes ln(K);
+  double al[2], d[1][2] = {{0.0, 0.0}};
+  bool act[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    act[k] = ln.on && sc[ln.c0 + k].active;
+    al[k] = act[k] ? sc[ln.c0 + k].alpha : 0.0;
+  }
+  if (act[0] || act[1])
+    for (int64_t i = ln.i0; i < n; i += U * ln.step) {
+      double r[2 * U], q[2 * U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t iu = i + u * ln.step;
+        const int64_t e = (iu < n ? iu : i) * K + ln.c0;
+        mu_load(R + e, r + 2 * u);
+        mu_load(Q + e, q + 2 * u);
       }
+#pragma unroll
+      for (int u = 0; u < 2 * U; ++u)
+        if (act[u & 1]) r[u] = r[u] - al[u & 1] * q[u];
+      float f[2 * U];
+      if (R32) cvt_n(r, f);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t iu = i + u * ln.step;
+        if (iu >= n) break;
+        const int64_t e = iu * K + ln.c0;
+        *(double2*)(R + e) = make_double2(r[2 * u], r[2 * u + 1]);
+        if (R32) *(float2*)(R32 + e) = make_float2(f[2 * u], f[2 * u + 1]);
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+          if (act[k]) d[0][k] += r[2 * u + k] * r[2 * u + k];
+      }
+    }
+  cols_reduce_v<2, 1>(d, K, part, maxb, ticket, epi);
+}
+
+template <typename ZT, bool FIRST>
+__global__ void __launch_bounds__(MROWS_BLOCK)
+    k_m_p_update_v(int64_t n, int K, double* __restrict__ P, const ZT* __restrict__ Z,
+                   double* __restrict__ X, const Scal* sc) {
+  constexpr int U = MU_ROWS;
+  const MuLanes ln(K);
+  double al[2], be[2];
+  bool owed[2], act[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const Scal* S = sc + ln.c0 + k;
+    al[k] = !FIRST && ln.on ? S->alpha : 0.0;
+    owed[k] = al[k] != 0.0;
+    act[k] = ln.on && (FIRST || S->active);
+    be[k] = !FIRST && act[k] ? S->beta : 0.0;
+  }
+  const bool anyx = owed[0] || owed[1], anyp = act[0] || act[1];
+  if (!anyx && !anyp) return;
+  for (int64_t i = ln.i0; i < n; i += U * ln.step) {
+    ZT zt[2 * U];
+    double z[2 * U], p[2 * U], x[2 * U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t iu = i + u * ln.step;
+      const int64_t e = (iu < n ? iu : i) * K + ln.c0;
+      zt[2 * u] = zt[2 * u + 1] = ZT(0);
+      if (anyp) mu_load(Z + e, zt + 2 * u);
+      p[2 * u] = p[2 * u + 1] = 0.0;
+      if (!FIRST) mu_load(P + e, p + 2 * u);
+      if (anyx) mu_load(X + e, x + 2 * u);
+    }
+    cvt_n(zt, z);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t iu = i + u * ln.step;
+      if (iu >= n) break;
+      const int64_t e = iu * K + ln.c0;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int m = 2 * u + k;
+        if (owed[k]) x[m] = x[m] + al[k] * p[m];
+        if (act[k]) p[m] = FIRST ? z[m] : z[m] + be[k] * p[m];
+      }
+      if (anyx) *(double2*)(X + e) = make_double2(x[2 * u], x[2 * u + 1]);
+      if (anyp) *(double2*)(P + e) = make_double2(p[2 * u], p[2 * u + 1]);
+    }
+  }
 }
 
 // End of a solve: the x updates still owed.
@@ -1191,8 +1333,8 @@ static void m_post(const amg_handle* H, const MultiWs& W, bool vec, int K, const
 
 // R32: the FP32 copy of R0 (FP32 hierarchies), read by the level-0
 // pre-smoother: each element is converted once, not once per gather.
-template <typename T>
-static int m_vcycle(const amg_handle* H, const MultiWs& W, const double* R0, double* Z0,
+template <typename T, typename ZT>
+static int m_vcycle(const amg_handle* H, const MultiWs& W, const double* R0, ZT* Z0,
                     bool dots, const double* Q, int beta_form, bool first, cudaStream_t s,
                     const float* R32) {
   const int K = W.K;
@@ -1266,12 +1408,39 @@ static int m_vcycle(const amg_handle* H, const MultiWs& W, const double* R0, dou
   return AMG_OK;
 }
 
-static int m_vcycle_any(const amg_handle* H, const MultiWs& W, const double* R0, double* Z0,
-                        bool dots, const double* Q, int beta_form, bool first, cudaStream_t s,
-                        const float* R32 = nullptr) {
-  if (H->opt.precision == AMG_PREC_F32)
-    return m_vcycle<float>(H, W, R0, Z0, dots, Q, beta_form, first, s, R32);
-  return m_vcycle<double>(H, W, R0, Z0, dots, Q, beta_form, first, s, nullptr);
+// Grid of the vector-column updates: 32 / (K / 2) rows a warp and pass.
+static int mgrid_mu(const amg_handle* H, int64_t rows, int K) {
+  const int rw = 32 / (K / 2);
+  return grid_for((rows + rw - 1) / rw * 32, MROWS_BLOCK, H->num_sms, MV_BLOCKS);
+}
+
+template <bool FIRST, typename ZT>
+static void m_p_update(const amg_handle* H, const MultiWs& W, const ZT* Z, double* X,
+                       cudaStream_t s) {
+  const int64_t n = H->L[0].n;
+  const int K = W.K;
+  if (K % 2 == 0 && ((uintptr_t)X & 15u) == 0)
+    k_m_p_update_v<ZT, FIRST><<<mgrid_mu(H, n, K), MROWS_BLOCK, 0, s>>>(n, K, W.P, Z, X, W.sc);
+  else
+    AMG_DISPATCH_KPL(K, (k_m_p_update<KPL, ZT, FIRST><<<mgrid(H, n), MROWS_BLOCK, 0, s>>>(
+                            n, K, W.P, Z, X, W.sc)));
+}
+
+// z of the iteration (FP32 V-cycles: FP32, in W.Z), with the dot products, then
+// p from it.
+template <bool FIRST>
+static int m_z_and_p(const amg_handle* H, const MultiWs& W, int beta_form, double* X,
+                     cudaStream_t s) {
+  if (H->opt.precision == AMG_PREC_F32) {
+    float* Z = (float*)W.Z;
+    AMG_TRY((m_vcycle<float, float>(H, W, W.R, Z, true, W.Q, beta_form, FIRST, s, W.R32)));
+    m_p_update<FIRST>(H, W, Z, X, s);
+  } else {
+    AMG_TRY((m_vcycle<double, double>(H, W, W.R, W.Z, true, W.Q, beta_form, FIRST, s, nullptr)));
+    m_p_update<FIRST>(H, W, W.Z, X, s);
+  }
+  AMG_LAUNCH_CHECK();
+  return AMG_OK;
 }
 
 // Workspace for K right-hand sides, kept in the handle (reallocated if K grows).
@@ -1352,7 +1521,9 @@ int vcycle_multi(amg_handle* H, int K, const double* R, double* Z, cudaStream_t 
     k_m_to_f32<<<grid_for((m + 3) / 4, 256, H->num_sms, 8), 256, 0, s>>>(m, R, W->R32, vec);
     AMG_LAUNCH_CHECK();
   }
-  return m_vcycle_any(H, *W, R, Z, false, nullptr, PCG_BETA_FR, true, s, W->R32);
+  if (H->opt.precision == AMG_PREC_F32)
+    return m_vcycle<float, double>(H, *W, R, Z, false, nullptr, PCG_BETA_FR, true, s, W->R32);
+  return m_vcycle<double, double>(H, *W, R, Z, false, nullptr, PCG_BETA_FR, true, s, nullptr);
 }
 
 int pcg_multi_run(amg_handle* H, int K, const double* B, double* X, const pcg_options* o,
@@ -1386,28 +1557,27 @@ int pcg_multi_run(amg_handle* H, int K, const double* B, double* X, const pcg_op
   MultiRrEpi re{W->sc, o->tol, o->maxit, W->nactive};
   int k = 0;
   if (act > 0) {
-    AMG_TRY(m_vcycle_any(H, *W, W->R, W->Z, true, W->Q, beta_form, true, s, W->R32));
-    AMG_CUDA_TRY(cudaMemcpyAsync(W->P, W->Z, sizeof(double) * n * K, cudaMemcpyDeviceToDevice, s));
+    AMG_TRY(m_z_and_p<true>(H, *W, beta_form, X, s));
     for (;;) {
       if (K % 2 == 0)  // two doubles a lane (the workspace is 16-byte aligned)
-        k_m_spmm_dot_v<<<gmv, MROWS_BLOCK, 0, s>>>(A, C, K, mv_split<double>(gmv, L0.A, K), W->P, W->Q, W->part, maxb,
-                                                  W->ticket, pe);
+        k_m_spmm_dot_v<<<gmv, MROWS_BLOCK, 0, s>>>(A, C, K, mv_split<double>(gmv, L0.A, K),
+                                                  W->P, W->Q, W->part, maxb, W->ticket, pe);
       else
         AMG_DISPATCH_KPL(K, (k_m_spmm_dot<KPL><<<gmv, MROWS_BLOCK, 0, s>>>(
                                 A, C, K, W->P, W->Q, W->part, maxb, W->ticket, pe)));
       AMG_LAUNCH_CHECK();
       AMG_CUDA_TRY(cudaMemsetAsync(W->nactive, 0, sizeof(int), s));
-      AMG_DISPATCH_KPL(K, (k_m_update<KPL><<<g, MROWS_BLOCK, 0, s>>>(
-                                  n, K, W->R, W->Q, W->sc, W->part, maxb, W->ticket, re,
-                                  W->R32)));
+      if (K % 2 == 0)
+        k_m_update_v<<<mgrid_mu(H, n, K), MROWS_BLOCK, 0, s>>>(n, K, W->R, W->Q, W->sc, W->part,
+                                                               maxb, W->ticket, re, W->R32);
+      else
+        AMG_DISPATCH_KPL(K, (k_m_update<KPL><<<g, MROWS_BLOCK, 0, s>>>(
+                                n, K, W->R, W->Q, W->sc, W->part, maxb, W->ticket, re, W->R32)));
       AMG_LAUNCH_CHECK();
       ++k;
       AMG_TRY(read_act());
       if (act == 0 || k >= o->maxit) break;
-      AMG_TRY(m_vcycle_any(H, *W, W->R, W->Z, true, W->Q, beta_form, false, s, W->R32));
-      AMG_DISPATCH_KPL(
-          K, (k_m_p_update<KPL><<<g, MROWS_BLOCK, 0, s>>>(n, K, W->P, W->Z, X, W->sc)));
-      AMG_LAUNCH_CHECK();
+      AMG_TRY(m_z_and_p<false>(H, *W, beta_form, X, s));
     }
     AMG_DISPATCH_KPL(K,
                      (k_m_x_pending<KPL><<<g, MROWS_BLOCK, 0, s>>>(n, K, X, W->P, W->sc)));
