@@ -288,8 +288,8 @@ struct PcgScalars {
   double* x;
 };
 
-// Coarsest blocks up to this many rows are factored and solved by one CUDA
-// block each; larger ones use kernels spread over the whole GPU.
+// Coarsest blocks up to this many rows are solved by one CUDA block each inside
+// the persistent small-level launch; larger ones by the whole grid.
 constexpr int64_t COARSE_SMALL = 1024;
 
 // Diagonal block of coarsest row i: b with brow[b] <= i < brow[b+1].

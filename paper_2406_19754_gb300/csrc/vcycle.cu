@@ -515,6 +515,10 @@ __global__ void k_coarse_y(int64_t nco, int nblk, const int64_t* __restrict__ br
 // the vector is converted to FP64 once per CTA instead of once per term.  One
 // row per warp took 33 (y) and 28 us (x).
 constexpr int64_t COARSE_PAIR_ROWS = 5632;  // 44 KB of shared memory
+// One CTA solves a block of m rows in m^2 / 2 clocks of its SM's FP64 pipe after
+// about 6 us, two launches of one warp per row over the GPU in 12 to 13 us (48
+// blocks of batched systems: 36 and 12.6 us), the same bits: equal at m = 160.
+constexpr int64_t COARSE_ONE_CTA = 160;
 
 template <bool TRANSPOSED, typename BT, typename XT>
 __global__ void __launch_bounds__(256)
@@ -768,7 +772,7 @@ static int coarse_solve(const amg_handle* H, const BT* b, XT* x, cudaStream_t s,
   }
   int64_t m = 0;  // largest block
   for (int k = 0; k < H->nblk; ++k) m = std::max(m, H->cblk_row[k + 1] - H->cblk_row[k]);
-  if (m <= COARSE_SMALL) {  // one CUDA block per diagonal block; 2m doubles <= 16 KB
+  if (m <= COARSE_ONE_CTA) {  // one CUDA block per diagonal block
     const size_t sm = sizeof(double) * 2 * (size_t)m;
     k_coarse<BT, XT><<<H->nblk, 1024, sm, s>>>(H->d_brow, H->d_bmat, H->Linv, H->LinvT, b, x,
                                                act);

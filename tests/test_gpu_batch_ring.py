@@ -48,3 +48,20 @@ def test_batched_ring_equals_per_lane(amg, case, precision, sweeps):
                 d = x1[o[k]:o[k + 1]] - x0[o[k]:o[k + 1]]
                 assert float(d.norm() / x0[o[k]:o[k + 1]].norm()) <= 1e-10
         assert min(s["iterations"] for s in s1) < max(s["iterations"] for s in s1)
+
+
+@pytest.mark.parametrize("max_coarse", [40, 130, 600])  # blocks of one CTA, of whole-grid rows
+@pytest.mark.parametrize("precision", ["f64", "f32"])
+def test_coarsest_blocks_by_rows(amg, max_coarse, precision):
+    # each system's part of the blocked V-cycle is that of the system alone (its
+    # coarsest block solved by one CTA in the small-level launch): the same bits
+    systems = [poisson3d(21, 20, 19), poisson3d(21, 20, 19)]
+    devs = [amg.csr_to_device(S) for S in systems]
+    Hb = amg.BatchHierarchy(devs, max_coarse=max_coarse, precision=precision)
+    Hs = amg.Hierarchy(*devs[0], max_coarse=max_coarse, precision=precision)
+    assert Hb.levels == Hs.levels
+    n = Hs.level_info(0)[0]
+    b = torch.as_tensor(uniform01(47, 2 * n), device="cuda")
+    z = Hb.vcycle(b)
+    for k in range(2):
+        assert torch.equal(z[k * n:(k + 1) * n], Hs.vcycle(b[k * n:(k + 1) * n].clone()))
