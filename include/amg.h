@@ -116,7 +116,7 @@ typedef struct amg_options {
                             every level */
   int coarse_solver;     /* 0 (default): dense Cholesky of the coarsest level;
                             1: PCG preconditioned by its l1-Jacobi scaling
-                            (Sec. 3, VBM/VMATCH coarsest solver), one CUDA block,
+                            (Sec. 3, VBM/VMATCH coarsest solver), one cluster or block,
                             FP64; not for batched systems */
   int coarse_maxit;      /* PCG coarsest solve: iteration cap, default 40 */
   double coarse_tol;     /* PCG coarsest solve: stop at ||r|| <= tol ||b||,

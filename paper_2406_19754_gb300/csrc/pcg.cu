@@ -163,7 +163,8 @@ struct RrEpi {
 // operations a row, 32 row-operations per SM every 16 clocks.  Each thread
 // takes four rows a step by 32-byte accesses, so enough bytes are in flight,
 // and r32 is rounded on the integer pipe (cvt_n); scalar rows with the
-// hardware conversion took 107 us for 16.8M rows with r32, 74 us without.
+// hardware conversion took 107 us for 16.8M rows with r32, 16-byte accesses 91,
+// these 85 (floor 70).
 __global__ void k_cg_update(int64_t n, double* __restrict__ x, double* __restrict__ r,
                             const double* __restrict__ p, const double* __restrict__ q, Reduce red,
                             PcgScalars* sc, float* __restrict__ r32,
