@@ -103,11 +103,12 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
       return;
     }
     if (ring.ended) return;
-    if (ring.slice) {
-      const double acc = ring_row_sum<double>(ring, p);
-      if (ring.has) {
-        q[ring.i] = acc;
-        d += ring.row<double>(0) * acc;
+    if (ring.slot[0].slice) {
+      double acc[1] = {0.0};
+      ring_row_sums<false>(ring, p, acc);
+      if (ring.slot[0].has) {
+        q[ring.slot[0].i] = acc[0];
+        d += ring.row<double>(0) * acc[0];
       }
     }
     if (ring.last) {

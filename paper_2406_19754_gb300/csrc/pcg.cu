@@ -113,11 +113,12 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
       if (ring.lane == 0) ring_fail(fail, &sc->status);
       break;
     }
-    if (ring.slice) {
-      const double acc = ring_row_sum<double>(ring, p);
-      if (ring.has) {
-        q[ring.i] = acc;
-        d[0] += ring.template row<double>(0) * acc;
+    if (ring.slot[0].slice) {
+      double acc[1] = {0.0};
+      ring_row_sums<false>(ring, p, acc);
+      if (ring.slot[0].has) {
+        q[ring.slot[0].i] = acc[0];
+        d[0] += ring.template row<double>(0) * acc[0];
       }
     }
     ring.release();

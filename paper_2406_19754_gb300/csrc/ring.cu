@@ -19,7 +19,7 @@ namespace amg {
 constexpr size_t RING_L1_SPLIT = 128 * 1024;
 
 RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows, bool dots,
-                   bool chunked) {
+                   bool chunked, bool pairs) {
   RingGeom none;
   if (M.C != 32 || M.tpr != 1 || (M.row0 != nullptr) != chunked || !M.rec || M.wmax <= 0 ||
       M.nslices <= 0)
@@ -35,10 +35,12 @@ RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows, 
   // values, index blocks, records, per-row vectors; every part starts on 128 bytes
   auto plan = [&](int q, int D) {
     RingGeom g;
-    g.tile = ring_tile(q);
-    size_t off = up((size_t)M.tile_w[q] * 32 * (size_t)vbytes);
+    const int f = pairs ? 2 : 1;  // (tile_w and tile_ix bound two tiles together)
+    g.tile = ring_tile(q) * f;
+    g.warps = pairs ? g.tile / 2 : g.tile;
+    size_t off = up((size_t)M.tile_w[q] * f * 32 * (size_t)vbytes);
     g.coff = (uint32_t)off;
-    off = up(off + (size_t)M.tile_ix[q]);
+    off = up(off + (size_t)M.tile_ix[q] * f);
     g.soff = (uint32_t)off;
     off = up(off + 16 * (size_t)(g.tile + 1));
     if (chunked) {
@@ -62,6 +64,14 @@ RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows, 
   const int q0 = dots || chunked || M.nslices >= 304 * ring_tile(0) ? 0
                  : M.nslices >= 304 * ring_tile(1)       ? 1
                                                          : 2;
+  if (pairs) {
+    const int c = ring_ctas(vbytes, 2);
+    if (M.nslices < 304 * 2 * ring_tile(0)) return none;
+    const size_t smem = c * (plan(0, 3).smem + 1024);
+    const RingGeom g = plan(0, stages ? stages : smem <= RING_L1_SPLIT ? 3 : 2);
+    const bool fits = g.smem <= RING_SMEM_PER_CTA && c * (g.smem + 1024) <= RING_SMEM_PER_SM;
+    return fits ? g : none;
+  }
   for (int ctas : {RING_CTAS_PER_SM, RING_CTAS_PER_SM - 1, 2})
     for (int q = q0; q < (chunked ? 1 : 3); ++q) {
       const int c = ctas * ring_tile(0) / ring_tile(q);  // the same number of warps

@@ -67,6 +67,11 @@ constexpr int RING_MAX_TILE = 8;  // slices per tile = consumer warps per CTA
 // row's gathers in flight together (256^3 FP32 solve 158.7 -> 175 and 193 ms).
 constexpr int RING_CTAS_PER_SM = 4;
 constexpr int RING_MAX_THREADS = (RING_MAX_TILE + 1) * 32;
+// CTAs per SM of a kernel with values of `vbytes` bytes and spw slices a warp
+// (FP64 rings of two do not fit four times).
+constexpr int ring_ctas(int vbytes, int spw) {
+  return vbytes == 8 && spw == 2 ? 3 : RING_CTAS_PER_SM;
+}
 constexpr unsigned long long RING_WAIT_NS = 1000000000ull;  // 1 s
 constexpr size_t RING_SMEM_PER_CTA = 112 * 1024;   // at least two CTAs per SM
 constexpr size_t RING_SMEM_PER_SM = 227 * 1024;
@@ -93,6 +98,7 @@ struct RingRows {
 struct RingGeom {
   int D = 0;            // stages per CTA (0: not eligible)
   int tile = 0;         // slices per tile
+  int warps = 0;        // consumer warps (tile, or tile / 2: two slices a warp)
   uint32_t stage = 0;   // bytes per stage
   uint32_t coff = 0;    // offset of the index blocks within a stage
   uint32_t soff = 0;    // offset of the slice records
@@ -101,7 +107,7 @@ struct RingGeom {
   uint32_t direct = 0;  // bit k: row vector k starts off a 16-byte boundary, no bulk copies
   int grid = 0;         // CTAs (ring_prepare)
   size_t smem = 0;      // dynamic shared memory per CTA
-  int threads() const { return (tile + 1) * 32; }
+  int threads() const { return (warps + 1) * 32; }
 };
 
 // Chunks of a batched level: chunk c is slices off[c] .. off[c + 1] - 1, all of
@@ -201,7 +207,19 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 //     if (ring.slice) { ... ring_row_sum(ring, g, init) of row ring.i ... }
 //     ring.release();
 //   }
-template <typename V, bool CHUNKED = false>
+// A consumer warp's slice of the current tile, this lane's row in it.
+template <typename V>
+struct RingSlot {
+  bool slice = false;     // there is a slice
+  bool has = false;       // this lane has a row: row i
+  uint32_t i = 0, j = 0;  // j: the row's place among the staged entries
+  const V* vals = nullptr;  // this lane's values
+  const int32_t* ixb = nullptr;
+  int wm = 0;  // (ELL width << 2) | IX_* code
+  __device__ __forceinline__ V val(int k) const { return vals[k * 32]; }
+};
+
+template <typename V, bool CHUNKED = false, int SPW = 1>
 struct TileRing {
   const SellView<V>& A;
   const RingGeom& g;
@@ -215,15 +233,10 @@ struct TileRing {
   uint32_t phase = 0;
   uint32_t t, ntiles;    // current tile, tiles (not CHUNKED)
   bool ended = false;    // CHUNKED: no more tiles
-  bool slice = false;    // this warp has a slice of the tile
-  bool has = false;      // this lane has a row: row i
   bool last = false;     // CHUNKED: last tile of its chunk
-  uint32_t i = 0, j = 0;  // j: the row's place among the staged entries
   int64_t chunk = 0;
   const unsigned char* st = nullptr;  // current stage
-  const V* vals = nullptr;            // this lane's values
-  const int32_t* ixb = nullptr;
-  int wm = 0;  // (ELL width << 2) | IX_* code
+  RingSlot<V> slot[SPW];              // this warp's slices
 
   __device__ __forceinline__ TileRing(const SellView<V>& A_, const RingGeom& g_,
                                       const RingRows& rows_, const RingChunks& ch_,
@@ -236,11 +249,10 @@ struct TileRing {
     lane = threadIdx.x & 31;
     ntiles = (uint32_t)((A.nslices + g.tile - 1) / g.tile);
     t = blockIdx.x;
-    j = threadIdx.x;
     if (threadIdx.x == 0) {
       for (int d = 0; d < g.D; ++d) {
         mbar_init(full(d), 1);
-        mbar_init(empty(d), (uint32_t)g.tile);
+        mbar_init(empty(d), (uint32_t)g.warps);
       }
       mbar_init_fence();
     }
@@ -251,7 +263,7 @@ struct TileRing {
   __device__ __forceinline__ uint32_t empty(int d) const {
     return bars + 8u * (uint32_t)(RING_MAX_STAGES + d);
   }
-  __device__ __forceinline__ bool producer() const { return warp == g.tile; }
+  __device__ __forceinline__ bool producer() const { return warp == g.warps; }
   __device__ __forceinline__ SliceRec load_rec(int64_t s) const {
     const longlong2 r = __ldg((const longlong2*)(A.rec + (s < A.nslices ? s : A.nslices)));
     return SliceRec{r.x, r.y};
@@ -409,38 +421,48 @@ struct TileRing {
   __device__ __forceinline__ bool wait() {
     if (!__all_sync(0xffffffffu, mbar_wait_bounded(full(stage), phase))) return false;
     st = base + (uint32_t)stage * g.stage;
+    uint32_t ns, r0, rows_, e0 = 0;  // the tile: slices, first row, rows, first staged row
     if constexpr (CHUNKED) {
       const RingTile& h = *(const RingTile*)(st + g.hoff);
       ended = h.ns < 0;
       if (ended) return true;
-      slice = warp < h.ns;
-      i = (uint32_t)h.r0 + threadIdx.x;
-      has = slice && (int)threadIdx.x < h.rows;
-      j = i - (uint32_t)h.e0;
+      ns = (uint32_t)h.ns;
+      r0 = (uint32_t)h.r0;
+      rows_ = (uint32_t)h.rows;
+      e0 = r0 - (uint32_t)h.e0;
       last = h.last != 0;
       chunk = h.chunk;
     } else {
       const uint32_t s0 = t * (uint32_t)g.tile;
-      slice = s0 + warp < (uint32_t)A.nslices;
-      i = s0 * 32 + threadIdx.x;
-      has = i < (uint32_t)A.n;
+      ns = (uint32_t)A.nslices - s0;
+      r0 = s0 * 32;
+      rows_ = (uint32_t)A.n - r0;
     }
-    if (slice) {
-      // low halves: differences within a tile
-      const int4* r = (const int4*)(st + g.soff);
-      const int4 r0 = r[0], rw = r[warp], rn = r[warp + 1];
-      vals = (const V*)(st + (uint32_t)(rw.x - r0.x) * (uint32_t)sizeof(V)) + lane;
-      ixb = (const int32_t*)(st + (g.coff + (uint32_t)((rw.z & ~3) - (r0.z & ~3))));
-      wm = (rn.x - rw.x) >> 5 << 2 | (rw.z & 3);
+    const int4* r = (const int4*)(st + g.soff);
+    const int4 rb = r[0];
+#pragma unroll
+    for (int m = 0; m < SPW; ++m) {
+      RingSlot<V>& o = slot[m];
+      const uint32_t k = (uint32_t)warp * SPW + m;
+      o.slice = k < ns;
+      const uint32_t u = k * 32 + lane;
+      o.i = r0 + u;
+      o.j = e0 + u;
+      o.has = u < rows_;
+      if (o.slice) {  // low halves: differences within a tile
+        const int4 rw = r[k], rn = r[k + 1];
+        o.vals = (const V*)(st + (uint32_t)(rw.x - rb.x) * (uint32_t)sizeof(V)) + lane;
+        o.ixb = (const int32_t*)(st + (g.coff + (uint32_t)((rw.z & ~3) - (rb.z & ~3))));
+        o.wm = (rn.x - rw.x) >> 5 << 2 | (rw.z & 3);
+      }
     }
     return true;
   }
 
-  __device__ __forceinline__ V val(int k) const { return vals[k * 32]; }
-  // this lane's entry (row i) of per-row vector k, of type X
+  // this lane's entry (row of slot m) of per-row vector k, of type X
   template <typename X>
-  __device__ __forceinline__ X row(int k) const {
-    return ((const X*)(st + g.roff[k]))[j];
+  __device__ __forceinline__ X row(int k, int m = 0) const {
+    return ((const X*)(st + g.roff[k]))[slot[m].j];
   }
 
   // every lane is done with the stage
@@ -515,62 +537,100 @@ struct IxClamp {
 };
 
 // acc + sum of a_k v[col_k] (NEG: acc - sum, by FMAs with the negated
-// values) for k = k0 .. k0 + N - 1, k ascending: the N gathers issue
-// together, then the FMAs follow in order.  Exactly N FMAs: on GB300's FP64
-// pipe a predicated-off FMA would still cost its cycles.
-template <int N, bool NEG, typename T, typename R, typename I>
-__device__ __forceinline__ T ring_chunk(const R& ring, const I& ix, int k0, T acc) {
-  int32_t o[N];
-  ix.load(k0, o);
-  T x[N];
+// values) for k = k0 .. k0 + N - 1, k ascending, of the rows in NS slices: all
+// gathers issue together, then the FMAs follow in order.  Exactly N FMAs a row:
+// on GB300's FP64 pipe a predicated-off FMA would still cost its cycles.
+template <int N, bool NEG, int NS, typename T, typename S, typename I>
+__device__ __forceinline__ void ring_chunk(const S* sl, const I (&ix)[NS], int k0, T* acc) {
+  T x[NS][N];
 #pragma unroll
-  for (int u = 0; u < N; ++u) x[u] = to_f(__ldg(ix.v + o[u]), T(0));
+  for (int m = 0; m < NS; ++m) {
+    int32_t o[N];
+    ix[m].load(k0, o);
 #pragma unroll
-  for (int u = 0; u < N; ++u) {
-    const T a = to_f(ring.val(k0 + u), T(0));
-    acc = fma(NEG ? -a : a, x[u], acc);
+    for (int u = 0; u < N; ++u) x[m][u] = to_f(__ldg(ix[m].v + o[u]), T(0));
   }
-  return acc;
+#pragma unroll
+  for (int m = 0; m < NS; ++m)
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+      const T a = to_f(sl[m].val(k0 + u), T(0));
+      acc[m] = fma(NEG ? -a : a, x[m][u], acc[m]);
+    }
 }
 
 // Chunks of 8 and one remainder chunk of the exact length (w is
 // warp-uniform).
-template <bool NEG, typename T, typename R, typename I>
-__device__ __forceinline__ T ring_chunks(const R& ring, const I& ix, int w, T acc) {
+template <bool NEG, int NS, typename T, typename S, typename I>
+__device__ __forceinline__ void ring_chunks(const S* sl, const I (&ix)[NS], int w, T* acc) {
   int k0 = 0;
-  for (; k0 + 8 <= w; k0 += 8) acc = ring_chunk<8, NEG>(ring, ix, k0, acc);
+  for (; k0 + 8 <= w; k0 += 8) ring_chunk<8, NEG, NS>(sl, ix, k0, acc);
   switch (w - k0) {
-    case 1: acc = ring_chunk<1, NEG>(ring, ix, k0, acc); break;
-    case 2: acc = ring_chunk<2, NEG>(ring, ix, k0, acc); break;
-    case 3: acc = ring_chunk<3, NEG>(ring, ix, k0, acc); break;
-    case 4: acc = ring_chunk<4, NEG>(ring, ix, k0, acc); break;
-    case 5: acc = ring_chunk<5, NEG>(ring, ix, k0, acc); break;
-    case 6: acc = ring_chunk<6, NEG>(ring, ix, k0, acc); break;
-    case 7: acc = ring_chunk<7, NEG>(ring, ix, k0, acc); break;
+    case 1: ring_chunk<1, NEG, NS>(sl, ix, k0, acc); break;
+    case 2: ring_chunk<2, NEG, NS>(sl, ix, k0, acc); break;
+    case 3: ring_chunk<3, NEG, NS>(sl, ix, k0, acc); break;
+    case 4: ring_chunk<4, NEG, NS>(sl, ix, k0, acc); break;
+    case 5: ring_chunk<5, NEG, NS>(sl, ix, k0, acc); break;
+    case 6: ring_chunk<6, NEG, NS>(sl, ix, k0, acc); break;
+    case 7: ring_chunk<7, NEG, NS>(sl, ix, k0, acc); break;
     default: break;
   }
-  return acc;
 }
 
-// init + sum_k a_k v[col_k] (NEG: init - sum) over the entries of this
-// lane's row i in the current stage, k ascending (the per-lane kernels'
-// order).
-template <typename T, bool NEG = false, typename R, typename X>
-__device__ __forceinline__ T ring_row_sum(const R& ring, const X* v, T init = T(0)) {
-  const int w = ring.wm >> 2;
-  const int32_t* c = ring.ixb;
-  switch (ring.wm & 3) {
-    case IX_OFFSET:
-      return ring_chunks<NEG>(ring, IxOffset<X>{v + ring.i, c}, w, init);
-    case IX_CLAMP:
-      return ring_chunks<NEG>(ring, IxClamp<X>{v, c, (int32_t)ring.i, ring.A.ncols - 1}, w,
-                              init);
-    case IX_DELTA:
-      return ring_chunks<NEG>(
-          ring, IxDelta<X>{v, c, (const uint16_t*)(c + ((w + 3) & ~3)) + ring.lane}, w, init);
-    default:
-      return ring_chunks<NEG>(ring, IxPlain<X>{v, c + ring.lane}, w, init);
+// acc[m] + sum_k a_k v[col_k] (NEG: - sum) over the entries of this lane's row
+// in each of NS slices of one width and coding, k ascending (the per-lane
+// kernels' order).
+template <bool NEG, int NS, typename T, typename S, typename X>
+__device__ __forceinline__ void ring_slots_sum(const S* sl, int ncols, int lane, const X* v,
+                                               T* acc) {
+  const int w = sl[0].wm >> 2;
+  switch (sl[0].wm & 3) {
+    case IX_OFFSET: {
+      IxOffset<X> ix[NS];
+#pragma unroll
+      for (int m = 0; m < NS; ++m) ix[m] = IxOffset<X>{v + sl[m].i, sl[m].ixb};
+      return ring_chunks<NEG, NS>(sl, ix, w, acc);
+    }
+    case IX_CLAMP: {
+      IxClamp<X> ix[NS];
+#pragma unroll
+      for (int m = 0; m < NS; ++m)
+        ix[m] = IxClamp<X>{v, sl[m].ixb, (int32_t)sl[m].i, ncols - 1};
+      return ring_chunks<NEG, NS>(sl, ix, w, acc);
+    }
+    case IX_DELTA: {
+      IxDelta<X> ix[NS];
+#pragma unroll
+      for (int m = 0; m < NS; ++m)
+        ix[m] = IxDelta<X>{v, sl[m].ixb,
+                           (const uint16_t*)(sl[m].ixb + ((w + 3) & ~3)) + lane};
+      return ring_chunks<NEG, NS>(sl, ix, w, acc);
+    }
+    default: {
+      IxPlain<X> ix[NS];
+#pragma unroll
+      for (int m = 0; m < NS; ++m) ix[m] = IxPlain<X>{v, sl[m].ixb + lane};
+      return ring_chunks<NEG, NS>(sl, ix, w, acc);
+    }
   }
+}
+
+// The same over this warp's slices of the tile; two of one width and coding (in
+// a stencil matrix nearly always) with all their gathers in flight at once.
+template <bool NEG, typename T, typename V, bool CH, int SPW, typename X>
+__device__ __forceinline__ void ring_row_sums(const TileRing<V, CH, SPW>& ring, const X* v,
+                                              T (&acc)[SPW]) {
+  const int nc = ring.A.ncols;
+  if constexpr (SPW == 2) {
+    if (ring.slot[1].slice && ring.slot[0].wm == ring.slot[1].wm) {
+      ring_slots_sum<NEG, 2>(ring.slot, nc, ring.lane, v, acc);
+      return;
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < SPW; ++m)
+    if (ring.slot[m].slice)
+      ring_slots_sum<NEG, 1>(ring.slot + m, nc, ring.lane, v, acc + m);
 }
 
 // A bounded wait gave up: the handle's sticky flag, and the PCG status
@@ -586,7 +646,7 @@ __device__ __forceinline__ void ring_fail(int* fail, int* status) {
 // for batched systems (M.row0), which only chunked kernels take.  The grid is
 // left to ring_prepare.  Host code.
 RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows,
-                   bool dots = false, bool chunked = false);
+                   bool dots = false, bool chunked = false, bool pairs = false);
 
 // Prepares kernel `fn` for a launch with geometry g on the current device
 // (shared-memory limit, once per device and kernel) and sets g.grid to the

@@ -158,15 +158,22 @@ __global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
 // thread over the warp's slices, then per block and over blocks, as there
 // (with this launch's grid).  The rows' own operands (s, r, b, agg, ...) come
 // with the tile (per-row vectors of the ring).
-template <typename V, typename T, typename BT, bool CH>
-__global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
+//
+// SPW = 2: a warp takes two slices of a tile of 16 and has both rows' gathers in
+// flight.  The FP32 pre-smoother waits for them most (9 of 17 cycles between a
+// warp's instructions, DRAM and issue slots half busy): 137 -> 108 us at 256^3.
+// On levels of at least 4,864 slices whose rings of twice the bytes fit four CTAs
+// an SM.  The post-smoothers, with four row operands a slice besides, gained
+// nothing (201 -> 205 us).
+template <typename V, typename T, typename BT, bool CH, int SPW>
+__global__ void __launch_bounds__(RING_MAX_THREADS, ring_ctas(sizeof(V), SPW))
     k_pre_ring(const __grid_constant__ SellView<V> Ah, const BT* __restrict__ b,
                T* __restrict__ r, const __grid_constant__ RingGeom g,
                const __grid_constant__ RingRows rows, const __grid_constant__ RingChunks ch,
                int* fail) {
   extern __shared__ unsigned char ring_smem[];
   if (*(volatile int*)fail) return;
-  TileRing<V, CH> ring(Ah, g, rows, ch, ring_smem);
+  TileRing<V, CH, SPW> ring(Ah, g, rows, ch, ring_smem);
   if (ring.producer()) {
     ring.produce(fail, nullptr);
     return;
@@ -177,12 +184,14 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
       return;
     }
     if (ring.ended) return;
-    if (ring.slice) {
-      const T bi = ring.has ? to_f(ring.template row<BT>(0), T(0)) : T(0);
-      // pre_slice's arithmetic: from b_i down by negated FMAs
-      const T acc = ring_row_sum<T, true>(ring, b, bi);
-      if (ring.has) r[ring.i] = acc;
-    }
+    T acc[SPW];
+#pragma unroll
+    for (int m = 0; m < SPW; ++m)
+      acc[m] = ring.slot[m].has ? to_f(ring.template row<BT>(0, m), T(0)) : T(0);
+    ring_row_sums<true>(ring, b, acc);  // pre_slice's arithmetic: from b_i down
+#pragma unroll
+    for (int m = 0; m < SPW; ++m)
+      if (ring.slot[m].has) r[ring.slot[m].i] = acc[m];
     ring.release();
   }
 }
@@ -213,33 +222,26 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
       break;
     }
     if (ring.ended) break;
-    if (ring.slice) {
-      const bool has = ring.has;
-      const int64_t i = ring.i;
-      // x_c of the row's own aggregate: gathered with the row's entries
-      const T xci = has ? __ldg(xc + ring.template row<int32_t>(3)) : T(0);
-      const T ri = has ? ring.template row<T>(1) : T(0);
+    const bool has = ring.slot[0].has;
+    // x_c of the row's own aggregate: gathered with the row's entries
+    const T xci = has ? __ldg(xc + ring.template row<int32_t>(3)) : T(0);
+    const BT bi = !MS && has ? ring.template row<BT>(2) : BT(0);
+    // post_slice's arithmetic (one sweep): from b_i + r_i down, then one FMA
+    T acc[1] = {!MS && has ? to_f(bi, T(0)) + ring.template row<T>(1) : T(0)};
+    ring_row_sums<!MS>(ring, xc, acc);
+    if (has) {
+      const uint32_t i = ring.slot[0].i;
+      const T si = ring.template row<T>(0);
       if constexpr (MS) {
-        const T acc = ring_row_sum<T>(ring, xc);
-        if (has) {
-          const T si = ring.template row<T>(0);
-          const T yi = ring.template row<T>(2) + xci;
-          const T ei = ri - acc;
-          x[i] = to_f(fma(si, ei, yi), XT(0));
-          e[i] = ei;
-        }
+        const T ei = ring.template row<T>(1) - acc[0];
+        const T yi = ring.template row<T>(2) + xci;
+        x[i] = to_f(fma(si, ei, yi), XT(0));
+        e[i] = ei;
       } else {
-        // post_slice's arithmetic (one sweep): from b_i + r_i down, then one FMA
-        const BT bi = has ? ring.template row<BT>(2) : BT(0);
-        const T init = has ? to_f(bi, T(0)) + ri : T(0);
-        const T acc = ring_row_sum<T, true>(ring, xc, init);
-        if (has) {
-          const XT zi = to_f(fma(ring.template row<T>(0), acc, xci), XT(0));
-          x[i] = zi;
-          if constexpr (NDOT > 0) d[0] += (double)bi * (double)zi;
-          if constexpr (NDOT > 1)
-            d[NDOT > 1 ? 1 : 0] += (double)zi * ring.template row<double>(4);
-        }
+        const XT zi = to_f(fma(si, acc[0], xci), XT(0));
+        x[i] = zi;
+        if constexpr (NDOT > 0) d[0] += (double)bi * (double)zi;
+        if constexpr (NDOT > 1) d[NDOT > 1 ? 1 : 0] += (double)zi * ring.template row<double>(4);
       }
     }
     if constexpr (CH && NDOT > 0) {
@@ -283,12 +285,13 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
       if (ring.lane == 0) ring_fail(fail, status);
       break;
     }
-    if (ring.slice) {
-      const T acc = ring_row_sum<T>(ring, r);
-      if (ring.has) {
-        const int64_t i = ring.i;
+    {
+      T acc[1] = {T(0)};
+      ring_row_sums<false>(ring, r, acc);
+      if (ring.slot[0].has) {
+        const int64_t i = ring.slot[0].i;
         const T ri = ring.template row<T>(1);
-        const T rn = ri - acc;
+        const T rn = ri - acc[0];
         r_out[i] = rn;
         const T si = ring.template row<T>(0);
         if constexpr (PRE) {
@@ -814,15 +817,29 @@ static int launch_pre(const amg_handle* H, const Level& L, const V* ah, const BT
       rows.add(b, (int)sizeof(BT));
       RingGeom g = ring_plan(L.A, (int)sizeof(V), ring_stages(H), rows, false, H->batched);
       if (g.D && H->batched) {
-        const auto fn = k_pre_ring<V, T, BT, true>;
+        const auto fn = k_pre_ring<V, T, BT, true, 1>;
         AMG_TRY(ring_prepare((const void*)fn, g, L.rch_n, H->num_sms));
         fn<<<g.grid, g.threads(), g.smem, s>>>(v, b, r, g, rows, RingChunks{L.rch_off, L.rch_n},
                                                H->wait_fail);
         AMG_LAUNCH_CHECK();
         return AMG_OK;
       }
+      // FP32 values, two slices a warp: more gathers in flight (k_pre_ring)
+      if constexpr (sizeof(V) == 4) {
+        if (!H->batched) {
+          RingGeom g2 = ring_plan(L.A, (int)sizeof(V), ring_stages(H), rows, false, false, true);
+          if (g2.D) {
+            const auto fn = k_pre_ring<V, T, BT, false, 2>;
+            AMG_TRY(ring_prepare((const void*)fn, g2, ring_tiles(g2, L.A), H->num_sms));
+            fn<<<g2.grid, g2.threads(), g2.smem, s>>>(v, b, r, g2, rows, RingChunks(),
+                                                      H->wait_fail);
+            AMG_LAUNCH_CHECK();
+            return AMG_OK;
+          }
+        }
+      }
       if (g.D) {
-        const auto fn = k_pre_ring<V, T, BT, false>;
+        const auto fn = k_pre_ring<V, T, BT, false, 1>;
         AMG_TRY(ring_prepare((const void*)fn, g, ring_tiles(g, L.A), H->num_sms));
         fn<<<g.grid, g.threads(), g.smem, s>>>(v, b, r, g, rows, RingChunks(), H->wait_fail);
         AMG_LAUNCH_CHECK();
