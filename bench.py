@@ -103,7 +103,7 @@ def _args():
     ap.add_argument("--no-ring", action="store_true",
                     help="per-lane loads instead of the shared-memory ring (stream_ring=0)")
     ap.add_argument("--ring-stages", type=int, default=0,
-                    help="stages per warp of the shared-memory ring (2..4; 0: the library's)")
+                    help="stages per CTA of the shared-memory ring (2..4; 0: the library's)")
     ap.add_argument("--compress", action="store_true",
                     help="2-byte column offsets in the kernels (compress_columns=1)")
     ap.add_argument("--tail-rows", type=int, default=None,
