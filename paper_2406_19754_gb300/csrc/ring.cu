@@ -16,6 +16,11 @@ namespace amg {
 // vector, else two: measured at 256^3 (FP32), the level-0 pre-smoother (9 KB
 // stages) took 0.136 ms with three against 0.143 with two, the level-1 one of
 // a diffusion matrix (18 KB stages) 0.092 against 0.080.
+//
+// Pairs (two slices a warp, tiles of 16): where two CTAs on each of 152 SMs have a
+// tile and four rings fit an SM.  256^3 FP32, level-0 pre-smoother: 137 us with one
+// slice a warp, 108 with two; four warps of two slices in six or seven CTAs an SM
+// 118 and 114.
 constexpr size_t RING_L1_SPLIT = 128 * 1024;
 
 RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows, bool dots,
@@ -65,7 +70,7 @@ RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows, 
                  : M.nslices >= 304 * ring_tile(1)       ? 1
                                                          : 2;
   if (pairs) {
-    const int c = ring_ctas(vbytes, 2);
+    const int c = RING_CTAS_PER_SM;
     if (M.nslices < 304 * 2 * ring_tile(0)) return none;
     const size_t smem = c * (plan(0, 3).smem + 1024);
     const RingGeom g = plan(0, stages ? stages : smem <= RING_L1_SPLIT ? 3 : 2);

@@ -21,7 +21,12 @@
 // What bounds it: with a ring per warp (every warp refilling its own two
 // stages slice by slice) the FP32 level-0 pre-smoother issued 241 warp
 // instructions a slice of 7 entries a row, more than half of them to manage
-// the ring, and its time did not move when a third of its bytes went.
+// the ring, and its time did not move when a third of its bytes went.  A tile a
+// CTA, operands always staged and 32-bit places take 156 (post-smoother 406 ->
+// 224).  What is left is the latency of the gathers in the FP32 pre-smoother and
+// sweeps (two slices a warp, SPW = 2) and the FP64 pipe in the FP64 kernels (86%
+// busy).  256^3, level 0: FP32 pre-smoother 179 -> 108 us, post-smoother 250 -> 201,
+// FP64 pre-smoother 249 -> 223, post-smoother 279 -> 250, product 250 -> 242.
 //
 // Column indices are a third of an FP64 operator's stream and half of an FP32
 // one's, and the columns of 32 consecutive rows say almost the same thing 32
@@ -29,10 +34,10 @@
 // columns (IX_* in common.cuh): one offset per ELL column where the rows share
 // their offsets (every slice of a stencil matrix: 4 bytes instead of 128),
 // 16-bit deltas from a base per ELL column where the columns lie close (A P
-// and the coarse levels: 68 instead of 128), else plain columns.  In the
+// and the coarse levels: 68 instead of 128), else plain columns.  In the FP32
 // per-lane kernels fewer index bytes did not pay (each load then carries less,
-// and their number bounds them); here the copies are whole blocks, so bytes
-// are what counts.
+// and their number bounds them: 142 -> 169 us); here the copies are whole blocks,
+// so bytes are what counts.
 //
 // Batched systems (CHUNKED): a CTA takes chunks of consecutive slices of one
 // system, leaves out those of systems that have stopped, and cuts each into
@@ -67,11 +72,6 @@ constexpr int RING_MAX_TILE = 8;  // slices per tile = consumer warps per CTA
 // row's gathers in flight together (256^3 FP32 solve 158.7 -> 175 and 193 ms).
 constexpr int RING_CTAS_PER_SM = 4;
 constexpr int RING_MAX_THREADS = (RING_MAX_TILE + 1) * 32;
-// CTAs per SM of a kernel with values of `vbytes` bytes and spw slices a warp
-// (FP64 rings of two do not fit four times).
-constexpr int ring_ctas(int vbytes, int spw) {
-  return vbytes == 8 && spw == 2 ? 3 : RING_CTAS_PER_SM;
-}
 constexpr unsigned long long RING_WAIT_NS = 1000000000ull;  // 1 s
 constexpr size_t RING_SMEM_PER_CTA = 112 * 1024;   // at least two CTAs per SM
 constexpr size_t RING_SMEM_PER_SM = 227 * 1024;
@@ -615,7 +615,8 @@ __device__ __forceinline__ void ring_slots_sum(const S* sl, int ncols, int lane,
   }
 }
 
-// The same over this warp's slices of the tile; two of one width and coding (in
+// The same over this warp's slices of the tile (with one slice a warp the caller
+// has looked that there is one); two of one width and coding (in
 // a stencil matrix nearly always) with all their gathers in flight at once.
 template <bool NEG, typename T, typename V, bool CH, int SPW, typename X>
 __device__ __forceinline__ void ring_row_sums(const TileRing<V, CH, SPW>& ring, const X* v,
@@ -629,7 +630,7 @@ __device__ __forceinline__ void ring_row_sums(const TileRing<V, CH, SPW>& ring, 
   }
 #pragma unroll
   for (int m = 0; m < SPW; ++m)
-    if (ring.slot[m].slice)
+    if (SPW == 1 || ring.slot[m].slice)
       ring_slots_sum<NEG, 1>(ring.slot + m, nc, ring.lane, v, acc + m);
 }
 
@@ -644,7 +645,8 @@ __device__ __forceinline__ void ring_fail(int* fail, int* status) {
 // D = 0 when M does not qualify.  stages: 2..RING_MAX_STAGES, or 0 for the
 // default.  dots: the kernel also sums dot products over its grid.  chunked:
 // for batched systems (M.row0), which only chunked kernels take.  The grid is
-// left to ring_prepare.  Host code.
+// left to ring_prepare.  pairs: for kernels with two slices a warp (FP32 values).
+// Host code.
 RingGeom ring_plan(const Sell& M, int vbytes, int stages, const RingRows& rows,
                    bool dots = false, bool chunked = false, bool pairs = false);
 

@@ -164,9 +164,10 @@ __global__ void __launch_bounds__(SELL_BLOCK, sell_blocks(TPR))
 // warp's instructions, DRAM and issue slots half busy): 137 -> 108 us at 256^3.
 // On levels of at least 4,864 slices whose rings of twice the bytes fit four CTAs
 // an SM.  The post-smoothers, with four row operands a slice besides, gained
-// nothing (201 -> 205 us).
+// nothing (201 -> 205 us).  The FP32 further sweeps take two as well (VMATCH
+// 200^3 28.9 -> 28.2 ms, SMATCH 22.2 -> 21.5).
 template <typename V, typename T, typename BT, bool CH, int SPW>
-__global__ void __launch_bounds__(RING_MAX_THREADS, ring_ctas(sizeof(V), SPW))
+__global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
     k_pre_ring(const __grid_constant__ SellView<V> Ah, const BT* __restrict__ b,
                T* __restrict__ r, const __grid_constant__ RingGeom g,
                const __grid_constant__ RingRows rows, const __grid_constant__ RingChunks ch,
@@ -188,7 +189,7 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, ring_ctas(sizeof(V), SPW))
 #pragma unroll
     for (int m = 0; m < SPW; ++m)
       acc[m] = ring.slot[m].has ? to_f(ring.template row<BT>(0, m), T(0)) : T(0);
-    ring_row_sums<true>(ring, b, acc);  // pre_slice's arithmetic: from b_i down
+    if (ring.slot[0].slice) ring_row_sums<true>(ring, b, acc);  // pre_slice: from b_i down
 #pragma unroll
     for (int m = 0; m < SPW; ++m)
       if (ring.slot[m].has) r[ring.slot[m].i] = acc[m];
@@ -222,26 +223,28 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
       break;
     }
     if (ring.ended) break;
-    const bool has = ring.slot[0].has;
-    // x_c of the row's own aggregate: gathered with the row's entries
-    const T xci = has ? __ldg(xc + ring.template row<int32_t>(3)) : T(0);
-    const BT bi = !MS && has ? ring.template row<BT>(2) : BT(0);
-    // post_slice's arithmetic (one sweep): from b_i + r_i down, then one FMA
-    T acc[1] = {!MS && has ? to_f(bi, T(0)) + ring.template row<T>(1) : T(0)};
-    ring_row_sums<!MS>(ring, xc, acc);
-    if (has) {
-      const uint32_t i = ring.slot[0].i;
-      const T si = ring.template row<T>(0);
-      if constexpr (MS) {
-        const T ei = ring.template row<T>(1) - acc[0];
-        const T yi = ring.template row<T>(2) + xci;
-        x[i] = to_f(fma(si, ei, yi), XT(0));
-        e[i] = ei;
-      } else {
-        const XT zi = to_f(fma(si, acc[0], xci), XT(0));
-        x[i] = zi;
-        if constexpr (NDOT > 0) d[0] += (double)bi * (double)zi;
-        if constexpr (NDOT > 1) d[NDOT > 1 ? 1 : 0] += (double)zi * ring.template row<double>(4);
+    if (ring.slot[0].slice) {
+      const bool has = ring.slot[0].has;
+      // x_c of the row's own aggregate: gathered with the row's entries
+      const T xci = has ? __ldg(xc + ring.template row<int32_t>(3)) : T(0);
+      const BT bi = !MS && has ? ring.template row<BT>(2) : BT(0);
+      // post_slice's arithmetic (one sweep): from b_i + r_i down, then one FMA
+      T acc[1] = {!MS && has ? to_f(bi, T(0)) + ring.template row<T>(1) : T(0)};
+      ring_row_sums<!MS>(ring, xc, acc);
+      if (has) {
+        const uint32_t i = ring.slot[0].i;
+        const T si = ring.template row<T>(0);
+        if constexpr (MS) {
+          const T ei = ring.template row<T>(1) - acc[0];
+          const T yi = ring.template row<T>(2) + xci;
+          x[i] = to_f(fma(si, ei, yi), XT(0));
+          e[i] = ei;
+        } else {
+          const XT zi = to_f(fma(si, acc[0], xci), XT(0));
+          x[i] = zi;
+          if constexpr (NDOT > 0) d[0] += (double)bi * (double)zi;
+          if constexpr (NDOT > 1) d[NDOT > 1 ? 1 : 0] += (double)zi * ring.template row<double>(4);
+        }
       }
     }
     if constexpr (CH && NDOT > 0) {
@@ -264,7 +267,7 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
 // last one on level 0 of PCG (NDOT > 0) the right-hand side and q of its dot
 // products (b, y) and (y, q), which otherwise take a pass of their own (50 us
 // on 8M rows).
-template <bool PRE, typename V, typename T, typename BT, typename YT, int NDOT>
+template <bool PRE, typename V, typename T, typename BT, typename YT, int NDOT, int SPW>
 __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
     k_sweep_ring(const __grid_constant__ SellView<V> Ah, const T* __restrict__ r,
                  T* __restrict__ r_out, YT* __restrict__ x, int first,
@@ -277,7 +280,7 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
 #pragma unroll
   for (int k = 0; k < ND; ++k) d[k] = 0.0;
   int* status = NDOT > 0 ? &sc->status : nullptr;
-  TileRing<V> ring(Ah, g, rows, ch, ring_smem);
+  TileRing<V, false, SPW> ring(Ah, g, rows, ch, ring_smem);
   const bool producer = ring.producer();
   if (producer) ring.produce(fail, status);
   while (!producer && ring.more()) {
@@ -285,26 +288,28 @@ __global__ void __launch_bounds__(RING_MAX_THREADS, RING_CTAS_PER_SM)
       if (ring.lane == 0) ring_fail(fail, status);
       break;
     }
-    {
-      T acc[1] = {T(0)};
-      ring_row_sums<false>(ring, r, acc);
-      if (ring.slot[0].has) {
-        const int64_t i = ring.slot[0].i;
-        const T ri = ring.template row<T>(1);
-        const T rn = ri - acc[0];
-        r_out[i] = rn;
-        const T si = ring.template row<T>(0);
-        if constexpr (PRE) {
-          const T xi = first ? si * to_f(ring.template row<BT>(2), T(0))
-                             : ring.template row<T>(2);
-          x[i] = sweep_pre_x(xi, si, ri);
-        } else {
-          const YT yi = sweep_post_y(ring.template row<YT>(2), si, rn);
-          x[i] = yi;
-          if constexpr (NDOT > 0) d[0] += ring.template row<double>(3) * (double)yi;
-          if constexpr (NDOT > 1)
-            d[NDOT > 1 ? 1 : 0] += (double)yi * ring.template row<double>(4);
-        }
+    T acc[SPW];
+#pragma unroll
+    for (int m = 0; m < SPW; ++m) acc[m] = T(0);
+    if (ring.slot[0].slice) ring_row_sums<false>(ring, r, acc);
+#pragma unroll
+    for (int m = 0; m < SPW; ++m) {
+      if (!ring.slot[m].has) continue;
+      const uint32_t i = ring.slot[m].i;
+      const T ri = ring.template row<T>(1, m);
+      const T rn = ri - acc[m];
+      r_out[i] = rn;
+      const T si = ring.template row<T>(0, m);
+      if constexpr (PRE) {
+        const T xi = first ? si * to_f(ring.template row<BT>(2, m), T(0))
+                           : ring.template row<T>(2, m);
+        x[i] = sweep_pre_x(xi, si, ri);
+      } else {
+        const YT yi = sweep_post_y(ring.template row<YT>(2, m), si, rn);
+        x[i] = yi;
+        if constexpr (NDOT > 0) d[0] += ring.template row<double>(3, m) * (double)yi;
+        if constexpr (NDOT > 1)
+          d[NDOT > 1 ? 1 : 0] += (double)yi * ring.template row<double>(4, m);
       }
     }
     ring.release();
@@ -985,15 +990,21 @@ static int launch_sweep(const amg_handle* H, const Level& L, const BT* b, const 
           constexpr int ND = decltype(nd)::value;
           if (ND > 0) rows.add(sd->r0, (int)sizeof(double));
           if (ND > 1) rows.add(sd->q, (int)sizeof(double));
+          auto go = [&](auto fn, RingGeom& g) -> int {
+            AMG_TRY(ring_prepare((const void*)fn, g, ring_tiles(g, L.A), H->num_sms));
+            fn<<<g.grid, g.threads(), g.smem, s>>>(v, r, r_out, x, first, g, rows, RingChunks(),
+                                                   H->wait_fail, H->red, H->sc);
+            AMG_LAUNCH_CHECK();
+            if (ND > 0) sd->fused = true;
+            return AMG_OK;
+          };
+          if constexpr (sizeof(V) == 4) {  // two slices a warp, as k_pre_ring
+            RingGeom g2 = ring_plan(L.A, (int)sizeof(V), ring_stages(H), rows, ND > 0, false, true);
+            if (g2.D) return go(k_sweep_ring<PRE, V, T, BT, YT, ND, 2>, g2);
+          }
           RingGeom g = ring_plan(L.A, (int)sizeof(V), ring_stages(H), rows, ND > 0);
           if (!g.D) return 1;
-          const auto fn = k_sweep_ring<PRE, V, T, BT, YT, ND>;
-          AMG_TRY(ring_prepare((const void*)fn, g, ring_tiles(g, L.A), H->num_sms));
-          fn<<<g.grid, g.threads(), g.smem, s>>>(v, r, r_out, x, first, g, rows, RingChunks(),
-                                                 H->wait_fail, H->red, H->sc);
-          AMG_LAUNCH_CHECK();
-          if (ND > 0) sd->fused = true;
-          return AMG_OK;
+          return go(k_sweep_ring<PRE, V, T, BT, YT, ND, 1>, g);
         };
         int rc = 1;
         if constexpr (!PRE && sizeof(YT) == 8) {
