@@ -263,7 +263,8 @@ int pcg_solve(amg_handle* H, const double* b, double* x, const pcg_options* o, p
  * amg_vcycle_apply returns for it, bit for bit; each matrix entry is read
  * once for all columns.  The first call for a given nrhs allocates the
  * handle's multi-RHS workspace.  Needs a hierarchy of at least two levels
- * built by amg_setup (AMG_ERR_UNSUPPORTED otherwise).  Asynchronous.
+ * built by amg_setup, without smooth_prolongator and with coarse_solver 0
+ * (AMG_ERR_UNSUPPORTED otherwise).  Asynchronous.
  */
 int amg_vcycle_apply_multi(amg_handle* H, int nrhs, const double* R, double* Z,
                            amg_stream_t stream);
@@ -274,7 +275,9 @@ int amg_vcycle_apply_multi(amg_handle* H, int nrhs, const double* R, double* Z,
  * n0 x nrhs; X holds the initial guesses and receives the solutions.  Each
  * column has its own alpha, beta and stopping test; converged columns are
  * frozen.  st: host array of nrhs stats or NULL.  o->res_history and
- * o->x_history must be NULL.  Synchronous.  Returns the worst column status.
+ * o->x_history must be NULL.  Hierarchies as for amg_vcycle_apply_multi
+ * (AMG_ERR_UNSUPPORTED otherwise).  Synchronous.  Returns the worst column
+ * status.
  */
 int pcg_solve_multi(amg_handle* H, int nrhs, const double* B, double* X, const pcg_options* o,
                     pcg_stats* st, amg_stream_t stream);

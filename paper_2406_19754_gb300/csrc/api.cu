@@ -349,17 +349,25 @@ int pcg_solve(amg_handle* H, const double* b, double* x, const pcg_options* o, p
   return pcg_run(H, b, x, op, st, (cudaStream_t)stream);
 }
 
+// What the blocked V-cycle (multi.cu) runs: at least two levels of one system,
+// aggregates as prolongators, the dense coarsest factor (which a hierarchy with
+// the PCG coarsest solve does not build).
+static bool multi_supported(const amg_handle* H) {
+  return H->L.size() >= 2 && !H->L[0].A.row0 && !H->opt.smooth_prolongator &&
+         H->opt.coarse_solver == 0;
+}
+
 int amg_vcycle_apply_multi(amg_handle* H, int nrhs, const double* R, double* Z,
                            amg_stream_t stream) {
   if (!H || !R || !Z || (const double*)Z == R || nrhs < 1 || nrhs > 64) return AMG_ERR_ARG;
-  if (H->L.size() < 2 || H->L[0].A.row0 || H->opt.smooth_prolongator) return AMG_ERR_UNSUPPORTED;
+  if (!multi_supported(H)) return AMG_ERR_UNSUPPORTED;
   return vcycle_multi(H, nrhs, R, Z, (cudaStream_t)stream);
 }
 
 int pcg_solve_multi(amg_handle* H, int nrhs, const double* B, double* X, const pcg_options* o,
                     pcg_stats* st, amg_stream_t stream) {
   if (!H || !B || !X || nrhs < 1 || nrhs > 64) return AMG_ERR_ARG;
-  if (H->L.size() < 2 || H->L[0].A.row0 || H->opt.smooth_prolongator) return AMG_ERR_UNSUPPORTED;
+  if (!multi_supported(H)) return AMG_ERR_UNSUPPORTED;
   pcg_options def;
   pcg_default_options(&def);
   const pcg_options* op = o ? o : &def;

@@ -147,9 +147,11 @@ static int tg_prepare(amg_handle* H, int K, int nsamples, cudaStream_t s, amg_tg
   }
   if (!T->inner) return AMG_ERR_OOM;  // an earlier call failed here
   TgWs& w = T->w;
-  // the blocked PCG needs two levels; a one-level inner hierarchy solves
-  // exactly, one column at a time
-  const int G = T->inner->L.size() > 1 ? (nsamples < TG_GROUP ? nsamples : TG_GROUP) : 1;
+  // the blocked PCG needs two levels and the dense coarsest factor; a one-level
+  // inner hierarchy solves exactly, and one with the PCG coarsest solve by its
+  // own V-cycle, one column at a time
+  const bool blocked = T->inner->L.size() > 1 && T->inner->opt.coarse_solver == 0;
+  const int G = blocked ? (nsamples < TG_GROUP ? nsamples : TG_GROUP) : 1;
   if (w.G < G) {
     for (double** p : {&w.e, &w.a, &w.c, &w.t, &w.t2, &w.eb, &w.cb, &w.ab}) {
       ar.release(*p);
