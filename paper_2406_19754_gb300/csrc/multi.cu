@@ -1443,38 +1443,27 @@ static int m_z_and_p(const amg_handle* H, const MultiWs& W, int beta_form, doubl
   return AMG_OK;
 }
 
-// Workspace for K right-hand sides, kept in the handle (reallocated if K grows).
-static int multi_ws(amg_handle* H, int K, MultiWs** out) {
+// The workspace's buffers, whichever are there, and the workspace itself.
+static void multi_drop(amg_handle* H) {
   MultiWs* W = (MultiWs*)H->multi;
-  if (W && W->K >= K) {
-    W->K = K;
-    *out = W;
-    return AMG_OK;
-  }
-  if (W) {  // grow: drop the old buffers
-    Arena& ar = H->arena;
-    for (void* p : {(void*)W->R, (void*)W->R32, (void*)W->Z, (void*)W->P, (void*)W->Q,
-                    (void*)W->cy,
-                    (void*)W->part, (void*)W->ticket, (void*)W->sc, (void*)W->nactive})
-      ar.release(p);
-    for (size_t l = 0; l < H->L.size(); ++l) {
-      ar.release(W->lb[l]);
-      ar.release(W->lx[l]);
-      ar.release(W->lr[l]);
-    }
-    delete[] W->lb;
-    delete[] W->lx;
-    delete[] W->lr;
-    if (W->sc_host) cudaFreeHost(W->sc_host);
-    delete W;
-    H->multi = nullptr;
-  }
-  W = new MultiWs();
-  H->multi = W;
+  Arena& ar = H->arena;
+  for (void* p : {(void*)W->R, (void*)W->R32, (void*)W->Z, (void*)W->P, (void*)W->Q, (void*)W->cy,
+                  (void*)W->part, (void*)W->ticket, (void*)W->sc, (void*)W->nactive})
+    ar.release(p);
+  for (void** v : {W->lb, W->lx, W->lr})
+    for (size_t l = 0; v && l < H->L.size(); ++l) ar.release(v[l]);
+  multi_free(H);
+}
+
+static int multi_alloc(amg_handle* H, MultiWs* W, int K) {
   W->K = K;
   Arena& ar = H->arena;
   const int64_t n = H->L[0].n;
   const size_t vb = H->opt.precision == AMG_PREC_F32 ? 4 : 8;
+  const size_t nl = H->L.size();
+  W->lb = new void*[nl]();
+  W->lx = new void*[nl]();
+  W->lr = new void*[nl]();
   AMG_TRY(ar.alloc_n(&W->R, n * K));
   if (H->opt.precision == AMG_PREC_F32 && H->L.size() > 1) AMG_TRY(ar.alloc_n(&W->R32, n * K));
   AMG_TRY(ar.alloc_n(&W->Z, n * K));
@@ -1487,15 +1476,29 @@ static int multi_ws(amg_handle* H, int K, MultiWs** out) {
   AMG_TRY(ar.alloc_n(&W->nactive, 1));
   AMG_CUDA_TRY(cudaMemset(W->ticket, 0, sizeof(unsigned)));
   AMG_CUDA_TRY(cudaMallocHost((void**)&W->sc_host, sizeof(Scal) * K));
-  const size_t nl = H->L.size();
-  W->lb = new void*[nl]();
-  W->lx = new void*[nl]();
-  W->lr = new void*[nl]();
   for (size_t l = 0; l < nl; ++l) {
     const size_t bytes = vb * (size_t)H->L[l].n * K;
     AMG_TRY(ar.alloc(&W->lb[l], bytes));
     AMG_TRY(ar.alloc(&W->lx[l], bytes));
     AMG_TRY(ar.alloc(&W->lr[l], bytes));
+  }
+  return AMG_OK;
+}
+
+// Workspace for K right-hand sides, kept in the handle (reallocated if K grows).
+static int multi_ws(amg_handle* H, int K, MultiWs** out) {
+  MultiWs* W = (MultiWs*)H->multi;
+  if (W && W->K >= K) {
+    W->K = K;
+    *out = W;
+    return AMG_OK;
+  }
+  if (W) multi_drop(H);  // grow
+  H->multi = W = new MultiWs();
+  const int rc = multi_alloc(H, W, K);
+  if (rc < 0) {  // a later call starts over
+    multi_drop(H);
+    return rc;
   }
   *out = W;
   return AMG_OK;
