@@ -21,7 +21,8 @@ namespace amg {
 constexpr int MROWS_BLOCK = 256;  // 8 warps = 8 rows in flight per block
 
 struct MultiWs {
-  int K = 0;
+  int K = 0;    // columns of the running call
+  int cap = 0;  // columns the buffers hold
   double *R = nullptr, *Z = nullptr, *P = nullptr, *Q = nullptr;  // N x K
   float* R32 = nullptr;  // FP32 copy of R for an FP32 V-cycle (else null)
   void** lb = nullptr;  // per level b, x, r (V-cycle type), host arrays of pointers
@@ -1456,7 +1457,7 @@ static void multi_drop(amg_handle* H) {
 }
 
 static int multi_alloc(amg_handle* H, MultiWs* W, int K) {
-  W->K = K;
+  W->K = W->cap = K;
   Arena& ar = H->arena;
   const int64_t n = H->L[0].n;
   const size_t vb = H->opt.precision == AMG_PREC_F32 ? 4 : 8;
@@ -1485,10 +1486,11 @@ static int multi_alloc(amg_handle* H, MultiWs* W, int K) {
   return AMG_OK;
 }
 
-// Workspace for K right-hand sides, kept in the handle (reallocated if K grows).
+// Workspace for K right-hand sides, kept in the handle and reallocated when K
+// exceeds every earlier one.
 static int multi_ws(amg_handle* H, int K, MultiWs** out) {
   MultiWs* W = (MultiWs*)H->multi;
-  if (W && W->K >= K) {
+  if (W && W->cap >= K) {
     W->K = K;
     *out = W;
     return AMG_OK;

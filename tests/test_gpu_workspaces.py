@@ -41,3 +41,15 @@ def test_multi_workspace_survives_a_failed_allocation(amg, precision):
     assert k >= 9  # vectors, partial sums, scalars, then three vectors a level
     assert torch.equal(H.pcg_multi(few)[0], want[0])
     assert torch.equal(H.pcg_multi(many)[0], want[1])
+
+
+def test_multi_workspace_keeps_its_capacity(amg):
+    # a call with fewer columns in between: the buffers of the larger one stay
+    n = 9 * 8 * 7
+    H = amg.Hierarchy(*amg.csr_to_device(poisson3d(9, 8, 7)), max_coarse=40)
+    B = torch.as_tensor(uniform01(53, n * 8), device="cuda").reshape(n, 8)
+    x = H.pcg_multi(B)[0]
+    H.pcg_multi(B[:, :3].contiguous())
+    out = []
+    assert not _fails_at(amg, 0, lambda: out.append(H.pcg_multi(B)[0]))
+    assert torch.equal(out[0], x)
