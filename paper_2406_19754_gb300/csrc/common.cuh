@@ -781,6 +781,8 @@ int pcg_run(amg_handle* H, const double* b, double* x, const pcg_options* o, pcg
 int vcycle_multi(amg_handle* H, int K, const double* R, double* Z, cudaStream_t s);
 int pcg_multi_run(amg_handle* H, int K, const double* B, double* X, const pcg_options* o,
                   pcg_stats* st, cudaStream_t s);
+// The workspace of pcg_multi_run for up to K columns, ahead of the calls.
+int multi_reserve(amg_handle* H, int K);
 void multi_free(amg_handle* H);
 
 // Two-grid loss for the learned smoother (twogrid.cu)

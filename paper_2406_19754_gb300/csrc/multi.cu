@@ -1506,6 +1506,11 @@ static int multi_ws(amg_handle* H, int K, MultiWs** out) {
   return AMG_OK;
 }
 
+int multi_reserve(amg_handle* H, int K) {
+  MultiWs* W = (MultiWs*)H->multi;
+  return W && W->cap >= K ? AMG_OK : multi_ws(H, K, &W);
+}
+
 void multi_free(amg_handle* H) {
   MultiWs* W = (MultiWs*)H->multi;
   if (!W) return;

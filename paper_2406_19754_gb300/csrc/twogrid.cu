@@ -126,57 +126,87 @@ void tg_free(amg_handle* H) {
   H->tg = nullptr;
 }
 
-static int tg_prepare(amg_handle* H, int K, int nsamples, cudaStream_t s, amg_tg** out) {
-  amg_tg* T = (amg_tg*)H->tg;
+// The inner solver and the vectors that do not depend on the group.
+static int tg_create(amg_handle* H, cudaStream_t s) {
   Arena& ar = H->arena;
-  if (!T) {
-    T = new amg_tg();
-    H->tg = T;
-    const Level& L1 = H->L[1];
-    amg_csr A1{L1.n, L1.nnz, L1.rowptr, L1.col, L1.val};
-    amg_options o = H->opt;
-    o.precision = AMG_PREC_F64;
-    o.autotune = 0;
-    AMG_TRY(amg_setup(&A1, &o, (amg_stream_t)s, &T->inner));
-    TgWs& w = T->w;
-    w.n = H->L[0].n;
-    w.nc = L1.n;
-    AMG_TRY(ar.alloc_n(&w.sbar, w.n));
-    AMG_TRY(ar.alloc_n(&w.dots, 2 * TG_GROUP));
-    AMG_CUDA_TRY(cudaMallocHost((void**)&w.dots_host, 2 * TG_GROUP * sizeof(double)));
+  amg_tg* T = new amg_tg();
+  H->tg = T;
+  TgWs& w = T->w;
+  const Level& L1 = H->L[1];
+  amg_csr A1{L1.n, L1.nnz, L1.rowptr, L1.col, L1.val};
+  amg_options o = H->opt;
+  o.precision = AMG_PREC_F64;
+  o.autotune = 0;
+  AMG_TRY(amg_setup(&A1, &o, (amg_stream_t)s, &T->inner));
+  w.n = H->L[0].n;
+  w.nc = L1.n;
+  AMG_TRY(ar.alloc_n(&w.sbar, w.n));
+  AMG_TRY(ar.alloc_n(&w.dots, 2 * TG_GROUP));
+  AMG_CUDA_TRY(cudaMallocHost((void**)&w.dots_host, 2 * TG_GROUP * sizeof(double)));
+  return AMG_OK;
+}
+
+// Releases the group's vectors (no group is then prepared).
+static void tg_drop_group(Arena& ar, TgWs& w) {
+  w.G = w.K = 0;
+  for (double** p : {&w.e, &w.a, &w.c, &w.t, &w.t2, &w.eb, &w.cb, &w.ab, &w.g, &w.y}) {
+    ar.release(*p);
+    *p = nullptr;
   }
-  if (!T->inner) return AMG_ERR_OOM;  // an earlier call failed here
+  for (auto* v : {&w.Ae, &w.Ac}) {
+    for (double* p : *v) ar.release(p);
+    v->clear();
+  }
+}
+
+// Vectors for groups of G samples and K cycles; G and K are stored once every
+// allocation has succeeded.
+static int tg_alloc_group(Arena& ar, TgWs& w, int G, int K) {
+  for (double** p : {&w.e, &w.a, &w.c, &w.t, &w.t2, &w.eb, &w.cb, &w.ab})
+    AMG_TRY(ar.alloc_n(p, w.n * G));
+  for (double** p : {&w.g, &w.y}) AMG_TRY(ar.alloc_n(p, w.nc * G));
+  for (auto* v : {&w.Ae, &w.Ac}) {
+    v->assign(K, nullptr);
+    for (double*& p : *v) AMG_TRY(ar.alloc_n(&p, w.n * G));
+  }
+  w.G = G;
+  w.K = K;
+  return AMG_OK;
+}
+
+static int tg_prepare(amg_handle* H, int K, int nsamples, cudaStream_t s, amg_tg** out) {
+  Arena& ar = H->arena;
+  if (!H->tg) {
+    const int rc = tg_create(H, s);
+    if (rc < 0) {  // a later call starts over
+      TgWs& w = ((amg_tg*)H->tg)->w;
+      ar.release(w.sbar);
+      ar.release(w.dots);
+      tg_free(H);
+      return rc;
+    }
+  }
+  amg_tg* T = (amg_tg*)H->tg;
   TgWs& w = T->w;
   // the blocked PCG needs two levels and the dense coarsest factor; a one-level
   // inner hierarchy solves exactly, and one with the PCG coarsest solve by its
   // own V-cycle, one column at a time
   const bool blocked = T->inner->L.size() > 1 && T->inner->opt.coarse_solver == 0;
   const int G = blocked ? (nsamples < TG_GROUP ? nsamples : TG_GROUP) : 1;
-  if (w.G < G) {
-    for (double** p : {&w.e, &w.a, &w.c, &w.t, &w.t2, &w.eb, &w.cb, &w.ab}) {
-      ar.release(*p);
-      *p = nullptr;
-      AMG_TRY(ar.alloc_n(p, w.n * G));
+  if (w.G < G || w.K < K) {
+    // a group of G holds up to eight times one sample's vectors: where they do
+    // not fit, smaller groups do
+    const int k = K > w.K ? K : w.K;
+    int rc = AMG_ERR_OOM;
+    for (int q = G > w.G ? G : w.G; q >= 1 && rc == AMG_ERR_OOM; q /= 2) {
+      tg_drop_group(ar, w);
+      rc = tg_alloc_group(ar, w, q, k);
+      if (rc == AMG_OK && q > 1) rc = multi_reserve(T->inner, q);
     }
-    for (double** p : {&w.g, &w.y}) {
-      ar.release(*p);
-      *p = nullptr;
-      AMG_TRY(ar.alloc_n(p, w.nc * G));
+    if (rc < 0) {
+      tg_drop_group(ar, w);
+      return rc;
     }
-    for (auto* v : {&w.Ae, &w.Ac}) {
-      for (double* p : *v) ar.release(p);
-      v->clear();
-    }
-    w.K = 0;
-    w.G = G;
-  }
-  while (w.K < K) {
-    double *p = nullptr, *q = nullptr;
-    AMG_TRY(ar.alloc_n(&p, w.n * w.G));
-    AMG_TRY(ar.alloc_n(&q, w.n * w.G));
-    w.Ae.push_back(p);
-    w.Ac.push_back(q);
-    ++w.K;
   }
   *out = T;
   return AMG_OK;

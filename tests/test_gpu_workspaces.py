@@ -4,7 +4,7 @@ one grows leaves the handle usable, for fewer columns or samples and for as many
 import pytest
 import torch
 
-from synthetic import poisson3d, uniform01
+from synthetic import poisson3d, standard_normal, uniform01
 
 pytestmark = pytest.mark.gpu
 
@@ -53,3 +53,31 @@ def test_multi_workspace_keeps_its_capacity(amg):
     out = []
     assert not _fails_at(amg, 0, lambda: out.append(H.pcg_multi(B)[0]))
     assert torch.equal(out[0], x)
+
+
+def test_twogrid_workspace_survives_a_failed_allocation(amg):
+    from paper_2406_19754_gb300 import learned
+
+    n = 12 * 11 * 10
+    A = amg.csr_to_device(poisson3d(12, 11, 10))
+    e0 = torch.as_tensor(standard_normal(54, 9 * n).reshape(9, n), device="cuda")
+    ref = amg.Hierarchy(*A, max_coarse=20)
+    want = {k: learned.twogrid_loss(ref, e0[:k], 2)[0] for k in (2, 9)}
+
+    def check(H, k):  # in groups of any size: inner solves to 1e-12
+        loss = learned.twogrid_loss(H, e0[:k], 2)[0]
+        assert abs(loss - want[k]) <= 1e-9 * abs(want[k])
+
+    # the inner hierarchy's set-up fails: the call ends, a later one starts over
+    H = amg.Hierarchy(*A, max_coarse=20)
+    for k in (0, 3, 40):
+        assert _fails_at(amg, k, lambda: check(H, 9))
+    check(H, 2)
+    # the growth to groups of eight fails at each of its allocations (ten vectors,
+    # two a cycle, the blocked workspace): a smaller group takes over
+    for k in range(36):
+        H = amg.Hierarchy(*A, max_coarse=20)
+        check(H, 2)
+        assert not _fails_at(amg, k, lambda: check(H, 9))
+        check(H, 2)
+        check(H, 9)
