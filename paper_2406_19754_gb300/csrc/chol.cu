@@ -195,26 +195,32 @@ __global__ void __launch_bounds__(TILE_THREADS)
 
 }  // namespace
 
+// Launches of up to this many diagonal blocks: gridDim.y ends there.
+constexpr int CHOL_GRID_BLOCKS = 65535;
+
 // Factors nblk diagonal blocks (block b: rows brow[b] .. brow[b+1], matrices
 // at bmat[b]; device arrays), the largest of `largest` rows.  Asynchronous;
 // a pivot <= 0 puts AMG_ERR_NOT_SPD into *status.
 int chol_blocks(int nblk, int64_t largest, const int64_t* brow, const int64_t* bmat,
                 double* dense, double* Linv, double* LinvT, int* status, int num_sms,
                 cudaStream_t s) {
-  k_inverse_init<<<dim3(grid_for(largest * largest, 256, num_sms, 8), nblk), 256, 0, s>>>(
-      brow, bmat, Linv, LinvT);
-  AMG_LAUNCH_CHECK();
   const unsigned pg = (unsigned)((largest + PANEL_THREADS - 1) / PANEL_THREADS);
-  for (int64_t kb = 0; kb < largest; kb += NB) {
-    k_chol_panel<<<dim3(pg, nblk), PANEL_THREADS, 0, s>>>(brow, bmat, dense, Linv, LinvT, kb,
+  for (; nblk > 0; nblk -= CHOL_GRID_BLOCKS, brow += CHOL_GRID_BLOCKS, bmat += CHOL_GRID_BLOCKS) {
+    const unsigned nb = (unsigned)(nblk < CHOL_GRID_BLOCKS ? nblk : CHOL_GRID_BLOCKS);
+    k_inverse_init<<<dim3(grid_for(largest * largest, 256, num_sms, 8), nb), 256, 0, s>>>(
+        brow, bmat, Linv, LinvT);
+    AMG_LAUNCH_CHECK();
+    for (int64_t kb = 0; kb < largest; kb += NB) {
+      k_chol_panel<<<dim3(pg, nb), PANEL_THREADS, 0, s>>>(brow, bmat, dense, Linv, LinvT, kb,
                                                           status);
-    AMG_LAUNCH_CHECK();
-    if (kb + NB >= largest) break;
-    const int64_t rt = (largest - kb - 1) / NB;  // row tiles of the largest block
-    const int64_t tiles = rt * ((kb + NB) / NB) + rt * (rt + 1) / 2;
-    k_chol_update<<<dim3(grid_for(tiles, 1, num_sms, 8), nblk), TILE_THREADS, 0, s>>>(
-        brow, bmat, dense, Linv, LinvT, kb);
-    AMG_LAUNCH_CHECK();
+      AMG_LAUNCH_CHECK();
+      if (kb + NB >= largest) break;
+      const int64_t rt = (largest - kb - 1) / NB;  // row tiles of the largest block
+      const int64_t tiles = rt * ((kb + NB) / NB) + rt * (rt + 1) / 2;
+      k_chol_update<<<dim3(grid_for(tiles, 1, num_sms, 8), nb), TILE_THREADS, 0, s>>>(
+          brow, bmat, dense, Linv, LinvT, kb);
+      AMG_LAUNCH_CHECK();
+    }
   }
   return AMG_OK;
 }
