@@ -457,7 +457,7 @@ int amg_pairwise_match(const amg_csr* A, int32_t* mate, int* rounds, amg_stream_
   if (rc < 0) return rc;
   if (!mate) return AMG_ERR_ARG;
   Arena ar;
-  rc = match_pairwise(ar, A->n, A->nnz, A->rowptr, A->col, A->val, mate, rounds, (cudaStream_t)stream);
+  rc = match_pairwise(ar, A->n, A->rowptr, A->col, A->val, mate, rounds, (cudaStream_t)stream);
   cudaStreamSynchronize((cudaStream_t)stream);
   ar.release_all();
   return rc;

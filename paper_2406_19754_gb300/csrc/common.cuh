@@ -695,8 +695,8 @@ int match_round_loop(int64_t n, const int64_t* rowptr, const int32_t* col, const
 // Arguments of a caller's CSR matrix: AMG_ERR_ARG for null pointers or
 // sizes that cannot describe one, AMG_ERR_UNSUPPORTED beyond int32 rows.
 int check_csr(const amg_csr* A);
-int match_pairwise(Arena& ar, int64_t n, int64_t nnz, const int64_t* rowptr,
-                   const int32_t* col, const double* val, int32_t* mate, int* rounds, cudaStream_t s);
+int match_pairwise(Arena& ar, int64_t n, const int64_t* rowptr, const int32_t* col,
+                   const double* val, int32_t* mate, int* rounds, cudaStream_t s);
 int set_level0_weights(amg_handle* H, const float* omega, cudaStream_t s);
 
 // V-cycle (vcycle.cu).  dots: 0 none; 1 (r, z); 2 (r, z) and (z, q).

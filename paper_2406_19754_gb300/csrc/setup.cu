@@ -280,9 +280,22 @@ int match_round_loop(int64_t n, const int64_t* rowptr, const int32_t* col, const
   return rc;
 }
 
+// Entries that a caller's matrix stores.  Its nnz field need not say so (nothing
+// else here writes by it), and the edge weights take one place an entry.
+static int stored_entries(int64_t n, const int64_t* rowptr, int64_t* nnz, cudaStream_t s) {
+  int64_t b = 0, e = 0;
+  AMG_CUDA_TRY(cudaMemcpyAsync(&b, rowptr, sizeof(b), cudaMemcpyDeviceToHost, s));
+  AMG_CUDA_TRY(cudaMemcpyAsync(&e, rowptr + n, sizeof(e), cudaMemcpyDeviceToHost, s));
+  AMG_CUDA_TRY(cudaStreamSynchronize(s));
+  if (e < b) return AMG_ERR_ARG;
+  *nnz = e - b;
+  return AMG_OK;
+}
+
+// nnz: the entries stored between rowptr[0] and rowptr[n].
 static int match_rounds(Arena& ar, int64_t n, int64_t nnz, const int64_t* rowptr,
-                        const int32_t* col, const double* val, const double* diag, int32_t* mate, int* rounds_out,
-                        int num_sms, cudaStream_t s) {
+                        const int32_t* col, const double* val, const double* diag,
+                        int32_t* mate, int* rounds_out, int num_sms, cudaStream_t s) {
   int32_t *cand = nullptr, *flag = nullptr, *wl = nullptr;
   int* cnt = nullptr;  // [0], [1]: frontier sizes; [2]: rounds with a non-empty frontier
   AMG_TRY(ar.alloc_n(&cand, n));
@@ -303,9 +316,11 @@ static int match_rounds(Arena& ar, int64_t n, int64_t nnz, const int64_t* rowptr
   return rc;
 }
 
-int match_pairwise(Arena& ar, int64_t n, int64_t nnz, const int64_t* rowptr,
-                   const int32_t* col, const double* val, int32_t* mate, int* rounds, cudaStream_t s) {
+int match_pairwise(Arena& ar, int64_t n, const int64_t* rowptr, const int32_t* col,
+                   const double* val, int32_t* mate, int* rounds, cudaStream_t s) {
   int dev = 0, sms = 0;
+  int64_t nnz = 0;
+  AMG_TRY(stored_entries(n, rowptr, &nnz, s));
   AMG_CUDA_TRY(cudaGetDevice(&dev));
   AMG_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   double* diag = nullptr;
@@ -1237,6 +1252,7 @@ int setup_hierarchy(amg_handle* H, const amg_csr* A, cudaStream_t s, const amg_h
     k_iota<<<g1, 256, 0, s>>>(n, comp);
     AMG_LAUNCH_CHECK();
     int64_t cn = n, nc = n, cnnz = H->L[l].nnz;
+    if (l == 0 && o.aggregation == 0) AMG_TRY(stored_entries(n, rp, &cnnz, s));
     const int64_t* crp = rp;
     const int32_t* cci = ci;
     const double* cva = va;
