@@ -302,11 +302,16 @@ static int match_rounds(Arena& ar, int64_t n, int64_t nnz, const int64_t* rowptr
   AMG_TRY(ar.alloc_n(&flag, n));
   AMG_TRY(ar.alloc_n(&wl, 2 * n));
   AMG_TRY(ar.alloc_n(&cnt, 4));
+  // every edge's weight once; where 8 bytes an entry are not to be had, the rounds
+  // compute them on every look
   double* w = nullptr;
-  AMG_TRY(ar.alloc_n(&w, nnz));
-  k_match_weights<<<grid_for(n, 256, num_sms, 8), 256, 0, s>>>(n, rowptr, col, val, diag, w);
-  AMG_LAUNCH_CHECK();
-  const int rc = match_round_loop(n, rowptr, col, val, diag, w, mate, cand, flag, wl, n, cnt,
+  int rc = ar.alloc_n(&w, nnz);
+  if (rc < 0 && rc != AMG_ERR_OOM) return rc;
+  if (w) {
+    k_match_weights<<<grid_for(n, 256, num_sms, 8), 256, 0, s>>>(n, rowptr, col, val, diag, w);
+    AMG_LAUNCH_CHECK();
+  }
+  rc = match_round_loop(n, rowptr, col, val, diag, w, mate, cand, flag, wl, n, cnt,
                                   rounds_out, num_sms, s);
   ar.release(w);
   ar.release(cand);
