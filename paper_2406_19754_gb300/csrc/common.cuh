@@ -79,6 +79,8 @@ struct Arena {
 
  private:
   void drop_kept();
+  int malloc_or_drop(void** p, size_t bytes);
+  int new_slab();
 };
 
 // ------------------------------------------------------------------ SELL

@@ -49,30 +49,38 @@ int Arena::alloc(void** p, size_t bytes) {
       pool.erase(it);
       return AMG_OK;
     }
-    if (small) {
-      if (slab_used + bytes > slab_bytes) {
-        void* s = nullptr;
-        const size_t size =
-            std::min(std::max(2 * slab_bytes, ARENA_SLAB_MIN), ARENA_SLAB_MAX);
-        const int rc = device_malloc(&s, size);
-        if (rc < 0) return rc;
-        slabs.push_back(s);
-        slab_bytes = size;
-        slab_used = 0;
-      }
+    // where no slab can be had, a block of its own
+    if (small && (slab_used + bytes <= slab_bytes || new_slab() == AMG_OK)) {
       *p = (unsigned char*)slabs.back() + slab_used;
       slab_used += bytes;
       blocks[*p] = Block{bytes, true};
       return AMG_OK;
     }
   }
+  const int rc = malloc_or_drop(p, bytes);
+  if (rc < 0) return rc;
+  blocks[*p] = Block{bytes, false};
+  return AMG_OK;
+}
+
+// cudaMalloc; what is kept may be what is missing.
+int Arena::malloc_or_drop(void** p, size_t bytes) {
   int rc = device_malloc(p, bytes);
-  if (rc == AMG_ERR_OOM && !kept.empty()) {  // what is kept may be what is missing
+  if (rc == AMG_ERR_OOM && !kept.empty()) {
     drop_kept();
     rc = device_malloc(p, bytes);
   }
+  return rc;
+}
+
+int Arena::new_slab() {
+  void* s = nullptr;
+  const size_t size = std::min(std::max(2 * slab_bytes, ARENA_SLAB_MIN), ARENA_SLAB_MAX);
+  const int rc = malloc_or_drop(&s, size);
   if (rc < 0) return rc;
-  blocks[*p] = Block{bytes, false};
+  slabs.push_back(s);
+  slab_bytes = size;
+  slab_used = 0;
   return AMG_OK;
 }
 
