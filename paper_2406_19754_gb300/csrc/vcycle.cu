@@ -1247,9 +1247,10 @@ static int vcycle_levels(const amg_handle* H, const double* r0, double* z0, int 
   // Levels lt .. coarsest run in one persistent launch (tail.cu) when the
   // handle allows it; the others get one launch per step.
   // Where they fit a cluster's shared memory they run there, and larger levels
-  // above them join the launch (not when timed per level).
+  // above them join the launch (not when timed per level).  While the barrier
+  // time-out is injected (amg_debug_tail_timeout) the launch with that barrier runs.
   const int ts = tail_start(H);
-  const int cs = ts >= 0 && !act ? ct_start(H) : -1;
+  const int cs = ts >= 0 && !act && !H->tail_debug ? ct_start(H) : -1;
   const bool cluster = cs > 0 && cs <= ts;
   const int lt = cluster && !prof ? cs : ts;
   const int ldown = lt >= 0 ? lt : nl - 1;
