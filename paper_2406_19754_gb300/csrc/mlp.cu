@@ -261,56 +261,10 @@ __device__ __forceinline__ float gelu_fast(float u) {
   return fmaf(-(ax * q), e, fmaxf(u, 0.0f));
 }
 
-// Two GELUs at once: the same operations, so the same bits, with the products
-// and FMAs as packed FP32 pairs (fma.rn.f32x2: one issue slot for both).  The
-// forward pass is bound by the issue of its 64 GELUs a row: 18 instead of 24
-// instructions a pair.
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pk(float lo, float hi) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void upk(f32x2 v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 gelu_fast2(float u0, float u1) {
-  constexpr float c = 0.3275911f * 0.70710678f, h = -0.5f * 1.44269504f;
-  const f32x2 u = pk(u0, u1), na = pk(-fabsf(u0), -fabsf(u1));
-  float d0, d1;
-  upk(fma2(pk(-c, -c), na, pk(1.0f, 1.0f)), d0, d1);
-  const f32x2 t = pk(rcp_approx(d0), rcp_approx(d1));
-  f32x2 q = fma2(pk(0.5307027145f, 0.5307027145f), t, pk(-0.7265760135f, -0.7265760135f));
-  q = fma2(q, t, pk(0.7107068705f, 0.7107068705f));
-  q = fma2(q, t, pk(-0.142248368f, -0.142248368f));
-  q = fma2(q, t, pk(0.127414796f, 0.127414796f));
-  q = mul2(t, q);
-  float e0, e1;
-  upk(mul2(u, mul2(u, pk(h, h))), e0, e1);
-  return fma2(mul2(na, q), pk(ex2_approx(e0), ex2_approx(e1)),
-              pk(fmaxf(u0, 0.0f), fmaxf(u1, 0.0f)));
-}
-
 // two floats rounded to FP16 (nearest even), lo in the low half
 __device__ __forceinline__ uint32_t pack_h2(float lo, float hi) {
   const __half2 h = __floats2half2_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&h);
-}
-
-__device__ __forceinline__ uint32_t pack_h2(f32x2 v) {
-  float lo, hi;
-  upk(v, lo, hi);
-  return pack_h2(lo, hi);
 }
 
 // d = A B + c (c is read, d written: a bias can enter as c without a copy)
@@ -335,8 +289,7 @@ __global__ void __launch_bounds__(TC_WARPS * 32, 5)
   const int g = lane >> 2, t = lane & 3;
   // B fragments: W1^T (k = feature, n = neuron; k >= 9 is zero) and W2^T
   uint32_t w1b[4][2], w2b[2][4][2];
-  float b1v[4][2], b2v[4][2];
-  f32x2 w3v[4][2];  // twice, for rows g and g + 8
+  float b1v[4][2], b2v[4][2], w3v[4][2];
   auto w1 = [&](int o, int k) { return k < NF ? params[OFF_W1 + o * NF + k] : 0.0f; };
 #pragma unroll
   for (int nt = 0; nt < 4; ++nt) {
@@ -353,8 +306,7 @@ __global__ void __launch_bounds__(TC_WARPS * 32, 5)
     for (int j = 0; j < 2; ++j) {  // this thread's accumulator columns 8 nt + 2 t + j
       b1v[nt][j] = params[OFF_B1 + 8 * nt + 2 * t + j];
       b2v[nt][j] = params[OFF_B2 + 8 * nt + 2 * t + j];
-      const float w3 = params[OFF_W3 + 8 * nt + 2 * t + j];
-      w3v[nt][j] = pk(w3, w3);
+      w3v[nt][j] = params[OFF_W3 + 8 * nt + 2 * t + j];
     }
   }
   const float b3 = params[OFF_B3];
@@ -393,10 +345,10 @@ __global__ void __launch_bounds__(TC_WARPS * 32, 5)
     for (int ks = 0; ks < 2; ++ks) {
       const float(&lo)[4] = c1[2 * ks];
       const float(&hi)[4] = c1[2 * ks + 1];
-      const uint32_t a0 = pack_h2(gelu_fast2(lo[0], lo[1]));
-      const uint32_t a1 = pack_h2(gelu_fast2(lo[2], lo[3]));
-      const uint32_t a2 = pack_h2(gelu_fast2(hi[0], hi[1]));
-      const uint32_t a3 = pack_h2(gelu_fast2(hi[2], hi[3]));
+      const uint32_t a0 = pack_h2(gelu_fast(lo[0]), gelu_fast(lo[1]));
+      const uint32_t a1 = pack_h2(gelu_fast(lo[2]), gelu_fast(lo[3]));
+      const uint32_t a2 = pack_h2(gelu_fast(hi[0]), gelu_fast(hi[1]));
+      const uint32_t a3 = pack_h2(gelu_fast(hi[2]), gelu_fast(hi[3]));
 #pragma unroll
       for (int nt = 0; nt < 4; ++nt) {
         if (ks == 0)
@@ -408,14 +360,14 @@ __global__ void __launch_bounds__(TC_WARPS * 32, 5)
       }
     }
     // z = GELU(U2) w3 + b3 per row
-    f32x2 z2 = pk(0.0f, 0.0f);  // partial z of rows g and g + 8 over this thread's columns
+    float zg = 0.0f, zg8 = 0.0f;  // partial z of rows g and g + 8 over this thread's columns
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
-      for (int j = 0; j < 2; ++j)
-        z2 = fma2(w3v[nt][j], gelu_fast2(c2[nt][j], c2[nt][2 + j]), z2);
-    float zg, zg8;
-    upk(z2, zg, zg8);
+      for (int j = 0; j < 2; ++j) {
+        zg = fmaf(w3v[nt][j], gelu_fast(c2[nt][j]), zg);
+        zg8 = fmaf(w3v[nt][j], gelu_fast(c2[nt][2 + j]), zg8);
+      }
     // the four threads of a group hold a row's 32 columns between them
 #pragma unroll
     for (int o = 1; o < 4; o <<= 1) {
