@@ -191,17 +191,8 @@ __global__ void k_match_expand(const int32_t* __restrict__ wl, const int* __rest
       const int32_t v = side == 0 ? i : m;
       for (int64_t e = rowptr[v]; e < rowptr[v + 1]; ++e) {
         const int32_t k = col[e];
-        // most neighbours are on the list already (or matched): look before the
-        // atomic; one counter update per converged group of lanes
-        if (k != v && mate[k] == -1 && *(volatile int32_t*)&flag[k] == 0 &&
-            atomicExch(&flag[k], 1) == 0) {
-          const unsigned m = __activemask();
-          const int lead = __ffs(m) - 1, lane = threadIdx.x & 31;
-          int base = 0;
-          if (lane == lead) base = atomicAdd(nwl_next, __popc(m));
-          base = __shfl_sync(m, base, lead);
-          wl_next[base + __popc(m & ((1u << lane) - 1u))] = k;
-        }
+        if (k != v && mate[k] == -1 && atomicExch(&flag[k], 1) == 0)
+          wl_next[atomicAdd(nwl_next, 1)] = k;
       }
     }
   }
