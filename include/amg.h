@@ -259,9 +259,10 @@ int pcg_solve(amg_handle* H, const double* b, double* x, const pcg_options* o, p
 /*
  * Z = B R for nrhs right-hand sides at once (Eq. amg applied column by
  * column).  R, Z: device float64, row-major n0 x nrhs (row i's nrhs values
- * contiguous), distinct.  1 <= nrhs <= 64.  Every column equals what
- * amg_vcycle_apply returns for it, bit for bit; each matrix entry is read
- * once for all columns.  The first call for a given nrhs allocates the
+ * contiguous), distinct.  1 <= nrhs <= 64.  The cycle is V(1,1) on every level
+ * (smooth_sweeps and variable_cycle are not taken up); with one sweep every
+ * column equals what amg_vcycle_apply returns for it, bit for bit.  Each matrix
+ * entry is read once for all columns.  The first call for a given nrhs allocates the
  * handle's multi-RHS workspace.  Needs a hierarchy of at least two levels
  * built by amg_setup, without smooth_prolongator and with coarse_solver 0
  * (AMG_ERR_UNSUPPORTED otherwise).  Asynchronous.
@@ -319,8 +320,9 @@ int pcg_solve_batch(amg_handle* H, const double* b, double* x, const pcg_options
  * omega = max(omega_max * sigmoid(z), 1e-3), omega_max = 1 unless set) maps
  * each row's stencil features to the l1-Jacobi damping weight omega_i, so
  * s_i = omega_i / d_i stays an A-convergent smoother and the V-cycle stays
- * SPD (Sec. 2.3, l1-Jacobi; the network itself is not in the paper).  Weights are FP32 on the device; 1409 parameters laid out as
- * W1[32][9], b1[32], W2[32][32], b2[32], W3[32], b3.
+ * SPD (Sec. 2.3, l1-Jacobi; the network itself is not in the paper).  Weights
+ * are FP32 on the device; 1409 parameters laid out as W1[32][9], b1[32],
+ * W2[32][32], b2[32], W3[32], b3.
  */
 typedef struct mlp_handle mlp_handle;
 
@@ -392,7 +394,9 @@ int mlp_adam_step(mlp_handle* M, double lr, double beta1, double beta2, double e
  * gradient: L = mean_j log(||E^K e0_j||_A / ||e0_j||_A) / K with
  * E = S (I - P A_1^-1 P^T A) S, S = I - diag(s) A (Eq. amg with two levels).
  * A_1^-1 is applied by PCG-AMG on levels >= 1 to 1e-12 (exactly when level 1
- * is the coarsest).  e0: device float64[nsamples][n0] initial errors.
+ * is the coarsest), up to eight samples at a time as the columns of
+ * pcg_solve_multi (fewer where the vectors do not fit; one with coarse_solver
+ * 1).  e0: device float64[nsamples][n0] initial errors.
  * loss: host.  domega: device float[n0] receiving dL/domega, or NULL.  Needs
  * >= 2 levels (AMG_ERR_UNSUPPORTED otherwise).  The first call builds the
  * inner solver.  Synchronous.

@@ -242,9 +242,11 @@ struct CtRows {
   } while (0)
 
 // x = L^-T (L^-1 b): row i of both factors sits in CTA i mod 16 (rows of all
-// lengths everywhere), one warp per row, summed as coarse_block_solve does.
+// lengths everywhere), one warp per row, summed as coarse_block_solve does.  Runs
+// after a wait that gave up too: its places come from P alone, and it holds a
+// cluster barrier.
 template <typename T>
-__device__ void ct_cholesky(const CtParams& P, unsigned char* sm, int rank, bool ok) {
+__device__ void ct_cholesky(const CtParams& P, unsigned char* sm, int rank) {
   const uint32_t smb = smem_addr(sm);
   const int n = P.nco, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double* full = (double*)(sm + P.o_full);
@@ -369,7 +371,8 @@ __device__ void ct_pcg(const CtParams& P, unsigned char* sm) {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(CT_THREADS, 1) k_cluster_tail(const __grid_constant__ CtParams P) {
+__global__ void __launch_bounds__(CT_THREADS, 1)
+    k_cluster_tail(const __grid_constant__ CtParams P) {
   extern __shared__ __align__(128) unsigned char sm[];
   const int rank = (int)cluster_rank();
   const uint32_t bar = smem_addr(sm) + P.o_bar;
@@ -411,7 +414,8 @@ __global__ void __launch_bounds__(CT_THREADS, 1) k_cluster_tail(const __grid_con
     cluster_barrier();
     bool c = false;
     for (int k = 2; k <= L.nu; ++k) {
-      if (ok) CT_BY_VALUE(L, R.template sweep<V>(true, c ? L.o_r2 : L.o_r, c ? L.o_r : L.o_r2, k == 2));
+      const uint32_t from = c ? L.o_r2 : L.o_r, to = c ? L.o_r : L.o_r2;
+      if (ok) CT_BY_VALUE(L, R.template sweep<V>(true, from, to, k == 2));
       cluster_barrier();
       c = !c;
     }
@@ -422,7 +426,7 @@ __global__ void __launch_bounds__(CT_THREADS, 1) k_cluster_tail(const __grid_con
   if (P.pcg == 0 || rank == 0)
     ok = __syncthreads_and(mbar_wait_bounded(bar + 8u * P.nlev, 0) && ok);
   if (P.pcg == 0)
-    ct_cholesky<T>(P, sm, rank, ok);
+    ct_cholesky<T>(P, sm, rank);
   else if (rank == 0 && ok)
     ct_pcg<T>(P, sm);
   cluster_barrier();
@@ -437,7 +441,8 @@ __global__ void __launch_bounds__(CT_THREADS, 1) k_cluster_tail(const __grid_con
       c = !c;
       for (int k = 2; k <= L.nu; ++k) {
         cluster_barrier();
-        if (ok) CT_BY_VALUE(L, R.template sweep<V>(false, c ? L.o_r2 : L.o_r, c ? L.o_r : L.o_r2, false));
+        const uint32_t from = c ? L.o_r2 : L.o_r, to = c ? L.o_r : L.o_r2;
+        if (ok) CT_BY_VALUE(L, R.template sweep<V>(false, from, to, false));
         c = !c;
       }
       if (l == 0) {

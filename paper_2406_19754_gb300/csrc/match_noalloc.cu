@@ -68,8 +68,8 @@ static int match_noalloc(const amg_csr* A, int32_t* mate, int* rounds_out, cudaS
   AMG_LAUNCH_CHECK();
   // the same round loop as amg_pairwise_match, on the static scratch (its
   // two frontiers NA_ROWS entries apart); it clears what must start at zero
-  return match_round_loop(n, A->rowptr, A->col, A->val, diag, nullptr, mate, cand, flag, wl, NA_ROWS,
-                          cnt, rounds_out, sms, s);
+  return match_round_loop(n, A->rowptr, A->col, A->val, diag, nullptr, mate, cand, flag, wl,
+                          NA_ROWS, cnt, rounds_out, sms, s);
 }
 
 }  // namespace amg

@@ -233,7 +233,8 @@ __global__ void k_p_update_x(int64_t n, double* __restrict__ p, const double* __
         st4_stream(x + i, double4_32a{xv.x + alpha * pv.x, xv.y + alpha * pv.y,
                                       xv.z + alpha * pv.z, xv.w + alpha * pv.w});
       } else {
-        const double2 x0 = __ldcs((const double2*)(x + i)), x1 = __ldcs((const double2*)(x + i + 2));
+        const double2 x0 = __ldcs((const double2*)(x + i));
+        const double2 x1 = __ldcs((const double2*)(x + i + 2));
         __stcs((double2*)(x + i), make_double2(x0.x + alpha * pv.x, x0.y + alpha * pv.y));
         __stcs((double2*)(x + i + 2), make_double2(x1.x + alpha * pv.z, x1.y + alpha * pv.w));
       }

@@ -301,7 +301,8 @@ __global__ void k_sell_fill32(int64_t n, int64_t ncols, int64_t nslices, const i
     }
   }
   __syncthreads();
-  if (tmax && threadIdx.x < 6 && tm[threadIdx.x] > 0) atomicMax(tmax + threadIdx.x, tm[threadIdx.x]);
+  if (tmax && threadIdx.x < 6 && tm[threadIdx.x] > 0)
+    atomicMax(tmax + threadIdx.x, tm[threadIdx.x]);
 }
 
 // Column compression, one thread per slice: for each ELL column k the base is

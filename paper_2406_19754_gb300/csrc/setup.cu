@@ -91,10 +91,11 @@ __device__ __forceinline__ double match_weight(double a, double di, double dj) {
 }
 
 // All edge weights once, into both rows' slots (0, never eligible, where there
-// is none); entry e's weight is w[e - rowptr[0]].  A row is re-examined whenever a neighbour is matched, and each
-// look at an edge from its larger endpoint searched the other row for the
-// stored value and divided again on the reduced-rate FP64 pipe (a 128^3
-// diffusion setup spent 7.3 ms in k_match_cand).
+// is none); entry e's weight is w[e - rowptr[0]].  A row is re-examined whenever
+// a neighbour is matched, and each look at an edge from its larger endpoint
+// searched the other row for the stored value and divided again on the
+// reduced-rate FP64 pipe (a 128^3 diffusion setup spent 7.3 ms in
+// k_match_cand).
 __global__ void k_match_weights(int64_t n, const int64_t* __restrict__ rowptr,
                                 const int32_t* __restrict__ col, const double* __restrict__ val,
                                 const double* __restrict__ diag, double* __restrict__ w) {
@@ -108,7 +109,8 @@ __global__ void k_match_weights(int64_t n, const int64_t* __restrict__ rowptr,
       double a;
       double c = 0.0;
       // the entry of the smaller row, found from either side
-      if (j != i && edge_value(rowptr, col, val, i, j, val[e], &a)) c = match_weight(a, di, diag[j]);
+      if (j != i && edge_value(rowptr, col, val, i, j, val[e], &a))
+        c = match_weight(a, di, diag[j]);
       w[e - e0] = c;
     }
   }

@@ -1018,11 +1018,13 @@ static int launch_sweep(const amg_handle* H, const Level& L, const BT* b, const 
       }
     }
     if constexpr (PRE) {
-      AMG_DISPATCH_TPR(sell_code(L.A, sizeof(V)), (k_sweep_pre<TPR, V, T, BT><<<grid, SELL_BLOCK, 0, s>>>(
-                                            v, sc, b, r, r_out, (T*)x, first)));
+      AMG_DISPATCH_TPR(sell_code(L.A, sizeof(V)),
+                       (k_sweep_pre<TPR, V, T, BT><<<grid, SELL_BLOCK, 0, s>>>(
+                           v, sc, b, r, r_out, (T*)x, first)));
     } else {
-      AMG_DISPATCH_TPR(sell_code(L.A, sizeof(V)), (k_sweep_post<TPR, V, T, YT><<<grid, SELL_BLOCK, 0, s>>>(
-                                            v, sc, r, r_out, x)));
+      AMG_DISPATCH_TPR(sell_code(L.A, sizeof(V)),
+                       (k_sweep_post<TPR, V, T, YT><<<grid, SELL_BLOCK, 0, s>>>(v, sc, r, r_out,
+                                                                                x)));
     }
     AMG_LAUNCH_CHECK();
     return AMG_OK;
@@ -1088,8 +1090,9 @@ static int launch_post_sm(const amg_handle* H, const Level& L, const BT* b, cons
     using V = decltype(vtag);
     const SellView<V> q = view<V>(L.AP, sm_vals<V>(L.AP));
     const SellView<V> p = view<V>(L.P, sm_vals<V>(L.P));
-    AMG_DISPATCH_TPR(sell_code(L.AP, sizeof(V)), (k_post_sm<TPR, V, T, BT, XT><<<grid, SELL_BLOCK, 0, s>>>(
-                                          q, p, b, sc, r, xc, in.xp, x, in.e)));
+    AMG_DISPATCH_TPR(sell_code(L.AP, sizeof(V)),
+                     (k_post_sm<TPR, V, T, BT, XT><<<grid, SELL_BLOCK, 0, s>>>(
+                         q, p, b, sc, r, xc, in.xp, x, in.e)));
     AMG_LAUNCH_CHECK();
     return AMG_OK;
   };
