@@ -118,10 +118,13 @@ static void destroy(amg_handle* H) {
 }
 
 // Order-independent fingerprint of a CSR sparsity pattern: the wrapping sum
-// of splitmix64 hashes of (row, row pointer) and (position, column).
+// of splitmix64 hashes of (row, row pointer) and (position, column).  out[1]:
+// the entries between the first and last row pointer (a caller's nnz field need
+// not say so).
 __global__ void k_pattern_hash(int64_t n, const int64_t* rowptr, const int32_t* col,
                                unsigned long long* out) {
   const int64_t nnz = rowptr[n] - rowptr[0];
+  if (blockIdx.x == 0 && threadIdx.x == 0) out[1] = (unsigned long long)nnz;
   unsigned long long h = 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= n + nnz;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -135,18 +138,21 @@ __global__ void k_pattern_hash(int64_t n, const int64_t* rowptr, const int32_t* 
   if ((threadIdx.x & 31) == 0) atomicAdd(out, h);
 }
 
-static int pattern_hash(const amg_csr* A, unsigned long long* h, cudaStream_t s, int num_sms) {
-  unsigned long long* d = nullptr;
-  AMG_CUDA_TRY(cudaMallocAsync((void**)&d, sizeof(*d), s));
-  AMG_CUDA_TRY(cudaMemsetAsync(d, 0, sizeof(*d), s));
+static int pattern_hash(const amg_csr* A, unsigned long long* h, int64_t* entries,
+                        cudaStream_t s, int num_sms) {
+  unsigned long long *d = nullptr, out[2] = {0, 0};
+  AMG_CUDA_TRY(cudaMallocAsync((void**)&d, sizeof(out), s));
+  AMG_CUDA_TRY(cudaMemsetAsync(d, 0, sizeof(out), s));
   k_pattern_hash<<<grid_for(A->n + A->nnz + 1, 256, num_sms, 4), 256, 0, s>>>(A->n, A->rowptr,
                                                                                A->col, d);
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h, d, sizeof(*h), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(out, d, sizeof(out), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   cudaFreeAsync(d, s);
   AMG_CUDA_TRY(e);
-  return AMG_OK;
+  *h = out[0];
+  *entries = (int64_t)out[1];
+  return *entries < 0 ? AMG_ERR_ARG : AMG_OK;
 }
 
 static int create(const amg_csr* A, const amg_options* opt, cudaStream_t s, amg_handle** out,
@@ -192,7 +198,8 @@ static int create(const amg_csr* A, const amg_options* opt, cudaStream_t s, amg_
   AMG_CUDA_TRY(cudaMemsetAsync(H->red.ticket, 0, sizeof(unsigned), s));
   AMG_TRY(ar.alloc_n(&H->sc, 1));
   AMG_CUDA_TRY(cudaMemsetAsync(H->sc, 0, sizeof(PcgScalars), s));
-  if (!systems) AMG_TRY(pattern_hash(A, &H->pattern, s, H->num_sms));
+  H->entries = A->nnz;
+  if (!systems) AMG_TRY(pattern_hash(A, &H->pattern, &H->entries, s, H->num_sms));
   ar.begin_reuse();
   AMG_TRY(setup_hierarchy(H, A, s, like));  // on error the caller destroys H
   AMG_CUDA_TRY(cudaStreamSynchronize(s));
@@ -245,7 +252,8 @@ int amg_update_values(amg_handle* H, const amg_csr* A, amg_stream_t stream) {
   if (A->n != H->L[0].n || A->nnz != H->L[0].nnz) return AMG_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   unsigned long long h = 0;
-  rc = pattern_hash(A, &h, s, H->num_sms);
+  int64_t entries = 0;
+  rc = pattern_hash(A, &h, &entries, s, H->num_sms);
   if (rc < 0) return rc;
   if (h != H->pattern) return AMG_ERR_ARG;
   amg_handle* T = nullptr;

@@ -382,6 +382,7 @@ struct amg_handle {
   int tail_grid = 0;
   int tail_debug = 0;  // amg_debug_tail_timeout
   unsigned long long pattern = 0;  // fingerprint of the level-0 sparsity (value updates)
+  int64_t entries = 0;  // level 0's, by its row pointers (set-up)
 };
 
 namespace amg {

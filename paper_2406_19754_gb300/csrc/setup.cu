@@ -1249,8 +1249,7 @@ int setup_hierarchy(amg_handle* H, const amg_csr* A, cudaStream_t s, const amg_h
     AMG_TRY(ar.alloc_n(&comp, n));
     k_iota<<<g1, 256, 0, s>>>(n, comp);
     AMG_LAUNCH_CHECK();
-    int64_t cn = n, nc = n, cnnz = H->L[l].nnz;
-    if (l == 0 && o.aggregation == 0) AMG_TRY(stored_entries(n, rp, &cnnz, s));
+    int64_t cn = n, nc = n, cnnz = l == 0 ? H->entries : H->L[l].nnz;
     const int64_t* crp = rp;
     const int32_t* cci = ci;
     const double* cva = va;
