@@ -524,15 +524,6 @@ __device__ __forceinline__ int next_pow2(int x) {
   return p;
 }
 
-// Entry t sorts before entry p: by key, equal keys (a row that stores a column
-// more than once) by place, so that every entry has a rank of its own.
-__device__ __forceinline__ bool grank_before(const ulonglong2& kt, int t, const ulonglong2& kp,
-                                             int p) {
-  if (kt.x != kp.x) return kt.x < kp.x;
-  if (kt.y != kp.y) return kt.y < kp.y;
-  return t < p;
-}
-
 // Rows of at most GAL_SMALL contributions, one warp each; the others are
 // listed for k_galerkin_warp (count pass) or skipped (fill pass).
 template <bool FILL>
@@ -598,7 +589,10 @@ __global__ void __launch_bounds__(GAL_SMALL_WARPS * 32) k_galerkin_small(GalArgs
         if constexpr (FILL) {
           v[u] = g.val[e];
           k[u].x = ((uint64_t)(uint32_t)J[u] << 32) | (uint32_t)min(row, j);
-          k[u].y = ((uint64_t)(uint32_t)max(row, j) << 1) | (uint64_t)(row > j ? 1 : 0);
+          // with the place last: a row that stores a column more than once gives
+          // equal keys, and every entry needs a rank of its own
+          k[u].y = (((uint64_t)(uint32_t)max(row, j) << 1) | (uint64_t)(row > j ? 1 : 0)) *
+                       GAL_SMALL + (uint64_t)p;
         }
       }
     }
@@ -625,8 +619,8 @@ __global__ void __launch_bounds__(GAL_SMALL_WARPS * 32) k_galerkin_small(GalArgs
       int r0 = 0, r1 = 0;
       for (int t = 0; t < total; ++t) {
         const ulonglong2 kt = key[t];
-        r0 += grank_before(kt, t, k[0], lane) ? 1 : 0;
-        r1 += grank_before(kt, t, k[1], lane + 32) ? 1 : 0;
+        r0 += gless(kt.x, kt.y, k[0].x, k[0].y) ? 1 : 0;
+        r1 += gless(kt.x, kt.y, k[1].x, k[1].y) ? 1 : 0;
       }
       if (J[0] >= 0) {
         sv[r0] = v[0];
