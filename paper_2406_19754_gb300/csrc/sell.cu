@@ -368,9 +368,17 @@ static int sell_from_csr32(Arena& ar, const int64_t* rowptr, const int32_t* col,
   AMG_TRY(ar.alloc_n(&out.col, out.nnz_pad));
   AMG_TRY(ar.alloc_n(&out.v64, out.nnz_pad));
   if (ring) {
-    AMG_TRY(ar.alloc_n(&out.rec, out.nslices + 1));
     out.ix_bytes = (total & 0xffffffffll) << 4;
-    AMG_TRY(ar.alloc_n(&out.ix, out.ix_bytes));
+    int rc = ar.alloc_n(&out.rec, out.nslices + 1);
+    if (rc == AMG_OK) rc = ar.alloc_n(&out.ix, out.ix_bytes);
+    if (rc == AMG_ERR_OOM) {  // up to 4 bytes an entry beside the plain columns: do without
+      ar.release(out.rec);
+      out.rec = nullptr;
+      out.ix_bytes = 0;
+      ring = false;
+    } else if (rc < 0) {
+      return rc;
+    }
   }
   k_sell_fill32<<<g, 256, 0, s>>>(out.n, out.ncols, out.nslices, out.row0, rowptr, col, val, pk,
                                   total, layout, out.sliceptr, out.col, out.v64, out.rec,
