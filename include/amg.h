@@ -394,9 +394,9 @@ int mlp_adam_step(mlp_handle* M, double lr, double beta1, double beta2, double e
  * gradient: L = mean_j log(||E^K e0_j||_A / ||e0_j||_A) / K with
  * E = S (I - P A_1^-1 P^T A) S, S = I - diag(s) A (Eq. amg with two levels).
  * A_1^-1 is applied by PCG-AMG on levels >= 1 to 1e-12 (exactly when level 1
- * is the coarsest), up to eight samples at a time as the columns of
- * pcg_solve_multi (fewer where the vectors do not fit; one with coarse_solver
- * 1).  e0: device float64[nsamples][n0] initial errors.
+ * is the coarsest), four, six or eight samples at a time as the columns of
+ * pcg_solve_multi, or one (fewer than four left, vectors that do not fit,
+ * coarse_solver 1).  e0: device float64[nsamples][n0] initial errors.
  * loss: host.  domega: device float[n0] receiving dL/domega, or NULL.  Needs
  * >= 2 levels (AMG_ERR_UNSUPPORTED otherwise).  The first call builds the
  * inner solver.  Synchronous.

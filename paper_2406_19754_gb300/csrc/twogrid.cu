@@ -13,8 +13,8 @@
 // (I - P A_c^-1 P^T A)^T = I - A P A_c^-1 P^T, run in reverse order over the
 // stored forward states, with d(S x)_i / d s_i = -(A x)_i.  All FP64.
 //
-// Samples run in lockstep, up to TG_GROUP at a time, so each coarse solve is
-// one blocked PCG over the group's right-hand sides (columns): the inner
+// Samples run in lockstep, up to TG_GROUP at a time (tg_group), so each coarse
+// solve is one blocked PCG over the group's right-hand sides (columns): the inner
 // hierarchy's levels are small (27,648 rows below a 48^3 problem) and an
 // iteration is bound by its launches, whatever the number of columns.  One
 // sample at a time, a 48^3 training step of 4 samples and 2 cycles ran 540
@@ -95,6 +95,17 @@ __global__ void k_tg_dot(int64_t n, const double* __restrict__ x, const double* 
 }
 
 constexpr int TG_GROUP = 8;
+
+// Samples of the next group when `left` are left: an even number from four to
+// TG_GROUP, else one, solved by itself.  The blocked solve of an odd number of
+// columns takes its per-column kernels, and two columns cost it nearly as much as
+// eight, while the single solve runs its loop on the device.  Two cycles of 24^3
+// and 80^3 diffusion problems: one sample 5.6 and 22 ms; blocked 2 samples 18 and
+// 77, 3 samples 65 and 373, 4 samples 16 and 80, 8 samples 16 and 95.
+static int tg_group(int left, int most) {
+  const int m = (left < most ? left : most) & ~1;
+  return m >= 4 ? m : 1;
+}
 
 // Work vectors of a group of G samples: each entry of e .. ab, Ae[k], Ac[k]
 // holds G fine vectors one after the other; g and y are nc x G row-major.
@@ -192,13 +203,14 @@ static int tg_prepare(amg_handle* H, int K, int nsamples, cudaStream_t s, amg_tg
   // inner hierarchy solves exactly, and one with the PCG coarsest solve by its
   // own V-cycle, one column at a time
   const bool blocked = T->inner->L.size() > 1 && T->inner->opt.coarse_solver == 0;
-  const int G = blocked ? (nsamples < TG_GROUP ? nsamples : TG_GROUP) : 1;
+  const int G = blocked ? tg_group(nsamples, TG_GROUP) : 1;
   if (w.G < G || w.K < K) {
     // a group of G holds up to eight times one sample's vectors: where they do
     // not fit, smaller groups do
     const int k = K > w.K ? K : w.K;
     int rc = AMG_ERR_OOM;
-    for (int q = G > w.G ? G : w.G; q >= 1 && rc == AMG_ERR_OOM; q /= 2) {
+    for (int q = G > w.G ? G : w.G; q >= 1 && rc == AMG_ERR_OOM;
+         q = q > 1 ? tg_group(q / 2, TG_GROUP) : 0) {
       tg_drop_group(ar, w);
       rc = tg_alloc_group(ar, w, q, k);
       if (rc == AMG_OK && q > 1) rc = multi_reserve(T->inner, q);
@@ -271,7 +283,7 @@ int twogrid_loss(amg_handle* H, int nsamples, int K, const double* e0, double* l
   AMG_CUDA_TRY(cudaMemsetAsync(w.sbar, 0, sizeof(double) * n, s));
   double total = 0.0;
   for (int j0 = 0; j0 < nsamples; j0 += m) {
-    m = nsamples - j0 < w.G ? nsamples - j0 : w.G;
+    m = tg_group(nsamples - j0, w.G);
     AMG_CUDA_TRY(cudaMemcpyAsync(w.e, e0 + (int64_t)j0 * n, sizeof(double) * n * m,
                                  cudaMemcpyDeviceToDevice, s));
     for (int q = 0; q < m; ++q) {
