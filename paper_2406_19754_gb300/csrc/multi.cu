@@ -482,7 +482,7 @@ __global__ void __launch_bounds__(MROWS_BLOCK, MV_BLOCKS)
       XT zv[KPL];
       cvt_n(zt, zv);
       double zd[KPL];
-      if constexpr (DOTS) cvt_n(zt, zd);
+      if constexpr (DOTS) cvt_n(zv, zd);  // (a copy where z is FP64)
 #pragma unroll
       for (int q = 0; q < KPL; ++q) {
         const int c = lane + 32 * q;
@@ -714,7 +714,7 @@ __global__ void __launch_bounds__(MROWS_BLOCK, DOTS ? MV_BLOCKS_DOTS : MV_BLOCKS
         st_cols(Z + i * K + c0, zv);
         if constexpr (DOTS) {
           double zd[VW];
-          cvt_n(xv, zd);
+          cvt_n(zv, zd);
 #pragma unroll
           for (int k = 0; k < VW; ++k) {
             d[0][k] += (double)bv[k] * zd[k];
@@ -1107,23 +1107,31 @@ __global__ void k_m_p_update(int64_t n, int K, double* __restrict__ P, const ZT*
     act[q] = c < K && (FIRST || sc[c].active);
     be[q] = !FIRST && act[q] ? sc[c].beta : 0.0;
   }
-  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += nw) {
-    ZT zt[KPL];
-    double z[KPL], p[KPL], x[KPL];
-    // every load of the row before the conversions
+  // two rows a pass, every load of both before the conversions
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += 2 * nw) {
+    ZT zt[2 * KPL];
+    double z[2 * KPL], p[2 * KPL], x[2 * KPL];
 #pragma unroll
-    for (int q = 0; q < KPL; ++q) {
-      const int64_t e = i * K + lane + 32 * q;
-      zt[q] = act[q] ? Z[e] : ZT(0);
-      p[q] = !FIRST && (owed[q] || act[q]) ? P[e] : 0.0;
-      x[q] = owed[q] ? X[e] : 0.0;
-    }
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int q = 0; q < KPL; ++q) {
+        const int m = u * KPL + q;
+        const int64_t e = (i + u * nw < n ? i + u * nw : i) * K + lane + 32 * q;
+        zt[m] = act[q] ? Z[e] : ZT(0);
+        p[m] = !FIRST && (owed[q] || act[q]) ? P[e] : 0.0;
+        x[m] = owed[q] ? X[e] : 0.0;
+      }
     cvt_n(zt, z);
 #pragma unroll
-    for (int q = 0; q < KPL; ++q) {
-      const int64_t e = i * K + lane + 32 * q;
-      if (owed[q]) X[e] = x[q] + al[q] * p[q];
-      if (act[q]) P[e] = FIRST ? z[q] : z[q] + be[q] * p[q];
+    for (int u = 0; u < 2; ++u) {
+      if (i + u * nw >= n) break;
+#pragma unroll
+      for (int q = 0; q < KPL; ++q) {
+        const int m = u * KPL + q;
+        const int64_t e = (i + u * nw) * K + lane + 32 * q;
+        if (owed[q]) X[e] = x[m] + al[q] * p[m];
+        if (act[q]) P[e] = FIRST ? z[m] : z[m] + be[q] * p[m];
+      }
     }
   }
 }
@@ -1415,24 +1423,35 @@ static int mgrid_mu(const amg_handle* H, int64_t rows, int K) {
   return grid_for((rows + rw - 1) / rw * 32, MROWS_BLOCK, H->num_sms, MV_BLOCKS);
 }
 
+// Whether the p and x updates take vector columns.
+static bool m_p_vector(int K, const double* X) {
+  return K % 2 == 0 && ((uintptr_t)X & 15u) == 0;
+}
+
 template <bool FIRST, typename ZT>
 static void m_p_update(const amg_handle* H, const MultiWs& W, const ZT* Z, double* X,
                        cudaStream_t s) {
   const int64_t n = H->L[0].n;
   const int K = W.K;
-  if (K % 2 == 0 && ((uintptr_t)X & 15u) == 0)
+  if (m_p_vector(K, X))
     k_m_p_update_v<ZT, FIRST><<<mgrid_mu(H, n, K), MROWS_BLOCK, 0, s>>>(n, K, W.P, Z, X, W.sc);
   else
     AMG_DISPATCH_KPL(K, (k_m_p_update<KPL, ZT, FIRST><<<mgrid(H, n), MROWS_BLOCK, 0, s>>>(
                             n, K, W.P, Z, X, W.sc)));
 }
 
-// z of the iteration (FP32 V-cycles: FP32, in W.Z), with the dot products, then
-// p from it.
+// z of the iteration (in W.Z; FP32 V-cycles: FP32 where vector columns read it, and
+// FP64 for the per-column update, which has too few loads in flight to hide the
+// conversions), with the dot products, then p from it.  33 columns of 100^3: 162.7 ms
+// with FP32 z, 159.0 with FP64, 156.6 with two rows a pass and z converted once.
 template <bool FIRST>
 static int m_z_and_p(const amg_handle* H, const MultiWs& W, int beta_form, double* X,
                      cudaStream_t s) {
-  if (H->opt.precision == AMG_PREC_F32) {
+  const bool f32 = H->opt.precision == AMG_PREC_F32;
+  if (f32 && !m_p_vector(W.K, X)) {
+    AMG_TRY((m_vcycle<float, double>(H, W, W.R, W.Z, true, W.Q, beta_form, FIRST, s, W.R32)));
+    m_p_update<FIRST>(H, W, W.Z, X, s);
+  } else if (f32) {
     float* Z = (float*)W.Z;
     AMG_TRY((m_vcycle<float, float>(H, W, W.R, Z, true, W.Q, beta_form, FIRST, s, W.R32)));
     m_p_update<FIRST>(H, W, Z, X, s);
