@@ -85,8 +85,9 @@ __global__ void __launch_bounds__(PANEL_THREADS)
     bool bad = false;
 #pragma unroll
     for (int k = 0; k < NB; ++k) {
+      if (k >= nb) break;  // (a 2-row block takes 2 steps, not 32)
       const double piv = __shfl_sync(0xffffffffu, r[k], k);
-      if (k < nb && !(piv > 0.0)) bad = true;
+      if (!(piv > 0.0)) bad = true;
       const double lkk = sqrt(piv);
       const double l = lane == k ? lkk : __ddiv_rn(r[k], lkk);
       r[k] = l;
