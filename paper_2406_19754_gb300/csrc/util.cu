@@ -50,7 +50,7 @@ int Arena::alloc(void** p, size_t bytes) {
       return AMG_OK;
     }
     // where no slab can be had, a block of its own
-    if (small && (slab_used + bytes <= slab_bytes || new_slab() == AMG_OK)) {
+    if (small && (slab_used + bytes <= slab_bytes || new_slab(bytes) == AMG_OK)) {
       *p = (unsigned char*)slabs.back() + slab_used;
       slab_used += bytes;
       blocks[*p] = Block{bytes, true};
@@ -73,9 +73,10 @@ int Arena::malloc_or_drop(void** p, size_t bytes) {
   return rc;
 }
 
-int Arena::new_slab() {
+int Arena::new_slab(size_t least) {
   void* s = nullptr;
-  const size_t size = std::min(std::max(2 * slab_bytes, ARENA_SLAB_MIN), ARENA_SLAB_MAX);
+  const size_t size =
+      std::max(least, std::min(std::max(2 * slab_bytes, ARENA_SLAB_MIN), ARENA_SLAB_MAX));
   const int rc = malloc_or_drop(&s, size);
   if (rc < 0) return rc;
   slabs.push_back(s);

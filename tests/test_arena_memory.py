@@ -44,33 +44,40 @@ bool nothing_held();
 #define WANT(c) do if (!(c)) { printf("line %d: %s\n", __LINE__, #c); return 1; } while (0)
 
 int main() {
-  const size_t M = 1 << 20;
+  const size_t M = 1 << 20, S = amg::ARENA_SLAB_MIN;
   amg::Arena ar;
   void *a, *b, *c;
   // a kept large block makes room for a slab
-  room = 9 * M;
+  room = 8 * M + S / 2;
   ar.begin_reuse();
   WANT(ar.alloc(&a, 8 * M) == AMG_OK);
   ar.release(a);
   WANT(ar.alloc(&b, 1000) == AMG_OK);
-  WANT(room == 7 * M);
-  WANT(ar.alloc(&a, 7 * M) == AMG_OK && room == 0);
+  WANT(room == 8 * M - S / 2);
+  WANT(ar.alloc(&a, room) == AMG_OK && room == 0);
   WANT(ar.alloc(&c, 1000) == AMG_OK);  // from the same slab
   WANT(ar.alloc(&c, 3 * M) == AMG_ERR_OOM);
   ar.end_reuse();
   ar.release_all();
-  WANT(room == 9 * M && nothing_held());
+  WANT(room == 8 * M + S / 2 && nothing_held());
   // less room than a slab: a block of its own, kept and used again
-  room = M;
+  room = S / 2;
   ar.begin_reuse();
-  WANT(ar.alloc(&a, M / 2) == AMG_OK && room == M / 2);
-  WANT(ar.alloc(&b, M / 2) == AMG_OK && room == 0);
+  WANT(ar.alloc(&a, S / 4) == AMG_OK && room == S / 4);
+  WANT(ar.alloc(&b, S / 4) == AMG_OK && room == 0);
   WANT(ar.alloc(&c, 256) == AMG_ERR_OOM);
   ar.release(a);
-  WANT(ar.alloc(&c, 256) == AMG_OK && room == M / 2 - 256);  // what was kept went back
+  WANT(ar.alloc(&c, 256) == AMG_OK && room == S / 4 - 256);  // what was kept went back
   ar.end_reuse();
   ar.release_all();
-  WANT(room == M && nothing_held());
+  WANT(room == S / 2 && nothing_held());
+  // a request larger than the first slab gets one that holds it
+  room = 4 * M;
+  ar.begin_reuse();
+  WANT(ar.alloc(&a, M) == AMG_OK && room == 3 * M);
+  ar.end_reuse();
+  ar.release_all();
+  WANT(room == 4 * M && nothing_held());
   return 0;
 }
 """
